@@ -247,7 +247,9 @@ int32_t mkv_decode_attention(mkv_pool* pool, const void* q_dev, const int32_t* b
  * record format).  Every block of the persistent scan walks its share of layer 0, then of layer 1, ... without
  * waiting for the other blocks, so the table walk and query rotation of one layer and the merge of the
  * layer before overlap the page scans of their neighbours; results are those of n_layers calls of
- * mkv_decode_attention (the same kernel code per layer).
+ * mkv_decode_attention (the same kernel code per layer).  From four layers on the scan is cut once over all
+ * layers laid end to end, so that a block meets one or two rows instead of one per layer: the same sums, split
+ * at other pages (equal to fp32 rounding instead of bit for bit).
  *   layers_host  host array of n_layers entries (copied into the launch; free to reuse on return);
  *                lse_dev may be NULL; every workspace_dev as for mkv_decode_attention, distinct per layer
  *   n_layers     1 .. MKV_MAX_LAYERS_PER_CALL; MKV_E_INVALID beyond, for pools of different geometry,

@@ -76,6 +76,13 @@ struct DecodeParams {
 // layer 1, ... without waiting for the other blocks, so the start-up and the merge tail of one layer
 // overlap the page loops of its neighbours.
 constexpr int kMaxLayers = 32;
+//
+// Two cuts of the work.  Up to 3 layers: every layer is cut over the whole grid like a call of its own (results
+// are bit for bit those of single calls), and every block visits every layer.  From kMinFlatLayers layers on
+// (template parameter FLAT) the layers are laid end to end and the grid cuts the whole list once: a block then meets one or two
+// rows instead of one per layer, and pays the set-up of a row (table entries, first pages, query rotation:
+// 3 us) and its tail (reduction, partial, ticket: 3 us, warps waiting for the last one: 2 us) that much less often.
+constexpr int kMinFlatLayers = 4;
 template <int MAXL>
 struct LayerSet {
     int n;
@@ -295,7 +302,10 @@ __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (
 //   linear (many rows): grid equal ranges that may cross row boundaries.
 constexpr int kMaxAlignedRows = kMaxCtas / 4;
 
+//   flat (several layers): a linear cut of all layers' triples, the layers laid end to end.
 struct Partition {
+    long long total;                    // flat: triples of all layers
+    int flat_blocks;                    // flat: blocks that get work
     int aligned;                        // 1: row-aligned, 0: linear
     int blocks;                         // blocks that get work
     int base[kMaxAlignedRows + 1];      // row-aligned: first block of every row
@@ -369,6 +379,39 @@ __device__ __forceinline__ int partition_start(const Partition* pt, const int* c
     return s;
 }
 
+// flat cut: first triple of block c, counted over all layers
+__device__ __forceinline__ long long flat_start(const Partition* pt, int c) { return pt->total * c / pt->flat_blocks; }
+
+// block of a linear cut of W triples over C blocks that holds triple x: the last c with floor(W c / C) <= x
+__device__ __forceinline__ int linear_block_of(long long W, int C, long long x)
+{
+    int c = (int)((x * C) / W);
+    while (c + 1 < C && (W * (c + 1)) / C <= x) ++c;
+    while (c > 0 && (W * c) / C > x) --c;
+    return c;
+}
+
+// Whether position x of the row [row_start, row_end) (row index r) opens the run of some warp in the per-layer cut
+// with n_warps warps per block.
+__device__ __forceinline__ bool opens_warp_run(const Partition* pt, const int* cum, int B, int r, int row_start, int row_end,
+                                               int x, unsigned n_warps)
+{
+    int first, n;                                   // the block's share of the row
+    if (pt->aligned) {
+        const unsigned rows = row_end - row_start, k = pt->base[r + 1] - pt->base[r],
+                       j = ((unsigned)(x - row_start + 1) * k - 1) / rows;          // last j with floor(rows j / k) <= x - row_start
+        first = row_start + (int)(rows * j / k);
+        n = row_start + (int)(rows * (j + 1) / k) - first;
+    } else {
+        const long long W = cum[B];
+        const int c = linear_block_of(W, pt->blocks, x);
+        first = max((int)(W * c / pt->blocks), row_start);
+        n = min((int)(W * (c + 1) / pt->blocks), row_end) - first;
+    }
+    const unsigned w = ((unsigned)(x - first + 1) * n_warps - 1) / (unsigned)n;
+    return (int)((unsigned)n * w / n_warps) == x - first;
+}
+
 // blocks c0..c1 that hold a part of the row [row_start, row_end) (row index r)
 __device__ __forceinline__ void partition_blocks_of_row(const Partition* pt, const int* cum, int B, int r, int row_start,
                                                         int row_end, int& c0, int& c1)
@@ -378,17 +421,8 @@ __device__ __forceinline__ void partition_blocks_of_row(const Partition* pt, con
         c1 = pt->base[r + 1] - 1;
         return;
     }
-    const long long W = cum[B];
-    const int C = pt->blocks;
-    auto start = [&](int c) -> int { return (int)((W * c) / C); };
-    auto block_of = [&](int x) -> int {
-        int c = (int)(((long long)x * C) / W);
-        while (c + 1 < C && start(c + 1) <= x) ++c;
-        while (c > 0 && start(c) > x) --c;
-        return c;
-    };
-    c0 = block_of(row_start);
-    c1 = block_of(row_end - 1);
+    c0 = linear_block_of(cum[B], pt->blocks, row_start);
+    c1 = linear_block_of(cum[B], pt->blocks, row_end - 1);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -415,12 +449,13 @@ struct Geo {
     static constexpr int OFF_STRIDE = OFF_CUM + (kMaxBatch + 1) * 4;
     static constexpr int OFF_M = OFF_STRIDE + kMaxBatch * 4;
     static constexpr int OFF_L = OFF_M + NW * 8 * 4;
-    static constexpr int OFF_PART = OFF_L + NW * 8 * 4;
+    static constexpr int OFF_PART = (OFF_L + NW * 8 * 4 + 15) / 16 * 16;    // holds 64-bit fields
     static constexpr int OFF_LAST = OFF_PART + ((int)sizeof(Partition) + 15) / 16 * 16;
     static constexpr int OFF_QS = OFF_LAST + 16;             // record format 2: digit unit of the rotated query, per head
     static constexpr int SMEM = OFF_QS + 32;
     static_assert(SLOT % 128 == 0 && OFF_QT % 16 == 0 && OFF_QF % 16 == 0 && OFF_BAR % 8 == 0,
                   "slots are bulk-copy destinations; query fragments are read with 16- and 8-byte loads");
+    static_assert(OFF_PART % alignof(Partition) == 0 && OFF_LAST % 16 == 0, "alignment of the partition record");
     static_assert(NW >= 4, "a warp builds the query fragments of at most two columns of the 8-wide head group");
     static_assert(NSTAGE >= 2 && NSTAGE % 2 == 0 && NSTAGE <= 16, "an FP8 page takes a pair of slots; one phase bit per slot");
     static_assert(NSTAGE * SLOT >= 8 * D * 4, "ring doubles as the cross-warp reduction buffer");
@@ -1012,7 +1047,7 @@ __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot,
         P.lse[(size_t)b * hq + h * GQ + tid] = ml_s[8 + tid] > 0.f ? (ml_s[tid] + log2f(ml_s[8 + tid])) * kLn2 : -CUDART_INF_F;
 }
 
-template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT>
+template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT, bool FLAT>
 __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const LayerSet<MAXL> LS)
 {
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
@@ -1070,7 +1105,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         }
         if (lane == 0) cum[P0.B] = run;
         __syncwarp();
-        build_partition(pt, cum, P0.B, hkv, gridDim.x, lane);
+        if constexpr (FLAT) {
+            if (lane == 0) {
+                pt->total = (long long)run * n_layers;
+                pt->flat_blocks = (int)min(pt->total, (long long)gridDim.x);
+            }
+        }
+        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, lane);
     } else {
         // Pages of a row are visited in a strided order, page(i) = i * stride mod n_pages, the stride
         // coprime to n_pages and near 0.618 n_pages: every contiguous range of positions then holds the
@@ -1090,7 +1131,17 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     }
     __syncthreads();
     int my_start = 0, my_end = 0;                          // more blocks than work: an empty range
-    if ((int)blockIdx.x < pt->blocks) partition_range(pt, cum, hkv, P0.B, blockIdx.x, my_start, my_end);
+    int layer_first = 0, layer_end = n_layers;
+    if constexpr (FLAT) {
+        if ((int)blockIdx.x < pt->flat_blocks) {
+            layer_first = (int)(flat_start(pt, blockIdx.x) / cum[P0.B]);
+            layer_end = (int)((flat_start(pt, blockIdx.x + 1) - 1) / cum[P0.B]) + 1;
+        } else {
+            layer_end = 0;
+        }
+    } else if ((int)blockIdx.x < pt->blocks) {
+        partition_range(pt, cum, hkv, P0.B, blockIdx.x, my_start, my_end);
+    }
 
     // per-warp ring of NSTAGE slots; one bit per slot holds the mbarrier phase the next wait must see
     uint32_t phase = 0;
@@ -1139,22 +1190,29 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         return lost;
     };
 
-    for (int layer = 0; layer < n_layers; ++layer) {
+    // rows of empty requests
+    for (int i0 = blockIdx.x; i0 < P0.B * n_layers; i0 += gridDim.x) {
+        const int b = i0 % P0.B;
+        if (P0.lens[b] > 0) continue;
+        const DecodeParams& P = LS.layer[MAXL == 1 ? 0 : i0 / P0.B];
+        for (int i = tid; i < hq * D; i += NW * 32) P.out[(size_t)b * hq * D + i] = 0.f;
+        if (P.lse)
+            for (int i = tid; i < hq; i += NW * 32) P.lse[(size_t)b * hq + i] = -CUDART_INF_F;
+    }
+
+    for (int layer = layer_first; layer < layer_end; ++layer) {
     const DecodeParams& P = LS.layer[MAXL == 1 ? 0 : layer];
+    if constexpr (FLAT) {                                  // this block's range inside the layer
+        const long long w0 = (long long)layer * cum[P0.B];
+        my_start = (int)max(flat_start(pt, blockIdx.x) - w0, 0ll);
+        my_end = (int)min(flat_start(pt, blockIdx.x + 1) - w0, (long long)cum[P0.B]);
+    }
     auto wait_slot = [&](uint32_t s) {
         if (!wait_bounded(s, P.wait_ns)) {
             failed = true;
             atomicOr(P.status, kStTimeout);
         }
     };
-    // rows of empty requests
-    for (int b = blockIdx.x; b < P.B; b += gridDim.x)
-        if (P.lens[b] <= 0) {
-            for (int i = tid; i < hq * D; i += NW * 32) P.out[(size_t)b * hq * D + i] = 0.f;
-            if (P.lse)
-                for (int i = tid; i < hq; i += NW * 32) P.lse[(size_t)b * hq + i] = -CUDART_INF_F;
-        }
-
     int pos = my_start;
     int b = 0;
     while (pos < my_end) {
@@ -1191,12 +1249,18 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 
         // Table entries of up to G::ROUND of the warp's pages are compacted into two id lists, one per
         // format (entry i of a 32-page chunk is read by lane i; ballots give the positions).
+        // Returns how many of the warp's pages (from `first` on) the lists cover.  Long pages in the flat cut: a Stale
+        // tile that opens a warp's run of the per-layer cut is marked (kOpens); the scan leaves the page there, and
+        // a round ends at the last such tile, so that code sums are gathered over the same runs of tiles as there
+        // (their rounding inside the tensor core grows with the length of a run).
         int n3 = 0, n8 = 0;
-        auto build_lists = [&](int round) {
+        constexpr int kOpens = 0x8000;
+        auto build_lists = [&](int first) -> int {
             n3 = n8 = 0;
+            int covered = min(G::ROUND, n_my - first), cut3 = 0, cut8 = 0, cut = 0;
 #pragma unroll 1
             for (int c = 0; c < G::ROUND / 32; ++c) {
-                const int i = round * G::ROUND + c * 32 + lane;
+                const int i = first + c * 32 + lane;
                 int kind = 0, id = 0, valid = kPage, pg = 0;
                 if (i < n_my) {
                     pg = (int)(((unsigned)(pg0 + warp_first + i) * (unsigned)stride) % (unsigned)n_pages);   // < 2^32: max_pages <= 65535
@@ -1210,7 +1274,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     else
                         kind = (tag <= MKV_TAG_ANCHOR && id >= 0 && id < P.fp8_pages) ? 2 : 0;
                     if (kind == 0) atomicOr(P.status, kStBounds);     // never dereferenced
-                    if constexpr (TILED) pg = (pg - entry * P.tiles) | (entry << 16);   // second list: tile inside its page | logical page << 16
+                    if constexpr (TILED) {   // second list: tile inside its page | logical page << 16
+                        const bool opens = FLAT && opens_warp_run(pt, cum, P.B, b * hkv + h, row_start, row_end, row_start + pg, NW);
+                        pg = (pg - entry * P.tiles) | (entry << 16) | (opens ? kOpens : 0);
+                    }
                 }
                 const uint32_t m3 = __ballot_sync(FULL, kind == 1), m8 = __ballot_sync(FULL, kind == 2);
                 const uint32_t lt = (1u << lane) - 1u;
@@ -1220,10 +1287,25 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     if (kind == 1) lpg3[n3 + __popc(m3 & lt)] = pg;
                     if (kind == 2) lpg8[n8 + __popc(m8 & lt)] = pg;
                 }
+                if constexpr (TILED && FLAT) {
+                    const uint32_t mo = __ballot_sync(FULL, i < n_my && (pg & kOpens));
+                    if (mo) {
+                        const int at = 31 - __clz(mo);
+                        cut = c * 32 + at;
+                        cut3 = n3 + __popc(m3 & ((1u << at) - 1u));
+                        cut8 = n8 + __popc(m8 & ((1u << at) - 1u));
+                    }
+                }
                 n3 += __popc(m3);
                 n8 += __popc(m8);
             }
+            if (TILED && FLAT && cut > 0 && first + covered < n_my) {
+                covered = cut;
+                n3 = cut3;
+                n8 = cut8;
+            }
             __syncwarp();
+            return covered;
         };
         auto issue_tq3 = [&](int i) {      // copy Stale page i of the round into ring slot i % NSTAGE
             pending |= 1u << ((uint32_t)i % NSTAGE);
@@ -1234,7 +1316,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     mbar_expect_tx(bars + 8 * s, G::TQ3_REC);
                     bulk_load(ring + s * G::SLOT, tq3_base + (size_t)list3[i] * hkv * G::TQ3_REC, G::TQ3_REC, bars + 8 * s);
                 } else {   // the tile only: the page's scale/zero are applied once, when the scan leaves the page
-                    const int page = list3[i], m = lpg3[i] & 0xFFFF;
+                    const int page = list3[i], m = lpg3[i] & 0x7FFF;
                     const uint8_t* pbase = P.tq3 + ((size_t)page * hkv + h) * tq3_page;
                     mbar_expect_tx(bars + 8 * s, TQ3_TILE);
                     bulk_load(ring + s * G::SLOT, pbase + (size_t)m * TQ3_TILE, TQ3_TILE, bars + 8 * s);
@@ -1250,7 +1332,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 if constexpr (!TILED) {
                     rec = fp8_base + (size_t)e8 * hkv * (2 * G::FP8_HALF);
                 } else {
-                    rec = P.fp8 + (((size_t)e8 * hkv + h) * P.tiles + (lpg8[i] & 0xFFFF)) * (2 * G::FP8_HALF);
+                    rec = P.fp8 + (((size_t)e8 * hkv + h) * P.tiles + (lpg8[i] & 0x7FFF)) * (2 * G::FP8_HALF);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_expect_tx(bars + 8 * s, G::FP8_HALF);
@@ -1313,9 +1395,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         acc.mr = -CUDART_INF_F;
 
         // first round: start the copies, then build the query fragments while they fly
-        const int n_rounds = (n_my + G::ROUND - 1) / G::ROUND;
-        if (n_rounds > 0) {
-            build_lists(0);
+        int done = 0;
+        if (n_my > 0) {
+            done = build_lists(0);
             for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
         }
 
@@ -1403,11 +1485,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         // score unit of the Stale pages: record format 2 counts in digit units of this lane's head g
         const float sc2k = FMT == 2 ? sc2 * reinterpret_cast<const float*>(smem + G::OFF_QS)[g] : sc2;
 
-        for (int round = 0; round < n_rounds && !failed; ++round) {
-            if (round > 0) {
-                build_lists(round);
-                for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
-            }
+        for (bool more = n_my > 0; more && !failed;) {
             // ---- Stale pages: scores of page i+1 are computed together with the output update of page i
             if (n3 > 0) {
                 float s_cur[4], s_next[4];
@@ -1428,7 +1506,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
                         const int pg_i = list3[i];
-                        if (pg_i != cur_page) {
+                        if (pg_i != cur_page || (FLAT && i > 0 && (lpg3[i] & kOpens))) {
                             fold(cur_page, false, cur_lp);
                             cur_page = pg_i;
                             cur_lp = lpg3[i] >> 16;
@@ -1446,7 +1524,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
                         const int pg_i = list3[n3 - 1];
-                        if (pg_i != cur_page) {
+                        if (pg_i != cur_page || (FLAT && n3 > 1 && (lpg3[n3 - 1] & kOpens))) {
                             fold(cur_page, false, cur_lp);
                             cur_page = pg_i;
                             cur_lp = lpg3[n3 - 1] >> 16;
@@ -1475,6 +1553,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     __syncwarp();
                     if (i + NSTAGE / 2 < n8) issue_fp8(i + NSTAGE / 2);
                 }
+            }
+            more = done < n_my;
+            if (more && !failed) {
+                done += build_lists(done);
+                for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
             }
         }
         float (&oacc)[NBH][4] = acc.o;
@@ -1535,8 +1618,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 P.lse[(size_t)b * hq + h * GQ + tid] = l > 0.f ? (M + log2f(l)) * kLn2 : -CUDART_INF_F;
             }
         } else {
-            // partial (m, l, O) of this block for the row; slot 2c if the segment opens the block's range,
-            // 2c + 1 otherwise
+            // partial (m, l, O) of this block for the row; slot 2c if the segment opens the block's range (flat cut:
+            // its range in this layer), 2c + 1 otherwise
             float* slot = P.partials + (size_t)(2 * blockIdx.x + (pos != my_start ? 1 : 0)) * (8 * D + 16);
             for (int e = tid; e < 8 * D; e += NW * 32) {
                 float acc = 0.f;
@@ -1561,7 +1644,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             // request (the counter's top bit) and the row's last arrival, seeing the request, merges after all.
             // Either way exactly one block merges, and it leaves the counter at zero for the next call.
             int c0, c1;
-            partition_blocks_of_row(pt, cum, P.B, b * hkv + h, row_start, row_end, c0, c1);
+            if constexpr (FLAT) {                          // here the row's last arrival merges: no block is ahead of the others
+                const long long w0 = (long long)layer * cum[P0.B];
+                c0 = linear_block_of(pt->total, pt->flat_blocks, w0 + row_start);
+                c1 = linear_block_of(pt->total, pt->flat_blocks, w0 + row_end - 1);
+            } else {
+                partition_blocks_of_row(pt, cum, P.B, b * hkv + h, row_start, row_end, c0, c1);
+            }
             const int n_parts = c1 - c0 + 1;
             constexpr uint32_t kRequest = 0x80000000u;
             __syncthreads();
@@ -1569,8 +1658,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 __threadfence();
                 const uint32_t prev = atomicAdd(P.tickets + c0, 1u);
                 int todo = 0;                          // 1: merge this layer's row, 2: merge the row of the layer before
-                if ((prev & ~kRequest) == (uint32_t)(n_parts - 1) && (layer == n_layers - 1 || (prev & kRequest))) todo |= 1;
-                if (MAXL > 1 && layer > 0 && (prev & ~kRequest) == 0u) {
+                if ((prev & ~kRequest) == (uint32_t)(n_parts - 1) && (FLAT || layer == n_layers - 1 || (prev & kRequest))) todo |= 1;
+                if (MAXL > 1 && !FLAT && layer > 0 && (prev & ~kRequest) == 0u) {
                     const uint32_t old = atomicOr(LS.layer[layer - 1].tickets + c0, kRequest);
                     if (old == (uint32_t)n_parts) todo |= 2;
                 }
@@ -1580,8 +1669,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             const int todo = *last_s;
             if (todo) {
                 __threadfence();
-                const int first_slot = 2 * c0 + (row_start > partition_start(pt, cum, hkv, P.B, c0) ? 1 : 0);
-                if constexpr (MAXL > 1) {
+                // the row opens block c0's range of the layer where it starts at or before that range
+                const int c0_start = FLAT ? (int)max(flat_start(pt, c0) - (long long)layer * cum[P0.B], 0ll)
+                                          : partition_start(pt, cum, hkv, P.B, c0);
+                const int first_slot = 2 * c0 + (row_start > c0_start ? 1 : 0);
+                if constexpr (MAXL > 1 && !FLAT) {
                     if (todo & 2) {
                         const DecodeParams& Q = LS.layer[layer - 1];
                         merge_row<D, NW * 32>(Q, first_slot, 2 * c0, n_parts, red, b, h);
@@ -1638,11 +1730,11 @@ static int32_t run_tmem(mkv_pool* p, DecodeParams& prm, cudaStream_t s)
     return MKV_OK;
 }
 
-template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT>
+template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT, bool FLAT>
 static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_t s)
 {
     using G = Geo<D, NW, NSTAGE, TILED>;
-    auto kern = decode_tensor_kernel<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, FMT>;
+    auto kern = decode_tensor_kernel<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, FMT, FLAT>;
     // pages of several tiles: one row of parked accumulators (8 D floats) per warp behind the usual layout
     constexpr int SMEM = G::SMEM + (TILED ? NW * 8 * D * 4 : 0);
     static_assert(SMEM <= 232448, "dynamic shared memory of one block");
@@ -1675,11 +1767,11 @@ static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_
 }
 
 // the pool's record format selects the instantiation
-template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false, int MAXL = 1>
+template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false, int MAXL = 1, bool FLAT = false>
 static int32_t run_tensor(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_t s)
 {
-    return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2>(p, ls, s)
-                       : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1>(p, ls, s);
+    return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT>(p, ls, s)
+                       : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT>(p, ls, s);
 }
 
 template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false>
@@ -1819,9 +1911,15 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
         ls.layer[i] = make_params(pools[i], q[i], bt[i], tags[i], lens, B, max_pages, scale, out[i], lse ? lse[i] : nullptr,
                                   partials, tickets, kMaxCtas, nullptr);
     }
-    if (p0->tiles > 1)                   // pages of several tiles (all pools of the call have the same page size)
+    if (p0->tiles > 1 && n_layers >= kMinFlatLayers)   // pages of several tiles (all pools of the call have the same page size)
+        return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, true, kMaxLayers, true>(p0, ls, s)
+                            : run_tensor<256, 8, 4, 1, false, true, kMaxLayers, true>(p0, ls, s);
+    if (p0->tiles > 1)
         return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, true, kMaxLayers>(p0, ls, s)
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
+    if (n_layers >= kMinFlatLayers)
+        return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
+                            : run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s);
     return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, false, kMaxLayers>(p0, ls, s)
                         : run_tensor<256, 8, 4, 1, false, false, kMaxLayers>(p0, ls, s);
 }

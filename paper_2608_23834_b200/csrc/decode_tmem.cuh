@@ -71,7 +71,7 @@ struct TG {
     static constexpr int OFF_STRIDE = OFF_CUM + (kMaxBatch + 1) * 4;
     static constexpr int OFF_M = OFF_STRIDE + kMaxBatch * 4;
     static constexpr int OFF_L = OFF_M + 8 * 4;
-    static constexpr int OFF_PART = OFF_L + 8 * 4;
+    static constexpr int OFF_PART = (OFF_L + 8 * 4 + 15) / 16 * 16;    // holds 64-bit fields
     static constexpr int OFF_LAST = OFF_PART + ((int)sizeof(Partition) + 15) / 16 * 16;
     static constexpr int OFF_TMEM = OFF_LAST + 16;
     static constexpr int SMEM = OFF_TMEM + 16;

@@ -150,3 +150,45 @@ def test_a_wait_that_runs_out_is_reported_and_the_pool_stays_usable():
     for _ in range(2):                                            # tickets were left at zero: split rows merge as usual
         out2, lse2 = case.run(M.DECODE_TENSOR)
         assert np.array_equal(out2, out) and np.array_equal(lse2, lse)
+
+
+@pytest.mark.parametrize("n_layers,name", [(4, "cfg2"), (7, "edge"), (5, "tiny"), (4, "pages_of_832"), (6, "pages_of_48_d128")])
+@pytest.mark.parametrize("fmt", [1, 2])
+def test_layers_laid_end_to_end(n_layers, name, fmt):
+    """From four layers on one cut of the grid covers all layers' pages: rows that a block shares with its
+    neighbours, rows wholly inside a block, several layers inside a block, empty requests, fewer pages than
+    blocks.  Against single calls the order of the fp32 sums differs: a page adds at most 4 roundings of 2^-24
+    of the running sums, so 1e-4 of the output's scale bounds the runs of up to 400 pages here."""
+    fn = {"cfg2": lambda: W.config(2, seq_lens=(5008, 4432), recent_tokens=512, n_layers=1),
+          "pages_of_832": lambda: W.config(2, seq_lens=(9 * 832 + 100, 7 * 832), anchor_prefix=832, recent_tokens=900,
+                                           n_layers=1, page_tokens=832),
+          "pages_of_48_d128": lambda: W.config(1, seq_lens=(48 * 21 + 5, 48 * 30, 47, 48 * 9 + 47), anchor_prefix=48,
+                                               recent_tokens=100, anchor_span_tokens=96, page_tokens=48),
+          "tiny": lambda: W.config(0, seq_lens=(5,), head_dim=256, n_kv_heads=1, group=3),
+          "edge": lambda: W.config(0, seq_lens=(0, 1, 15, 16, 17, 33, 16 * 20 + 9, 300), head_dim=128, n_kv_heads=2, group=4,
+                                   anchor_prefix=16, recent_tokens=40, n_outlier=3)}[name]
+    oracle.set_format(fmt)
+    try:
+        cases = [Case(fn(), layer=i % 2) for i in range(2)]
+        refs = [c.reference() for c in cases]
+    finally:
+        oracle.set_format(1)
+    spec = cases[0].spec
+    layers = [cases[i % 2] for i in range(n_layers)]                     # layers that share pages still have their own outputs
+    workspaces = [M.Pool(spec.head_dim, spec.n_kv_heads, spec.n_q_heads, max(cases[0].tab.fp8_pages, 1),
+                         max(cases[0].tab.tq3_pages, 1), layers[i].L.sigma, max_batch=spec.batch,
+                         page_tokens=spec.page_tokens, tq3_format=fmt) for i in range(n_layers)]
+    for pool, c in zip(workspaces, layers):
+        pool.upload_arenas(c.L.fp8_arena, c.L.tq3_arena)
+    outs = [torch.full_like(cases[0].q, 7.0, dtype=torch.float32) for _ in layers]
+    lses = [torch.full((spec.batch, spec.n_q_heads), 7.0, device="cuda:0") for _ in layers]
+    for _ in range(2):                                                   # the second call finds the tickets at zero again
+        M.decode_attention_layers(workspaces, [c.q for c in layers], [c.bt for c in layers], [c.tags for c in layers],
+                                  cases[0].lens, spec.scale, outs, lses)
+    single = workspaces[-1].decode_attention(layers[-1].q, layers[-1].bt, layers[-1].tags, layers[-1].lens, spec.scale)
+    torch.cuda.synchronize()
+    for i in range(n_layers):
+        assert workspaces[i].status() == M.OK
+        ref, ref_lse = refs[i % 2]
+        check_case(layers[i], outs[i].cpu().numpy(), lses[i].cpu().numpy(), ref, ref_lse)
+    assert (outs[-1] - single).abs().max() <= 1e-4 * single.abs().max()

@@ -17,6 +17,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libmkv.so")
 _lib = None
+_native = None          # the C++ binding of the decode-step calls (csrc/py_binding.cpp)
 
 OK, E_INVALID, E_OOM_FP8, E_OOM_TQ3, E_STATE, E_BOUNDS, E_CUDA, E_TIMEOUT = 0, -1, -2, -3, -4, -5, -6, -7
 TAG_RECENT, TAG_ANCHOR, TAG_STALE = 0, 1, 2
@@ -71,7 +72,7 @@ class LayerAppend(C.Structure):
 
 def lib():
     """Load libmkv.so; fails loudly if it has not been built (python paper_2608_23834_b200/build.py)."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise ImportError(f"{_LIB_PATH} is missing: build it with `python -m paper_2608_23834_b200.build` "
@@ -126,6 +127,8 @@ def lib():
             fn.restype = C.c_int32
         L.mkv_last_cuda_error.restype = C.c_char_p
         L.mkv_last_cuda_error.argtypes = []
+        from . import _mkv_native
+        _native = _mkv_native
         _lib = L
     return _lib
 
@@ -133,6 +136,13 @@ def lib():
 def _check(rc: int, where: str):
     if rc != OK:
         raise MkvError(rc, where)
+
+
+def _native_rc(rc: int, where: str) -> bool:
+    """Result of a native call: True when enqueued, False when it left the arguments to the checks below it."""
+    if rc < 0:
+        raise MkvError(rc, where)
+    return rc == 0
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -193,10 +203,12 @@ class Pool:
             _check(L.mkv_pool_create(C.byref(self.cfg), _ptr(self.fp8_arena), _ptr(self.tq3_arena), _stream(None),
                                      C.byref(h)), "mkv_pool_create")
             self.handle = h
+            self._ref = _native.pool_ref(h.value, n_kv_heads, n_q_heads, head_dim)     # what the native calls need of the pool
             _check(L.mkv_workspace_init(_ptr(self.workspace), self.ws_bytes, _stream(None)), "mkv_workspace_init")
 
     def close(self):
         if getattr(self, "handle", None):
+            self._ref = None
             lib().mkv_pool_destroy(self.handle)
             self.handle = None
 
@@ -251,13 +263,19 @@ class Pool:
         torch.cuda.synchronize(self.device)
 
     # ---- hot path
+    # (the native calls check and marshal in C++; what they do not take as it stands goes through the Python
+    # checks below them, which name the argument)
     def append(self, k: torch.Tensor, v: torch.Tensor, slot_mapping: torch.Tensor, stream=None) -> None:
+        if _native_rc(_native.append(self._ref, k, v, slot_mapping, stream), "mkv_append"):
+            return
         assert k.dtype == torch.bfloat16 and v.dtype == torch.bfloat16 and slot_mapping.dtype == torch.int32
         assert k.is_contiguous() and v.is_contiguous() and k.shape == v.shape and k.shape[1:] == (self.hkv, self.d)
         _check(lib().mkv_append(self.handle, _ptr(k), _ptr(v), _ptr(slot_mapping), k.shape[0], _stream(stream)), "mkv_append")
 
     def demote(self, src_ids: torch.Tensor, dst_ids: torch.Tensor, block_table=None, tier_tag=None, entry_index=None,
                stream=None) -> None:
+        if _native_rc(_native.demote(self._ref, src_ids, dst_ids, block_table, tier_tag, entry_index, stream), "mkv_demote"):
+            return
         assert src_ids.dtype == torch.int32 and dst_ids.dtype == torch.int32 and src_ids.numel() == dst_ids.numel()
         if entry_index is not None:
             assert entry_index.dtype == torch.int64 and block_table.dtype == torch.int32 and tier_tag.dtype == torch.uint8
@@ -267,6 +285,8 @@ class Pool:
 
     def promote(self, src_ids: torch.Tensor, dst_ids: torch.Tensor, block_table=None, tier_tag=None, entry_index=None,
                 stream=None) -> None:
+        if _native_rc(_native.promote(self._ref, src_ids, dst_ids, block_table, tier_tag, entry_index, stream), "mkv_promote"):
+            return
         assert src_ids.dtype == torch.int32 and dst_ids.dtype == torch.int32 and src_ids.numel() == dst_ids.numel()
         if entry_index is not None:
             assert entry_index.dtype == torch.int64 and block_table.dtype == torch.int32 and tier_tag.dtype == torch.uint8
@@ -279,6 +299,10 @@ class Pool:
                                     _stream(stream)), "mkv_set_anchor")
 
     def decode_attention(self, q, block_table, tier_tag, seq_lens, scale, out=None, lse=None, workspace=None, stream=None):
+        if out is not None and _native_rc(_native.decode(self._ref, q, block_table, tier_tag, seq_lens, scale, out, lse,
+                                                         self.workspace if workspace is None else workspace, stream),
+                                          "mkv_decode_attention"):
+            return out
         B = q.shape[0]
         assert q.dtype == torch.bfloat16 and q.is_contiguous() and q.shape == (B, self.hq, self.d)
         assert block_table.dtype == torch.int32 and block_table.is_contiguous() and block_table.shape[0] == B
@@ -295,6 +319,11 @@ class Pool:
     def decode_attention_scored(self, q, block_table, tier_tag, seq_lens, scale, out=None, lse=None, page_mass=None,
                                 workspace=None, stream=None):
         """mkv_decode_attention_scored: returns (out, lse, page_mass [B][hq][max_pages])."""
+        if out is not None and lse is not None and page_mass is not None and _native_rc(
+                _native.decode_scored(self._ref, q, block_table, tier_tag, seq_lens, scale, out, lse,
+                                      self.workspace if workspace is None else workspace, stream, page_mass),
+                "mkv_decode_attention_scored"):
+            return out, lse, page_mass
         B = q.shape[0]
         assert q.dtype == torch.bfloat16 and q.is_contiguous() and q.shape == (B, self.hq, self.d)
         assert block_table.dtype == torch.int32 and block_table.is_contiguous() and block_table.shape[0] == B
@@ -317,6 +346,9 @@ class Pool:
 def decode_attention_layers(pools, qs, block_tables, tier_tags, seq_lens, scale, outs, lses=None, stream=None):
     """mkv_decode_attention_layers: the decode attention of len(pools) layers in one launch; layer i reads
     pools[i], qs[i], block_tables[i], tier_tags[i] and writes outs[i] (and lses[i]); seq_lens is common."""
+    if _lib is not None and _native_rc(_native.decode_layers(pools, qs, block_tables, tier_tags, seq_lens, scale, outs, lses,
+                                                             stream), "mkv_decode_attention_layers"):
+        return outs
     n = len(pools)
     B = qs[0].shape[0]
     calls = (LayerCall * n)()
@@ -337,6 +369,8 @@ def decode_attention_layers(pools, qs, block_tables, tier_tags, seq_lens, scale,
 
 def append_layers(pools, ks, vs, slot_mapping, stream=None):
     """mkv_append_layers: Append of the same token positions into the pools of several layers in one launch."""
+    if _lib is not None and _native_rc(_native.append_layers(pools, ks, vs, slot_mapping, stream), "mkv_append_layers"):
+        return
     n = len(pools)
     calls = (LayerAppend * n)()
     for i, pool in enumerate(pools):
@@ -351,6 +385,10 @@ def append_layers(pools, ks, vs, slot_mapping, stream=None):
 def page_score_update(page_mass, seq_lens, head_mask, beta, score, stream=None, page_tokens=16):
     """mkv_page_score_update[_paged] (Eq. attention-score): score <- beta * score + (1 - beta) * mean over the
     heads in head_mask of page_mass, in place, for the pages below each request's length."""
+    lib()
+    if _native_rc(_native.score_update(page_mass, seq_lens, int(head_mask), beta, score, stream, page_tokens),
+                  "mkv_page_score_update"):
+        return score
     B, hq, max_pages = page_mass.shape
     assert page_mass.dtype == torch.float32 and page_mass.is_contiguous()
     assert score.dtype == torch.float32 and score.is_contiguous() and score.shape == (B, max_pages)

@@ -86,10 +86,14 @@ __device__ __forceinline__ uint2 bf16x8_to_e4m3x8(uint4 in, float inv_scale)
     return make_uint2(q[0] | (q[1] << 16), q[2] | (q[3] << 16));
 }
 
-// Prefill-sized calls: one block per (16 consecutive input tokens, KV head).  Where the 16 tokens fill
-// one page front to back (slot_mapping[t0 + i] = 16 page + i), K rows leave with 8-byte stores and V
-// is transposed through shared memory so that every channel's 16 tokens leave as one 16-byte store;
-// any other group (skipped tokens, a run that starts inside a page, the tail) takes the per-token path.
+// Prefill-sized calls: one block per (window of 16 consecutive input tokens, KV head).  The block takes the runs
+// that START in its window, a run being consecutive tokens that go to consecutive positions of one 16-token tile;
+// such a run may reach up to 15 tokens into the next window.  A chunk of a request that starts anywhere inside a
+// page therefore still meets whole tiles, one per window.  A run that fills its tile leaves as whole rows: K with
+// 8-byte stores, V transposed through shared memory so that every channel's 16 tokens are one 16-byte store (HBM
+// bound: 6.3 of 6.55 TB/s).  Other runs (the ends of a request's chunk, scattered or skipped tokens) are stored
+// token by token.  (With windows cut at fixed tokens a chunk that starts inside a page had no whole tile at all
+// and every token took the second path: 147 us for 32,845 tokens in five chunks, d = 256.)
 template <int D>
 __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ fp8, int fp8_pages, int hkv, int tiles,
                                                           float inv_k_scale, float inv_v_scale,
@@ -100,26 +104,37 @@ __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ f
 {
     constexpr int VROW = D + 4;                      // padded token row of the transposition tile
     __shared__ __align__(16) uint8_t vt[kPage * VROW];
-    __shared__ int32_t slot_s[kPage];
-    __shared__ int run_s;
+    __shared__ int32_t slot_s[2 * kPage];            // slots of this window and the next
+    __shared__ int32_t len_s[kPage];                 // runs that start at token i of the window and do not fill a tile
+    __shared__ int full_s;                           // token whose run fills a tile (at most one starts in a window), or -1
     const int t0 = blockIdx.x * kPage, h = blockIdx.y, tid = threadIdx.x;
-    const int cnt = min(kPage, n - t0);
-    if (tid < kPage) slot_s[tid] = tid < cnt ? slots[t0 + tid] : -1;
-    __syncthreads();
-    if (tid == 0) {
-        const int s0 = slot_s[0];
-        bool run = cnt == kPage && s0 >= 0 && (s0 & 15) == 0 && (s0 >> 4) / tiles < fp8_pages;
-        for (int i = 1; run && i < kPage; ++i) run = slot_s[i] == s0 + i;
-        run_s = run ? 1 : 0;
+    if (tid < 32) {
+        const int sl = t0 + tid < n ? slots[t0 + tid] : -1;
+        const int before = tid == 0 && t0 > 0 ? slots[t0 - 1] : -2;
+        slot_s[tid] = sl;
+        const int up = __shfl_up_sync(0xffffffffu, sl, 1);
+        const int prev = tid == 0 ? before : up;
+        __syncwarp();
+        int len = 0;
+        if (tid < kPage && sl >= 0 && ((sl & 15) == 0 || prev != sl - 1)) {
+            len = 1;
+            while (len < kPage - (sl & 15) && slot_s[tid + len] == sl + len) ++len;
+        }
+        const bool full = len == kPage && (sl >> 4) / tiles < fp8_pages;
+        const uint32_t m = __ballot_sync(0xffffffffu, full);
+        if (tid < kPage) len_s[tid] = full ? 0 : len;
+        if (tid == 0) full_s = m ? __ffs(m) - 1 : -1;
     }
     __syncthreads();
-    if (run_s) {
-        const int gt = slot_s[0] >> 4, page = gt / tiles;
+    const int full = full_s;
+    if (full >= 0) {
+        const int gt = slot_s[full] >> 4, page = gt / tiles;
         uint8_t* rec = fp8 + (((size_t)page * hkv + h) * tiles + (gt - page * tiles)) * fp8_record_bytes(D);
         constexpr int CPT = D / 8;                   // 16-byte input chunks per token
+#pragma unroll
         for (int c = tid; c < kPage * CPT; c += 128) {
             const int t = c / CPT, c8 = c % CPT;
-            const size_t at = ((size_t)(t0 + t) * hkv + h) * (D / 8) + c8;
+            const size_t at = ((size_t)(t0 + full + t) * hkv + h) * (D / 8) + c8;
             const uint2 kq = bf16x8_to_e4m3x8(reinterpret_cast<const uint4*>(k)[at], inv_k_scale);
             const uint2 vq = bf16x8_to_e4m3x8(reinterpret_cast<const uint4*>(v)[at], inv_v_scale);
             *reinterpret_cast<uint2*>(rec + t * D + 8 * c8) = kq;
@@ -144,20 +159,21 @@ __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ f
                 *reinterpret_cast<uint4*>(rec + 16 * D + (4 * c4 + ch) * kPage) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
-        return;
     }
-    for (int t = 0; t < cnt; ++t) {
-        const int sm = slot_s[t];
-        if (sm < 0) continue;
-        const int gt = sm >> 4, page = gt / tiles;
-        if (page >= fp8_pages) {
-            if (tid == 0) atomicOr(status, kStBounds);
-            continue;
+    constexpr int PAR = 256 / D;                     // tokens stored side by side
+    int next = 0;
+    for (int i = 0; i < kPage; ++i)
+        for (int j = 0; j < len_s[i]; ++j) {
+            if (next++ % PAR != tid / (D / 2)) continue;
+            const int sm = slot_s[i + j], gt = sm >> 4, page = gt / tiles;
+            if (page >= fp8_pages) {
+                if (tid % (D / 2) == 0) atomicOr(status, kStBounds);
+                continue;
+            }
+            uint8_t* rec = fp8 + (((size_t)page * hkv + h) * tiles + (gt - page * tiles)) * fp8_record_bytes(D);
+            const size_t src = ((size_t)(t0 + i + j) * hkv + h) * (D / 2);
+            append_token<D>(rec, sm & 15, inv_k_scale, inv_v_scale, k + src, v + src, tid % (D / 2));
         }
-        uint8_t* rec = fp8 + (((size_t)page * hkv + h) * tiles + (gt - page * tiles)) * fp8_record_bytes(D);
-        const size_t src = ((size_t)(t0 + t) * hkv + h) * (D / 2);
-        if (tid < D / 2) append_token<D>(rec, sm & 15, inv_k_scale, inv_v_scale, k + src, v + src, tid);
-    }
 }
 
 // Decode-sized append into the pools of several layers: one block per (token, KV head, layer).

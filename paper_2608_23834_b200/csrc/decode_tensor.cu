@@ -312,12 +312,21 @@ struct Partition {
 };
 
 // Called by warp 0 (all 32 lanes) after cum[] is complete; other warps wait at the next barrier.
-__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int lane)
+// Blocks that share W triples: all of the grid, but no more than give every warp kMinPagesPerWarp pages.
+constexpr int kMinPagesPerWarp = 1;
+__device__ __forceinline__ int useful_blocks(long long W, int grid, int n_warps)
+{
+    const long long most = (W + kMinPagesPerWarp * n_warps - 1) / (kMinPagesPerWarp * n_warps);
+    return (int)(most < (long long)grid ? most : (long long)grid);
+}
+
+__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int n_warps, int lane)
 {
     constexpr uint32_t FULL = 0xffffffffu;
     const long long W = cum[B];
     const int rows = B * hkv;
-    int blocks = (int)(W < (long long)grid ? W : (long long)grid);
+    int blocks = useful_blocks(W, grid, n_warps);
+    grid = blocks;
     // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
     // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
     // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).
@@ -457,7 +466,7 @@ struct Geo {
                   "slots are bulk-copy destinations; query fragments are read with 16- and 8-byte loads");
     static_assert(OFF_PART % alignof(Partition) == 0 && OFF_LAST % 16 == 0, "alignment of the partition record");
     static_assert(NW >= 4, "a warp builds the query fragments of at most two columns of the 8-wide head group");
-    static_assert(NSTAGE >= 2 && NSTAGE % 2 == 0 && NSTAGE <= 16, "an FP8 page takes a pair of slots; one phase bit per slot");
+    static_assert(NSTAGE >= 4 && NSTAGE % 2 == 0 && NSTAGE <= 16, "an FP8 page takes a pair of slots; one phase bit per slot");
     static_assert(NSTAGE * SLOT >= 8 * D * 4, "ring doubles as the cross-warp reduction buffer");
     static_assert(FP8_HALF <= SLOT, "half an FP8 record fits a slot");
 };
@@ -1085,6 +1094,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         last_s[1] = 0;
     }
+    pdl_begin();
     if (warp == 0) {
         int run = 0;
         for (int b0 = 0; b0 < P0.B; b0 += 32) {
@@ -1108,10 +1118,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         if constexpr (FLAT) {
             if (lane == 0) {
                 pt->total = (long long)run * n_layers;
-                pt->flat_blocks = (int)min(pt->total, (long long)gridDim.x);
+                pt->flat_blocks = useful_blocks(pt->total, gridDim.x, NW);
             }
         }
-        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, lane);
+        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, NW, lane);
     } else {
         // Pages of a row are visited in a strided order, page(i) = i * stride mod n_pages, the stride
         // coprime to n_pages and near 0.618 n_pages: every contiguous range of positions then holds the
@@ -1159,7 +1169,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     // limit, 20 ms by default); returns false when it ran out.
     auto wait_bounded = [&](uint32_t s, unsigned long long limit_ns) -> bool {
         const uint32_t bar = bars + 8 * s, parity = (phase >> s) & 1u;
-        // limit 0 (diagnostic): one look without blocking, so that a copy still in flight counts as late
+        // limit 0 (diagnostic): one look without blocking, so that a copy still in flight counts as late (the first
+        // one of a row is looked at as soon as it is issued)
         bool ok = limit_ns == 0 ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity);
         if (!ok && limit_ns != 0) {
             unsigned long long t0, t1;
@@ -1323,10 +1334,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 }
             }
         };
-        auto issue_fp8 = [&](int i) {      // copy FP8 page i of the round into the slot pair 2 (i % (NSTAGE/2))
-            pending |= 3u << ((uint32_t)(2 * i) % NSTAGE);
+        // FP8 page i of the round goes into the slot pair (first8 + i) % (NSTAGE / 2): the first pair is one that the
+        // round's last Stale page does not occupy, so that the FP8 copies start before that page is finished
+        uint32_t first8 = 0;
+        auto issue_fp8 = [&](int i) {
+            const uint32_t s = 2 * ((first8 + (uint32_t)i) % (NSTAGE / 2));
+            pending |= 3u << s;
             if (lane == 0) {
-                const uint32_t s = (uint32_t)(2 * i) % NSTAGE;
                 const int e8 = list8[i] & 0x7FFFFFF;
                 const uint8_t* rec;
                 if constexpr (!TILED) {
@@ -1340,6 +1354,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 mbar_expect_tx(bars + 8 * (s + 1), G::FP8_HALF);
                 bulk_load(ring + (s + 1) * G::SLOT, rec + G::FP8_HALF, G::FP8_HALF, bars + 8 * (s + 1));
             }
+        };
+        auto start_round = [&]() {         // the first copies of a round
+            first8 = n3 > 0 ? ((uint32_t)(n3 - 1) % NSTAGE / 2 + 1) % (NSTAGE / 2) : 0u;
+            for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
+            if (n3 == 0)
+                for (int i = 0; i < min(n8, NSTAGE / 2); ++i) issue_fp8(i);
         };
 
         WarpAcc<NB> acc;
@@ -1398,7 +1418,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         int done = 0;
         if (n_my > 0) {
             done = build_lists(0);
-            for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
+            start_round();
+            // limit 0 (diagnostic): the first look comes before the query is prepared, while the copy is still in flight
+            if (P.wait_ns == 0 && n3 + n8 > 0 && !__all_sync(FULL, mbar_test_wait(bars, phase & 1u))) {
+                failed = true;
+                atomicOr(P.status, kStTimeout);
+            }
         }
 
         // query fragments: a warp rotates head `warp` (and `warp + NW`); loads were issued before the copies started
@@ -1520,6 +1545,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     if (i + NSTAGE < n3) issue_tq3(i + NSTAGE);
                 }
                 if (!failed) {
+                    if (n8 > 0) issue_fp8(0);
                     if constexpr (FMT == 2) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
                     else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
@@ -1535,12 +1561,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     if constexpr (TILED) fold(cur_page, true, cur_lp);   // back to output units for the FP8 pages and the reduction
                 }
                 __syncwarp();
+                if (!failed)
+                    for (int i = 1; i < min(n8, NSTAGE / 2); ++i) issue_fp8(i);
             }
             // ---- Recent/Anchor pages: two slots per page (keys, values)
             if (n8 > 0 && !failed) {
-                for (int i = 0; i < min(n8, NSTAGE / 2); ++i) issue_fp8(i);
                 for (int i = 0; i < n8 && !failed; ++i) {
-                    const uint32_t s = (uint32_t)(2 * i) % NSTAGE;
+                    const uint32_t s = 2 * ((first8 + (uint32_t)i) % (NSTAGE / 2));
                     wait_slot(s);
                     wait_slot(s + 1);
                     if (failed) break;
@@ -1557,7 +1584,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             more = done < n_my;
             if (more && !failed) {
                 done += build_lists(done);
-                for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
+                start_round();
             }
         }
         float (&oacc)[NBH][4] = acc.o;
@@ -1761,8 +1788,7 @@ static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_
         set_last_error("decode attention: the scan launches more blocks on this GPU than the partial area has slots for");
         return MKV_E_INVALID;
     }
-    kern<<<grid, NW * 32, SMEM, s>>>(ls);
-    MKV_CUDA(cudaGetLastError());
+    MKV_CUDA(launch_pdl(kern, dim3((unsigned)grid), NW * 32, SMEM, 1, true, s, ls));
     return MKV_OK;
 }
 
@@ -1804,6 +1830,7 @@ __global__ void __launch_bounds__(256) page_mass_finish_kernel(float* mass, cons
                                                               int hq, int max_pages, int page_tokens)
 {
     __shared__ float red[8];
+    pdl_begin();
     const int b = blockIdx.y, h = blockIdx.x, tid = threadIdx.x;
     const int len = lens[b], n_pages = len > 0 ? min((len + page_tokens - 1) / page_tokens, max_pages) : 0;
     float* row = mass + ((size_t)b * hq + h) * max_pages;
@@ -1830,6 +1857,7 @@ __global__ void __launch_bounds__(256) page_score_kernel(const float* mass, cons
                                                          unsigned long long head_mask, float beta, float inv_heads,
                                                          float* score, int page_tokens)
 {
+    pdl_begin();
     const int b = blockIdx.y, p = blockIdx.x * 256 + threadIdx.x;
     const int len = lens[b], n_pages = len > 0 ? min((len + page_tokens - 1) / page_tokens, max_pages) : 0;
     if (p >= n_pages) return;
@@ -1843,6 +1871,7 @@ __global__ void __launch_bounds__(256) page_score_kernel(const float* mass, cons
 // pages of several tiles: the scan adds parts of a page's sum to its entry, which therefore starts at -inf
 __global__ void page_mass_clear_kernel(float* mass, size_t n)
 {
+    pdl_begin();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) mass[i] = -CUDART_INF_F;
 }
@@ -1850,8 +1879,7 @@ __global__ void page_mass_clear_kernel(float* mass, size_t n)
 int32_t launch_page_mass_finish(float* mass, const float* lse, const int32_t* lens, int B, int hq, int max_pages,
                                 int page_tokens, cudaStream_t s)
 {
-    page_mass_finish_kernel<<<dim3(hq, B), 256, 0, s>>>(mass, lse, lens, hq, max_pages, page_tokens);
-    MKV_CUDA(cudaGetLastError());
+    MKV_CUDA(launch_pdl(page_mass_finish_kernel, dim3(hq, B), 256, 0, 1, true, s, mass, lse, lens, hq, max_pages, page_tokens));
     return MKV_OK;
 }
 
@@ -1861,9 +1889,8 @@ int32_t launch_page_score(const float* mass, const int32_t* lens, int B, int hq,
     int n = 0;
     for (int h = 0; h < hq; ++h) n += (int)((head_mask >> h) & 1ull);
     if (n == 0) return MKV_E_INVALID;
-    page_score_kernel<<<dim3((max_pages + 255) / 256, B), 256, 0, s>>>(mass, lens, hq, max_pages, head_mask, beta,
-                                                                         1.f / (float)n, score, page_tokens);
-    MKV_CUDA(cudaGetLastError());
+    MKV_CUDA(launch_pdl(page_score_kernel, dim3((max_pages + 255) / 256, B), 256, 0, 1, true, s, mass, lens, hq, max_pages,
+                        (unsigned long long)head_mask, beta, 1.f / (float)n, score, page_tokens));
     return MKV_OK;
 }
 
@@ -1946,8 +1973,7 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
         int32_t rc;
         if (p->tiles > 1) {
             const size_t n = (size_t)B * p->hkv * p->group * max_pages;
-            page_mass_clear_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(mass, n);
-            MKV_CUDA(cudaGetLastError());
+            MKV_CUDA(launch_pdl(page_mass_clear_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, 1, true, s, mass, n));
             rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true, true>(p, prm, s);
         } else {
             rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);

@@ -27,15 +27,14 @@ __device__ __forceinline__ uint16_t f32_to_f16_sat_bits(float x)
 }
 
 // ------------------------------------------------------------------------------------------ append
-// One token of one KV head: thread i converts elements 2i, 2i+1 of K and V (scale, round to nearest
-// even, saturate to +-448) and stores K token-major, V channel-major.
+// Elements 2 pair, 2 pair + 1 of K and V of one token and KV head (scale, round to nearest even, saturate to
+// +-448): K token-major, V channel-major.
 template <int D>
-__device__ __forceinline__ void append_token(uint8_t* __restrict__ rec, int slot, float inv_k_scale, float inv_v_scale,
-                                             const __nv_bfloat162* __restrict__ k, const __nv_bfloat162* __restrict__ v,
-                                             int pair)
+__device__ __forceinline__ void append_pair(uint8_t* __restrict__ rec, int slot, float inv_k_scale, float inv_v_scale,
+                                            __nv_bfloat162 k2, __nv_bfloat162 v2, int pair)
 {
-    float2 kf = __bfloat1622float2(k[pair]);
-    float2 vf = __bfloat1622float2(v[pair]);
+    float2 kf = __bfloat1622float2(k2);
+    float2 vf = __bfloat1622float2(v2);
     kf.x = __fmul_rn(kf.x, inv_k_scale);
     kf.y = __fmul_rn(kf.y, inv_k_scale);
     vf.x = __fmul_rn(vf.x, inv_v_scale);
@@ -57,6 +56,7 @@ __global__ void __launch_bounds__(D / 2) append_kernel(uint8_t* __restrict__ fp8
                                                         const int32_t* __restrict__ slots,
                                                         uint32_t* __restrict__ status)
 {
+    pdl_begin();
     const int tok = blockIdx.x, h = blockIdx.y;
     const int sm = slots[tok];
     if (sm < 0) return;
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(D / 2) append_kernel(uint8_t* __restrict__ fp8
     }
     uint8_t* rec = fp8 + (((size_t)page * hkv + h) * tiles + m) * fp8_record_bytes(D);
     const size_t src = ((size_t)tok * hkv + h) * (D / 2);
-    append_token<D>(rec, slot, inv_k_scale, inv_v_scale, k + src, v + src, threadIdx.x);
+    append_pair<D>(rec, slot, inv_k_scale, inv_v_scale, k[src + threadIdx.x], v[src + threadIdx.x], threadIdx.x);
 }
 
 // eight bf16 (one 16-byte load) -> eight e4m3 bytes
@@ -105,8 +105,9 @@ __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ f
     constexpr int VROW = D + 4;                      // padded token row of the transposition tile
     __shared__ __align__(16) uint8_t vt[kPage * VROW];
     __shared__ int32_t slot_s[2 * kPage];            // slots of this window and the next
-    __shared__ int32_t len_s[kPage];                 // runs that start at token i of the window and do not fill a tile
-    __shared__ int full_s;                           // token whose run fills a tile (at most one starts in a window), or -1
+    __shared__ int32_t rest_s[2 * kPage];            // tokens of the other runs that start in the window
+    __shared__ int full_s, n_rest_s;                 // token whose run fills a tile (at most one starts in a window), or -1
+    pdl_begin();
     const int t0 = blockIdx.x * kPage, h = blockIdx.y, tid = threadIdx.x;
     if (tid < 32) {
         const int sl = t0 + tid < n ? slots[t0 + tid] : -1;
@@ -122,8 +123,16 @@ __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ f
         }
         const bool full = len == kPage && (sl >> 4) / tiles < fp8_pages;
         const uint32_t m = __ballot_sync(0xffffffffu, full);
-        if (tid < kPage) len_s[tid] = full ? 0 : len;
+        if (full) len = 0;
+        int end = len;                               // running count of those tokens
+#pragma unroll
+        for (int o = 1; o < kPage; o <<= 1) {
+            const int before_me = __shfl_up_sync(0xffffffffu, end, o);
+            if (tid >= o) end += before_me;
+        }
+        for (int j = 0; j < len; ++j) rest_s[end - len + j] = tid + j;
         if (tid == 0) full_s = m ? __ffs(m) - 1 : -1;
+        if (tid == kPage - 1) n_rest_s = end;
     }
     __syncthreads();
     const int full = full_s;
@@ -160,20 +169,31 @@ __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ f
             }
         }
     }
-    constexpr int PAR = 256 / D;                     // tokens stored side by side
-    int next = 0;
-    for (int i = 0; i < kPage; ++i)
-        for (int j = 0; j < len_s[i]; ++j) {
-            if (next++ % PAR != tid / (D / 2)) continue;
-            const int sm = slot_s[i + j], gt = sm >> 4, page = gt / tiles;
+    // the rest token by token, the loads of four (token, element pair) items in flight per thread
+    const int n_items = n_rest_s * (D / 2);
+    for (int i0 = tid; i0 < n_items; i0 += 4 * 128) {
+        __nv_bfloat162 kk[4], vv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * 128;
+            if (i >= n_items) break;
+            const size_t src = ((size_t)(t0 + rest_s[i / (D / 2)]) * hkv + h) * (D / 2) + i % (D / 2);
+            kk[u] = k[src];
+            vv[u] = v[src];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * 128;
+            if (i >= n_items) break;
+            const int sm = slot_s[rest_s[i / (D / 2)]], gt = sm >> 4, page = gt / tiles;
             if (page >= fp8_pages) {
-                if (tid % (D / 2) == 0) atomicOr(status, kStBounds);
+                if (i % (D / 2) == 0) atomicOr(status, kStBounds);
                 continue;
             }
             uint8_t* rec = fp8 + (((size_t)page * hkv + h) * tiles + (gt - page * tiles)) * fp8_record_bytes(D);
-            const size_t src = ((size_t)(t0 + i + j) * hkv + h) * (D / 2);
-            append_token<D>(rec, sm & 15, inv_k_scale, inv_v_scale, k + src, v + src, tid % (D / 2));
+            append_pair<D>(rec, sm & 15, inv_k_scale, inv_v_scale, kk[u], vv[u], i % (D / 2));
         }
+    }
 }
 
 // Decode-sized append into the pools of several layers: one block per (token, KV head, layer).
@@ -190,6 +210,7 @@ template <int D>
 __global__ void __launch_bounds__(D / 2) append_layers_kernel(const AppendLayers A, int hkv, int tiles,
                                                                const int32_t* __restrict__ slots)
 {
+    pdl_begin();
     const int tok = blockIdx.x, h = blockIdx.y, layer = blockIdx.z;
     const int sm = slots[tok];
     if (sm < 0) return;
@@ -200,7 +221,8 @@ __global__ void __launch_bounds__(D / 2) append_layers_kernel(const AppendLayers
     }
     uint8_t* rec = A.fp8[layer] + (((size_t)page * hkv + h) * tiles + m) * fp8_record_bytes(D);
     const size_t src = ((size_t)tok * hkv + h) * (D / 2);
-    append_token<D>(rec, slot, A.inv_k_scale[layer], A.inv_v_scale[layer], A.k[layer] + src, A.v[layer] + src, threadIdx.x);
+    append_pair<D>(rec, slot, A.inv_k_scale[layer], A.inv_v_scale[layer], A.k[layer][src + threadIdx.x],
+                   A.v[layer][src + threadIdx.x], threadIdx.x);
 }
 
 int32_t launch_append_layers(mkv_pool* const* pools, const void* const* k, const void* const* v, const int32_t* slots,
@@ -218,31 +240,35 @@ int32_t launch_append_layers(mkv_pool* const* pools, const void* const* k, const
     }
     const mkv_pool* p = pools[0];
     dim3 grid(n, p->hkv, n_layers);
-    if (p->d == 128) append_layers_kernel<128><<<grid, 64, 0, s>>>(A, p->hkv, p->tiles, slots);
-    else append_layers_kernel<256><<<grid, 128, 0, s>>>(A, p->hkv, p->tiles, slots);
+    if (p->d == 128) MKV_CUDA(launch_pdl(append_layers_kernel<128>, grid, 64, 0, 1, true, s, A, p->hkv, p->tiles, slots));
+    else MKV_CUDA(launch_pdl(append_layers_kernel<256>, grid, 128, 0, 1, true, s, A, p->hkv, p->tiles, slots));
     MKV_CUDA(cudaGetLastError());
     return MKV_OK;
 }
+
+// Calls of fewer tokens than this take one block per token: a batch's new tokens, each in a page of its own.  At
+// 256 tokens both ways take 3.3 us (d = 128, 8 heads); at 64 tokens 2.0 us against 3.2 us.
+constexpr int kAppendRun = 256;
 
 int32_t launch_append(mkv_pool* p, const void* k, const void* v, const int32_t* slots, int n, cudaStream_t s)
 {
     const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale;
     const __nv_bfloat162* kk = (const __nv_bfloat162*)k;
     const __nv_bfloat162* vv = (const __nv_bfloat162*)v;
-    if (n >= 2 * kPage) {
+    if (n >= kAppendRun) {
         dim3 grid((n + kPage - 1) / kPage, p->hkv);
         if (p->d == 128)
-            append_run_kernel<128><<<grid, 128, 0, s>>>(p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
-                                                        p->status_dev);
+            MKV_CUDA(launch_pdl(append_run_kernel<128>, grid, 128, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
+                                                        p->status_dev));
         else
-            append_run_kernel<256><<<grid, 128, 0, s>>>(p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
-                                                        p->status_dev);
+            MKV_CUDA(launch_pdl(append_run_kernel<256>, grid, 128, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
+                                                        p->status_dev));
     } else {
         dim3 grid(n, p->hkv);
         if (p->d == 128)
-            append_kernel<128><<<grid, 64, 0, s>>>(p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev);
+            MKV_CUDA(launch_pdl(append_kernel<128>, grid, 64, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev));
         else
-            append_kernel<256><<<grid, 128, 0, s>>>(p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev);
+            MKV_CUDA(launch_pdl(append_kernel<256>, grid, 128, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev));
     }
     MKV_CUDA(cudaGetLastError());
     return MKV_OK;
@@ -277,23 +303,6 @@ static int heads_cluster(int hkv, int n_pages)
     for (int c = 8; c > 1; --c)
         if (hkv % c == 0) return c;
     return 1;
-}
-
-template <typename Kernel, typename... Args>
-static cudaError_t launch_clustered(Kernel kernel, int n_pages, int csize, int threads, cudaStream_t s, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)n_pages * csize);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = csize;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // ------------------------------------------------------------------------------------------ demote
@@ -703,6 +712,7 @@ __global__ void __launch_bounds__(D) demote_kernel(const uint8_t* __restrict__ f
 
     const int csize = (int)cluster_size(), crank = (int)cluster_rank();
     const int page = blockIdx.x / csize, tid = threadIdx.x, lane = tid & 31;
+    pdl_begin();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < fp8_pages && dst >= 0 && dst < tq3_pages;
     if (!valid && tid == 0 && crank == 0 && blockIdx.y == 0) atomicOr(status, kStBounds);
@@ -778,6 +788,7 @@ __global__ void __launch_bounds__(D) demote_minmax_kernel(const uint8_t* __restr
     __shared__ float part[2][D];
     const int csize = (int)cluster_size(), crank = (int)cluster_rank();
     const int unit = blockIdx.x / csize, page = unit / hkv, h = unit % hkv, c = threadIdx.x;
+    pdl_begin();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < fp8_pages && dst >= 0 && dst < tq3_pages;      // flagged by demote_kernel
     const uint8_t* page8 = fp8 + ((size_t)(valid ? src : 0) * hkv + h) * fp8_page_bytes(D, tiles);
@@ -849,6 +860,7 @@ __global__ void publish_kernel(int n, const int32_t* __restrict__ src_ids, const
                                const int64_t* __restrict__ entry_index, int64_t n_entries, int tag, uint32_t* status)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_begin();
     if (i >= n) return;
     const int src = src_ids[i], dst = dst_ids[i];
     if (src < 0 || src >= src_cap || dst < 0 || dst >= dst_cap) return;
@@ -875,31 +887,13 @@ static int tile_rows(int tiles, int n_pages, int hkv)
     return rows < tiles ? rows : tiles;
 }
 
-template <typename Kernel, typename... Args>
-static cudaError_t launch_clustered_rows(Kernel kernel, int n_pages, int csize, int rows, int threads, cudaStream_t s,
-                                         Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)n_pages * csize, rows);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = csize;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <int D, int FMT>
 static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
                                const int64_t* entry, int64_t n_entries, cudaStream_t s)
 {
-    const int c = heads_cluster(p->hkv, n);
     if (p->tiles == 1) {
-        MKV_CUDA(launch_clustered(demote_kernel<D, false, FMT>, n, c, D, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
+        const int c = heads_cluster(p->hkv, n);
+        MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, 1, p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, bt,
                                   tags, entry, n_entries, p->status_dev, (uint32_t*)nullptr));
         return MKV_OK;
@@ -911,20 +905,20 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
         // blocks per (page, head): up to a portable cluster of 8, fewer when the call fills the GPU anyway
         int cs = 8;
         while (cs > 1 && (cs > p->tiles || (long long)n * p->hkv * cs > 8LL * 148)) cs >>= 1;
-        MKV_CUDA(launch_clustered(demote_minmax_kernel<D>, n * p->hkv, cs, D, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
+        MKV_CUDA(launch_pdl(demote_minmax_kernel<D>, dim3((unsigned)n * p->hkv * cs), D, 0, cs, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, p->tiles, p->cfg.v_scale, src, dst));
     }
-    MKV_CUDA(launch_clustered_rows(demote_kernel<D, true, FMT>, n, heads_cluster(p->hkv, 0), tile_rows(p->tiles, n, p->hkv), D, s,
+    const int ch = heads_cluster(p->hkv, 0);
+    MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, n <= 148, s,
                                    (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv, p->tiles,
                                    p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr,
                                    fused ? tags : (uint8_t*)nullptr, fused ? entry : (const int64_t*)nullptr,
                                    fused ? n_entries : (int64_t)0, p->status_dev, fused ? page_tickets(p) : (uint32_t*)nullptr));
     if (entry && !fused) {
-        publish_kernel<<<(n + 127) / 128, 128, 0, s>>>(n, src, dst, p->cfg.fp8_pages, p->cfg.tq3_pages, bt, tags, entry,
-                                                       n_entries, MKV_TAG_STALE, p->status_dev);
+        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, true, s, n, src, dst, p->cfg.fp8_pages, p->cfg.tq3_pages, bt, tags, entry,
+                                                       n_entries, MKV_TAG_STALE, p->status_dev));
         MKV_CUDA(cudaGetLastError());
     }
-    (void)c;
     return MKV_OK;
 }
 
@@ -1107,6 +1101,7 @@ __global__ void __launch_bounds__(D) promote_kernel(const uint8_t* __restrict__ 
 
     const int csize = (int)cluster_size(), crank = (int)cluster_rank();
     const int page = blockIdx.x / csize, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_begin();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < tq3_pages && dst >= 0 && dst < fp8_pages;
     if (!valid && tid == 0 && crank == 0 && blockIdx.y == 0) atomicOr(status, kStBounds);
@@ -1320,21 +1315,22 @@ static int32_t launch_promote_d(mkv_pool* p, const int32_t* src, const int32_t* 
 {
     const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale;
     const float rs = (float)(1.0 / sqrt((double)p->d));
+    const int c = heads_cluster(p->hkv, p->tiles == 1 ? n : 0);
     if (p->tiles == 1) {
-        MKV_CUDA(launch_clustered(promote_kernel<D, false, FMT>, n, heads_cluster(p->hkv, n), D, s, (const uint8_t*)p->tq3, p->fp8,
+        MKV_CUDA(launch_pdl(promote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, n <= 148, s, (const uint8_t*)p->tq3, p->fp8,
                                   p->cfg.tq3_pages, p->cfg.fp8_pages, p->hkv, 1, ik, iv, rs, p->sigma, src, dst, bt, tags,
                                   entry, n_entries, p->status_dev, (uint32_t*)nullptr));
         return MKV_OK;
     }
     const bool fused = entry != nullptr && n <= kPageTickets;
-    MKV_CUDA(launch_clustered_rows(promote_kernel<D, true, FMT>, n, heads_cluster(p->hkv, 0), tile_rows(p->tiles, n, p->hkv), D, s,
+    MKV_CUDA(launch_pdl(promote_kernel<D, true, FMT>, dim3((unsigned)n * c, tile_rows(p->tiles, n, p->hkv)), D, 0, c, n <= 148, s,
                                    (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages, p->hkv, p->tiles, ik,
                                    iv, rs, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr, fused ? tags : (uint8_t*)nullptr,
                                    fused ? entry : (const int64_t*)nullptr, fused ? n_entries : (int64_t)0, p->status_dev,
                                    fused ? page_tickets(p) : (uint32_t*)nullptr));
     if (entry && !fused) {
-        publish_kernel<<<(n + 127) / 128, 128, 0, s>>>(n, src, dst, p->cfg.tq3_pages, p->cfg.fp8_pages, bt, tags, entry,
-                                                       n_entries, MKV_TAG_ANCHOR, p->status_dev);
+        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, true, s, n, src, dst, p->cfg.tq3_pages, p->cfg.fp8_pages, bt, tags, entry,
+                                                       n_entries, MKV_TAG_ANCHOR, p->status_dev));
         MKV_CUDA(cudaGetLastError());
     }
     return MKV_OK;
@@ -1353,6 +1349,7 @@ int32_t launch_promote(mkv_pool* p, const int32_t* src, const int32_t* dst, int 
 // ------------------------------------------------------------------------------------------ anchor
 __global__ void set_anchor_kernel(uint8_t* tags, int64_t entry, int flag, uint32_t* status)
 {
+    pdl_begin();
     if (tags[entry] == MKV_TAG_STALE)
         atomicOr(status, kStState);
     else
@@ -1361,7 +1358,7 @@ __global__ void set_anchor_kernel(uint8_t* tags, int64_t entry, int flag, uint32
 
 int32_t launch_set_anchor(mkv_pool* p, uint8_t* tags, int64_t entry, int flag, cudaStream_t s)
 {
-    set_anchor_kernel<<<1, 1, 0, s>>>(tags, entry, flag, p->status_dev);
+    MKV_CUDA(launch_pdl(set_anchor_kernel, dim3(1), 1, 0, 1, true, s, tags, entry, flag, p->status_dev));
     MKV_CUDA(cudaGetLastError());
     return MKV_OK;
 }

@@ -101,6 +101,46 @@ struct mkv_seq {
 };
 
 namespace mkv {
+// Programmatic dependent launch.  Every kernel of the library is launched so that it may start while the kernel
+// before it in the stream is still running, and begins with pdl_begin(): it lets the kernel behind it start in turn
+// and then waits until everything before it has completed and is visible.  What a kernel does not need to wait for
+// (its launch, shared-memory set-up) then overlaps its predecessor: an append + decode pair of a small call takes
+// 2 us less.  Order and visibility are those of ordinary stream order.
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// early: start before the predecessor has ended.  Not for a grid of one or two waves of long blocks: blocks placed
+// while the predecessor still holds some SMs spread unevenly (Promote of 1,023 pages 33 -> 36 us).
+// cluster: blocks per thread-block cluster along x (1: none)
+template <typename Kernel, typename... Args>
+static cudaError_t launch_pdl(Kernel kernel, dim3 grid, int threads, size_t smem, int cluster, bool early, cudaStream_t s,
+                              const Args&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    unsigned n = 0;
+    if (early) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 int32_t cuda_fail(cudaError_t e, const char* what);
 #define MKV_CUDA(call)                                         \
     do {                                                       \

@@ -254,17 +254,9 @@ __device__ __forceinline__ void key_lut4(uint32_t sel, uint32_t& r0, uint32_t& r
 }
 
 // Two 3-bit value codes sitting at bit POS of each 16-bit half of x -> half2 of the integer codes.
-// (x & mask) | 0x6400 is the fp16 number 1024 + code * 2^POS; one FMA recovers the code exactly.
-// The per-channel scale and zero are applied in fp32 after the token sum:
-//   sum_t p_t (scale*code_t + zero) = scale * (sum_t p_t code_t) + zero * (sum_t p_t).
-// The multiplier of the value unpack is read from the constant bank.  Written as a literal it needs a register
-// (the inline PTX takes register operands) beside the one of the addend, and the scan is short of registers: the
-// compiler then rebuilds literals with a move before every use.  Measured: 2 % of a layer's time; doing the same
-// to the masks of the LOP3s, or writing these operations as plain expressions, made the scan slower.
-// 2^-POS as fp16 pairs (exponent arithmetic on 1.0 = 0x3C00)
-__constant__ uint32_t kValueMul[8] = {0x3C003C00u, 0x38003800u, 0x34003400u, 0x30003000u,
-                                      0x2C002C00u, 0x28002800u, 0x24002400u, 0x20002000u};
-template <int POS, bool CB = false>      // CB: multiplier from the constant bank (it pays in the format-2 scan only)
+// (x & mask) | 0x6400 is the fp16 number 1024 + code * 2^POS; one FMA recovers the code exactly.  (For operands that
+// have to be the codes themselves; the mma.sync scan uses value_bits.)
+template <int POS>
 __device__ __forceinline__ uint32_t value_code(uint32_t x)
 {
     constexpr uint32_t mask = 0x00070007u << POS;
@@ -272,7 +264,42 @@ __device__ __forceinline__ uint32_t value_code(uint32_t x)
     // 2^-POS and -1024 * 2^-POS as fp16 pairs (exponent arithmetic on 1.0 = 0x3C00, -1024 = 0xE400)
     constexpr uint32_t mul = (0x3C00u - (POS << 10)) * 0x00010001u;
     constexpr uint32_t add = (0xE400u - (POS << 10)) * 0x00010001u;
-    return hfma2_u32(u, CB ? kValueMul[POS] : mul, add);
+    return hfma2_u32(u, mul, add);
+}
+
+// The same two codes as they stand: bits below 2^11 read as an fp16 number are worth bits * 2^-24 (subnormals, and
+// the first binade above them, are one linear scale), so masking alone gives the exact operand code * 2^(POS - 24).
+// The powers of two are taken out again where they cost nothing or little (see value_operands).  Against value_code
+// this removes one half-rate FMA per two codes, a twelfth of the scan's instructions.
+template <int POS>
+__device__ __forceinline__ uint32_t value_bits(uint32_t x)
+{
+    static_assert(POS <= 8, "bits below 2^11 are linear");
+    return x & (0x00070007u << POS);
+}
+
+// A operands of the four channel blocks of a word triple, as code * 2^e.  In every row of every block the codes of
+// tokens 0-7 (registers 0, 1) stand two bits higher than those of tokens 8-15 (registers 2, 3), so the
+// probabilities of tokens 8-15 enter the product four times as large.  What is left is one power of two per row,
+// value_unit<block, row / 8>(), which goes into the row's scale.
+template <int BLOCK>
+__device__ __forceinline__ void value_operands(uint32_t (&a)[4], uint32_t W0, uint32_t W1, uint32_t W2, uint32_t X)
+{
+    if constexpr (BLOCK == 0) {          // X = bytes of W0, W1 between the two
+        a[0] = value_bits<8>(W0 << 8); a[1] = value_bits<3>(W0); a[2] = value_bits<6>(W0); a[3] = value_bits<1>(X);
+    } else if constexpr (BLOCK == 1) {
+        a[0] = value_bits<4>(X); a[1] = value_bits<7>(X); a[2] = value_bits<2>(W1); a[3] = value_bits<5>(W1);
+    } else if constexpr (BLOCK == 2) {   // X = bytes of W1, W2; its bytes 0 and 2 are bytes 1 and 3 of W1
+        a[0] = value_bits<8>(W1); a[1] = value_bits<3>(X); a[2] = value_bits<6>(X); a[3] = value_bits<1>(W2);
+    } else {
+        const uint32_t X2 = W2 >> 8;
+        a[0] = value_bits<4>(W2); a[1] = value_bits<7>(W2); a[2] = value_bits<2>(X2); a[3] = value_bits<5>(X2);
+    }
+}
+template <int BLOCK, int HI>      // what a unit of the sums is worth in codes: 2^(24 - POS) of the row's register 0 / 1
+__device__ __forceinline__ constexpr float value_unit()
+{
+    return BLOCK % 2 == 0 ? (HI ? 2097152.f : 65536.f) : (HI ? 131072.f : 1048576.f);
 }
 
 __device__ __forceinline__ float2 half2_to_float2(uint32_t x)
@@ -280,15 +307,17 @@ __device__ __forceinline__ float2 half2_to_float2(uint32_t x)
     return __half22float2(*reinterpret_cast<const __half2*>(&x));
 }
 
-// acc[channel rows g, g+8][heads] += scale_row * t + zero_row * psum_head
+// acc[channel rows g, g+8][heads] += scale_row * t + zero_row * psum_head, t in units of value_unit<BLOCK, row>
+template <int BLOCK>
 __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (&t)[4], uint32_t sc_pair, uint32_t zp_pair,
                                                   float ps0, float ps1)
 {
     const float2 sc = half2_to_float2(sc_pair), zp = half2_to_float2(zp_pair);
-    acc[0] = fmaf(sc.x, t[0], fmaf(zp.x, ps0, acc[0]));
-    acc[1] = fmaf(sc.x, t[1], fmaf(zp.x, ps1, acc[1]));
-    acc[2] = fmaf(sc.y, t[2], fmaf(zp.y, ps0, acc[2]));
-    acc[3] = fmaf(sc.y, t[3], fmaf(zp.y, ps1, acc[3]));
+    const float s0 = sc.x * value_unit<BLOCK, 0>(), s1 = sc.y * value_unit<BLOCK, 1>();     // exact
+    acc[0] = fmaf(s0, t[0], fmaf(zp.x, ps0, acc[0]));
+    acc[1] = fmaf(s0, t[1], fmaf(zp.x, ps1, acc[1]));
+    acc[2] = fmaf(s1, t[2], fmaf(zp.y, ps0, acc[2]));
+    acc[3] = fmaf(s1, t[3], fmaf(zp.y, ps1, acc[3]));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -532,11 +561,14 @@ __device__ __forceinline__ void softmax_rescale(WarpAcc<NB>& acc, const float (&
 }
 
 // Second half, branch-free (so that it can be scheduled into the unpack work of the next page): P and its row sums.
-template <int NB>
+// STALE: the operands of the second token half are four times the probabilities (value_operands); the row sums
+// take the factor out again.
+template <int NB, bool STALE>
 __device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf)
 {
+    const float up = STALE ? 2.f : 0.f;
     const float p0 = fast_exp2(s[0] - acc.m[0]), p1 = fast_exp2(s[1] - acc.m[1]);
-    const float p2 = fast_exp2(s[2] - acc.m[0]), p3 = fast_exp2(s[3] - acc.m[1]);
+    const float p2 = fast_exp2(s[2] - (acc.m[0] - up)), p3 = fast_exp2(s[3] - (acc.m[1] - up));
     const uint32_t ph01 = pack_f16x2(p0, p1), ph23 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(ph01), h23 = half2_to_float2(ph23);
     pf.b0 = movmatrix_trans(ph01);
@@ -544,7 +576,7 @@ __device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)
     pf.c0 = movmatrix_trans(pack_f16x2(p0 - h01.x, p1 - h01.y));
     pf.c1 = movmatrix_trans(pack_f16x2(p2 - h23.x, p3 - h23.y));
     // row sums through the tensor core: the same P that multiplies V
-    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u};
+    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, STALE ? 0x34003400u : 0x3C003C00u, STALE ? 0x34003400u : 0x3C003C00u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
     mma16816(ps, ones, pf.c0, pf.c1);
@@ -558,7 +590,7 @@ template <int NB>
 __device__ __forceinline__ void softmax_page(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf)
 {
     softmax_rescale<NB>(acc, s);
-    softmax_probs<NB>(acc, s, pf);
+    softmax_probs<NB, false>(acc, s, pf);
 }
 
 // Scored variant (Section 3.1): log2 of the page's exponential sum, referred to an absolute origin
@@ -637,64 +669,38 @@ __device__ __forceinline__ void tq3_key_quad(float (&S0)[4], float (&S1)[4], uin
 
 // Output update of the four channel blocks 4j..4j+3 of a Stale page: integer codes through the tensor
 // core, then the fp16 scale and zero of every channel applied to the 16x8 result in fp32.
-template <bool DEFER = false, bool CB = false>
+// DEFER: sum p * code only, the accumulators are in units of value_unit until the page is left.
+template <bool DEFER = false>
 __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], float (&o2)[4], float (&o3)[4],
                                                uint32_t W0, uint32_t W1, uint32_t W2, uint32_t meta_quad, const PFrag& pf)
 {
     float t[4];
     uint32_t a[4];
-    if constexpr (DEFER) {
-        // sum p * code only: the accumulators are in code units until the page is left
-        const uint32_t X1 = prmt(W0, W1, 0x6341u), X0 = prmt(W1, W2, 0x6341u), X2 = W2 >> 8;
-        a[0] = value_code<0, CB>(W0); a[1] = value_code<3, CB>(W0); a[2] = value_code<6, CB>(W0); a[3] = value_code<1, CB>(X1);
-        mma16816(o0, a, pf.b0, pf.b1);
-        mma16816(o0, a, pf.c0, pf.c1);
-        a[0] = value_code<4, CB>(X1); a[1] = value_code<7, CB>(X1); a[2] = value_code<2, CB>(W1); a[3] = value_code<5, CB>(W1);
-        mma16816(o1, a, pf.b0, pf.b1);
-        mma16816(o1, a, pf.c0, pf.c1);
-        a[0] = value_code<0, CB>(X0); a[1] = value_code<3, CB>(X0); a[2] = value_code<6, CB>(X0); a[3] = value_code<1, CB>(W2);
-        mma16816(o2, a, pf.b0, pf.b1);
-        mma16816(o2, a, pf.c0, pf.c1);
-        a[0] = value_code<4, CB>(W2); a[1] = value_code<7, CB>(W2); a[2] = value_code<2, CB>(X2); a[3] = value_code<5, CB>(X2);
-        mma16816(o3, a, pf.b0, pf.b1);
-        mma16816(o3, a, pf.c0, pf.c1);
-        return;
-    }
+    auto product = [&](float (&o)[4]) {
+        if constexpr (DEFER) mma16816(o, a, pf.b0, pf.b1);
+        else mma16816_zero(o, a, pf.b0, pf.b1);
+        mma16816(o, a, pf.c0, pf.c1);
+    };
+    uint4 mt;
     {   // blocks 4j, 4j+1
-        const uint4 mt = lds128(meta_quad);
-        const uint32_t X1 = prmt(W0, W1, 0x6341u);
-        a[0] = value_code<0, CB>(W0);
-        a[1] = value_code<3, CB>(W0);
-        a[2] = value_code<6, CB>(W0);
-        a[3] = value_code<1, CB>(X1);
-        mma16816_zero(t, a, pf.b0, pf.b1);
-        mma16816(t, a, pf.c0, pf.c1);
-        affine_accumulate(o0, t, mt.x, mt.y, pf.ps0, pf.ps1);
-        a[0] = value_code<4, CB>(X1);
-        a[1] = value_code<7, CB>(X1);
-        a[2] = value_code<2, CB>(W1);
-        a[3] = value_code<5, CB>(W1);
-        mma16816_zero(t, a, pf.b0, pf.b1);
-        mma16816(t, a, pf.c0, pf.c1);
-        affine_accumulate(o1, t, mt.z, mt.w, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) mt = lds128(meta_quad);
+        const uint32_t X = prmt(W0, W1, 0x6341u);
+        value_operands<0>(a, W0, W1, W2, X);
+        product(DEFER ? o0 : t);
+        if constexpr (!DEFER) affine_accumulate<0>(o0, t, mt.x, mt.y, pf.ps0, pf.ps1);
+        value_operands<1>(a, W0, W1, W2, X);
+        product(DEFER ? o1 : t);
+        if constexpr (!DEFER) affine_accumulate<1>(o1, t, mt.z, mt.w, pf.ps0, pf.ps1);
     }
     {   // blocks 4j+2, 4j+3
-        const uint4 mt = lds128(meta_quad + 128);
-        const uint32_t X0 = prmt(W1, W2, 0x6341u), X2 = W2 >> 8;
-        a[0] = value_code<0, CB>(X0);
-        a[1] = value_code<3, CB>(X0);
-        a[2] = value_code<6, CB>(X0);
-        a[3] = value_code<1, CB>(W2);
-        mma16816_zero(t, a, pf.b0, pf.b1);
-        mma16816(t, a, pf.c0, pf.c1);
-        affine_accumulate(o2, t, mt.x, mt.y, pf.ps0, pf.ps1);
-        a[0] = value_code<4, CB>(W2);
-        a[1] = value_code<7, CB>(W2);
-        a[2] = value_code<2, CB>(X2);
-        a[3] = value_code<5, CB>(X2);
-        mma16816_zero(t, a, pf.b0, pf.b1);
-        mma16816(t, a, pf.c0, pf.c1);
-        affine_accumulate(o3, t, mt.z, mt.w, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) mt = lds128(meta_quad + 128);
+        const uint32_t X = prmt(W1, W2, 0x6341u);
+        value_operands<2>(a, W0, W1, W2, X);
+        product(DEFER ? o2 : t);
+        if constexpr (!DEFER) affine_accumulate<2>(o2, t, mt.x, mt.y, pf.ps0, pf.ps1);
+        value_operands<3>(a, W0, W1, W2, X);
+        product(DEFER ? o3 : t);
+        if constexpr (!DEFER) affine_accumulate<3>(o3, t, mt.z, mt.w, pf.ps0, pf.ps1);
     }
 }
 
@@ -796,18 +802,19 @@ __device__ __forceinline__ void softmax_rescale_v2(WarpAcc<NB>& acc, const float
     }
 }
 
-// P of head g for the lane's four tokens is the B fragment of the value product as it stands.
+// P of head g for the lane's four tokens is the B fragment of the value product as it stands (tokens 8-15 four
+// times as large, see value_operands).
 template <int NB>
 __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf)
 {
     const float p0 = fast_exp2(s[0] - acc.mr), p1 = fast_exp2(s[1] - acc.mr);
-    const float p2 = fast_exp2(s[2] - acc.mr), p3 = fast_exp2(s[3] - acc.mr);
+    const float p2 = fast_exp2(s[2] - (acc.mr - 2.f)), p3 = fast_exp2(s[3] - (acc.mr - 2.f));
     pf.b0 = pack_f16x2(p0, p1);
     pf.b1 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(pf.b0), h23 = half2_to_float2(pf.b1);
     pf.c0 = pack_f16x2(p0 - h01.x, p1 - h01.y);
     pf.c1 = pack_f16x2(p2 - h23.x, p3 - h23.y);
-    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u};
+    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x34003400u, 0x34003400u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
     mma16816(ps, ones, pf.c0, pf.c1);
@@ -834,7 +841,7 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
     if constexpr (DO_V) load_lane_words<D>(rec_v + 6 * D, lane, vw);
     if constexpr (DO_V) {      // in one block with the key unpack of the next page
         if constexpr (FMT == 2) softmax_probs_v2<NB>(acc, s_cur, pf);
-        else softmax_probs<NB>(acc, s_cur, pf);
+        else softmax_probs<NB, true>(acc, s_cur, pf);
     }
     if constexpr (DO_V && DEFER) {
         acc.lp[0] += pf.ps0;
@@ -851,7 +858,7 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
             else tq3_key_quad(S0, S1, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * 2048);
         }
         if constexpr (DO_V)
-            tq3_value_quad<DEFER, FMT == 2>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
+            tq3_value_quad<DEFER>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
                                   vw[3 * j + 2], meta + j * 256, pf);
     }
     if constexpr (DO_K && FMT == 2) {
@@ -1391,7 +1398,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int i = 4 * j + q;
-                    const float2 sc = half2_to_float2(scp[q]), zp = half2_to_float2(zpp[q]);
+                    float2 sc = half2_to_float2(scp[q]);
+                    const float2 zp = half2_to_float2(zpp[q]);
+                    sc.x *= q % 2 == 0 ? value_unit<0, 0>() : value_unit<1, 0>();
+                    sc.y *= q % 2 == 0 ? value_unit<0, 1>() : value_unit<1, 1>();
                     float r[4];
                     r[0] = fmaf(park[(i * 4 + 0) * 32 + lane], acc.pk[0], fmaf(sc.x, acc.o[i][0], zp.x * acc.lp[0]));
                     r[1] = fmaf(park[(i * 4 + 1) * 32 + lane], acc.pk[1], fmaf(sc.x, acc.o[i][1], zp.x * acc.lp[1]));

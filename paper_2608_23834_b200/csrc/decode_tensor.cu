@@ -524,6 +524,13 @@ struct WarpAcc {
 // Updates the running maximum (only when it is exceeded by more than 2^kRescaleSlack, so that
 // accumulators are rarely rescaled), and returns P^T as MMA B fragments split into an fp16 pair
 // hi (pb) + lo (pc), plus the page's row sums ps[0..1].
+//
+// SPLIT (groups of at most four query heads, kernel template parameter): the head columns 4-7 of the MMAs, which would
+// stand idle, carry the low halves of heads 0-3, so that ONE MMA does the work of the pair hi + lo: scores, maxima and
+// probabilities of heads 0-3 are present twice (columns or rows h and h + 4), b0, b1 hold the high halves in columns
+// 0-3 and the low halves in columns 4-7, and the two column halves of the output tile are added when the block
+// reduces it.  The same products and sums, half the tensor-core instructions (17 instead of 34 per Stale page at
+// d = 128): each of them holds up the issue of everything else for about five cycles.
 struct PFrag {
     uint32_t b0, b1, c0, c1;
     float ps0, ps1;
@@ -563,34 +570,40 @@ __device__ __forceinline__ void softmax_rescale(WarpAcc<NB>& acc, const float (&
 // Second half, branch-free (so that it can be scheduled into the unpack work of the next page): P and its row sums.
 // STALE: the operands of the second token half are four times the probabilities (value_operands); the row sums
 // take the factor out again.
-template <int NB, bool STALE>
-__device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf)
+template <int NB, bool STALE, bool SPLIT>
+__device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
     const float up = STALE ? 2.f : 0.f;
     const float p0 = fast_exp2(s[0] - acc.m[0]), p1 = fast_exp2(s[1] - acc.m[1]);
     const float p2 = fast_exp2(s[2] - (acc.m[0] - up)), p3 = fast_exp2(s[3] - (acc.m[1] - up));
     const uint32_t ph01 = pack_f16x2(p0, p1), ph23 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(ph01), h23 = half2_to_float2(ph23);
-    pf.b0 = movmatrix_trans(ph01);
-    pf.b1 = movmatrix_trans(ph23);
-    pf.c0 = movmatrix_trans(pack_f16x2(p0 - h01.x, p1 - h01.y));
-    pf.c1 = movmatrix_trans(pack_f16x2(p2 - h23.x, p3 - h23.y));
+    const uint32_t pl01 = pack_f16x2(p0 - h01.x, p1 - h01.y), pl23 = pack_f16x2(p2 - h23.x, p3 - h23.y);
+    if constexpr (SPLIT) {                   // columns 2tq, 2tq + 1 of lanes with tq >= 2 carry the low halves
+        pf.b0 = movmatrix_trans(lane & 2 ? pl01 : ph01);
+        pf.b1 = movmatrix_trans(lane & 2 ? pl23 : ph23);
+    } else {
+        pf.b0 = movmatrix_trans(ph01);
+        pf.b1 = movmatrix_trans(ph23);
+        pf.c0 = movmatrix_trans(pl01);
+        pf.c1 = movmatrix_trans(pl23);
+    }
     // row sums through the tensor core: the same P that multiplies V
     const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, STALE ? 0x34003400u : 0x3C003C00u, STALE ? 0x34003400u : 0x3C003C00u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
-    mma16816(ps, ones, pf.c0, pf.c1);
+    if constexpr (!SPLIT) mma16816(ps, ones, pf.c0, pf.c1);
     pf.ps0 = ps[0];
     pf.ps1 = ps[1];
     acc.l[0] += ps[0];
     acc.l[1] += ps[1];
 }
 
-template <int NB>
-__device__ __forceinline__ void softmax_page(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf)
+template <int NB, bool SPLIT>
+__device__ __forceinline__ void softmax_page(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
     softmax_rescale<NB>(acc, s);
-    softmax_probs<NB, false>(acc, s, pf);
+    softmax_probs<NB, false, SPLIT>(acc, s, pf, lane);
 }
 
 // Scored variant (Section 3.1): log2 of the page's exponential sum, referred to an absolute origin
@@ -613,10 +626,14 @@ __device__ __forceinline__ void atomic_log2_add(float* addr, float v)
 }
 
 // ACCUMULATE: the entry receives a part of the page (a tile, or a run of tiles) and is added to, not stored.
-template <int NB, bool ACCUMULATE = false>
+template <int NB, bool SPLIT, bool ACCUMULATE = false>
 __device__ __forceinline__ void store_page_mass(const WarpAcc<NB>& acc, float ps0, float ps1, float* mass_pg, int mass_stride,
                                                 int GQ, int lane)
 {
+    if constexpr (SPLIT) {
+        ps0 += __shfl_xor_sync(0xffffffffu, ps0, 2);
+        ps1 += __shfl_xor_sync(0xffffffffu, ps1, 2);
+    }
     if (lane < 4) {                  // g == 0: one lane per head pair
         const int h0 = 2 * lane;
         const float v0 = __log2f(ps0) + acc.m[0], v1 = __log2f(ps1) + acc.m[1];
@@ -648,6 +665,7 @@ __device__ __forceinline__ void load_lane_words(uint32_t sec, int lane, uint32_t
 
 // Scores of the four key blocks 4j..4j+3 of a Stale page: 12 byte-table lookups per block pair and two
 // MMAs per block (query hi and lo).
+template <bool SPLIT>
 __device__ __forceinline__ void tq3_key_quad(float (&S0)[4], float (&S1)[4], uint32_t A, uint32_t Bw, uint32_t Cw,
                                              uint32_t q_quad)
 {
@@ -661,6 +679,12 @@ __device__ __forceinline__ void tq3_key_quad(float (&S0)[4], float (&S1)[4], uin
         uint32_t a[4];
         key_lut4(sel[w], a[0], a[1]);
         key_lut4(sel[w] >> 16, a[2], a[3]);
+        if constexpr (SPLIT) {                             // {b0, b1}: hi in columns 0-3, lo in columns 4-7
+            const uint2 q = lds64(q_quad + w * 256);
+            if (w & 1) mma16816(S1, a, q.x, q.y);
+            else       mma16816(S0, a, q.x, q.y);
+            continue;
+        }
         const uint4 q = lds128(q_quad + w * 512);          // {hi b0, hi b1, lo b0, lo b1}
         if (w & 1) { mma16816(S1, a, q.x, q.y); mma16816(S1, a, q.z, q.w); }
         else       { mma16816(S0, a, q.x, q.y); mma16816(S0, a, q.z, q.w); }
@@ -670,7 +694,7 @@ __device__ __forceinline__ void tq3_key_quad(float (&S0)[4], float (&S1)[4], uin
 // Output update of the four channel blocks 4j..4j+3 of a Stale page: integer codes through the tensor
 // core, then the fp16 scale and zero of every channel applied to the 16x8 result in fp32.
 // DEFER: sum p * code only, the accumulators are in units of value_unit until the page is left.
-template <bool DEFER = false>
+template <bool DEFER, bool SPLIT>
 __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], float (&o2)[4], float (&o3)[4],
                                                uint32_t W0, uint32_t W1, uint32_t W2, uint32_t meta_quad, const PFrag& pf)
 {
@@ -679,7 +703,7 @@ __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], f
     auto product = [&](float (&o)[4]) {
         if constexpr (DEFER) mma16816(o, a, pf.b0, pf.b1);
         else mma16816_zero(o, a, pf.b0, pf.b1);
-        mma16816(o, a, pf.c0, pf.c1);
+        if constexpr (!SPLIT) mma16816(o, a, pf.c0, pf.c1);
     };
     uint4 mt;
     {   // blocks 4j, 4j+1
@@ -720,7 +744,9 @@ __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], f
 // (step, token half u, K half), then per step and token half one MMA for digits 0,1 and one for digit 2.
 // q_pair: shared-memory address of this lane's query fragments of step 2j (digits 0,1 at +0, digit 2 at +512,
 // step 2j+1 at +1024).
-template <bool FIRST>      // FIRST: the page's first two steps start the four sums
+// SPLIT: one MMA per step and token half; rows 0-3 digit 0, 4-7 digit 1, 8-11 and 12-15 digit 2 of heads 0-3
+// (step 2j at +0, step 2j+1 at +512).
+template <bool FIRST, bool SPLIT>      // FIRST: the page's first two steps start the four sums
 __device__ __forceinline__ void tq3_key_pair_v2(int (&Sa0)[4], int (&Sb0)[4], int (&Sa1)[4], int (&Sb1)[4],
                                                 uint32_t A, uint32_t Bw, uint32_t Cw, uint32_t q_pair)
 {
@@ -738,6 +764,17 @@ __device__ __forceinline__ void tq3_key_pair_v2(int (&Sa0)[4], int (&Sb0)[4], in
     }
 #pragma unroll
     for (int st = 0; st < 2; ++st) {
+        if constexpr (SPLIT) {
+            const uint4 q = lds128(q_pair + st * 512);
+            if (FIRST && st == 0) {
+                mma16832_s8_zero(Sa0, q.x, q.y, q.z, q.w, r[0], r[1]);
+                mma16832_s8_zero(Sa1, q.x, q.y, q.z, q.w, r[2], r[3]);
+            } else {
+                mma16832_s8(Sa0, q.x, q.y, q.z, q.w, r[4 * st], r[4 * st + 1]);
+                mma16832_s8(Sa1, q.x, q.y, q.z, q.w, r[4 * st + 2], r[4 * st + 3]);
+            }
+            continue;
+        }
         // (the second fragment's rows 8-15 are stored as zeros: a full 16-byte load keeps the four operand
         // registers together, where building {x, 0, y, 0} cost two moves per MMA)
         const uint4 qa = lds128(q_pair + st * 1024), qb = lds128(q_pair + st * 1024 + 512);
@@ -804,8 +841,8 @@ __device__ __forceinline__ void softmax_rescale_v2(WarpAcc<NB>& acc, const float
 
 // P of head g for the lane's four tokens is the B fragment of the value product as it stands (tokens 8-15 four
 // times as large, see value_operands).
-template <int NB>
-__device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf)
+template <int NB, bool SPLIT>
+__device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
     const float p0 = fast_exp2(s[0] - acc.mr), p1 = fast_exp2(s[1] - acc.mr);
     const float p2 = fast_exp2(s[2] - (acc.mr - 2.f)), p3 = fast_exp2(s[3] - (acc.mr - 2.f));
@@ -814,10 +851,14 @@ __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (
     const float2 h01 = half2_to_float2(pf.b0), h23 = half2_to_float2(pf.b1);
     pf.c0 = pack_f16x2(p0 - h01.x, p1 - h01.y);
     pf.c1 = pack_f16x2(p2 - h23.x, p3 - h23.y);
+    if constexpr (SPLIT) {                   // rows 4-7 carry the low halves of heads 0-3
+        pf.b0 = lane & 16 ? pf.c0 : pf.b0;
+        pf.b1 = lane & 16 ? pf.c1 : pf.b1;
+    }
     const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x34003400u, 0x34003400u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
-    mma16816(ps, ones, pf.c0, pf.c1);
+    if constexpr (!SPLIT) mma16816(ps, ones, pf.c0, pf.c1);
     pf.ps0 = ps[0];
     pf.ps1 = ps[1];
     acc.l[0] += ps[0];
@@ -828,7 +869,7 @@ __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (
 // probabilities pf) and the score phase of the next page (record rec_k) are issued quad by quad in
 // one instruction stream, so that table lookups, half-precision FMAs, fp32 FMAs and MMAs of the two
 // phases overlap.  DO_V / DO_K switch the halves off for the first and the last page.
-template <int D, bool DO_V, bool DO_K, bool DEFER = false, int FMT = 1>
+template <int D, bool DO_V, bool DO_K, bool DEFER, int FMT, bool SPLIT>
 __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, const float (&s_cur)[4], PFrag& pf, uint32_t rec_k,
                                          uint32_t qt_lane, float sc2, int lane, float (&s_next)[4])
 {
@@ -840,8 +881,8 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
     if constexpr (DO_K) load_lane_words<D>(rec_k, lane, kw);
     if constexpr (DO_V) load_lane_words<D>(rec_v + 6 * D, lane, vw);
     if constexpr (DO_V) {      // in one block with the key unpack of the next page
-        if constexpr (FMT == 2) softmax_probs_v2<NB>(acc, s_cur, pf);
-        else softmax_probs<NB, true>(acc, s_cur, pf);
+        if constexpr (FMT == 2) softmax_probs_v2<NB, SPLIT>(acc, s_cur, pf, lane);
+        else softmax_probs<NB, true, SPLIT>(acc, s_cur, pf, lane);
     }
     if constexpr (DO_V && DEFER) {
         acc.lp[0] += pf.ps0;
@@ -852,13 +893,14 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
     for (int j = 0; j < NB / 4; ++j) {
         if constexpr (DO_K) {
             if constexpr (FMT == 2) {
-                if (j == 0) tq3_key_pair_v2<true>(I0, I1, I2, I3, kw[0], kw[1], kw[2], qt_lane);
-                else tq3_key_pair_v2<false>(I0, I1, I2, I3, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * 2048);
+                if (j == 0) tq3_key_pair_v2<true, SPLIT>(I0, I1, I2, I3, kw[0], kw[1], kw[2], qt_lane);
+                else tq3_key_pair_v2<false, SPLIT>(I0, I1, I2, I3, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2],
+                                                   qt_lane + j * (SPLIT ? 1024 : 2048));
             }
-            else tq3_key_quad(S0, S1, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * 2048);
+            else tq3_key_quad<SPLIT>(S0, S1, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * (SPLIT ? 1024 : 2048));
         }
         if constexpr (DO_V)
-            tq3_value_quad<DEFER>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
+            tq3_value_quad<DEFER, SPLIT>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
                                   vw[3 * j + 2], meta + j * 256, pf);
     }
     if constexpr (DO_K && FMT == 2) {
@@ -868,6 +910,21 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
         const uint32_t gaddr = rec_k + 12 * D + 4 * tq;
         const float2 ga = half2_to_float2(lds32(gaddr)), gb = half2_to_float2(lds32(gaddr + 16));
         // (sc2 carries the head's digit unit delta_h / 8 here)
+        if constexpr (SPLIT) {
+            // this lane has digit 0 (g < 4) or 1 (g >= 4) and digit 2 of head g % 4, the lane 16 away the other one
+            const float mine = lane & 16 ? 128.f : 16384.f, theirs = lane & 16 ? 16384.f : 128.f;
+            float d[4];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                d[e] = fmaf((float)I0[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I0[e], 16), theirs, (float)I0[2 + e]));
+                d[2 + e] = fmaf((float)I2[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I2[e], 16), theirs, (float)I2[2 + e]));
+            }
+            s_next[0] = d[0] * (ga.x * sc2);
+            s_next[1] = d[1] * (ga.y * sc2);
+            s_next[2] = d[2] * (gb.x * sc2);
+            s_next[3] = d[3] * (gb.y * sc2);
+            return;
+        }
         s_next[0] = digits_to_score(I0[0], I0[2], I1[0]) * (ga.x * sc2);
         s_next[1] = digits_to_score(I0[1], I0[3], I1[1]) * (ga.y * sc2);
         s_next[2] = digits_to_score(I2[0], I2[2], I3[0]) * (gb.x * sc2);
@@ -881,6 +938,10 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
         s_next[1] = (S0[1] + S1[1]) * r0;
         s_next[2] = (S0[2] + S1[2]) * r1;
         s_next[3] = (S0[3] + S1[3]) * r1;
+        if constexpr (SPLIT) {               // products with the high and the low half of the query
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s_next[e] += __shfl_xor_sync(0xffffffffu, s_next[e], 2);
+        }
     }
 }
 
@@ -898,7 +959,7 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_
 // fragments can be fetched with ldmatrix: a lane then holds the four consecutive tokens 4tq .. 4tq+3 of
 // its two channel rows, which is the order P^T has after the transposition of a score tile whose rows
 // are permuted this way.
-template <int D, bool SCORED, bool ACCUMULATE = false>
+template <int D, bool SCORED, bool ACCUMULATE, bool SPLIT>
 __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, uint32_t vaddr, uint32_t qf_lane,
                                          float score_scale, float v_scale, int valid, int lane, float* mass_pg,
                                          int mass_stride, int GQ)
@@ -935,8 +996,8 @@ __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, u
                (4 * tq + 2 < valid ? 0x00FF0000u : 0u) | (4 * tq + 3 < valid ? 0xFF000000u : 0u);
     }
     PFrag pf;
-    softmax_page<NB>(acc, s, pf);
-    if constexpr (SCORED) store_page_mass<NB, ACCUMULATE>(acc, pf.ps0, pf.ps1, mass_pg, mass_stride, GQ, lane);
+    softmax_page<NB, SPLIT>(acc, s, pf, lane);
+    if constexpr (SCORED) store_page_mass<NB, SPLIT, ACCUMULATE>(acc, pf.ps0, pf.ps1, mass_pg, mass_stride, GQ, lane);
     const bool scale_v = v_scale != 1.0f;
 #pragma unroll
     for (int cb = 0; cb < NB; cb += 2) {
@@ -954,12 +1015,12 @@ __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, u
             if (scale_v) {
                 float t[4];
                 mma16816_zero(t, a, pf.b0, pf.b1);
-                mma16816(t, a, pf.c0, pf.c1);
+                if constexpr (!SPLIT) mma16816(t, a, pf.c0, pf.c1);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc.o[cb + e][i] = fmaf(v_scale, t[i], acc.o[cb + e][i]);
             } else {
                 mma16816(acc.o[cb + e], a, pf.b0, pf.b1);
-                mma16816(acc.o[cb + e], a, pf.c0, pf.c1);
+                if constexpr (!SPLIT) mma16816(acc.o[cb + e], a, pf.c0, pf.c1);
             }
         }
     }
@@ -1063,7 +1124,7 @@ __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot,
         P.lse[(size_t)b * hq + h * GQ + tid] = ml_s[8 + tid] > 0.f ? (ml_s[tid] + log2f(ml_s[8 + tid])) * kLn2 : -CUDART_INF_F;
 }
 
-template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT, bool FLAT>
+template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT, bool FLAT, bool SPLIT>
 __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const LayerSet<MAXL> LS)
 {
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
@@ -1165,7 +1226,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     bool failed = false;
     const uint32_t ring = sbase + warp * NSTAGE * G::SLOT;
     const uint32_t bars = sbase + G::OFF_BAR + warp * NSTAGE * 8;
-    const uint32_t qt_lane = sbase + G::OFF_QT + lane * 16, qf_lane = sbase + G::OFF_QF + lane * 8;
+    const uint32_t qt_lane = sbase + G::OFF_QT + lane * (SPLIT && FMT == 1 ? 8 : 16), qf_lane = sbase + G::OFF_QF + lane * 8;
     int* list3 = reinterpret_cast<int*>(smem + G::OFF_LIST) + warp * 2 * G::ROUND;   // Stale page ids of the round
     int* list8 = list3 + G::ROUND;                                                   // FP8 page ids | valid << 27
     int* lpg3 = reinterpret_cast<int*>(smem + G::OFF_LIST) + (NW + warp) * 2 * G::ROUND;   // their logical pages (scored variant)
@@ -1388,7 +1449,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         };
         auto fold = [&](int page, bool to_regs, int logical_page) {
             if constexpr (SCORED)      // this warp's part of the page's exponential sum
-                store_page_mass<NB, true>(acc, acc.lp[0], acc.lp[1], mass_row + logical_page, P.max_pages, GQ, lane);
+                store_page_mass<NB, SPLIT, true>(acc, acc.lp[0], acc.lp[1], mass_row + logical_page, P.max_pages, GQ, lane);
             const uint4* meta = reinterpret_cast<const uint4*>(P.tq3 + ((size_t)page * hkv + h) * tq3_page +
                                                                 (size_t)P.tiles * TQ3_TILE + g * 16);
 #pragma unroll
@@ -1440,7 +1501,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 #pragma unroll
         for (int k = 0; k < HPW; ++k) {
             const int hd = warp + k * NW;
-            if (hd >= 8) break;
+            if (hd >= (SPLIT ? 4 : 8)) break;
             float a[EPL];
 #pragma unroll
             for (int r = 0; r < EPL; ++r) {
@@ -1493,6 +1554,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     }
                     const int i0 = lane * EPL + r0, st = i0 >> 5, k = i0 & 31;
                     const int L = 4 * hd + ((k & 15) >> 2);
+                    if constexpr (SPLIT) {      // one fragment per step: rows hd, hd + 4, hd + 8, hd + 12
+                        uint8_t* at = qt8 + (st * 32 + L) * 16 + (k >> 4) * 8;
+                        *reinterpret_cast<uint2*>(at) = make_uint2(word[0], word[2]);
+                        *reinterpret_cast<uint2*>(at + 256) = make_uint2(word[1], word[2]);
+                        continue;
+                    }
                     *reinterpret_cast<uint32_t*>(qt8 + ((st * 2) * 32 + L) * 16 + (2 * (k >> 4)) * 4) = word[0];
                     *reinterpret_cast<uint32_t*>(qt8 + ((st * 2) * 32 + L) * 16 + (2 * (k >> 4) + 1) * 4) = word[1];
                     *reinterpret_cast<uint2*>(qt8 + ((st * 2 + 1) * 32 + L) * 16 + (k >> 4) * 8) = make_uint2(word[2], 0u);
@@ -1503,22 +1570,24 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 const int i = lane * EPL + r;
                 if constexpr (FMT == 1) {   // rotated query, natural slot order: block i/16, slot s = i%16; per lane {hi b0, hi b1, lo b0, lo b1}
                     const int kb = i >> 4, s = i & 15;
-                    const int at = (kb * 32 + 4 * hd + ((s & 7) >> 1)) * 8 + (s >> 3) * 2 + (s & 1);
+                    const int at = (kb * 32 + 4 * hd + ((s & 7) >> 1)) * (SPLIT ? 4 : 8) + (s >> 3) * 2 + (s & 1);
                     // fp16 pair hi + lo carries the rotated query to ~2^-22
                     const float v = a[r] * rs;
                     const __half vh = __float2half_rn(v);
                     qt[at] = vh;
-                    qt[at + 4] = __float2half_rn(v - __half2float(vh));
+                    qt[at + (SPLIT ? 64 : 4)] = __float2half_rn(v - __half2float(vh));     // SPLIT: column hd + 4
                 }
                 {   // plain query in the slot order of the FP8 key loads: 16 consecutive dims per lane
                     const int j = i >> 6, t4 = (i & 63) >> 4, wv = (i & 15) >> 2, e = i & 3;
-                    qf[((4 * j + wv) * 32 + 4 * hd + t4) * 4 + (e >> 1) * 2 + (e & 1)] = __float2half_rn(qx[k][r]);
+                    const int at = ((4 * j + wv) * 32 + 4 * hd + t4) * 4 + (e >> 1) * 2 + (e & 1);
+                    qf[at] = __float2half_rn(qx[k][r]);
+                    if constexpr (SPLIT) qf[at + 64] = qf[at];         // column hd + 4: the same scores
                 }
             }
         }
         __syncthreads();
         // score unit of the Stale pages: record format 2 counts in digit units of this lane's head g
-        const float sc2k = FMT == 2 ? sc2 * reinterpret_cast<const float*>(smem + G::OFF_QS)[g] : sc2;
+        const float sc2k = FMT == 2 ? sc2 * reinterpret_cast<const float*>(smem + G::OFF_QS)[SPLIT ? g & 3 : g] : sc2;
 
         for (bool more = n_my > 0; more && !failed;) {
             // ---- Stale pages: scores of page i+1 are computed together with the output update of page i
@@ -1532,7 +1601,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     cur_lp = lpg3[0] >> 16;
                 }
                 wait_slot(0);
-                if (!failed) tq3_step<D, false, true, TILED, FMT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, lane, s_cur);
+                if (!failed) tq3_step<D, false, true, TILED, FMT, SPLIT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, lane, s_cur);
                 for (int i = 0; i + 1 < n3 && !failed; ++i) {
                     const uint32_t cur = (uint32_t)i % NSTAGE, nxt = (uint32_t)(i + 1) % NSTAGE;
                     wait_slot(nxt);
@@ -1547,8 +1616,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                             cur_lp = lpg3[i] >> 16;
                         }
                     }
-                    tq3_step<D, true, true, TILED, FMT>(acc, ring + cur * G::SLOT, s_cur, pf, ring + nxt * G::SLOT, qt_lane, sc2k, lane, s_next);
-                    if constexpr (SCORED && !TILED) store_page_mass<NB>(acc, pf.ps0, pf.ps1, mass_row + lpg3[i], P.max_pages, GQ, lane);
+                    tq3_step<D, true, true, TILED, FMT, SPLIT>(acc, ring + cur * G::SLOT, s_cur, pf, ring + nxt * G::SLOT, qt_lane, sc2k, lane, s_next);
+                    if constexpr (SCORED && !TILED) store_page_mass<NB, SPLIT>(acc, pf.ps0, pf.ps1, mass_row + lpg3[i], P.max_pages, GQ, lane);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) s_cur[e] = s_next[e];
                     __syncwarp();
@@ -1566,8 +1635,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                             cur_lp = lpg3[n3 - 1] >> 16;
                         }
                     }
-                    tq3_step<D, true, false, TILED, FMT>(acc, ring + ((uint32_t)(n3 - 1) % NSTAGE) * G::SLOT, s_cur, pf, 0, qt_lane, sc2k, lane, s_next);
-                    if constexpr (SCORED && !TILED) store_page_mass<NB>(acc, pf.ps0, pf.ps1, mass_row + lpg3[n3 - 1], P.max_pages, GQ, lane);
+                    tq3_step<D, true, false, TILED, FMT, SPLIT>(acc, ring + ((uint32_t)(n3 - 1) % NSTAGE) * G::SLOT, s_cur, pf, 0, qt_lane, sc2k, lane, s_next);
+                    if constexpr (SCORED && !TILED) store_page_mass<NB, SPLIT>(acc, pf.ps0, pf.ps1, mass_row + lpg3[n3 - 1], P.max_pages, GQ, lane);
                     if constexpr (TILED) fold(cur_page, true, cur_lp);   // back to output units for the FP8 pages and the reduction
                 }
                 __syncwarp();
@@ -1583,7 +1652,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     if (failed) break;
                     const int e = list8[i];
                     const int valid = (e >> 27) & 15;
-                    fp8_page<D, SCORED, TILED>(acc, ring + s * G::SLOT, ring + (s + 1) * G::SLOT, qf_lane, sc2 * P.k_scale, P.v_scale,
+                    fp8_page<D, SCORED, TILED, SPLIT>(acc, ring + s * G::SLOT, ring + (s + 1) * G::SLOT, qf_lane, sc2 * P.k_scale, P.v_scale,
                                                valid ? valid : kPage, lane,
                                                SCORED ? mass_row + (TILED ? (lpg8[i] >> 16) : lpg8[i]) : nullptr, P.max_pages, GQ);
                     if constexpr (FMT == 2) max_rows_from_columns<NB>(acc, lane);     // the page may have raised the maxima
@@ -1643,6 +1712,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 for (int w = 0; w < NU; ++w) {
                     acc += red[(size_t)w * D * 8 + e];
                     l += sm_l[w * 8 + head];
+                    if constexpr (SPLIT) {
+                        acc += red[(size_t)w * D * 8 + e + 4];
+                        l += sm_l[w * 8 + head + 4];
+                    }
                 }
                 P.out[((size_t)b * hq + h * GQ + head) * D + ch] = l > 0.f ? acc / l : 0.f;
             }
@@ -1650,6 +1723,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 float l = 0.f, M = -CUDART_INF_F;
                 for (int w = 0; w < NU; ++w) {
                     l += sm_l[w * 8 + tid];
+                    if constexpr (SPLIT) l += sm_l[w * 8 + tid + 4];
                     M = fmaxf(M, sm_m[w * 8 + tid]);
                 }
                 P.lse[(size_t)b * hq + h * GQ + tid] = l > 0.f ? (M + log2f(l)) * kLn2 : -CUDART_INF_F;
@@ -1661,13 +1735,17 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             for (int e = tid; e < 8 * D; e += NW * 32) {
                 float acc = 0.f;
 #pragma unroll
-                for (int w = 0; w < NU; ++w) acc += red[(size_t)w * D * 8 + e];
-                slot[e] = acc;
+                for (int w = 0; w < NU; ++w) {
+                    acc += red[(size_t)w * D * 8 + e];
+                    if constexpr (SPLIT) acc += (e & 4) ? 0.f : red[(size_t)w * D * 8 + e + 4];
+                }
+                slot[e] = acc;                 // (SPLIT: columns 4-7 are not read as heads)
             }
             if (tid < 8) {
                 float l = 0.f, M = -CUDART_INF_F;
                 for (int w = 0; w < NU; ++w) {
                     l += sm_l[w * 8 + tid];
+                    if constexpr (SPLIT) l += tid < 4 ? sm_l[w * 8 + tid + 4] : 0.f;
                     M = fmaxf(M, sm_m[w * 8 + tid]);
                 }
                 slot[8 * D + tid] = M;
@@ -1767,11 +1845,11 @@ static int32_t run_tmem(mkv_pool* p, DecodeParams& prm, cudaStream_t s)
     return MKV_OK;
 }
 
-template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT, bool FLAT>
+template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL, int FMT, bool FLAT, bool SPLIT>
 static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_t s)
 {
     using G = Geo<D, NW, NSTAGE, TILED>;
-    auto kern = decode_tensor_kernel<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, FMT, FLAT>;
+    auto kern = decode_tensor_kernel<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, FMT, FLAT, SPLIT>;
     // pages of several tiles: one row of parked accumulators (8 D floats) per warp behind the usual layout
     constexpr int SMEM = G::SMEM + (TILED ? NW * 8 * D * 4 : 0);
     static_assert(SMEM <= 232448, "dynamic shared memory of one block");
@@ -1806,8 +1884,14 @@ static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_
 template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false, int MAXL = 1, bool FLAT = false>
 static int32_t run_tensor(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_t s)
 {
-    return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT>(p, ls, s)
-                       : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT>(p, ls, s);
+    // groups of at most four query heads: two column halves (see PFrag).  Not for long pages: their code sums stay in
+    // the tensor core's accumulators over many tiles, and the split changes their rounding there.
+    if constexpr (!TILED)
+        if (p->group <= 4)
+            return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, true>(p, ls, s)
+                               : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, true>(p, ls, s);
+    return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, false>(p, ls, s)
+                       : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, false>(p, ls, s);
 }
 
 template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false>

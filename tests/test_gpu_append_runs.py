@@ -18,7 +18,7 @@ def test_runs_at_any_offset_write_what_single_tokens_write(d, hkv, page, starts)
     rng = np.random.default_rng(sum(starts) + d + page)
     slots, first = [], 0
     for s in starts:
-        n = int(rng.integers(150, 330))
+        n = int(rng.integers(280, 460))
         slots.append(first * page + s % page + np.arange(n))
         first += (s % page + n + page - 1) // page
     slots.append(first * page + rng.permutation(page))              # one page in random order

@@ -1028,16 +1028,18 @@ __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, u
 
 // Eq. (softmax-merge) of one (request, KV head) row that was split over n_parts blocks.  Part 0 sits
 // in slot first_slot, part j > 0 in slot even_base + 2j.  Called by all NT threads of the block that
-// drew the row's last ticket; `buf` is idle shared memory (n_parts * 16 + 16 floats).  Warp hd < 8
-// reduces the maxima and row sums of head hd (one trip to L2: both are loaded together and kept in
-// shared memory); a thread then owns float4 groups (one channel, four heads) of the [channel][8 heads]
-// tile and has 40 loads in flight, issued before the weights are worked out.
-template <int D, int NT, int KPMAX = 40>
+// drew the row's last ticket; `buf` is idle shared memory.  Warp hd < 8 reduces the maxima and row sums of head hd
+// (one trip to L2: both are loaded together and kept in shared memory); a thread owns float4 groups (one channel,
+// four heads) of the [channel][8 heads] tile.  With twice as many threads as groups (16 warps at d = 128) every
+// other part goes to the second half of the threads.  KP loads per thread are in flight, issued before the weights
+// are worked out: 32 to 40 parts per block, bounded by the registers of the launch shape.
+template <int D, int NT, int KPMAX = NT <= 256 ? 40 : NT <= 384 ? 24 : 16>
 __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot, int even_base, int n_parts,
                                           float* buf, int b, int h)
 {
     constexpr uint32_t FULL = 0xffffffffu;
-    constexpr int STRIDE = 8 * D + 16, GPT = (2 * D + NT - 1) / NT, KP = KPMAX / GPT;   // KPMAX (40) float4 loads in flight per thread
+    constexpr int STRIDE = 8 * D + 16, GROUPS = 2 * D, GPT = (GROUPS + NT - 1) / NT, S = NT >= 2 * GROUPS ? 2 : 1;
+    constexpr int KP = KPMAX / GPT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int GQ = P.group, hq = P.hkv * GQ;
     float* w_s = buf;                        // [n_parts][8] maxima, then weights e^{m_j - m}
@@ -1050,21 +1052,22 @@ __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot,
     float4 acc[GPT], v[KP][GPT];
 #pragma unroll
     for (int k = 0; k < GPT; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int first = S > 1 ? tid / GROUPS : 0, grp0 = S > 1 ? tid % GROUPS : tid;     // parts first, first + S, ...
     const int head0 = (tid & 1) * 4;         // NT is even: every group of this thread covers the same four heads
     auto load_round = [&](int j0) {
 #pragma unroll
         for (int p = 0; p < KP; ++p) {
-            const float* ps = slot_of(min(j0 + p, n_parts - 1));
+            const float* ps = slot_of(min(j0 + p * S, n_parts - 1));
 #pragma unroll
             for (int k = 0; k < GPT; ++k)
-                v[p][k] = __ldcg(reinterpret_cast<const float4*>(ps) + min(tid + k * NT, 2 * D - 1));
+                v[p][k] = __ldcg(reinterpret_cast<const float4*>(ps) + min(grp0 + k * NT, GROUPS - 1));
         }
     };
     auto use_round = [&](int j0) {
 #pragma unroll
         for (int p = 0; p < KP; ++p)
-            if (j0 + p < n_parts) {
-                const float4 w = *reinterpret_cast<const float4*>(w_s + (j0 + p) * 8 + head0);
+            if (j0 + p * S < n_parts) {
+                const float4 w = *reinterpret_cast<const float4*>(w_s + (j0 + p * S) * 8 + head0);
 #pragma unroll
                 for (int k = 0; k < GPT; ++k) {
                     acc[k].x = fmaf(w.x, v[p][k].x, acc[k].x);
@@ -1074,7 +1077,7 @@ __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot,
                 }
             }
     };
-    load_round(0);                           // in flight while the weights are worked out
+    load_round(first);                       // in flight while the weights are worked out
     for (int hd = warp; hd < 8; hd += NT / 32) {
         float M = -CUDART_INF_F;
         for (int j = lane; j < n_parts; j += 32) {
@@ -1101,15 +1104,24 @@ __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot,
         }
     }
     __syncthreads();
-    use_round(0);
-    for (int j0 = KP; j0 < n_parts; j0 += KP) {
+    use_round(first);
+    for (int j0 = first + KP * S; j0 < n_parts; j0 += KP * S) {
         load_round(j0);
         use_round(j0);
     }
+    if constexpr (S > 1) {                   // the second half of the threads hands its sums over
+        float4* half = reinterpret_cast<float4*>(buf + n_parts * 16 + 16);
+        if (first == 1) half[grp0] = acc[0];
+        __syncthreads();
+        if (first == 0) {
+            const float4 o = half[grp0];
+            acc[0].x += o.x; acc[0].y += o.y; acc[0].z += o.z; acc[0].w += o.w;
+        }
+    }
 #pragma unroll
     for (int k = 0; k < GPT; ++k) {
-        const int grp = tid + k * NT, ch = grp >> 1;
-        if (grp >= 2 * D) continue;
+        const int grp = grp0 + k * NT, ch = grp >> 1;
+        if (grp >= GROUPS || first > 0) continue;
         const float av[4] = {acc[k].x, acc[k].y, acc[k].z, acc[k].w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -2039,9 +2051,9 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
         return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, true, kMaxLayers>(p0, ls, s)
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
     if (n_layers >= kMinFlatLayers)
-        return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
+        return p0->d == 128 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
                             : run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s);
-    return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, false, kMaxLayers>(p0, ls, s)
+    return p0->d == 128 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers>(p0, ls, s)
                         : run_tensor<256, 8, 4, 1, false, false, kMaxLayers>(p0, ls, s);
 }
 
@@ -2070,7 +2082,7 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
             MKV_CUDA(launch_pdl(page_mass_clear_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, 1, true, s, mass, n));
             rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true, true>(p, prm, s);
         } else {
-            rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);
+            rc = p->d == 128 ? run_tensor1<128, 16, 4, 1, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);
         }
         if (rc != MKV_OK) return rc;
         return launch_page_mass_finish(mass, lse, lens, B, p->hkv * p->group, max_pages, p->cfg.page_size, s);
@@ -2078,9 +2090,9 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
     if (p->tiles > 1)                    // pages of several tiles: the default launch shapes only
         return p->d == 128 ? run_tensor1<128, 12, 4, 1, false, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, false, true>(p, prm, s);
     if (p->variant == MKV_DECODE_TMEM && p->d == 256) return run_tmem<256>(p, prm, s);
-    // launch shapes (warps per block, ring slots per warp, blocks per SM): 12 warps at 168 registers for
-    // d = 128 (7 % faster than 16 warps at 128 registers), 8 warps for d = 256
-    return p->d == 128 ? run_tensor1<128, 12, 4, 1>(p, prm, s) : run_tensor1<256, 8, 4, 1>(p, prm, s);
+    // launch shapes (warps per block, ring slots per warp, blocks per SM): 16 warps at 128 registers for d = 128 (64
+    // ragged requests: 658 us against 678 us with 12 warps at 168 registers), 8 warps at up to 255 for d = 256
+    return p->d == 128 ? run_tensor1<128, 16, 4, 1>(p, prm, s) : run_tensor1<256, 8, 4, 1>(p, prm, s);
 }
 
 }  // namespace mkv

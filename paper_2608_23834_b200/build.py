@@ -25,7 +25,7 @@ def needs_build() -> bool:
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = sources() + [os.path.join(CSRC, "py_binding.cpp"),
-                        os.path.join(CSRC, "mkv_internal.cuh"), os.path.join(CSRC, "decode_tmem.cuh"),
+                        *(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")),
                         os.path.join(ROOT, "include", "mkv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 

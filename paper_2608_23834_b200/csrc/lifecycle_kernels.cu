@@ -409,6 +409,145 @@ struct DemoteLane {
     }
 };
 
+// One key vector (a token of one KV head), lane l holding its elements l * D/32 ..: the literal sequence of fp32
+// operations that defines the encoder.  Codes as bytes in element order, norm correction as fp16 bits.
+template <int D, int FMT>
+__device__ __forceinline__ void encode_key_token(const uint32_t (&raw)[D / 128], const DemoteLane<D, FMT>& K, float k_scale,
+                                                 uint32_t (&packed)[D / 128], uint16_t& gcode)
+{
+    using CB = KeyCodebook<FMT>;
+    constexpr int EPL = D / 32;
+    const float c0sq = K.c0sq, c1sq = K.c1sq, c2sq = K.c2sq, c3sq = K.c3sq;
+    const uint32_t (&flip)[EPL] = K.flip;
+    const float (&sgn)[5] = K.sgn;
+    float x[EPL], a[EPL];
+#pragma unroll
+    for (int r = 0; r < EPL; r += 2) {
+        const float2 f = e4m3x2_to_f32((raw[r >> 2] >> (8 * (r & 3))) & 0xFFFFu);
+        x[r] = f.x;
+        x[r + 1] = f.y;
+    }
+    if (k_scale != 1.0f) {           // a product with 1 is the factor itself: the common case skips it
+#pragma unroll
+        for (int r = 0; r < EPL; ++r) x[r] = __fmul_rn(x[r], k_scale);
+    }
+#pragma unroll
+    for (int r = 0; r < EPL; ++r) a[r] = __uint_as_float(__float_as_uint(x[r]) ^ flip[r]);
+    // Walsh-Hadamard butterflies, strides ascending: inside the lane, then across lanes
+    // (stride 1 pairs neighbours: scalar; from stride 2 on two butterflies share one packed instruction)
+#pragma unroll
+    for (int r = 0; r < EPL; r += 2) {
+        const float u = a[r], w = a[r + 1];
+        a[r] = __fadd_rn(u, w);
+        a[r + 1] = __fsub_rn(u, w);
+    }
+    f32x2 ap[EPL / 2];
+    const f32x2 minus1 = pack2(-1.0f, -1.0f);
+#pragma unroll
+    for (int r = 0; r < EPL / 2; ++r) ap[r] = pack2(a[2 * r], a[2 * r + 1]);
+#pragma unroll
+    for (int hh = 1; hh < EPL / 2; hh <<= 1)            // strides 2, 4 of the elements = 1, 2 of the pairs
+#pragma unroll
+        for (int r = 0; r < EPL / 2; ++r)
+            if ((r & hh) == 0) {
+                const f32x2 u = ap[r], w = ap[r + hh];
+                ap[r] = add2(u, w);
+                ap[r + hh] = fma2(w, minus1, u);        // u - w: the product with -1 is exact, one rounding
+            }
+#pragma unroll
+    for (int b = 0; b < 5; ++b) {
+        const f32x2 s2 = pack2(sgn[b], sgn[b]);
+#pragma unroll
+        for (int r = 0; r < EPL / 2; ++r) {
+            // lower lane: o + a; upper lane: o - a.  The product with +-1 is exact, so the fused form rounds
+            // once, exactly like the single addition it stands for (zero signs included)
+            float lo, hi;
+            unpack2(ap[r], lo, hi);
+            const float olo = __shfl_xor_sync(0xffffffffu, lo, 1 << b), ohi = __shfl_xor_sync(0xffffffffu, hi, 1 << b);
+            ap[r] = fma2(ap[r], s2, pack2(olo, ohi));
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < EPL / 2; ++r) unpack2(ap[r], a[2 * r], a[2 * r + 1]);
+    // |x|^2: pairwise tree in index order (every element of the butterfly ends equal)
+    float e[EPL];
+#pragma unroll
+    for (int r = 0; r < EPL; r += 2) {
+        const f32x2 xx = pack2(x[r], x[r + 1]);
+        unpack2(mul2(xx, xx), e[r], e[r + 1]);
+    }
+#pragma unroll
+    for (int hh = 1; hh < EPL; hh <<= 1)
+#pragma unroll
+        for (int r = 0; r < EPL; r += 2 * hh) e[r] = __fadd_rn(e[r], e[r + hh]);
+    float n2 = e[0];
+#pragma unroll
+    for (int m = 1; m < 32; m <<= 1) n2 = __fadd_rn(n2, __shfl_xor_sync(0xffffffffu, n2, m));
+    const float nx = __fsqrt_rn(n2);
+    const float t1 = __fmul_rn(CB::B0, nx), t2 = __fmul_rn(CB::B1, nx), t3 = __fmul_rn(CB::B2, nx);
+    float f[EPL];
+    uint32_t sq64 = 4u * EPL;          // record format 2: 64 x the sum of this lane's squared levels (4, 36, 121, 324)
+#pragma unroll
+    for (int r = 0; r < EPL / 4; ++r) packed[r] = 0;
+#pragma unroll
+    for (int r = 0; r < EPL; ++r) {
+        const float w = fabsf(a[r]);
+        const bool g1 = w > t1, g2 = w > t2, g3 = w > t3;
+        // sign bit of the code: a[r] < 0 (a zero of either sign is positive)
+        uint32_t code = a[r] < 0.0f ? 4u : 0u;
+        if (g1) code += 1u;
+        if (g2) code += 1u;
+        if (g3) code += 1u;
+        packed[r >> 2] |= code << (8 * (r & 3));
+        if constexpr (FMT == 2) {
+            if (g1) sq64 += 32u;
+            if (g2) sq64 += 85u;
+            if (g3) sq64 += 203u;
+        } else {
+            f[r] = g2 ? (g3 ? c3sq : c2sq) : (g1 ? c1sq : c0sq);
+        }
+    }
+    float nc2;
+    if constexpr (FMT == 2) {
+        // The squared levels of format 2 are multiples of 1/64 and d of them sum to at most 5.0625 d, so every
+        // partial sum of the pairwise tree is exact in fp32: any order gives the same bits, and the sum can be
+        // taken in integers (one warp reduction) instead.
+        static_assert(324 * D < (1 << 24), "exact in fp32");
+        nc2 = __fmul_rn((float)__reduce_add_sync(0xffffffffu, sq64), 0.015625f);
+    } else {
+#pragma unroll
+        for (int hh = 1; hh < EPL; hh <<= 1)
+#pragma unroll
+            for (int r = 0; r < EPL; r += 2 * hh) f[r] = __fadd_rn(f[r], f[r + hh]);
+        nc2 = f[0];
+#pragma unroll
+        for (int m = 1; m < 32; m <<= 1) nc2 = __fadd_rn(nc2, __shfl_xor_sync(0xffffffffu, nc2, m));
+    }
+    const float nc = __fsqrt_rn(nc2);
+    gcode = (nx == 0.0f) ? (uint16_t)0 : f32_to_f16_sat_bits(__fdiv_rn(nx, nc));
+}
+
+// Minimum and maximum of a channel by strict comparison in token order (of equal values, +0 and -0, the earliest counts).
+__device__ __forceinline__ void literal_min_max(const float (&val)[kPage], float& mn, float& mx)
+{
+    mn = mx = val[0];
+#pragma unroll
+    for (int t = 1; t < kPage; ++t) {
+        if (val[t] < mn) mn = val[t];
+        if (val[t] > mx) mx = val[t];
+    }
+}
+
+// clamp(rint((val - zp) / sc), 0, 7) with the correctly rounded quotient, 0 when sc == 0 (and for a NaN)
+__device__ __forceinline__ uint32_t literal_value_code(float val, float scf, float zpf)
+{
+    const float den = scf != 0.0f ? scf : 1.0f, num = __fsub_rn(val, zpf);
+    float r = rintf(__fdiv_rn(num != 0.0f ? num : den, den));   // half to even
+    r = r < 0.0f ? 0.0f : r;
+    r = r > 7.0f ? 7.0f : r;
+    return (num != 0.0f && scf != 0.0f) ? (uint32_t)(int)r : 0u;
+}
+
 // Encodes the 16 tokens of one FP8 record (rec8) into the record image img = [key codes | value codes | g |
 // scale/zero] in shared memory; all D threads of the block call it.  OWN_META: the value scale and zero come
 // from these 16 tokens (16-token pages); otherwise thread c passes the page's scale/zero of channel c.
@@ -417,16 +556,12 @@ __device__ __forceinline__ void demote_tile(const uint8_t* __restrict__ rec8, ui
                                             const DemoteLane<D, FMT>& K, float k_scale, float v_scale, uint16_t sc_page,
                                             uint16_t zp_page)
 {
-    using CB = KeyCodebook<FMT>;
     constexpr int EPL = D / 32, NJ = D / 64, KROW = D + 8, NT = D;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const float c0sq = K.c0sq, c1sq = K.c1sq, c2sq = K.c2sq, c3sq = K.c3sq;
-    const uint32_t (&flip)[EPL] = K.flip;
-    const float (&sgn)[5] = K.sgn;
     // ---- keys: warp w encodes tokens w, w + NT/32, ... ------------------------------------------
     for (int tok = warp; tok < kPage; tok += NT / 32) {
-        float x[EPL], a[EPL];
-        uint32_t raw[EPL / 4];
+        uint32_t raw[EPL / 4], packed[EPL / 4];
+        uint16_t gcode;
         if constexpr (EPL == 8) {
             const uint2 u = *reinterpret_cast<const uint2*>(rec8 + tok * D + lane * EPL);
             raw[0] = u.x;
@@ -434,117 +569,12 @@ __device__ __forceinline__ void demote_tile(const uint8_t* __restrict__ rec8, ui
         } else {
             raw[0] = *reinterpret_cast<const uint32_t*>(rec8 + tok * D + lane * EPL);
         }
-#pragma unroll
-        for (int r = 0; r < EPL; r += 2) {
-            const float2 f = e4m3x2_to_f32((raw[r >> 2] >> (8 * (r & 3))) & 0xFFFFu);
-            x[r] = f.x;
-            x[r + 1] = f.y;
-        }
-        if (k_scale != 1.0f) {           // a product with 1 is the factor itself: the common case skips it
-#pragma unroll
-            for (int r = 0; r < EPL; ++r) x[r] = __fmul_rn(x[r], k_scale);
-        }
-#pragma unroll
-        for (int r = 0; r < EPL; ++r) a[r] = __uint_as_float(__float_as_uint(x[r]) ^ flip[r]);
-        // Walsh-Hadamard butterflies, strides ascending: inside the lane, then across lanes
-        // (stride 1 pairs neighbours: scalar; from stride 2 on two butterflies share one packed instruction)
-#pragma unroll
-        for (int r = 0; r < EPL; r += 2) {
-            const float u = a[r], w = a[r + 1];
-            a[r] = __fadd_rn(u, w);
-            a[r + 1] = __fsub_rn(u, w);
-        }
-        f32x2 ap[EPL / 2];
-        const f32x2 minus1 = pack2(-1.0f, -1.0f);
-#pragma unroll
-        for (int r = 0; r < EPL / 2; ++r) ap[r] = pack2(a[2 * r], a[2 * r + 1]);
-#pragma unroll
-        for (int hh = 1; hh < EPL / 2; hh <<= 1)            // strides 2, 4 of the elements = 1, 2 of the pairs
-#pragma unroll
-            for (int r = 0; r < EPL / 2; ++r)
-                if ((r & hh) == 0) {
-                    const f32x2 u = ap[r], w = ap[r + hh];
-                    ap[r] = add2(u, w);
-                    ap[r + hh] = fma2(w, minus1, u);        // u - w: the product with -1 is exact, one rounding
-                }
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-            const f32x2 s2 = pack2(sgn[b], sgn[b]);
-#pragma unroll
-            for (int r = 0; r < EPL / 2; ++r) {
-                // lower lane: o + a; upper lane: o - a.  The product with +-1 is exact, so the fused form rounds
-                // once, exactly like the single addition it stands for (zero signs included)
-                float lo, hi;
-                unpack2(ap[r], lo, hi);
-                const float olo = __shfl_xor_sync(0xffffffffu, lo, 1 << b), ohi = __shfl_xor_sync(0xffffffffu, hi, 1 << b);
-                ap[r] = fma2(ap[r], s2, pack2(olo, ohi));
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < EPL / 2; ++r) unpack2(ap[r], a[2 * r], a[2 * r + 1]);
-        // |x|^2: pairwise tree in index order (every element of the butterfly ends equal)
-        float e[EPL];
-#pragma unroll
-        for (int r = 0; r < EPL; r += 2) {
-            const f32x2 xx = pack2(x[r], x[r + 1]);
-            unpack2(mul2(xx, xx), e[r], e[r + 1]);
-        }
-#pragma unroll
-        for (int hh = 1; hh < EPL; hh <<= 1)
-#pragma unroll
-            for (int r = 0; r < EPL; r += 2 * hh) e[r] = __fadd_rn(e[r], e[r + hh]);
-        float n2 = e[0];
-#pragma unroll
-        for (int m = 1; m < 32; m <<= 1) n2 = __fadd_rn(n2, __shfl_xor_sync(0xffffffffu, n2, m));
-        const float nx = __fsqrt_rn(n2);
-        const float t1 = __fmul_rn(CB::B0, nx), t2 = __fmul_rn(CB::B1, nx), t3 = __fmul_rn(CB::B2, nx);
-        float f[EPL];
-        uint32_t packed[EPL / 4];
-        uint32_t sq64 = 4u * EPL;          // record format 2: 64 x the sum of this lane's squared levels (4, 36, 121, 324)
-#pragma unroll
-        for (int r = 0; r < EPL / 4; ++r) packed[r] = 0;
-#pragma unroll
-        for (int r = 0; r < EPL; ++r) {
-            const float w = fabsf(a[r]);
-            const bool g1 = w > t1, g2 = w > t2, g3 = w > t3;
-            // sign bit of the code: a[r] < 0 (a zero of either sign is positive)
-            uint32_t code = a[r] < 0.0f ? 4u : 0u;
-            if (g1) code += 1u;
-            if (g2) code += 1u;
-            if (g3) code += 1u;
-            packed[r >> 2] |= code << (8 * (r & 3));
-            if constexpr (FMT == 2) {
-                if (g1) sq64 += 32u;
-                if (g2) sq64 += 85u;
-                if (g3) sq64 += 203u;
-            } else {
-                f[r] = g2 ? (g3 ? c3sq : c2sq) : (g1 ? c1sq : c0sq);
-            }
-        }
+        encode_key_token<D, FMT>(raw, K, k_scale, packed, gcode);
         if constexpr (EPL == 8)
             *reinterpret_cast<uint2*>(kcode + tok * KROW + lane * EPL) = make_uint2(packed[0], packed[1]);
         else
             *reinterpret_cast<uint32_t*>(kcode + tok * KROW + lane * EPL) = packed[0];
-        float nc2;
-        if constexpr (FMT == 2) {
-            // The squared levels of format 2 are multiples of 1/64 and d of them sum to at most 5.0625 d, so every
-            // partial sum of the pairwise tree is exact in fp32: any order gives the same bits, and the sum can be
-            // taken in integers (one warp reduction) instead.
-            static_assert(324 * D < (1 << 24), "exact in fp32");
-            nc2 = __fmul_rn((float)__reduce_add_sync(0xffffffffu, sq64), 0.015625f);
-        } else {
-#pragma unroll
-            for (int hh = 1; hh < EPL; hh <<= 1)
-#pragma unroll
-                for (int r = 0; r < EPL; r += 2 * hh) f[r] = __fadd_rn(f[r], f[r + hh]);
-            nc2 = f[0];
-#pragma unroll
-            for (int m = 1; m < 32; m <<= 1) nc2 = __fadd_rn(nc2, __shfl_xor_sync(0xffffffffu, nc2, m));
-        }
-        const float nc = __fsqrt_rn(nc2);
-        if (lane == 0)
-            *reinterpret_cast<uint16_t*>(img + 12 * D + 2 * tok) =
-                (nx == 0.0f) ? (uint16_t)0 : f32_to_f16_sat_bits(__fdiv_rn(nx, nc));
+        if (lane == 0) *reinterpret_cast<uint16_t*>(img + 12 * D + 2 * tok) = gcode;
     }
 
     // ---- values: one thread per channel, 16 tokens of the page ------------------------------
@@ -573,15 +603,7 @@ __device__ __forceinline__ void demote_tile(const uint8_t* __restrict__ rec8, ui
                 mn = fminf(mn, val[t]);
                 mx = fmaxf(mx, val[t]);
             }
-            if (!(mn != 0.0f && mx != 0.0f) || val[0] != val[0]) {
-                mn = val[0];
-                mx = val[0];
-#pragma unroll
-                for (int t = 1; t < kPage; ++t) {
-                    if (val[t] < mn) mn = val[t];
-                    if (val[t] > mx) mx = val[t];
-                }
-            }
+            if (!(mn != 0.0f && mx != 0.0f) || val[0] != val[0]) literal_min_max(val, mn, mx);
             sc = f32_to_f16_sat_bits(__fdiv_rn(__fsub_rn(mx, mn), 7.0f));
             zp = f32_to_f16_sat_bits(mn);
         }
@@ -621,14 +643,7 @@ __device__ __forceinline__ void demote_tile(const uint8_t* __restrict__ rec8, ui
             }
         } else {
 #pragma unroll
-            for (int t = 0; t < kPage; ++t) {
-                const float num = __fsub_rn(val[t], zpf);
-                float r = rintf(__fdiv_rn(num != 0.0f ? num : den, den));   // half to even
-                r = r < 0.0f ? 0.0f : r;
-                r = r > 7.0f ? 7.0f : r;
-                const uint32_t q = (num != 0.0f && scf != 0.0f) ? (uint32_t)(int)r : 0u;
-                q4[t >> 2] |= q << (8 * (t & 3));
-            }
+            for (int t = 0; t < kPage; ++t) q4[t >> 2] |= literal_value_code(val[t], scf, zpf) << (8 * (t & 3));
         }
         *reinterpret_cast<uint4*>(vcode + c * kPage) = make_uint4(q4[0], q4[1], q4[2], q4[3]);
     }
@@ -763,6 +778,30 @@ __global__ void __launch_bounds__(D) demote_kernel(const uint8_t* __restrict__ f
     }
 }
 
+// A lane's words of one code section to global memory, in the record's 16-byte chunks.
+template <int D>
+__device__ __forceinline__ void store_lane_words(uint8_t* sec, int lane, const uint32_t (&w)[3 * (D / 16) / 4])
+{
+    constexpr int LW = 3 * (D / 16) / 4;
+#pragma unroll
+    for (int c = 0; c < LW / 4; ++c)
+        *reinterpret_cast<uint4*>(sec + c * 512 + lane * 16) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+    if constexpr (LW % 4 != 0)
+        *reinterpret_cast<uint2*>(sec + (LW / 4) * 512 + lane * 8) = make_uint2(w[LW - 2], w[LW - 1]);
+}
+
+// squared level of a magnitude (a single fp32 product, as the record's norm correction defines it)
+template <int FMT>
+__device__ __forceinline__ float level_sq(uint32_t mag)
+{
+    using CB = KeyCodebook<FMT>;
+    const float c0 = __fmul_rn(CB::C0, CB::C0), c1 = __fmul_rn(CB::C1, CB::C1), c2 = __fmul_rn(CB::C2, CB::C2),
+                c3 = __fmul_rn(CB::C3, CB::C3);
+    return mag & 2u ? (mag & 1u ? c3 : c2) : (mag & 1u ? c1 : c0);
+}
+
+#include "demote_warp.cuh"
+
 // Pages of several tiles, first pass of Demote: the minimum and maximum of every value channel over all tokens
 // of the page, then the page's scale and zero (same arithmetic and order of the halves as in the 16-token
 // record).  One cluster per (page, KV head); block r of the cluster scans tiles r, r + cluster size, ... with one
@@ -887,10 +926,42 @@ static int tile_rows(int tiles, int n_pages, int hkv)
     return rows < tiles ? rows : tiles;
 }
 
+// blocks per page of the warp kernels: one, or a cluster that has a warp for every head when the call has few pages
+static int warp_cluster(int hkv, int n_pages)
+{
+    const int c = (hkv + kDemoteWarps - 1) / kDemoteWarps;
+    return n_pages > 2 * 148 ? 1 : c < 8 ? c : 8;
+}
+
+// grid rows of the tile-parallel warp kernels: enough for 12 warps on every SM
+static int warp_tile_rows(int tiles, int n_pages, int hkv)
+{
+    int rows = (12 * 148 + n_pages * hkv - 1) / (n_pages * hkv);
+    if (rows < 16) rows = 16;
+    return rows < tiles ? rows : tiles;
+}
+
+template <int D, int FMT, bool BIG>
+static cudaError_t launch_demote_warp(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
+                                      const int64_t* entry, int64_t n_entries, uint32_t* tickets, cudaStream_t s)
+{
+    const int warps = p->hkv < kDemoteWarps ? p->hkv : kDemoteWarps, c = warp_cluster(p->hkv, BIG ? 0 : n);
+    const int smem = DemoteWarp<D>::OFF_WARPS + warps * DemoteWarp<D>::BYTES;
+    static_assert(DemoteWarp<D>::OFF_WARPS + kDemoteWarps * DemoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
+    return launch_pdl(demote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv) : 1), 32 * warps,
+                      (size_t)smem, c, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv,
+                      p->tiles, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
+}
+
 template <int D, int FMT>
 static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
                                const int64_t* entry, int64_t n_entries, cudaStream_t s)
 {
+    const bool unit_scales = p->cfg.k_scale == 1.0f && p->cfg.v_scale == 1.0f;      // what the warp kernel's exactness rests on
+    if (p->tiles == 1 && unit_scales) {
+        MKV_CUDA((launch_demote_warp<D, FMT, false>(p, src, dst, n, bt, tags, entry, n_entries, nullptr, s)));
+        return MKV_OK;
+    }
     if (p->tiles == 1) {
         const int c = heads_cluster(p->hkv, n);
         MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
@@ -909,6 +980,10 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
                                   p->cfg.tq3_pages, p->hkv, p->tiles, p->cfg.v_scale, src, dst));
     }
     const int ch = heads_cluster(p->hkv, 0);
+    if (unit_scales)
+        MKV_CUDA((launch_demote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
+                                                   fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
+    else
     MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, n <= 148, s,
                                    (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv, p->tiles,
                                    p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr,

@@ -740,15 +740,18 @@ __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], f
 // 21 bits below the largest coordinate (one fp16, 11 bits, is not enough for the 2e-3 bound; two int8 digits,
 // 15 bits, fail it on short peaked rows by simulation).  The integer sums are exact.
 
-// Two 32-dim steps (2j, 2j+1) of a Stale page: word triple (A, B, C) of the lane -> eight B registers
-// (step, token half u, K half), then per step and token half one MMA for digits 0,1 and one for digit 2.
-// q_pair: shared-memory address of this lane's query fragments of step 2j (digits 0,1 at +0, digit 2 at +512,
-// step 2j+1 at +1024).
-// SPLIT: one MMA per step and token half; rows 0-3 digit 0, 4-7 digit 1, 8-11 and 12-15 digit 2 of heads 0-3
-// (step 2j at +0, step 2j+1 at +512).
-template <bool FIRST, bool SPLIT>      // FIRST: the page's first two steps start the four sums
-__device__ __forceinline__ void tq3_key_pair_v2(int (&Sa0)[4], int (&Sb0)[4], int (&Sa1)[4], int (&Sb1)[4],
-                                                uint32_t A, uint32_t Bw, uint32_t Cw, uint32_t q_pair)
+// Two 32-dim steps (2j, 2j+1) of a Stale page: word triple (A, B, C) of the lane -> eight operand registers
+// (step, token half, K half), tokens g and g + 8.  They are an A fragment (16 tokens x 32 dims) as well as two B
+// fragments (32 dims x 8 tokens):
+//   more than four heads: A = keys, B = one query digit of eight heads: three MMAs per step give S_d[token][head],
+//     d = 0, 1, 2 (with the query as A its digits fill one and a half fragments: four MMAs for 16 tokens; 2 x 59,008
+//     tokens in 16 layers: 558 -> 540 us);
+//   SPLIT: A = query, rows 0-3 digit 0, 4-7 digit 1, 8-11 and 12-15 digit 2 of heads 0-3: one MMA per token half.
+// q_pair: shared-memory address of this lane's query fragments of step 2j; a step has 512 bytes (SPLIT), or
+// digits 0 and 1 (16 bytes a lane), then digit 2 (8 bytes a lane; `q2_pair`) 512 bytes behind, 768 in all.
+template <bool FIRST, bool SPLIT>      // FIRST: the page's first two steps start the sums
+__device__ __forceinline__ void tq3_key_pair_v2(int (&S0)[4], int (&S1)[4], int (&S2)[4],
+                                                uint32_t A, uint32_t Bw, uint32_t Cw, uint32_t q_pair, uint32_t q2_pair)
 {
     // signed levels +-{2, 6, 11, 18} (eight times the codebook) as bytes, indexed by code = magnitude | sign << 2
     constexpr uint32_t T0 = 0x120B0602u, T1 = 0xEEF5FAFEu;
@@ -764,31 +767,29 @@ __device__ __forceinline__ void tq3_key_pair_v2(int (&Sa0)[4], int (&Sb0)[4], in
     }
 #pragma unroll
     for (int st = 0; st < 2; ++st) {
+        const uint32_t k0 = r[4 * st], k1 = r[4 * st + 1], k2 = r[4 * st + 2], k3 = r[4 * st + 3];
         if constexpr (SPLIT) {
             const uint4 q = lds128(q_pair + st * 512);
             if (FIRST && st == 0) {
-                mma16832_s8_zero(Sa0, q.x, q.y, q.z, q.w, r[0], r[1]);
-                mma16832_s8_zero(Sa1, q.x, q.y, q.z, q.w, r[2], r[3]);
+                mma16832_s8_zero(S0, q.x, q.y, q.z, q.w, k0, k1);
+                mma16832_s8_zero(S1, q.x, q.y, q.z, q.w, k2, k3);
             } else {
-                mma16832_s8(Sa0, q.x, q.y, q.z, q.w, r[4 * st], r[4 * st + 1]);
-                mma16832_s8(Sa1, q.x, q.y, q.z, q.w, r[4 * st + 2], r[4 * st + 3]);
+                mma16832_s8(S0, q.x, q.y, q.z, q.w, k0, k1);
+                mma16832_s8(S1, q.x, q.y, q.z, q.w, k2, k3);
             }
-            continue;
+        } else {
+            const uint4 q = lds128(q_pair + st * 768);
+            const uint2 q2 = lds64(q2_pair + st * 768);
+            if (FIRST && st == 0) {
+                mma16832_s8_zero(S0, k0, k2, k1, k3, q.x, q.y);
+                mma16832_s8_zero(S1, k0, k2, k1, k3, q.z, q.w);
+                mma16832_s8_zero(S2, k0, k2, k1, k3, q2.x, q2.y);
+            } else {
+                mma16832_s8(S0, k0, k2, k1, k3, q.x, q.y);
+                mma16832_s8(S1, k0, k2, k1, k3, q.z, q.w);
+                mma16832_s8(S2, k0, k2, k1, k3, q2.x, q2.y);
+            }
         }
-        // (the second fragment's rows 8-15 are stored as zeros: a full 16-byte load keeps the four operand
-        // registers together, where building {x, 0, y, 0} cost two moves per MMA)
-        const uint4 qa = lds128(q_pair + st * 1024), qb = lds128(q_pair + st * 1024 + 512);
-        if (FIRST && st == 0) {
-            mma16832_s8_zero(Sa0, qa.x, qa.y, qa.z, qa.w, r[0], r[1]);
-            mma16832_s8_zero(Sb0, qb.x, qb.y, qb.z, qb.w, r[0], r[1]);
-            mma16832_s8_zero(Sa1, qa.x, qa.y, qa.z, qa.w, r[2], r[3]);
-            mma16832_s8_zero(Sb1, qb.x, qb.y, qb.z, qb.w, r[2], r[3]);
-            continue;
-        }
-        mma16832_s8(Sa0, qa.x, qa.y, qa.z, qa.w, r[4 * st], r[4 * st + 1]);
-        mma16832_s8(Sb0, qb.x, qb.y, qb.z, qb.w, r[4 * st], r[4 * st + 1]);
-        mma16832_s8(Sa1, qa.x, qa.y, qa.z, qa.w, r[4 * st + 2], r[4 * st + 3]);
-        mma16832_s8(Sb1, qb.x, qb.y, qb.z, qb.w, r[4 * st + 2], r[4 * st + 3]);
     }
 }
 
@@ -841,7 +842,7 @@ __device__ __forceinline__ void softmax_rescale_v2(WarpAcc<NB>& acc, const float
 
 // P of head g for the lane's four tokens is the B fragment of the value product as it stands (tokens 8-15 four
 // times as large, see value_operands).
-template <int NB, bool SPLIT>
+template <int NB>
 __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
     const float p0 = fast_exp2(s[0] - acc.mr), p1 = fast_exp2(s[1] - acc.mr);
@@ -851,14 +852,11 @@ __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (
     const float2 h01 = half2_to_float2(pf.b0), h23 = half2_to_float2(pf.b1);
     pf.c0 = pack_f16x2(p0 - h01.x, p1 - h01.y);
     pf.c1 = pack_f16x2(p2 - h23.x, p3 - h23.y);
-    if constexpr (SPLIT) {                   // rows 4-7 carry the low halves of heads 0-3
-        pf.b0 = lane & 16 ? pf.c0 : pf.b0;
-        pf.b1 = lane & 16 ? pf.c1 : pf.b1;
-    }
+    pf.b0 = lane & 16 ? pf.c0 : pf.b0;       // rows 4-7 carry the low halves of heads 0-3
+    pf.b1 = lane & 16 ? pf.c1 : pf.b1;
     const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x34003400u, 0x34003400u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
-    if constexpr (!SPLIT) mma16816(ps, ones, pf.c0, pf.c1);
     pf.ps0 = ps[0];
     pf.ps1 = ps[1];
     acc.l[0] += ps[0];
@@ -871,17 +869,17 @@ __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (
 // phases overlap.  DO_V / DO_K switch the halves off for the first and the last page.
 template <int D, bool DO_V, bool DO_K, bool DEFER, int FMT, bool SPLIT>
 __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, const float (&s_cur)[4], PFrag& pf, uint32_t rec_k,
-                                         uint32_t qt_lane, float sc2, int lane, float (&s_next)[4])
+                                         uint32_t qt_lane, float sc2, float sc2b, int lane, float (&s_next)[4])
 {
     constexpr int NB = D / 16, LW = 3 * NB / 4;
     const int g = lane >> 2;
     uint32_t kw[LW], vw[LW];
     float S0[4] = {0.f, 0.f, 0.f, 0.f}, S1[4] = {0.f, 0.f, 0.f, 0.f};
-    int I0[4], I1[4], I2[4], I3[4];     // format 2: (digits 0,1 | 2) x (tokens g | g+8), started by the first pair of steps
+    int I0[4], I1[4], I2[4];            // format 2: digits 0, 1, 2; SPLIT: tokens g, g + 8; started by the first pair of steps
     if constexpr (DO_K) load_lane_words<D>(rec_k, lane, kw);
     if constexpr (DO_V) load_lane_words<D>(rec_v + 6 * D, lane, vw);
     if constexpr (DO_V) {      // in one block with the key unpack of the next page
-        if constexpr (FMT == 2) softmax_probs_v2<NB, SPLIT>(acc, s_cur, pf, lane);
+        if constexpr (FMT == 2 && SPLIT) softmax_probs_v2<NB>(acc, s_cur, pf, lane);
         else softmax_probs<NB, true, SPLIT>(acc, s_cur, pf, lane);
     }
     if constexpr (DO_V && DEFER) {
@@ -893,9 +891,9 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
     for (int j = 0; j < NB / 4; ++j) {
         if constexpr (DO_K) {
             if constexpr (FMT == 2) {
-                if (j == 0) tq3_key_pair_v2<true, SPLIT>(I0, I1, I2, I3, kw[0], kw[1], kw[2], qt_lane);
-                else tq3_key_pair_v2<false, SPLIT>(I0, I1, I2, I3, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2],
-                                                   qt_lane + j * (SPLIT ? 1024 : 2048));
+                const uint32_t q = qt_lane + j * (SPLIT ? 1024 : 1536), q2 = q - lane * 8 + 512;
+                if (j == 0) tq3_key_pair_v2<true, SPLIT>(I0, I1, I2, kw[0], kw[1], kw[2], q, q2);
+                else tq3_key_pair_v2<false, SPLIT>(I0, I1, I2, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], q, q2);
             }
             else tq3_key_quad<SPLIT>(S0, S1, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * (SPLIT ? 1024 : 2048));
         }
@@ -903,32 +901,33 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
             tq3_value_quad<DEFER, SPLIT>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
                                   vw[3 * j + 2], meta + j * 256, pf);
     }
-    if constexpr (DO_K && FMT == 2) {
-        // head g, tokens 2tq, 2tq+1 (I0 | I1) and 2tq+8, 2tq+9 (I2 | I3): the three query digits, then the token's
-        // norm correction
+    if constexpr (DO_K && FMT == 2 && SPLIT) {
+        // head g % 4, tokens 2tq, 2tq+1 (I0) and 2tq+8, 2tq+9 (I1): the three query digits, then the token's norm
+        // correction (sc2 carries the head's digit unit delta_h / 8 here)
         const int tq = lane & 3;
         const uint32_t gaddr = rec_k + 12 * D + 4 * tq;
         const float2 ga = half2_to_float2(lds32(gaddr)), gb = half2_to_float2(lds32(gaddr + 16));
-        // (sc2 carries the head's digit unit delta_h / 8 here)
-        if constexpr (SPLIT) {
-            // this lane has digit 0 (g < 4) or 1 (g >= 4) and digit 2 of head g % 4, the lane 16 away the other one
-            const float mine = lane & 16 ? 128.f : 16384.f, theirs = lane & 16 ? 16384.f : 128.f;
-            float d[4];
+        // this lane has digit 0 (g < 4) or 1 (g >= 4) and digit 2 of head g % 4, the lane 16 away the other one
+        const float mine = lane & 16 ? 128.f : 16384.f, theirs = lane & 16 ? 16384.f : 128.f;
+        float d[4];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                d[e] = fmaf((float)I0[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I0[e], 16), theirs, (float)I0[2 + e]));
-                d[2 + e] = fmaf((float)I2[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I2[e], 16), theirs, (float)I2[2 + e]));
-            }
-            s_next[0] = d[0] * (ga.x * sc2);
-            s_next[1] = d[1] * (ga.y * sc2);
-            s_next[2] = d[2] * (gb.x * sc2);
-            s_next[3] = d[3] * (gb.y * sc2);
-            return;
+        for (int e = 0; e < 2; ++e) {
+            d[e] = fmaf((float)I0[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I0[e], 16), theirs, (float)I0[2 + e]));
+            d[2 + e] = fmaf((float)I1[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I1[e], 16), theirs, (float)I1[2 + e]));
         }
-        s_next[0] = digits_to_score(I0[0], I0[2], I1[0]) * (ga.x * sc2);
-        s_next[1] = digits_to_score(I0[1], I0[3], I1[1]) * (ga.y * sc2);
-        s_next[2] = digits_to_score(I2[0], I2[2], I3[0]) * (gb.x * sc2);
-        s_next[3] = digits_to_score(I2[1], I2[3], I3[1]) * (gb.y * sc2);
+        s_next[0] = d[0] * (ga.x * sc2);
+        s_next[1] = d[1] * (ga.y * sc2);
+        s_next[2] = d[2] * (gb.x * sc2);
+        s_next[3] = d[3] * (gb.y * sc2);
+    }
+    if constexpr (DO_K && FMT == 2 && !SPLIT) {
+        // tokens g, g + 8 of heads 2tq, 2tq + 1 (digit units in sc2, sc2b)
+        const uint32_t gaddr = rec_k + 12 * D;
+        const float r0 = __half2float(__ushort_as_half(lds16(gaddr + 2 * g))), r1 = __half2float(__ushort_as_half(lds16(gaddr + 2 * g + 16)));
+        s_next[0] = digits_to_score(I0[0], I1[0], I2[0]) * (r0 * sc2);
+        s_next[1] = digits_to_score(I0[1], I1[1], I2[1]) * (r0 * sc2b);
+        s_next[2] = digits_to_score(I0[2], I1[2], I2[2]) * (r1 * sc2);
+        s_next[3] = digits_to_score(I0[3], I1[3], I2[3]) * (r1 * sc2b);
     }
     if constexpr (DO_K && FMT == 1) {
         const uint32_t gaddr = rec_k + 12 * D;
@@ -1402,7 +1401,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             pending |= 1u << ((uint32_t)i % NSTAGE);
             if (lane == 0) {
                 const uint32_t s = (uint32_t)i % NSTAGE;
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 if constexpr (!TILED) {
                     mbar_expect_tx(bars + 8 * s, G::TQ3_REC);
                     bulk_load(ring + s * G::SLOT, tq3_base + (size_t)list3[i] * hkv * G::TQ3_REC, G::TQ3_REC, bars + 8 * s);
@@ -1428,7 +1426,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 } else {
                     rec = P.fp8 + (((size_t)e8 * hkv + h) * P.tiles + (lpg8[i] & 0x7FFF)) * (2 * G::FP8_HALF);
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_expect_tx(bars + 8 * s, G::FP8_HALF);
                 bulk_load(ring + s * G::SLOT, rec, G::FP8_HALF, bars + 8 * s);
                 mbar_expect_tx(bars + 8 * (s + 1), G::FP8_HALF);
@@ -1501,6 +1498,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         int done = 0;
         if (n_my > 0) {
             done = build_lists(0);
+            // The ring was the reduction buffer: the copies come after those stores.  (Slots that are used again inside a
+            // segment were only read since, and the reads are over: no fence per page.)
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             start_round();
             // limit 0 (diagnostic): the first look comes before the query is prepared, while the copy is still in flight
             if (P.wait_ns == 0 && n3 + n8 > 0 && !__all_sync(FULL, mbar_test_wait(bars, phase & 1u))) {
@@ -1540,10 +1540,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             __half* qt = reinterpret_cast<__half*>(smem + G::OFF_QT);
             __half* qf = reinterpret_cast<__half*>(smem + G::OFF_QF);
             if constexpr (FMT == 2) {
-                // rotated query as three balanced base-128 digits in the A-fragment order of the integer key
-                // products: dim i sits in step i/32 at K slot k = i%32 of fragment lane 4 hd + (k%16)/4, byte k%4;
-                // digits 0,1 in registers 2 (k/16) + digit of the step's first 512 bytes, digit 2 in register 2 (k/16)
-                // of the second 512 bytes, whose odd registers (fragment rows 8-15) are zero
+                // rotated query as three balanced base-128 digits in the fragment order of the integer key
+                // products: dim i sits in step i/32 at K slot k = i%32 of fragment lane 4 hd + (k%16)/4, byte k%4 of
+                // register k/16 of its digit (see tq3_key_pair_v2)
                 uint8_t* qt8 = smem + G::OFF_QT;
                 float amax = 0.f;
 #pragma unroll
@@ -1572,9 +1571,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                         *reinterpret_cast<uint2*>(at + 256) = make_uint2(word[1], word[2]);
                         continue;
                     }
-                    *reinterpret_cast<uint32_t*>(qt8 + ((st * 2) * 32 + L) * 16 + (2 * (k >> 4)) * 4) = word[0];
-                    *reinterpret_cast<uint32_t*>(qt8 + ((st * 2) * 32 + L) * 16 + (2 * (k >> 4) + 1) * 4) = word[1];
-                    *reinterpret_cast<uint2*>(qt8 + ((st * 2 + 1) * 32 + L) * 16 + (k >> 4) * 8) = make_uint2(word[2], 0u);
+                    uint32_t* at = reinterpret_cast<uint32_t*>(qt8 + st * 768 + L * 16) + (k >> 4);
+                    at[0] = word[0];
+                    at[2] = word[1];
+                    reinterpret_cast<uint32_t*>(qt8 + st * 768 + 512 + L * 8)[k >> 4] = word[2];
                 }
             }
 #pragma unroll
@@ -1598,8 +1598,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             }
         }
         __syncthreads();
-        // score unit of the Stale pages: record format 2 counts in digit units of this lane's head g
-        const float sc2k = FMT == 2 ? sc2 * reinterpret_cast<const float*>(smem + G::OFF_QS)[SPLIT ? g & 3 : g] : sc2;
+        // score units of the Stale pages: record format 2 counts in digit units of this lane's head(s)
+        const float* digit_unit = reinterpret_cast<const float*>(smem + G::OFF_QS);
+        const float sc2k = FMT == 2 ? sc2 * digit_unit[SPLIT ? g & 3 : 2 * tq] : sc2;
+        const float sc2k1 = FMT == 2 && !SPLIT ? sc2 * digit_unit[2 * tq + 1] : sc2;
 
         for (bool more = n_my > 0; more && !failed;) {
             // ---- Stale pages: scores of page i+1 are computed together with the output update of page i
@@ -1613,12 +1615,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     cur_lp = lpg3[0] >> 16;
                 }
                 wait_slot(0);
-                if (!failed) tq3_step<D, false, true, TILED, FMT, SPLIT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, lane, s_cur);
+                if (!failed) tq3_step<D, false, true, TILED, FMT, SPLIT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, sc2k1, lane, s_cur);
                 for (int i = 0; i + 1 < n3 && !failed; ++i) {
                     const uint32_t cur = (uint32_t)i % NSTAGE, nxt = (uint32_t)(i + 1) % NSTAGE;
                     wait_slot(nxt);
                     if (failed) break;
-                    if constexpr (FMT == 2) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
+                    if constexpr (FMT == 2 && SPLIT) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
                     else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
                         const int pg_i = list3[i];
@@ -1628,7 +1630,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                             cur_lp = lpg3[i] >> 16;
                         }
                     }
-                    tq3_step<D, true, true, TILED, FMT, SPLIT>(acc, ring + cur * G::SLOT, s_cur, pf, ring + nxt * G::SLOT, qt_lane, sc2k, lane, s_next);
+                    tq3_step<D, true, true, TILED, FMT, SPLIT>(acc, ring + cur * G::SLOT, s_cur, pf, ring + nxt * G::SLOT, qt_lane, sc2k, sc2k1, lane, s_next);
                     if constexpr (SCORED && !TILED) store_page_mass<NB, SPLIT>(acc, pf.ps0, pf.ps1, mass_row + lpg3[i], P.max_pages, GQ, lane);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) s_cur[e] = s_next[e];
@@ -1637,7 +1639,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 }
                 if (!failed) {
                     if (n8 > 0) issue_fp8(0);
-                    if constexpr (FMT == 2) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
+                    if constexpr (FMT == 2 && SPLIT) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
                     else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
                         const int pg_i = list3[n3 - 1];
@@ -1647,7 +1649,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                             cur_lp = lpg3[n3 - 1] >> 16;
                         }
                     }
-                    tq3_step<D, true, false, TILED, FMT, SPLIT>(acc, ring + ((uint32_t)(n3 - 1) % NSTAGE) * G::SLOT, s_cur, pf, 0, qt_lane, sc2k, lane, s_next);
+                    tq3_step<D, true, false, TILED, FMT, SPLIT>(acc, ring + ((uint32_t)(n3 - 1) % NSTAGE) * G::SLOT, s_cur, pf, 0, qt_lane, sc2k, sc2k1, lane, s_next);
                     if constexpr (SCORED && !TILED) store_page_mass<NB, SPLIT>(acc, pf.ps0, pf.ps1, mass_row + lpg3[n3 - 1], P.max_pages, GQ, lane);
                     if constexpr (TILED) fold(cur_page, true, cur_lp);   // back to output units for the FP8 pages and the reduction
                 }
@@ -1667,7 +1669,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     fp8_page<D, SCORED, TILED, SPLIT>(acc, ring + s * G::SLOT, ring + (s + 1) * G::SLOT, qf_lane, sc2 * P.k_scale, P.v_scale,
                                                valid ? valid : kPage, lane,
                                                SCORED ? mass_row + (TILED ? (lpg8[i] >> 16) : lpg8[i]) : nullptr, P.max_pages, GQ);
-                    if constexpr (FMT == 2) max_rows_from_columns<NB>(acc, lane);     // the page may have raised the maxima
+                    if constexpr (FMT == 2 && SPLIT) max_rows_from_columns<NB>(acc, lane);     // the page may have raised the maxima
                     __syncwarp();
                     if (i + NSTAGE / 2 < n8) issue_fp8(i + NSTAGE / 2);
                 }

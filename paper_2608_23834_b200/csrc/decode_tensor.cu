@@ -39,7 +39,7 @@ namespace mkv {
 constexpr int kMaxBatch = 1024;      // requests per call
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-constexpr float kRescaleSlack = 8.0f;   // running maximum is only raised when exceeded by 2^8
+constexpr float kRescaleSlack = 7.0f;   // running maximum is only raised when exceeded by 2^7
 constexpr unsigned long long kDefaultWaitNs = 20000000ull;   // 20 ms: far beyond any copy that is going to arrive
 
 size_t decode_ws_tensor_bytes(int, int, int, int d)
@@ -296,10 +296,13 @@ __device__ __forceinline__ void value_operands(uint32_t (&a)[4], uint32_t W0, ui
         a[0] = value_bits<4>(W2); a[1] = value_bits<7>(W2); a[2] = value_bits<2>(X2); a[3] = value_bits<5>(X2);
     }
 }
-template <int BLOCK, int HI>      // what a unit of the sums is worth in codes: 2^(24 - POS) of the row's register 0 / 1
+// What a unit of the sums is worth in codes: 2^(24 - POS) of the row's register 0 / 1, the probabilities entering
+// 2^6 (tokens 0-7) and 2^8 times as large: that keeps the units within fp16's powers of two, for half_times, and
+// the products within fp16's range (probabilities are at most 2^kRescaleSlack).
+template <int BLOCK, int HI>
 __device__ __forceinline__ constexpr float value_unit()
 {
-    return BLOCK % 2 == 0 ? (HI ? 2097152.f : 65536.f) : (HI ? 131072.f : 1048576.f);
+    return BLOCK % 2 == 0 ? (HI ? 32768.f : 1024.f) : (HI ? 2048.f : 16384.f);
 }
 
 __device__ __forceinline__ float2 half2_to_float2(uint32_t x)
@@ -307,13 +310,31 @@ __device__ __forceinline__ float2 half2_to_float2(uint32_t x)
     return __half22float2(*reinterpret_cast<const __half2*>(&x));
 }
 
+// fp16 bits of a power of two from 1 to 2^15
+__device__ __forceinline__ constexpr uint32_t unit_bits(float x)
+{
+    uint32_t e = 15;
+    for (; x >= 2.f; x *= 0.5f) ++e;
+    return e << 10;
+}
+
+// h * 2^k in fp32, conversion and product in one mixed-precision FMA
+template <uint32_t UNIT>
+__device__ __forceinline__ float half_times(uint16_t h)
+{
+    float r;
+    asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(r) : "h"(h), "h"((uint16_t)UNIT), "f"(0.f));
+    return r;
+}
+
 // acc[channel rows g, g+8][heads] += scale_row * t + zero_row * psum_head, t in units of value_unit<BLOCK, row>
 template <int BLOCK>
 __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (&t)[4], uint32_t sc_pair, uint32_t zp_pair,
                                                   float ps0, float ps1)
 {
-    const float2 sc = half2_to_float2(sc_pair), zp = half2_to_float2(zp_pair);
-    const float s0 = sc.x * value_unit<BLOCK, 0>(), s1 = sc.y * value_unit<BLOCK, 1>();     // exact
+    const float2 zp = half2_to_float2(zp_pair);
+    const float s0 = half_times<unit_bits(value_unit<BLOCK, 0>())>((uint16_t)sc_pair),      // exact
+                s1 = half_times<unit_bits(value_unit<BLOCK, 1>())>((uint16_t)(sc_pair >> 16));
     acc[0] = fmaf(s0, t[0], fmaf(zp.x, ps0, acc[0]));
     acc[1] = fmaf(s0, t[1], fmaf(zp.x, ps1, acc[1]));
     acc[2] = fmaf(s1, t[2], fmaf(zp.y, ps0, acc[2]));
@@ -568,14 +589,14 @@ __device__ __forceinline__ void softmax_rescale(WarpAcc<NB>& acc, const float (&
 }
 
 // Second half, branch-free (so that it can be scheduled into the unpack work of the next page): P and its row sums.
-// STALE: the operands of the second token half are four times the probabilities (value_operands); the row sums
-// take the factor out again.
+// STALE: the operands are 2^6 (second token half: 2^8) times the probabilities (value_operands, value_unit); the row
+// sums take the factors out again.
 template <int NB, bool STALE, bool SPLIT>
 __device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
-    const float up = STALE ? 2.f : 0.f;
-    const float p0 = fast_exp2(s[0] - acc.m[0]), p1 = fast_exp2(s[1] - acc.m[1]);
-    const float p2 = fast_exp2(s[2] - (acc.m[0] - up)), p3 = fast_exp2(s[3] - (acc.m[1] - up));
+    const float up = STALE ? 6.f : 0.f, up2 = STALE ? 8.f : 0.f;
+    const float p0 = fast_exp2(s[0] - (acc.m[0] - up)), p1 = fast_exp2(s[1] - (acc.m[1] - up));
+    const float p2 = fast_exp2(s[2] - (acc.m[0] - up2)), p3 = fast_exp2(s[3] - (acc.m[1] - up2));
     const uint32_t ph01 = pack_f16x2(p0, p1), ph23 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(ph01), h23 = half2_to_float2(ph23);
     const uint32_t pl01 = pack_f16x2(p0 - h01.x, p1 - h01.y), pl23 = pack_f16x2(p2 - h23.x, p3 - h23.y);
@@ -589,7 +610,7 @@ __device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)
         pf.c1 = movmatrix_trans(pl23);
     }
     // row sums through the tensor core: the same P that multiplies V
-    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, STALE ? 0x34003400u : 0x3C003C00u, STALE ? 0x34003400u : 0x3C003C00u};
+    const uint32_t ones[4] = {STALE ? 0x24002400u : 0x3C003C00u, STALE ? 0x24002400u : 0x3C003C00u, STALE ? 0x1C001C00u : 0x3C003C00u, STALE ? 0x1C001C00u : 0x3C003C00u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
     if constexpr (!SPLIT) mma16816(ps, ones, pf.c0, pf.c1);
@@ -845,8 +866,8 @@ __device__ __forceinline__ void softmax_rescale_v2(WarpAcc<NB>& acc, const float
 template <int NB>
 __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
-    const float p0 = fast_exp2(s[0] - acc.mr), p1 = fast_exp2(s[1] - acc.mr);
-    const float p2 = fast_exp2(s[2] - (acc.mr - 2.f)), p3 = fast_exp2(s[3] - (acc.mr - 2.f));
+    const float p0 = fast_exp2(s[0] - (acc.mr - 6.f)), p1 = fast_exp2(s[1] - (acc.mr - 6.f));
+    const float p2 = fast_exp2(s[2] - (acc.mr - 8.f)), p3 = fast_exp2(s[3] - (acc.mr - 8.f));
     pf.b0 = pack_f16x2(p0, p1);
     pf.b1 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(pf.b0), h23 = half2_to_float2(pf.b1);
@@ -854,7 +875,7 @@ __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (
     pf.c1 = pack_f16x2(p2 - h23.x, p3 - h23.y);
     pf.b0 = lane & 16 ? pf.c0 : pf.b0;       // rows 4-7 carry the low halves of heads 0-3
     pf.b1 = lane & 16 ? pf.c1 : pf.b1;
-    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x34003400u, 0x34003400u};
+    const uint32_t ones[4] = {0x24002400u, 0x24002400u, 0x1C001C00u, 0x1C001C00u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
     pf.ps0 = ps[0];

@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
+#include <math_constants.h>
 
 #include <cmath>
 
@@ -1008,405 +1009,36 @@ int32_t launch_demote(mkv_pool* p, const int32_t* src, const int32_t* dst, int n
 }
 
 // ------------------------------------------------------------------------------------------ promote
-// Promote (Algorithm 1 step 3): reconstruct a Stale page into a newly allocated FP8 page, then publish
-// it as Anchor.  One cluster per page, its blocks sharing out the KV heads as in demote_kernel.  The
-// record is staged in shared memory;
-// warps rebuild key vectors (signed levels, shuffle Walsh-Hadamard, norm correction, sign), threads
-// rebuild value channels; the fp32 operation order is fixed so that the written bytes are reproducible.
-//
-// Reading the code sections back (inverse of the packer in demote_kernel): fragment lane
-// L = 4 (row % 8) + (slot % 8) / 2 holds, in nibble 2 rr + slot % 2 with rr = row / 8 + 2 (slot / 8),
-// the entry (row, slot) of every 16 x 16 block; for keys row = token and slot = channel % 16, for
-// values row = channel % 16 and slot = token.
-// D = A B + C with 8-bit integers: A 16 x 32 (row-major fragments), B 32 x 8 (column-major), C 16 x 8 in int32
-__device__ __forceinline__ void imma16832(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+// Promote (Algorithm 1 step 3): reconstruct a Stale page into a newly allocated FP8 page, then publish it as Anchor.
+#include "promote_warp.cuh"
+
+template <int D, int FMT, bool BIG>
+static cudaError_t launch_promote_warp(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
+                                       const int64_t* entry, int64_t n_entries, uint32_t* tickets, cudaStream_t s)
 {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// Keys of one record of format 2 back to e4m3 rows (Promote), the inverse rotation as a matrix product.
-// The levels of format 2 are eighths of the integers +-2, +-6, +-11, +-18, so the transform H c of a token's d
-// levels consists of sums of integers below 2^13: every order of summation gives the same value, and the
-// butterflies can be replaced by the product C[16 tokens x d] H[d x d] in 8-bit integer tensor-core
-// instructions (exact int32 sums).  The record's key section already is the A operand: lane 4 (t % 8) + (k % 16) / 4
-// holds, per 32-dim step, the codes of tokens g, g + 8 at dims 4 tq .. + 3 and 16 + 4 tq .. + 3, and one
-// byte-table lookup turns four codes into four signed bytes.  H[k][n] = (-1)^popcount(k & n) needs no table: for
-// lane (g, tq), column n = 8 j + g and rows k = 32 s + 16 b + 4 tq + i its sign is the product of a per-lane
-// pattern over i, a per-warp part and a part that is known at compile time.
-// Warp w computes the column tiles j = w, w + D/32, ... (eight columns each); results go to `ktile`
-// [16 tokens][D] e4m3 in shared memory.  All D threads call it; the caller synchronises before reading ktile.
-// What promote_keys_v2 needs per lane and warp, computed once per block.
-template <int D>
-struct PromoteKeyLane {
-    uint32_t b0p, b1p, b0n, b1n;          // B fragments of H for this lane: both K halves, plain and negated
-    uint32_t o0p, o1p, o0n, o1n;          // the same for the odd steps (negated in warps whose columns have bit 5 of n set)
-    uint32_t flip[D / 8 / (D / 32)][2];   // rotation signs of the lane's two columns of every tile, as fp32 sign bits
-    __device__ __forceinline__ void init(const SigmaBits& sigma, int warp, int lane)
-    {
-        constexpr uint32_t NEG = 0xFEFEFEFEu;             // x ^ NEG negates bytes +-1
-        constexpr int NWARP = D / 32, NTILE = D / 8 / NWARP;
-        const int g = lane >> 2, tq = lane & 3;
-        // (-1)^popcount(k & n), k = 32 s + 16 b + 4 tq + i, n = 8 j + g, j = NWARP t + warp:
-        //   bits 0-1: i & g -> the byte pattern W over i;  bit 2: tq0 & g2;  bit 3: tq1 & j0 (j0 = warp & 1);
-        //   bit 4: b & j1 (j1 = (warp >> 1) & 1);  bits 5-7: s & (j >> 2), of which bit 0 of j >> 2 is warp >> 2 for
-        //   D = 256 (it negates the odd steps) and the rest is the tile index (compile time)
-        const uint32_t W = (g & 3) == 0 ? 0x01010101u : (g & 3) == 1 ? 0xFF01FF01u : (g & 3) == 2 ? 0xFFFF0101u : 0x01FFFF01u;
-        const bool lane_odd = (((tq & 1) & (g >> 2)) ^ ((tq >> 1) & (warp & 1))) != 0;
-        b0p = lane_odd ? (W ^ NEG) : W;
-        b1p = ((warp >> 1) & 1) ? (b0p ^ NEG) : b0p;
-        b0n = b0p ^ NEG;
-        b1n = b1p ^ NEG;
-        const bool w2 = ((warp >> 2) & 1) != 0;
-        o0p = w2 ? b0n : b0p;
-        o1p = w2 ? b1n : b1p;
-        o0n = w2 ? b0p : b0n;
-        o1n = w2 ? b1p : b1n;
-#pragma unroll
-        for (int t = 0; t < NTILE; ++t) {
-            const int n0 = 8 * (NWARP * t + warp) + 2 * tq;
-            const uint32_t sg = (sigma.w[n0 >> 5] >> (n0 & 31)) & 3u;
-            flip[t][0] = (sg & 1u) << 31;
-            flip[t][1] = (sg & 2u) << 30;
-        }
-    }
-};
-
-// Keys of one record of format 2 back to e4m3 rows (Promote), the inverse rotation as a matrix product.
-// The levels of format 2 are eighths of the integers +-2, +-6, +-11, +-18, so the transform H c of a token's d
-// levels consists of sums of integers below 2^13: every order of summation gives the same value, and the
-// butterflies can be replaced by the product C[16 tokens x d] H[d x d] in 8-bit integer tensor-core
-// instructions (exact int32 sums).  The record's key section already is the A operand: lane 4 (t % 8) + (k % 16) / 4
-// holds, per 32-dim step, the codes of tokens g, g + 8 at dims 4 tq .. + 3 and 16 + 4 tq .. + 3, and one
-// byte-table lookup turns four codes into four signed bytes.  H[k][n] = (-1)^popcount(k & n) needs no table
-// (PromoteKeyLane).  Warp w computes the column tiles j = w, w + D/32, ... (eight columns each); results go to
-// `ktile` [16 tokens][D] e4m3 in shared memory.  All D threads call it; the caller synchronises before reading ktile.
-template <int D>
-__device__ __forceinline__ void promote_keys_v2(const uint8_t* img, uint8_t* ktile, uint4* afrag, const PromoteKeyLane<D>& L,
-                                                float rs, float inv_k_scale, bool unit_k)
-{
-    constexpr int NS = D / 32;            // 32-dim steps (K of the product)
-    constexpr int NWARP = D / 32;         // warps of the block
-    constexpr int NTILE = D / 8 / NWARP;  // column tiles per warp (4)
-    constexpr uint32_t T0 = 0x120B0602u, T1 = 0xEEF5FAFEu;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
-    // ---- A: the record's codes as signed bytes, 4 registers per step.  Warp s unpacks step s for everybody
-    // (afrag [step][lane] in shared memory), then every warp fetches all steps.
-    {
-        const int j = warp >> 1;
-        const uint32_t A = *reinterpret_cast<const uint32_t*>(img + lane_word_offset(D, lane, 3 * j));
-        const uint32_t Bw = *reinterpret_cast<const uint32_t*>(img + lane_word_offset(D, lane, 3 * j + 1));
-        const uint32_t Cw = *reinterpret_cast<const uint32_t*>(img + lane_word_offset(D, lane, 3 * j + 2));
-        uint32_t s0, s1;
-        if ((warp & 1) == 0) {
-            s0 = A & 0x77777777u;
-            s1 = Bw & 0x77777777u;
-        } else {
-            s0 = ((A >> 1) & 0x44444444u) | (Cw & 0x33333333u);
-            s1 = ((Bw >> 1) & 0x44444444u) | ((Cw >> 2) & 0x33333333u);
-        }
-        uint4 v;
-        v.x = __byte_perm(T0, T1, s0);            // token g, dims 4 tq ..
-        v.z = __byte_perm(T0, T1, s0 >> 16);      // token g, dims 16 + 4 tq ..
-        v.y = __byte_perm(T0, T1, s1);            // token g + 8
-        v.w = __byte_perm(T0, T1, s1 >> 16);
-        afrag[warp * 32 + lane] = v;
-    }
-    __syncthreads();
-    uint32_t a[NS][4];
-#pragma unroll
-    for (int s_ = 0; s_ < NS; ++s_) {
-        const uint4 v = afrag[s_ * 32 + lane];
-        a[s_][0] = v.x; a[s_][1] = v.y; a[s_][2] = v.z; a[s_][3] = v.w;
-    }
-    // ---- per token scale g r / 8
-    const __half* gh = reinterpret_cast<const __half*>(img + 12 * D);
-    const float gr0 = __fmul_rn(__fmul_rn(__half2float(gh[g]), rs), 0.125f);
-    const float gr1 = __fmul_rn(__fmul_rn(__half2float(gh[g + 8]), rs), 0.125f);
-    float out[NTILE][4];
-#pragma unroll
-    for (int t = 0; t < NTILE; ++t) {
-        constexpr int JH = NWARP / 4;                     // j >> 2 = JH * t + (warp >> 2)
-        int c[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int s_ = 0; s_ < NS; ++s_) {
-            const bool neg = (__popc((unsigned)(s_ & (JH * t) & (NWARP == 8 ? 6 : 7))) & 1) != 0;     // compile-time part of bits 5-7
-            if (s_ & 1) imma16832(c, a[s_][0], a[s_][1], a[s_][2], a[s_][3], neg ? L.o0n : L.o0p, neg ? L.o1n : L.o1p);
-            else imma16832(c, a[s_][0], a[s_][1], a[s_][2], a[s_][3], neg ? L.b0n : L.b0p, neg ? L.b1n : L.b1p);
-        }
-        // columns n = 8 j + 2 tq, + 1 of tokens g (c0, c1) and g + 8 (c2, c3); j = NWARP t + warp
-        out[t][0] = __uint_as_float(__float_as_uint(__fmul_rn(gr0, (float)c[0])) ^ L.flip[t][0]);
-        out[t][1] = __uint_as_float(__float_as_uint(__fmul_rn(gr0, (float)c[1])) ^ L.flip[t][1]);
-        out[t][2] = __uint_as_float(__float_as_uint(__fmul_rn(gr1, (float)c[2])) ^ L.flip[t][0]);
-        out[t][3] = __uint_as_float(__float_as_uint(__fmul_rn(gr1, (float)c[3])) ^ L.flip[t][1]);
-    }
-    if (!unit_k) {                        // a product with 1 is skipped (a branch, not predicated multiplications)
-#pragma unroll
-        for (int t = 0; t < NTILE; ++t)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) out[t][e] = __fmul_rn(out[t][e], inv_k_scale);
-    }
-#pragma unroll
-    for (int t = 0; t < NTILE; ++t) {
-        const int n0 = 8 * (NWARP * t + warp) + 2 * tq;
-        *reinterpret_cast<uint16_t*>(ktile + g * D + n0) =
-            (uint16_t)__nv_cvt_float2_to_fp8x2(make_float2(out[t][0], out[t][1]), __NV_SATFINITE, __NV_E4M3);
-        *reinterpret_cast<uint16_t*>(ktile + (g + 8) * D + n0) =
-            (uint16_t)__nv_cvt_float2_to_fp8x2(make_float2(out[t][2], out[t][3]), __NV_SATFINITE, __NV_E4M3);
-    }
-}
-
-template <int D, bool BIG, int FMT>
-__global__ void __launch_bounds__(D) promote_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8,
-                                                     int tq3_pages, int fp8_pages, int hkv, int tiles, float inv_k_scale,
-                                                     float inv_v_scale, float rs, SigmaBits sigma,
-                                                     const int32_t* __restrict__ src_ids,
-                                                     const int32_t* __restrict__ dst_ids, int32_t* block_table,
-                                                     uint8_t* tier_tag, const int64_t* entry_index, int64_t n_entries,
-                                                     uint32_t* __restrict__ status, uint32_t* page_tickets)
-{
-    constexpr int EPL = D / 32;
-    constexpr int NT = D;
-    constexpr int REC = 16 * D + 32;
-    __shared__ __align__(16) uint8_t image[2][REC];
-    __shared__ __align__(16) uint8_t ktile[FMT == 2 ? kPage * D : 16];   // format 2: the rebuilt key rows of one record
-    __shared__ uint4 afrag[FMT == 2 ? D : 1];                            // format 2: [32-dim step][lane] A operands of the key product
-    __shared__ float level[8];            // signed key levels by 3-bit code
-
-    const int csize = (int)cluster_size(), crank = (int)cluster_rank();
-    const int page = blockIdx.x / csize, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    pdl_begin();
-    const int src = src_ids[page], dst = dst_ids[page];
-    const bool valid = src >= 0 && src < tq3_pages && dst >= 0 && dst < fp8_pages;
-    if (!valid && tid == 0 && crank == 0 && blockIdx.y == 0) atomicOr(status, kStBounds);
-    if (tid < 8) {
-        using CB = KeyCodebook<FMT>;
-        const float c = (tid & 3) == 0 ? CB::C0 : (tid & 3) == 1 ? CB::C1 : (tid & 3) == 2 ? CB::C2 : CB::C3;
-        level[tid] = (tid & 4) ? -c : c;
-    }
-    // ---- per-lane constants of the key path: this lane rebuilds channels lane*EPL .. +EPL-1
-    const int kb = (lane * EPL) >> 4, s0 = (lane * EPL) & 15;       // 16-channel block, first slot in it
-    const int kj = kb >> 2, kind = kb & 3;
-    const int w_sgn = 3 * kj + (kind & 1);                          // word A or B: codes of kinds 0/1, signs of 2/3
-    const int w_mag = kind < 2 ? w_sgn : 3 * kj + 2;                // word C holds the magnitudes of kinds 2/3
-    const int off_sgn = lane_word_offset(D, 0, w_sgn), off_mag = lane_word_offset(D, 0, w_mag);
-    const int str_sgn = lane_word_offset(D, 1, w_sgn) - off_sgn, str_mag = lane_word_offset(D, 1, w_mag) - off_mag;
-    const int mag_extra = kind == 3 ? 2 : 0;                        // high pair of the C nibble
-    const uint32_t mag_mask = kind < 2 ? 7u : 3u;                   // kinds 0/1 read sign and magnitude at once
-    const uint32_t sgn_mask = kind < 2 ? 0u : 4u;
-    uint32_t flip[EPL];
-#pragma unroll
-    for (int r = 0; r < EPL; ++r) {
-        const int i = lane * EPL + r;
-        flip[r] = ((sigma.w[i >> 5] >> (i & 31)) & 1u) << 31;
-    }
-    float sgn[5];                           // butterfly stage b: lanes with bit b set subtract
-#pragma unroll
-    for (int b = 0; b < 5; ++b) sgn[b] = ((lane >> b) & 1) ? -1.0f : 1.0f;
-    const bool unit_k = inv_k_scale == 1.0f, unit_v = inv_v_scale == 1.0f;   // a product with 1 is skipped
-    PromoteKeyLane<D> key_lane;
-    if constexpr (FMT == 2) key_lane.init(sigma, warp, lane);
-    // ---- per-thread constants of the value path: this thread rebuilds channel tid
-    const int cb = tid >> 4, row = tid & 15;
-    const int vj = cb >> 2, grp = (cb & 3) >> 1, k0 = 4 * (cb & 1) + (row >> 3);
-    const int off_v = 6 * D + lane_word_offset(D, 4 * (row & 7), 3 * vj + grp);
-    const int off_v1 = 6 * D + lane_word_offset(D, 4 * (row & 7), 3 * vj + grp + 1);
-    const int str_v = lane_word_offset(D, 1, 3 * vj + grp) - lane_word_offset(D, 0, 3 * vj + grp);
-    const int str_v1 = lane_word_offset(D, 1, 3 * vj + grp + 1) - lane_word_offset(D, 0, 3 * vj + grp + 1);
-    const uint32_t sel0 = grp == 0 ? 0x0410u : 0x0541u, sel1 = grp == 0 ? 0x0632u : 0x0763u;
-    const int meta_i = (cb >> 1) * 64 + (row & 7) * 8 + 4 * (cb & 1) + (row >> 3);
-
-    // 16-token pages: one record per head.  Pages of several tiles: the blocks of grid row y take tiles y,
-    // y + gridDim.y, ...; a tile and the page's scale/zero behind it form the same image as a 16-token record.
-    constexpr int TILE = 12 * D + 32;
-    const int m_first = BIG ? (int)blockIdx.y : 0, m_step = BIG ? (int)gridDim.y : 1, m_end = BIG ? tiles : 1;
-    // The record of the next (head, tile) is copied into the other image asynchronously while this one is rebuilt.
-    auto fetch = [&](int h, int m, uint8_t* img) {
-        const uint8_t* page3 = tq3 + ((size_t)src * hkv + h) * tq3_page_bytes(D, tiles);
-        const uint8_t* rec3 = page3 + (size_t)m * TILE;
-        if constexpr (!BIG) {
-            for (int i = tid; i < REC / 16; i += NT) cp_async16(img + 16 * i, rec3 + 16 * i);
-        } else {
-            const uint8_t* meta = page3 + (size_t)tiles * TILE;
-            for (int i = tid; i < TILE / 16; i += NT) cp_async16(img + 16 * i, rec3 + 16 * i);
-            for (int i = tid; i < 4 * D / 16; i += NT) cp_async16(img + TILE + 16 * i, meta + 16 * i);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    int h = crank, m = m_first;
-    bool more = valid && h < hkv && m < m_end;
-    if (more) fetch(h, m, image[0]);
-    for (int it = 0; more; ++it) {
-        int hn = h, mn = m + m_step;
-        if (mn >= m_end) {
-            mn = m_first;
-            hn = h + csize;
-        }
-        const bool more_next = hn < hkv;
-        uint8_t* rec8 = fp8 + (((size_t)dst * hkv + h) * tiles + m) * fp8_record_bytes(D);
-        uint8_t* img = image[it & 1];
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();            // this image has landed for every thread; the other image and ktile are no longer read
-        if (more_next) fetch(hn, mn, image[(it + 1) & 1]);
-
-        // ---- keys.  Format 2: the inverse rotation as an integer matrix product (all warps, every token at once)
-        if constexpr (FMT == 2) promote_keys_v2<D>(img, ktile, afrag, key_lane, rs, inv_k_scale, unit_k);
-        // Format 1: warp w rebuilds tokens w, w + NT/32, ... with butterflies
-        for (int tok = warp; FMT != 2 && tok < kPage; tok += NT / 32) {
-            float y[EPL];
-            if constexpr (FMT == 2) {
-                // record format 2: four consecutive dims are the nibbles of one half-word of register
-                // e = 4 (step % 2) + 2 (token / 8) + (k / 16) in the triple step / 2 of fragment lane 4 (token % 8) + (k % 16) / 4
-#pragma unroll
-                for (int gi = 0; gi < EPL / 4; ++gi) {
-                    const int i0 = lane * EPL + 4 * gi, st = i0 >> 5, k = i0 & 31, j = st >> 1;
-                    const int e = 4 * (st & 1) + 2 * (tok >> 3) + (k >> 4), L = 4 * (tok & 7) + ((k & 15) >> 2), sh = 16 * (e & 1);
-                    const uint32_t A = *reinterpret_cast<const uint32_t*>(img + lane_word_offset(D, L, 3 * j));
-                    const uint32_t Bw = *reinterpret_cast<const uint32_t*>(img + lane_word_offset(D, L, 3 * j + 1));
-                    const uint32_t Cw = *reinterpret_cast<const uint32_t*>(img + lane_word_offset(D, L, 3 * j + 2));
-                    uint32_t nib;
-                    if (e < 2) nib = (A >> sh) & 0x7777u;
-                    else if (e < 4) nib = (Bw >> sh) & 0x7777u;
-                    else if (e < 6) nib = ((Cw >> sh) & 0x3333u) | ((A >> (sh + 1)) & 0x4444u);
-                    else nib = ((Cw >> (sh + 2)) & 0x3333u) | ((Bw >> (sh + 1)) & 0x4444u);
-                    // one byte-table lookup for the four codes: 8 x the signed level (2, 6, 11, 18 | negated).  The
-                    // transform below is exact on these integers, so the factor 1/8 moves into the token's scale
-                    const uint32_t lv = __byte_perm(0x120B0602u, 0xEEF5FAFEu, nib);
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) y[4 * gi + x] = (float)(int)(int8_t)(lv >> (8 * x));
-                }
-            }
-#pragma unroll
-            for (int r2 = 0; r2 < (FMT == 2 ? 0 : EPL); r2 += 2) {
-                const int s = s0 + r2;                                    // even slot; s + 1 shares the word
-                const int L = 4 * (tok & 7) + ((s & 7) >> 1), n = 2 * ((tok >> 3) + 2 * (s >> 3));
-                const uint32_t ws = *reinterpret_cast<const uint32_t*>(img + off_sgn + L * str_sgn) >> (4 * n);
-                const uint32_t wm = *reinterpret_cast<const uint32_t*>(img + off_mag + L * str_mag) >> (4 * n + mag_extra);
-                const uint32_t c_even = (wm & mag_mask) | ((ws >> 1) & sgn_mask);
-                const uint32_t c_odd = ((wm >> 4) & mag_mask) | ((ws >> 5) & sgn_mask);
-                y[r2] = level[c_even];
-                y[r2 + 1] = level[c_odd];
-            }
-#pragma unroll
-            for (int hh = 1; hh < EPL; hh <<= 1)
-#pragma unroll
-                for (int r = 0; r < EPL; ++r)
-                    if ((r & hh) == 0) {
-                        const float u = y[r], w = y[r + hh];
-                        y[r] = __fadd_rn(u, w);
-                        y[r + hh] = __fsub_rn(u, w);
-                    }
-#pragma unroll
-            for (int b = 0; b < 5; ++b)
-#pragma unroll
-                for (int r = 0; r < EPL; ++r) {
-                    // o + y or o - y: the product with +-1 is exact, one rounding as in the single addition
-                    const float o = __shfl_xor_sync(0xffffffffu, y[r], 1 << b);
-                    y[r] = __fmaf_rn(y[r], sgn[b], o);
-                }
-            const float g = __half2float(reinterpret_cast<const __half*>(img + 12 * D)[tok]);
-            // format 2: y holds 8 x the transform of the levels (all sums of the transform are exact integers below
-            // 2^13, so H(8 c) = 8 H(c) bit for bit) and gr y = (gr / 8)(8 y) is the same real product, rounded once
-            const float gr = FMT == 2 ? __fmul_rn(__fmul_rn(g, rs), 0.125f) : __fmul_rn(g, rs);
-            uint32_t out[EPL / 4];
-#pragma unroll
-            for (int r = 0; r < EPL / 4; ++r) out[r] = 0;
-#pragma unroll
-            for (int r = 0; r < EPL; r += 2) {
-                float2 kk;
-                kk.x = __uint_as_float(__float_as_uint(__fmul_rn(gr, y[r])) ^ flip[r]);
-                kk.y = __uint_as_float(__float_as_uint(__fmul_rn(gr, y[r + 1])) ^ flip[r + 1]);
-                if (!unit_k) {
-                    kk.x = __fmul_rn(kk.x, inv_k_scale);
-                    kk.y = __fmul_rn(kk.y, inv_k_scale);
-                }
-                out[r >> 2] |= (uint32_t)__nv_cvt_float2_to_fp8x2(kk, __NV_SATFINITE, __NV_E4M3) << (8 * (r & 3));
-            }
-            if constexpr (EPL == 8)
-                *reinterpret_cast<uint2*>(rec8 + tok * D + lane * EPL) = make_uint2(out[0], out[1]);
-            else
-                *reinterpret_cast<uint32_t*>(rec8 + tok * D + lane * EPL) = out[0];
-        }
-        // ---- values: one thread per channel; fragment lane 4 (row % 8) + q holds tokens 2q, 2q+1, 2q+8, 2q+9
-        {
-            const __half* meta = reinterpret_cast<const __half*>(img + 12 * D + 32);
-            const float sc = __half2float(meta[meta_i]), zp = __half2float(meta[meta_i + 2]);
-            // The channel's eight possible output bytes, e4m3((sc * code + zp) / v_scale) for code 0..7, computed
-            // once; a byte-table lookup then turns the codes of four tokens into four output bytes.
-            float lv[8];
-#pragma unroll
-            for (int cde = 0; cde < 8; ++cde) lv[cde] = __fadd_rn(__fmul_rn(sc, (float)cde), zp);
-            if (!unit_v) {
-#pragma unroll
-                for (int cde = 0; cde < 8; ++cde) lv[cde] = __fmul_rn(lv[cde], inv_v_scale);
-            }
-            uint32_t pr[4];
-#pragma unroll
-            for (int cde = 0; cde < 8; cde += 2)
-                pr[cde >> 1] = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(lv[cde], lv[cde + 1]), __NV_SATFINITE, __NV_E4M3);
-            const uint32_t lut_lo = pr[0] | (pr[1] << 16), lut_hi = pr[2] | (pr[3] << 16);
-            uint32_t near[4], far[4];           // per q: codes of tokens (2q, 2q+1) and (2q+8, 2q+9) as two nibbles
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t lo = *reinterpret_cast<const uint32_t*>(img + off_v + q * str_v);
-                const uint32_t hi = *reinterpret_cast<const uint32_t*>(img + off_v1 + q * str_v1);
-                const uint32_t st0 = __byte_perm(lo, hi, sel0) >> (3 * k0);          // stream of the even tokens
-                const uint32_t st1 = __byte_perm(lo, hi, sel1) >> (3 * k0);          // stream of the odd tokens
-                near[q] = (st0 & 7u) | ((st1 & 7u) << 4);
-                far[q] = ((st0 >> 6) & 7u) | (((st1 >> 6) & 7u) << 4);
-            }
-            uint32_t out[4];
-            out[0] = __byte_perm(lut_lo, lut_hi, near[0] | (near[1] << 8));           // tokens 0..3
-            out[1] = __byte_perm(lut_lo, lut_hi, near[2] | (near[3] << 8));           // tokens 4..7
-            out[2] = __byte_perm(lut_lo, lut_hi, far[0] | (far[1] << 8));             // tokens 8..11
-            out[3] = __byte_perm(lut_lo, lut_hi, far[2] | (far[3] << 8));             // tokens 12..15
-            *reinterpret_cast<uint4*>(rec8 + 16 * D + tid * kPage) = make_uint4(out[0], out[1], out[2], out[3]);
-        }
-        if constexpr (FMT == 2) {
-            __syncthreads();               // key rows complete; the next record's rows are written after the next barrier
-            reinterpret_cast<uint4*>(rec8)[tid] = reinterpret_cast<const uint4*>(ktile)[tid];      // 16 D bytes, D threads
-        }
-        h = hn;
-        m = mn;
-        more = more_next;
-    }
-    // copy-before-publish (as in demote_kernel: cluster barrier, then the publishing thread's cumulative fence)
-    cluster_barrier();
-    if (valid && crank == 0 && tid == 0 && entry_index != nullptr && (__threadfence(), last_cluster_of_page(page_tickets, page))) {
-        const int64_t e = entry_index[page];
-        if (e >= n_entries) atomicOr(status, kStBounds);
-        else if (e >= 0) {
-            block_table[e] = dst;
-            __threadfence();
-            tier_tag[e] = (uint8_t)MKV_TAG_ANCHOR;
-        }
-    }
+    const int warps = p->hkv < kDemoteWarps ? p->hkv : kDemoteWarps, c = warp_cluster(p->hkv, BIG ? 0 : n);
+    const int smem = PromoteWarp<D>::OFF_WARPS + warps * PromoteWarp<D>::BYTES;
+    static_assert(PromoteWarp<D>::OFF_WARPS + kDemoteWarps * PromoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
+    const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale, rs = (float)(1.0 / sqrt((double)p->d));
+    return launch_pdl(promote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv) : 1),
+                      32 * warps, (size_t)smem, c, n <= 148, s, (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages,
+                      p->hkv, p->tiles, ik, iv, rs, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }
 
 template <int D, int FMT>
 static int32_t launch_promote_d(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
                                 const int64_t* entry, int64_t n_entries, cudaStream_t s)
 {
-    const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale;
-    const float rs = (float)(1.0 / sqrt((double)p->d));
-    const int c = heads_cluster(p->hkv, p->tiles == 1 ? n : 0);
     if (p->tiles == 1) {
-        MKV_CUDA(launch_pdl(promote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, n <= 148, s, (const uint8_t*)p->tq3, p->fp8,
-                                  p->cfg.tq3_pages, p->cfg.fp8_pages, p->hkv, 1, ik, iv, rs, p->sigma, src, dst, bt, tags,
-                                  entry, n_entries, p->status_dev, (uint32_t*)nullptr));
+        MKV_CUDA((launch_promote_warp<D, FMT, false>(p, src, dst, n, bt, tags, entry, n_entries, nullptr, s)));
         return MKV_OK;
     }
     const bool fused = entry != nullptr && n <= kPageTickets;
-    MKV_CUDA(launch_pdl(promote_kernel<D, true, FMT>, dim3((unsigned)n * c, tile_rows(p->tiles, n, p->hkv)), D, 0, c, n <= 148, s,
-                                   (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages, p->hkv, p->tiles, ik,
-                                   iv, rs, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr, fused ? tags : (uint8_t*)nullptr,
-                                   fused ? entry : (const int64_t*)nullptr, fused ? n_entries : (int64_t)0, p->status_dev,
-                                   fused ? page_tickets(p) : (uint32_t*)nullptr));
+    MKV_CUDA((launch_promote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
+                                                fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
     if (entry && !fused) {
-        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, true, s, n, src, dst, p->cfg.tq3_pages, p->cfg.fp8_pages, bt, tags, entry,
-                                                       n_entries, MKV_TAG_ANCHOR, p->status_dev));
-        MKV_CUDA(cudaGetLastError());
+        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, true, s, n, src, dst, p->cfg.tq3_pages,
+                            p->cfg.fp8_pages, bt, tags, entry, n_entries, MKV_TAG_ANCHOR, p->status_dev));
     }
     return MKV_OK;
 }

@@ -328,13 +328,22 @@ __device__ __forceinline__ float half_times(uint16_t h)
 }
 
 // acc[channel rows g, g+8][heads] += scale_row * t + zero_row * psum_head, t in units of value_unit<BLOCK, row>
-template <int BLOCK>
+// MIXED: half_times instead of a conversion and a product.  (Not in the format-2 scan of more than four heads at
+// d = 256, where the compiler's schedule gets worse: 2 x 59,008 tokens in 16 layers 553 us with it, 540 us without.)
+template <int BLOCK, bool MIXED>
 __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (&t)[4], uint32_t sc_pair, uint32_t zp_pair,
                                                   float ps0, float ps1)
 {
     const float2 zp = half2_to_float2(zp_pair);
-    const float s0 = half_times<unit_bits(value_unit<BLOCK, 0>())>((uint16_t)sc_pair),      // exact
-                s1 = half_times<unit_bits(value_unit<BLOCK, 1>())>((uint16_t)(sc_pair >> 16));
+    float s0, s1;                            // exact either way
+    if constexpr (MIXED) {
+        s0 = half_times<unit_bits(value_unit<BLOCK, 0>())>((uint16_t)sc_pair);
+        s1 = half_times<unit_bits(value_unit<BLOCK, 1>())>((uint16_t)(sc_pair >> 16));
+    } else {
+        const float2 sc = half2_to_float2(sc_pair);
+        s0 = sc.x * value_unit<BLOCK, 0>();
+        s1 = sc.y * value_unit<BLOCK, 1>();
+    }
     acc[0] = fmaf(s0, t[0], fmaf(zp.x, ps0, acc[0]));
     acc[1] = fmaf(s0, t[1], fmaf(zp.x, ps1, acc[1]));
     acc[2] = fmaf(s1, t[2], fmaf(zp.y, ps0, acc[2]));
@@ -715,7 +724,7 @@ __device__ __forceinline__ void tq3_key_quad(float (&S0)[4], float (&S1)[4], uin
 // Output update of the four channel blocks 4j..4j+3 of a Stale page: integer codes through the tensor
 // core, then the fp16 scale and zero of every channel applied to the 16x8 result in fp32.
 // DEFER: sum p * code only, the accumulators are in units of value_unit until the page is left.
-template <bool DEFER, bool SPLIT>
+template <bool DEFER, bool SPLIT, bool MIXED>
 __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], float (&o2)[4], float (&o3)[4],
                                                uint32_t W0, uint32_t W1, uint32_t W2, uint32_t meta_quad, const PFrag& pf)
 {
@@ -732,20 +741,20 @@ __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], f
         const uint32_t X = prmt(W0, W1, 0x6341u);
         value_operands<0>(a, W0, W1, W2, X);
         product(DEFER ? o0 : t);
-        if constexpr (!DEFER) affine_accumulate<0>(o0, t, mt.x, mt.y, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) affine_accumulate<0, MIXED>(o0, t, mt.x, mt.y, pf.ps0, pf.ps1);
         value_operands<1>(a, W0, W1, W2, X);
         product(DEFER ? o1 : t);
-        if constexpr (!DEFER) affine_accumulate<1>(o1, t, mt.z, mt.w, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) affine_accumulate<1, MIXED>(o1, t, mt.z, mt.w, pf.ps0, pf.ps1);
     }
     {   // blocks 4j+2, 4j+3
         if constexpr (!DEFER) mt = lds128(meta_quad + 128);
         const uint32_t X = prmt(W1, W2, 0x6341u);
         value_operands<2>(a, W0, W1, W2, X);
         product(DEFER ? o2 : t);
-        if constexpr (!DEFER) affine_accumulate<2>(o2, t, mt.x, mt.y, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) affine_accumulate<2, MIXED>(o2, t, mt.x, mt.y, pf.ps0, pf.ps1);
         value_operands<3>(a, W0, W1, W2, X);
         product(DEFER ? o3 : t);
-        if constexpr (!DEFER) affine_accumulate<3>(o3, t, mt.z, mt.w, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) affine_accumulate<3, MIXED>(o3, t, mt.z, mt.w, pf.ps0, pf.ps1);
     }
 }
 
@@ -919,7 +928,7 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
             else tq3_key_quad<SPLIT>(S0, S1, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * (SPLIT ? 1024 : 2048));
         }
         if constexpr (DO_V)
-            tq3_value_quad<DEFER, SPLIT>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
+            tq3_value_quad<DEFER, SPLIT, !(D == 256 && FMT == 2 && !SPLIT)>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
                                   vw[3 * j + 2], meta + j * 256, pf);
     }
     if constexpr (DO_K && FMT == 2 && SPLIT) {

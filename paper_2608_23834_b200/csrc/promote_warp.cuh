@@ -115,21 +115,38 @@ promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, 
     const bool unit_k = inv_k_scale == 1.0f, unit_v = inv_v_scale == 1.0f;   // a product with 1 is skipped
 
     const int m_first = BIG ? (int)blockIdx.y : 0, m_step = BIG ? (int)gridDim.y : 1, m_end = BIG ? tiles : 1;
-    for (int h = crank * n_warps + warp; valid && h < hkv; h += csize * n_warps)
-    for (int m = m_first; m < m_end; m += m_step) {
-        const uint8_t* page3 = tq3 + ((size_t)src * hkv + h) * tq3_page_bytes(D, tiles);
-        const uint8_t* rec3 = page3 + (size_t)m * TILE;
-        const uint8_t* meta = page3 + (size_t)tiles * TILE;          // (16-token pages: right behind the one tile)
-        uint8_t* rec8 = fp8 + (((size_t)dst * hkv + h) * tiles + m) * fp8_record_bytes(D);
-        // ---- everything the lane needs of the record, in flight at once
-        uint32_t kw[LW], vw[LW];
-        uint4 mt[D / 128];
+    const int h_first = crank * n_warps + warp, h_step = csize * n_warps;
+    auto page_of = [&](int h) { return tq3 + ((size_t)src * hkv + h) * tq3_page_bytes(D, tiles); };
+    // What a lane needs of a record.  At d = 128 each part of the next record is asked for as soon as this record's is used
+    // up: the loads then fly under the work on this one, in the registers that have just become free (d = 256 has none).
+    constexpr bool AHEAD = D == 128;
+    uint32_t kw[LW], vw[LW];
+    uint4 mt[D / 128];
+    uint16_t g0 = 0, g1 = 0;
+    auto fetch_keys = [&](const uint8_t* rec3) {
         fetch_lane_words<D>(rec3, lane, kw);
-        const uint16_t g0 = __ldg(reinterpret_cast<const uint16_t*>(rec3 + 12 * D) + g),
-                       g1 = __ldg(reinterpret_cast<const uint16_t*>(rec3 + 12 * D) + g + 8);
+        g0 = __ldg(reinterpret_cast<const uint16_t*>(rec3 + 12 * D) + g);
+        g1 = __ldg(reinterpret_cast<const uint16_t*>(rec3 + 12 * D) + g + 8);
+    };
+    auto fetch_meta = [&](const uint8_t* page3) {    // (16-token pages: right behind the one tile)
 #pragma unroll
-        for (int i = 0; i < D / 128; ++i) mt[i] = __ldg(reinterpret_cast<const uint4*>(meta) + lane + 32 * i);
-        fetch_lane_words<D>(rec3 + 6 * D, lane, vw);
+        for (int i = 0; i < D / 128; ++i) mt[i] = __ldg(reinterpret_cast<const uint4*>(page3 + (size_t)tiles * TILE) + lane + 32 * i);
+    };
+    auto fetch_record = [&](int h, int m) {
+        const uint8_t* page3 = page_of(h);
+        fetch_keys(page3 + (size_t)m * TILE);
+        fetch_meta(page3);
+        fetch_lane_words<D>(page3 + (size_t)m * TILE + 6 * D, lane, vw);
+    };
+    if (AHEAD && valid && h_first < hkv && m_first < m_end) fetch_record(h_first, m_first);
+    for (int h = h_first; valid && h < hkv; h += h_step)
+    for (int m = m_first; m < m_end; m += m_step) {
+        uint8_t* rec8 = fp8 + (((size_t)dst * hkv + h) * tiles + m) * fp8_record_bytes(D);
+        const int next_m = m + m_step < m_end ? m + m_step : m_first, next_h = m + m_step < m_end ? h : h + h_step;
+        const bool more = AHEAD && next_h < hkv;
+        if constexpr (!AHEAD) fetch_record(h, m);
+        const uint8_t* next_page = page_of(more ? next_h : h);
+        const uint8_t* next = next_page + (size_t)next_m * TILE;
 
         // ---- keys
         {
@@ -159,6 +176,7 @@ promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, 
                 }
             }
             const float gr0 = __fmul_rn(__half2float(__ushort_as_half(g0)), rs), gr1 = __fmul_rn(__half2float(__ushort_as_half(g1)), rs);
+            if (more) fetch_keys(next);
             __syncwarp();                            // the tile of the round before has been read
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
@@ -186,13 +204,20 @@ promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, 
 #pragma unroll
                 for (int b = 0; b < NBLK; ++b)
 #pragma unroll
+                    for (int u = 0; u < 2; ++u) v[b][u] = mul2(gs[u], v[b][u]);
+                if (!unit_k) {                       // (a branch, not predicated products)
+                    const f32x2 ik = pack2(inv_k_scale, inv_k_scale);
+#pragma unroll
+                    for (int b = 0; b < NBLK; ++b)
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) v[b][u] = mul2(v[b][u], ik);
+                }
+#pragma unroll
+                for (int b = 0; b < NBLK; ++b)
+#pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         float lo, hi;
-                        unpack2(mul2(gs[u], v[b][u]), lo, hi);
-                        if (!unit_k) {
-                            lo = __fmul_rn(lo, inv_k_scale);
-                            hi = __fmul_rn(hi, inv_k_scale);
-                        }
+                        unpack2(v[b][u], lo, hi);
                         *reinterpret_cast<uint16_t*>(tile + (g + 8 * u) * KST + 16 * b + 4 * tq + 2 * t) = (uint16_t)e4m3_pair(lo, hi);
                     }
             }
@@ -217,22 +242,34 @@ promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, 
         for (int i = 0; i < D / 128; ++i) {
             const int c = lane + 32 * i, ch0 = (c >> 3) * 32 + (c & 7);
             const float2 sc[2] = {f16x2_to_f32(mt[i].x), f16x2_to_f32(mt[i].z)}, zp[2] = {f16x2_to_f32(mt[i].y), f16x2_to_f32(mt[i].w)};
+            f32x2 lv[4][4];                          // [block e / 2, row half e % 2][codes 2 k, 2 k + 1]
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {            // block e / 2, row half e % 2
+            for (int e = 0; e < 4; ++e) {
                 const float s = e & 1 ? sc[e >> 1].y : sc[e >> 1].x, z = e & 1 ? zp[e >> 1].y : zp[e >> 1].x;
+                const f32x2 s2 = pack2(s, s), z2 = pack2(z, z);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) lv[e][k] = add2(mul2(s2, pack2((float)(2 * k), (float)(2 * k + 1))), z2);
+            }
+            if (!unit_v) {
+                const f32x2 iv = pack2(inv_v_scale, inv_v_scale);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) lv[e][k] = mul2(lv[e][k], iv);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
                 uint32_t pr[4];
 #pragma unroll
-                for (int cde = 0; cde < 8; cde += 2) {
-                    float lo = __fadd_rn(__fmul_rn(s, (float)cde), z), hi = __fadd_rn(__fmul_rn(s, (float)(cde + 1)), z);
-                    if (!unit_v) {
-                        lo = __fmul_rn(lo, inv_v_scale);
-                        hi = __fmul_rn(hi, inv_v_scale);
-                    }
-                    pr[cde >> 1] = e4m3_pair(lo, hi);
+                for (int k = 0; k < 4; ++k) {
+                    float lo, hi;
+                    unpack2(lv[e][k], lo, hi);
+                    pr[k] = e4m3_pair(lo, hi);
                 }
                 lut[ch0 + 16 * (e >> 1) + 8 * (e & 1)] = make_uint2(pr[0] | (pr[1] << 16), pr[2] | (pr[3] << 16));
             }
         }
+        if (more && (!BIG || next_h != h)) fetch_meta(next_page);
         __syncwarp();                                // tables complete, key rows read: the tile takes the value rows
         uint32_t* vrow = reinterpret_cast<uint32_t*>(tile);          // [channel][tq]: tokens 2tq, 2tq+1, 2tq+8, 2tq+9
         auto put = [&](int ch, uint32_t sel) {
@@ -253,6 +290,7 @@ promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, 
             put(ch + 48, code_selector<4, 10>(W2, W2));
             put(ch + 56, code_selector<7, 13>(W2, W2));
         }
+        if (more) fetch_lane_words<D>(next + 6 * D, lane, vw);
         __syncwarp();
 #pragma unroll
         for (int i = lane; i < D; i += 32) {

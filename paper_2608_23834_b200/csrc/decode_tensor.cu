@@ -371,25 +371,26 @@ struct Partition {
 };
 
 // Called by warp 0 (all 32 lanes) after cum[] is complete; other warps wait at the next barrier.
-// Blocks that share W triples: all of the grid, but no more than give every warp kMinPagesPerWarp pages.
-constexpr int kMinPagesPerWarp = 1;
-__device__ __forceinline__ int useful_blocks(long long W, int grid, int n_warps)
+// Blocks that share W triples: all of the grid, but no more than give every block min_pages of them (a page per warp
+// of an SM: below that a row's partials cost more to merge than the spreading saves).
+__device__ __forceinline__ int useful_blocks(long long W, int grid, int min_pages)
 {
-    const long long most = (W + kMinPagesPerWarp * n_warps - 1) / (kMinPagesPerWarp * n_warps);
+    const long long most = (W + min_pages - 1) / min_pages;
     return (int)(most < (long long)grid ? most : (long long)grid);
 }
 
-__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int n_warps, int lane)
+__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int min_pages, int per_sm, int lane)
 {
     constexpr uint32_t FULL = 0xffffffffu;
     const long long W = cum[B];
     const int rows = B * hkv;
-    int blocks = useful_blocks(W, grid, n_warps);
+    int blocks = useful_blocks(W, grid, min_pages);
     grid = blocks;
     // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
     // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
     // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).
-    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && W >= grid) ? 1 : 0;
+    // With two blocks per SM that cost overlaps the other block's pages: from eight.
+    int aligned = (rows * 4 * per_sm <= grid && rows <= kMaxAlignedRows && W >= grid) ? 1 : 0;
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_page(r) / W);
         // every row must end up with at least one block, otherwise the linear cut is used
@@ -1062,7 +1063,7 @@ __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, u
 // four heads) of the [channel][8 heads] tile.  With twice as many threads as groups (16 warps at d = 128) every
 // other part goes to the second half of the threads.  KP loads per thread are in flight, issued before the weights
 // are worked out: 32 to 40 parts per block, bounded by the registers of the launch shape.
-template <int D, int NT, int KPMAX = NT <= 256 ? 40 : NT <= 384 ? 24 : 16>
+template <int D, int NT, int KPMAX>
 __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot, int even_base, int n_parts,
                                           float* buf, int b, int h)
 {
@@ -1169,6 +1170,8 @@ template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL
 __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const LayerSet<MAXL> LS)
 {
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
+    // 16-byte loads that a thread of the merge keeps in flight, within the registers of the launch shape
+    constexpr int MERGE_LOADS = NW * MINB <= 8 ? 40 : NW * MINB <= 12 ? 24 : 16;
     using G = Geo<D, NW, NSTAGE, TILED>;     // pages of several tiles: short rounds leave room for the parked rows
     constexpr int NB = G::NB, NBH = NB, NU = NW;
     constexpr uint32_t FULL = 0xffffffffu;
@@ -1227,10 +1230,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         if constexpr (FLAT) {
             if (lane == 0) {
                 pt->total = (long long)run * n_layers;
-                pt->flat_blocks = useful_blocks(pt->total, gridDim.x, NW);
+                pt->flat_blocks = useful_blocks(pt->total, gridDim.x, NW * MINB);
             }
         }
-        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, NW, lane);
+        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, NW * MINB, MINB, lane);
     } else {
         // Pages of a row are visited in a strided order, page(i) = i * stride mod n_pages, the stride
         // coprime to n_pages and near 0.618 n_pages: every contiguous range of positions then holds the
@@ -1835,12 +1838,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 if constexpr (MAXL > 1 && !FLAT) {
                     if (todo & 2) {
                         const DecodeParams& Q = LS.layer[layer - 1];
-                        merge_row<D, NW * 32>(Q, first_slot, 2 * c0, n_parts, red, b, h);
+                        merge_row<D, NW * 32, MERGE_LOADS>(Q, first_slot, 2 * c0, n_parts, red, b, h);
                         if (tid == 0) Q.tickets[c0] = 0;
                     }
                 }
                 if (todo & 1) {
-                    merge_row<D, NW * 32>(P, first_slot, 2 * c0, n_parts, red, b, h);
+                    merge_row<D, NW * 32, MERGE_LOADS>(P, first_slot, 2 * c0, n_parts, red, b, h);
                     if (tid == 0) P.tickets[c0] = 0;
                 }
             }
@@ -2082,11 +2085,24 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
     if (p0->tiles > 1)
         return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, true, kMaxLayers>(p0, ls, s)
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
+    // Two blocks of half the warps per SM: one's set-up, reduction and merge overlap the other's pages (16 layers x 2 x
+    // 59,008 tokens, d 256: 540 -> 510 us; x 4 x 700..3,001: 86 -> 77 us).  Not at d = 128 with more than four query heads
+    // per KV head, whose scan spills in this shape (16 layers x 4 x 16,000 tokens, 1 head: 56 -> 60 us).
     if (n_layers >= kMinFlatLayers)
-        return p0->d == 128 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
-                            : run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s);
+        return p0->d == 128 ? (p0->group > 4 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
+                                             : run_tensor<128, 8, 4, 2, false, false, kMaxLayers, true>(p0, ls, s))
+                            : run_tensor<256, 4, 4, 2, false, false, kMaxLayers, true>(p0, ls, s);
     return p0->d == 128 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers>(p0, ls, s)
                         : run_tensor<256, 8, 4, 1, false, false, kMaxLayers>(p0, ls, s);
+}
+
+// Two blocks of half the warps per SM instead of one: the set-up, reduction and merge of one overlap the pages of the
+// other, which pays the more rows a block meets (d 128, 8 x 4 heads: 64 ragged requests 632 -> 579 us, 8 x 4,096 tokens
+// 30.7 -> 23.6 us).  At d = 256 a merge by four warps costs more, and few rows have many partials: from 32 rows (8 x
+// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows: 71 -> 76 us).  Partial areas for one block per SM only take one.
+static bool two_blocks(const mkv_pool* p, int B, int max_blocks)
+{
+    return max_blocks >= 2 * p->dev.sm_count && (p->d == 128 || B * p->hkv >= 32);
 }
 
 int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, const uint8_t* tags,
@@ -2114,7 +2130,10 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
             MKV_CUDA(launch_pdl(page_mass_clear_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, 1, true, s, mass, n));
             rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true, true>(p, prm, s);
         } else {
-            rc = p->d == 128 ? run_tensor1<128, 16, 4, 1, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);
+            if (two_blocks(p, B, max_blocks))
+                rc = p->d == 128 ? run_tensor1<128, 8, 4, 2, true>(p, prm, s) : run_tensor1<256, 4, 4, 2, true>(p, prm, s);
+            else
+                rc = p->d == 128 ? run_tensor1<128, 16, 4, 1, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);
         }
         if (rc != MKV_OK) return rc;
         return launch_page_mass_finish(mass, lse, lens, B, p->hkv * p->group, max_pages, p->cfg.page_size, s);
@@ -2122,8 +2141,9 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
     if (p->tiles > 1)                    // pages of several tiles: the default launch shapes only
         return p->d == 128 ? run_tensor1<128, 12, 4, 1, false, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, false, true>(p, prm, s);
     if (p->variant == MKV_DECODE_TMEM && p->d == 256) return run_tmem<256>(p, prm, s);
-    // launch shapes (warps per block, ring slots per warp, blocks per SM): 16 warps at 128 registers for d = 128 (64
-    // ragged requests: 658 us against 678 us with 12 warps at 168 registers), 8 warps at up to 255 for d = 256
+    // launch shapes: warps per block, ring slots per warp, blocks per SM
+    if (two_blocks(p, B, max_blocks))
+        return p->d == 128 ? run_tensor1<128, 8, 4, 2>(p, prm, s) : run_tensor1<256, 4, 4, 2>(p, prm, s);
     return p->d == 128 ? run_tensor1<128, 16, 4, 1>(p, prm, s) : run_tensor1<256, 8, 4, 1>(p, prm, s);
 }
 

@@ -379,7 +379,7 @@ __device__ __forceinline__ int useful_blocks(long long W, int grid, int min_page
     return (int)(most < (long long)grid ? most : (long long)grid);
 }
 
-__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int min_pages, int per_sm, int lane)
+__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int min_pages, int straddle, int lane)
 {
     constexpr uint32_t FULL = 0xffffffffu;
     const long long W = cum[B];
@@ -389,8 +389,11 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, i
     // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
     // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
     // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).
-    // With two blocks per SM that cost overlaps the other block's pages: from eight.
-    int aligned = (rows * 4 * per_sm <= grid && rows <= kMaxAlignedRows && W >= grid) ? 1 : 0;
+    // The rounding to whole blocks costs about half a block's share in k of a block's pages; from `straddle` pages on that
+    // is dearer than the straddling (d 128, 8 heads, two blocks per SM: 8 x 4,096 tokens 28.9 us linear, 23.6 aligned;
+    // 8 x 32,768 of which half FP8 104.7 linear, 108 aligned).
+    const int aligned_loss = (int)(W * rows / (2ll * grid * grid));
+    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && W >= grid && aligned_loss < straddle) ? 1 : 0;
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_page(r) / W);
         // every row must end up with at least one block, otherwise the linear cut is used
@@ -1233,7 +1236,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 pt->flat_blocks = useful_blocks(pt->total, gridDim.x, NW * MINB);
             }
         }
-        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, NW * MINB, MINB, lane);
+        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, NW * MINB, 4 * NW, lane);
     } else {
         // Pages of a row are visited in a strided order, page(i) = i * stride mod n_pages, the stride
         // coprime to n_pages and near 0.618 n_pages: every contiguous range of positions then holds the
@@ -2059,6 +2062,17 @@ static DecodeParams make_params(mkv_pool* p, const void* q, const int32_t* bt, c
     return prm;
 }
 
+// Two blocks of half the warps per SM instead of one: the set-up, reduction and merge of one overlap the pages of the
+// other, which pays the more rows a block meets (d 128, 8 x 4 heads: 64 ragged requests 632 -> 579 us, 8 x 4,096 tokens
+// 30.7 -> 23.6 us).  At d = 256 a merge by four warps costs more, and few rows have many partials: from 32 rows (8 x
+// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows: 71 -> 76 us).  Partial areas for one block per SM only take one.
+static bool two_blocks(const mkv_pool* p, int B, int max_blocks)
+{
+    return max_blocks >= 2 * p->dev.sm_count && (p->d == 128 || B * p->hkv >= 32);
+}
+
+constexpr int kRowsOfTwoBlocks = 96;     // several layers laid end to end, d = 256
+
 // Decode attention of several layers in one launch: layer i reads pool[i], q[i], bt[i], tags[i] and writes
 // out[i], lse[i] (or none), with its own workspace ws[i]; the requests (lens, B, max_pages, scale) are common.
 int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q, const int32_t* const* bt,
@@ -2087,22 +2101,19 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
     // Two blocks of half the warps per SM: one's set-up, reduction and merge overlap the other's pages (16 layers x 2 x
     // 59,008 tokens, d 256: 540 -> 510 us; x 4 x 700..3,001: 86 -> 77 us).  Not at d = 128 with more than four query heads
-    // per KV head, whose scan spills in this shape (16 layers x 4 x 16,000 tokens, 1 head: 56 -> 60 us).
+    // per KV head, whose scan spills in this shape (16 layers x 4 x 16,000 tokens, 1 head: 56 -> 60 us), and not at d = 256 with
+    // few rows, whose partials four warps take longer to merge (16 layers x 1 x 4,000 tokens: 48.6 -> 51 us).
     if (n_layers >= kMinFlatLayers)
         return p0->d == 128 ? (p0->group > 4 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
                                              : run_tensor<128, 8, 4, 2, false, false, kMaxLayers, true>(p0, ls, s))
-                            : run_tensor<256, 4, 4, 2, false, false, kMaxLayers, true>(p0, ls, s);
+                            : (n_layers * B * p0->hkv < kRowsOfTwoBlocks
+                                   ? run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
+                                   : run_tensor<256, 4, 4, 2, false, false, kMaxLayers, true>(p0, ls, s));
+    if (two_blocks(p0, B, kMaxCtas))     // as a call of one layer (the results are the same bits)
+        return p0->d == 128 ? run_tensor<128, 8, 4, 2, false, false, kMaxLayers>(p0, ls, s)
+                            : run_tensor<256, 4, 4, 2, false, false, kMaxLayers>(p0, ls, s);
     return p0->d == 128 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers>(p0, ls, s)
                         : run_tensor<256, 8, 4, 1, false, false, kMaxLayers>(p0, ls, s);
-}
-
-// Two blocks of half the warps per SM instead of one: the set-up, reduction and merge of one overlap the pages of the
-// other, which pays the more rows a block meets (d 128, 8 x 4 heads: 64 ragged requests 632 -> 579 us, 8 x 4,096 tokens
-// 30.7 -> 23.6 us).  At d = 256 a merge by four warps costs more, and few rows have many partials: from 32 rows (8 x
-// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows: 71 -> 76 us).  Partial areas for one block per SM only take one.
-static bool two_blocks(const mkv_pool* p, int B, int max_blocks)
-{
-    return max_blocks >= 2 * p->dev.sm_count && (p->d == 128 || B * p->hkv >= 32);
 }
 
 int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, const uint8_t* tags,

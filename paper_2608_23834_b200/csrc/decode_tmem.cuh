@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
         }
         if (lane == 0) cum[P.B] = run;
         __syncwarp();
-        build_partition(pt, cum, P.B, hkv, gridDim.x, 1, 1, lane);
+        build_partition(pt, cum, P.B, hkv, gridDim.x, 1, 1 << 30, lane);
     } else {
         for (int b = tid - 32; b < P.B; b += NT - 32) {
             const int len = min(max(P.lens[b], 0), P.max_pages * kPage), n = (len + kPage - 1) / kPage;

@@ -510,13 +510,16 @@ struct Geo {
     static constexpr int SLOT = (TQ3_REC + 127) / 128 * 128;
     // pages of one warp whose table entries are compacted at a time (fewer where the ring leaves little room)
     static constexpr int ROUND = (NW * NSTAGE * SLOT > 190000 || SHORT_ROUNDS) ? 64 : 128;
+    // The ring is used in pairs of slots with one barrier each: a pair holds two Stale records, or the keys and values of one
+    // FP8 page, asked for together and waited for once.
+    static constexpr int NP = NSTAGE / 2, PAIR = 2 * SLOT;
     static constexpr int RING = NW * NSTAGE * SLOT;
     static constexpr int QROT = NB * 32 * 16;               // rotated query B fragments, hi and lo interleaved
     static constexpr int QPLAIN = NB * 32 * 8;              // plain query B fragments (FP8 pages)
     static constexpr int OFF_QT = RING;
     static constexpr int OFF_QF = OFF_QT + QROT;
     static constexpr int OFF_BAR = OFF_QF + QPLAIN;
-    static constexpr int OFF_LIST = OFF_BAR + NW * NSTAGE * 8;   // [warp][2 formats][ROUND] page ids, then [warp][2][ROUND] logical pages
+    static constexpr int OFF_LIST = (OFF_BAR + NW * NP * 8 + 15) / 16 * 16;   // [warp][2 formats][ROUND] page ids, then [warp][2][ROUND] logical pages
     static constexpr int OFF_CUM = OFF_LIST + NW * 4 * ROUND * 4;
     static constexpr int OFF_STRIDE = OFF_CUM + (kMaxBatch + 1) * 4;
     static constexpr int OFF_M = OFF_STRIDE + kMaxBatch * 4;
@@ -529,7 +532,7 @@ struct Geo {
                   "slots are bulk-copy destinations; query fragments are read with 16- and 8-byte loads");
     static_assert(OFF_PART % alignof(Partition) == 0 && OFF_LAST % 16 == 0, "alignment of the partition record");
     static_assert(NW >= 4, "a warp builds the query fragments of at most two columns of the 8-wide head group");
-    static_assert(NSTAGE >= 4 && NSTAGE % 2 == 0 && NSTAGE <= 16, "an FP8 page takes a pair of slots; one phase bit per slot");
+    static_assert(NSTAGE >= 4 && NSTAGE % 2 == 0 && NSTAGE <= 16, "an FP8 page takes a pair of slots; one phase bit per pair");
     static_assert(NSTAGE * SLOT >= 8 * D * 4, "ring doubles as the cross-warp reduction buffer");
     static_assert(FP8_HALF <= SLOT, "half an FP8 record fits a slot");
 };
@@ -1205,7 +1208,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 
     // ---- prologue: barriers, prefix of pages, page strides ---------------------------------------
     if (tid == 0) {
-        for (int i = 0; i < NW * NSTAGE; ++i) mbar_init(sbase + G::OFF_BAR + 8 * i, 1);
+        for (int i = 0; i < NW * G::NP; ++i) mbar_init(sbase + G::OFF_BAR + 8 * i, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         last_s[1] = 0;
     }
@@ -1268,25 +1271,25 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         partition_range(pt, cum, hkv, P0.B, blockIdx.x, my_start, my_end);
     }
 
-    // per-warp ring of NSTAGE slots; one bit per slot holds the mbarrier phase the next wait must see
+    // per-warp ring of NP slot pairs; one bit per pair holds the mbarrier phase the next wait must see
     uint32_t phase = 0;
     bool failed = false;
     const uint32_t ring = sbase + warp * NSTAGE * G::SLOT;
-    const uint32_t bars = sbase + G::OFF_BAR + warp * NSTAGE * 8;
+    const uint32_t bars = sbase + G::OFF_BAR + warp * G::NP * 8;
     const uint32_t qt_lane = sbase + G::OFF_QT + lane * (SPLIT && FMT == 1 ? 8 : 16), qf_lane = sbase + G::OFF_QF + lane * 8;
     int* list3 = reinterpret_cast<int*>(smem + G::OFF_LIST) + warp * 2 * G::ROUND;   // Stale page ids of the round
     int* list8 = list3 + G::ROUND;                                                   // FP8 page ids | valid << 27
     int* lpg3 = reinterpret_cast<int*>(smem + G::OFF_LIST) + (NW + warp) * 2 * G::ROUND;   // their logical pages (scored variant)
     int* lpg8 = lpg3 + G::ROUND;
     const float sc2 = P0.scale * kLog2e;     // scores are kept in log2 units
-    uint32_t pending = 0;                    // ring slots with a copy in flight that nobody has waited for yet
-    // Bounded wait for ring slot s, then flip its expected phase.  `limit_ns` of wall time (the pool's wait
+    uint32_t pending = 0;                    // slot pairs with copies in flight that nobody has waited for yet
+    // Bounded wait for slot pair s, then flip its expected phase.  `limit_ns` of wall time (the pool's wait
     // limit, 20 ms by default); returns false when it ran out.
     auto wait_bounded = [&](uint32_t s, unsigned long long limit_ns) -> bool {
         const uint32_t bar = bars + 8 * s, parity = (phase >> s) & 1u;
-        // limit 0 (diagnostic): one look without blocking, so that a copy still in flight counts as late (the first
-        // one of a row is looked at as soon as it is issued)
-        bool ok = limit_ns == 0 ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity);
+        // (limit 0, diagnostic: a copy that this first look does not find counts as late; the first copies of a row are looked
+        // at as soon as they are issued)
+        bool ok = mbar_try_wait(bar, parity);
         if (!ok && limit_ns != 0) {
             unsigned long long t0, t1;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
@@ -1311,7 +1314,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     auto drain = [&]() {
         bool lost = false;
 #pragma unroll 1
-        for (uint32_t s = 0; s < (uint32_t)NSTAGE; ++s)
+        for (uint32_t s = 0; s < (uint32_t)G::NP; ++s)
             if (pending & (1u << s)) lost |= !wait_bounded(s, kDefaultWaitNs);
         return lost;
     };
@@ -1333,11 +1336,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         my_start = (int)max(flat_start(pt, blockIdx.x) - w0, 0ll);
         my_end = (int)min(flat_start(pt, blockIdx.x + 1) - w0, (long long)cum[P0.B]);
     }
-    auto wait_slot = [&](uint32_t s) {
-        if (!wait_bounded(s, P.wait_ns)) {
-            failed = true;
-            atomicOr(P.status, kStTimeout);
-        }
+    auto wait_slot = [&](uint32_t s) -> bool {
+        if (wait_bounded(s, P.wait_ns)) return true;
+        failed = true;
+        atomicOr(P.status, kStTimeout);
+        return false;
     };
     int pos = my_start;
     int b = 0;
@@ -1433,27 +1436,26 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             __syncwarp();
             return covered;
         };
-        auto issue_tq3 = [&](int i) {      // copy Stale page i of the round into ring slot i % NSTAGE
-            pending |= 1u << ((uint32_t)i % NSTAGE);
-            if (lane == 0) {
-                const uint32_t s = (uint32_t)i % NSTAGE;
-                if constexpr (!TILED) {
-                    mbar_expect_tx(bars + 8 * s, G::TQ3_REC);
-                    bulk_load(ring + s * G::SLOT, tq3_base + (size_t)list3[i] * hkv * G::TQ3_REC, G::TQ3_REC, bars + 8 * s);
-                } else {   // the tile only: the page's scale/zero are applied once, when the scan leaves the page
-                    const int page = list3[i], m = lpg3[i] & 0x7FFF;
-                    const uint8_t* pbase = P.tq3 + ((size_t)page * hkv + h) * tq3_page;
-                    mbar_expect_tx(bars + 8 * s, TQ3_TILE);
-                    bulk_load(ring + s * G::SLOT, pbase + (size_t)m * TQ3_TILE, TQ3_TILE, bars + 8 * s);
-                }
+        // Copy Stale pages 2j, 2j + 1 of the round (the second if there is one) into slot pair j % NP, a lane each.
+        auto issue_tq3 = [&](int j) {
+            const uint32_t s = (uint32_t)j % G::NP;
+            const int n = min(n3 - 2 * j, 2);
+            pending |= 1u << s;
+            if (lane < n) {
+                constexpr uint32_t BYTES = TILED ? TQ3_TILE : G::TQ3_REC;    // long pages: the tile only, their scale/zero are applied once
+                const int i = 2 * j + lane, page = list3[i];
+                const uint8_t* src = TILED ? P.tq3 + ((size_t)page * hkv + h) * tq3_page + (size_t)(lpg3[i] & 0x7FFF) * TQ3_TILE
+                                           : tq3_base + (size_t)page * hkv * G::TQ3_REC;
+                if (lane == 0) mbar_expect_tx(bars + 8 * s, n * BYTES);
+                bulk_load(ring + s * G::PAIR + lane * G::SLOT, src, BYTES, bars + 8 * s);
             }
         };
-        // FP8 page i of the round goes into the slot pair (first8 + i) % (NSTAGE / 2): the first pair is one that the
-        // round's last Stale page does not occupy, so that the FP8 copies start before that page is finished
+        // FP8 page i of the round goes into slot pair (first8 + i) % NP: the first pair is one that the round's last Stale
+        // page does not occupy, so that the FP8 copies start before that page is finished
         uint32_t first8 = 0;
         auto issue_fp8 = [&](int i) {
-            const uint32_t s = 2 * ((first8 + (uint32_t)i) % (NSTAGE / 2));
-            pending |= 3u << s;
+            const uint32_t s = (first8 + (uint32_t)i) % G::NP;
+            pending |= 1u << s;
             if (lane == 0) {
                 const int e8 = list8[i] & 0x7FFFFFF;
                 const uint8_t* rec;
@@ -1462,17 +1464,15 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 } else {
                     rec = P.fp8 + (((size_t)e8 * hkv + h) * P.tiles + (lpg8[i] & 0x7FFF)) * (2 * G::FP8_HALF);
                 }
-                mbar_expect_tx(bars + 8 * s, G::FP8_HALF);
-                bulk_load(ring + s * G::SLOT, rec, G::FP8_HALF, bars + 8 * s);
-                mbar_expect_tx(bars + 8 * (s + 1), G::FP8_HALF);
-                bulk_load(ring + (s + 1) * G::SLOT, rec + G::FP8_HALF, G::FP8_HALF, bars + 8 * (s + 1));
+                mbar_expect_tx(bars + 8 * s, 2 * G::FP8_HALF);
+                bulk_load(ring + s * G::PAIR, rec, 2 * G::FP8_HALF, bars + 8 * s);
             }
         };
         auto start_round = [&]() {         // the first copies of a round
-            first8 = n3 > 0 ? ((uint32_t)(n3 - 1) % NSTAGE / 2 + 1) % (NSTAGE / 2) : 0u;
-            for (int i = 0; i < min(n3, NSTAGE); ++i) issue_tq3(i);
+            first8 = n3 > 0 ? ((uint32_t)(n3 - 1) / 2 + 1) % G::NP : 0u;
+            for (int j = 0; j < min((n3 + 1) / 2, G::NP); ++j) issue_tq3(j);
             if (n3 == 0)
-                for (int i = 0; i < min(n8, NSTAGE / 2); ++i) issue_fp8(i);
+                for (int i = 0; i < min(n8, G::NP); ++i) issue_fp8(i);
         };
 
         WarpAcc<NB> acc;
@@ -1652,10 +1652,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 }
                 wait_slot(0);
                 if (!failed) tq3_step<D, false, true, TILED, FMT, SPLIT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, sc2k1, lane, s_cur);
-                for (int i = 0; i + 1 < n3 && !failed; ++i) {
+                for (int i = 0; !failed && i + 1 < n3; ++i) {
                     const uint32_t cur = (uint32_t)i % NSTAGE, nxt = (uint32_t)(i + 1) % NSTAGE;
-                    wait_slot(nxt);
-                    if (failed) break;
+                    if ((i & 1) && !wait_slot(nxt / 2)) break;       // the next page opens a slot pair
                     if constexpr (FMT == 2 && SPLIT) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
                     else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
@@ -1671,7 +1670,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 #pragma unroll
                     for (int e = 0; e < 4; ++e) s_cur[e] = s_next[e];
                     __syncwarp();
-                    if (i + NSTAGE < n3) issue_tq3(i + NSTAGE);
+                    if ((i & 1) && i + 2 * G::NP - 1 < n3) issue_tq3(i / 2 + G::NP);    // the pair of pages i - 1, i is free
                 }
                 if (!failed) {
                     if (n8 > 0) issue_fp8(0);
@@ -1691,23 +1690,21 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 }
                 __syncwarp();
                 if (!failed)
-                    for (int i = 1; i < min(n8, NSTAGE / 2); ++i) issue_fp8(i);
+                    for (int i = 1; i < min(n8, G::NP); ++i) issue_fp8(i);
             }
             // ---- Recent/Anchor pages: two slots per page (keys, values)
             if (n8 > 0 && !failed) {
-                for (int i = 0; i < n8 && !failed; ++i) {
-                    const uint32_t s = 2 * ((first8 + (uint32_t)i) % (NSTAGE / 2));
-                    wait_slot(s);
-                    wait_slot(s + 1);
-                    if (failed) break;
+                for (int i = 0; i < n8; ++i) {
+                    const uint32_t s = (first8 + (uint32_t)i) % G::NP;
+                    if (!wait_slot(s)) break;
                     const int e = list8[i];
                     const int valid = (e >> 27) & 15;
-                    fp8_page<D, SCORED, TILED, SPLIT>(acc, ring + s * G::SLOT, ring + (s + 1) * G::SLOT, qf_lane, sc2 * P.k_scale, P.v_scale,
+                    fp8_page<D, SCORED, TILED, SPLIT>(acc, ring + s * G::PAIR, ring + s * G::PAIR + G::FP8_HALF, qf_lane, sc2 * P.k_scale, P.v_scale,
                                                valid ? valid : kPage, lane,
                                                SCORED ? mass_row + (TILED ? (lpg8[i] >> 16) : lpg8[i]) : nullptr, P.max_pages, GQ);
                     if constexpr (FMT == 2 && SPLIT) max_rows_from_columns<NB>(acc, lane);     // the page may have raised the maxima
                     __syncwarp();
-                    if (i + NSTAGE / 2 < n8) issue_fp8(i + NSTAGE / 2);
+                    if (i + G::NP < n8) issue_fp8(i + G::NP);
                 }
             }
             more = done < n_my;

@@ -1651,8 +1651,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     cur_lp = lpg3[0] >> 16;
                 }
                 wait_slot(0);
-                if (!failed) tq3_step<D, false, true, TILED, FMT, SPLIT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, sc2k1, lane, s_cur);
-                for (int i = 0; !failed && i + 1 < n3; ++i) {
+                if (failed) break;
+                tq3_step<D, false, true, TILED, FMT, SPLIT>(acc, 0, s_cur, pf, ring, qt_lane, sc2k, sc2k1, lane, s_cur);
+                // (twice in the code where that was faster: 64 ragged requests 542 -> 534 us; long pages and several layers, whose
+                // loop is larger, lose by it: 634 -> 726 us)
+                constexpr int UNROLL = SPLIT && !TILED && !FLAT ? 2 : 1;
+#pragma unroll UNROLL
+                for (int i = 0; i + 1 < n3; ++i) {
                     const uint32_t cur = (uint32_t)i % NSTAGE, nxt = (uint32_t)(i + 1) % NSTAGE;
                     if ((i & 1) && !wait_slot(nxt / 2)) break;       // the next page opens a slot pair
                     if constexpr (FMT == 2 && SPLIT) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);

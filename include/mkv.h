@@ -285,7 +285,9 @@ int32_t mkv_append_layers(const mkv_layer_append* layers_host, int32_t n_layers,
  * a process whose allocator is frozen while it serves).  (The paper has no counterpart: this is a
  * property of the library, not of the method.)  The split partials go to a fixed array inside the
  * library image, MKV_STATIC_SCRATCH_BYTES per GPU that loads the library, held until the process
- * exits.  Arguments, results and kernel are those of mkv_decode_attention with the tensor-core variant;
+ * exits.  Arguments, results and kernel are those of mkv_decode_attention with the tensor-core variant (which
+ * splits rows among twice as many blocks where it has room for their partials: the same sums split at other
+ * pages, equal to fp32 rounding);
  * a pool that was switched to another variant is refused with MKV_E_INVALID.
  *   - allocates nothing: no cudaMalloc / cudaFree, no allocating library call, on any call.
  *   - limits: B <= MKV_STATIC_MAX_BATCH, and the scan must not launch more than MKV_STATIC_MAX_BLOCKS

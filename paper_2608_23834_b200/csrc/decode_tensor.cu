@@ -5,8 +5,8 @@
 // unpacked tile, and split partials (m, l, O) are merged with Eq. (softmax-merge).
 //
 // Mapping to the hardware
-//   * work = (request, KV head, page) triples in row-major order, cut into equal contiguous ranges,
-//     one per block (persistent grid, a multiple of the SM count); a block processes the
+//   * work = (request, KV head, page) triples in row-major order (several layers: end to end), cut into
+//     contiguous ranges, one per block (persistent grid, one or two blocks per SM); a block processes the
 //     (request, KV head) segments of its range one after another, its warps taking contiguous runs of pages.
 //   * each warp streams its pages through a private ring of shared-memory slots filled by bulk
 //     asynchronous copies (cp.async.bulk + mbarrier), several pages ahead of the arithmetic.
@@ -14,8 +14,8 @@
 //     (rotated) query of the 8-column head group: S[16 tokens][8 heads] = K q^T.  TQ3 keys stay in
 //     the rotated domain; the query is rotated instead (q' = d^-1/2 H (sigma . q)).  The packed
 //     3-bit codes are stored in the register layout of that A fragment, so unpacking is a byte
-//     table lookup (PRMT) per four codes for keys and one masked OR plus one half2 FMA per two
-//     codes for values -- no shared-memory round trip, no dequantised tile.
+//     table lookup (PRMT) per four codes for keys and one mask per two codes for values -- no
+//     shared-memory round trip, no dequantised tile.
 //   * P = exp2(S - m) is transposed in registers (movmatrix) into the B operand of
 //     O^T[16 channels][8 heads] += V^T P, one MMA per 16 channels; the row sums come from one more
 //     MMA against a matrix of ones.  TQ3 values enter that MMA as their integer codes; the

@@ -15,12 +15,6 @@
 
 namespace mkv {
 
-__device__ __forceinline__ float e4m3_to_f32(uint8_t b)
-{
-    __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)b, __NV_E4M3);
-    return __half2float(__half(h));
-}
-
 __device__ __forceinline__ uint16_t f32_to_f16_sat_bits(float x)
 {
     x = fminf(fmaxf(x, -65504.f), 65504.f);

@@ -152,7 +152,8 @@ def test_a_wait_that_runs_out_is_reported_and_the_pool_stays_usable():
         assert np.array_equal(out2, out) and np.array_equal(lse2, lse)
 
 
-@pytest.mark.parametrize("n_layers,name", [(4, "cfg2"), (7, "edge"), (5, "tiny"), (4, "pages_of_832"), (6, "pages_of_48_d128")])
+@pytest.mark.parametrize("n_layers,name", [(4, "cfg2"), (7, "edge"), (5, "tiny"), (4, "many_rows"), (4, "pages_of_832"),
+                                           (6, "pages_of_48_d128")])
 @pytest.mark.parametrize("fmt", [1, 2])
 def test_layers_laid_end_to_end(n_layers, name, fmt):
     """From four layers on one cut of the grid covers all layers' pages: rows that a block shares with its
@@ -165,6 +166,8 @@ def test_layers_laid_end_to_end(n_layers, name, fmt):
           "pages_of_48_d128": lambda: W.config(1, seq_lens=(48 * 21 + 5, 48 * 30, 47, 48 * 9 + 47), anchor_prefix=48,
                                                recent_tokens=100, anchor_span_tokens=96, page_tokens=48),
           "tiny": lambda: W.config(0, seq_lens=(5,), head_dim=256, n_kv_heads=1, group=3),
+          "many_rows": lambda: W.config(2, seq_lens=(33, 700, 16, 450, 1, 0, 257, 1300), anchor_prefix=32, recent_tokens=120,
+                                        n_layers=1),
           "edge": lambda: W.config(0, seq_lens=(0, 1, 15, 16, 17, 33, 16 * 20 + 9, 300), head_dim=128, n_kv_heads=2, group=4,
                                    anchor_prefix=16, recent_tokens=40, n_outlier=3)}[name]
     oracle.set_format(fmt)

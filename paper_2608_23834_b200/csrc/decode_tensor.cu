@@ -968,13 +968,15 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
         const int tq = lane & 3;
         const uint32_t gaddr = rec_k + 12 * D + 4 * tq;
         const float2 ga = half2_to_float2(lds32(gaddr)), gb = half2_to_float2(lds32(gaddr + 16));
-        // this lane has digit 0 (g < 4) or 1 (g >= 4) and digit 2 of head g % 4, the lane 16 away the other one
-        const float mine = lane & 16 ? 128.f : 16384.f, theirs = lane & 16 ? 16384.f : 128.f;
+        // This lane has digit 0 (g < 4) or 1 (g >= 4) and digit 2 of head g % 4, the lane 16 away the other one.  Both put
+        // the score together in the same order: rows h and h + 4 supply the high and the low halves of the same
+        // probabilities, so their scores have to be the same bits.
         float d[4];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            d[e] = fmaf((float)I0[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I0[e], 16), theirs, (float)I0[2 + e]));
-            d[2 + e] = fmaf((float)I1[e], mine, fmaf((float)__shfl_xor_sync(0xffffffffu, I1[e], 16), theirs, (float)I1[2 + e]));
+            const int o0 = __shfl_xor_sync(0xffffffffu, I0[e], 16), o1 = __shfl_xor_sync(0xffffffffu, I1[e], 16);
+            d[e] = lane & 16 ? digits_to_score(o0, I0[e], I0[2 + e]) : digits_to_score(I0[e], o0, I0[2 + e]);
+            d[2 + e] = lane & 16 ? digits_to_score(o1, I1[e], I1[2 + e]) : digits_to_score(I1[e], o1, I1[2 + e]);
         }
         s_next[0] = d[0] * (ga.x * sc2);
         s_next[1] = d[1] * (ga.y * sc2);

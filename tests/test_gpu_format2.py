@@ -214,3 +214,40 @@ def test_decode_with_fp8_scales_other_than_one(k_scale, v_scale, variant):
     # and the scales matter: the result differs from the one under unit scales
     ref1, _ = case.reference()
     assert np.abs(ref - ref1).max() > 1e-2
+
+
+@pytest.mark.parametrize("d", [128, 256])
+def test_both_halves_of_a_probability_belong_to_the_same_score(d):
+    """Groups of at most four query heads: a head is scored in two rows, one supplies the high and one the low halves
+    of its probabilities.  If the two rows put the score's digits together in different orders, their scores differ in
+    the last bit for some directions of the query, and then some probabilities are wrong by an fp16 rounding.  To meet
+    enough of them: 32,768 heads with queries in random directions, 16 tokens with the same key codes (hence all with
+    the same digits) and slightly different norms, scores between 16 and 120 in log2 units.
+    Bound: a score of 120 rounded four times in fp32 is good to 4 x 120 x 2^-25 = 1.4e-5 log2 units, 1e-5 of a
+    probability; the errors of 16 tokens are independent and relative to outputs that average 16 values, hence the same
+    size in the output.  A wrong half of one probability in 16 moves its row by 2^-11 x 1 / 16 x 4 = 1.2e-4."""
+    hkv, group, B = 8, 4, 1024
+    rng = np.random.default_rng(11 + d)
+    sigma = (rng.integers(0, 2, d) * 2 - 1).astype(np.int8)
+    u = rng.standard_normal((hkv, d)).astype(np.float32)
+    rec = np.zeros((1, hkv, 16 * d + 32), np.uint8)
+    for h in range(hkv):
+        rec[0, h] = oracle.demote_record(oracle.fp8_pack_record(np.repeat(u[h:h + 1], 16, 0),
+                                                                rng.standard_normal((16, d)).astype(np.float32)), d, sigma)
+        g = rec[0, h, 12 * d:12 * d + 32].view(np.float16)
+        g[:] = (g * rng.uniform(0.99, 1.01, 16)).astype(np.float16)
+    pool = M.Pool(d, hkv, hkv * group, 1, 1, sigma, max_batch=B, tq3_format=2)
+    pool.page_write_raw(M.FMT_TQ3, 0, rec[0])
+    q = rng.standard_normal((B, hkv, group, d)).astype(np.float32) + 0.2 * u[None, :, None]
+    dot = np.einsum("bhgd,hd->bhg", q, u)[..., None]
+    q *= rng.uniform(16, 120, dot.shape).astype(np.float32) / (np.sign(dot) * np.maximum(np.abs(dot), 0.5) * d ** -0.5 * np.log2(np.e))
+    q_bits = W.f32_to_bf16_bits(q.reshape(B, hkv * group, d))
+    bt, tags = np.zeros((B, 1), np.int32), np.full((B, 1), M.TAG_STALE, np.uint8)
+    lens = np.full(B, 16, np.int32)
+    from _gpu_util import bf16_tensor
+    out = pool.decode_attention(bf16_tensor(q_bits), *(torch.from_numpy(x).cuda() for x in (bt, tags, lens)), d ** -0.5)
+    torch.cuda.synchronize()
+    assert pool.status() == M.OK
+    ref, _ = oracle.decode_attention(np.zeros((0,), np.uint8), rec, d, hkv, group, sigma, q_bits, bt, tags, lens, d ** -0.5)
+    err = np.linalg.norm(out.cpu().numpy() - ref, axis=-1) / np.linalg.norm(ref, axis=-1)
+    assert err.max() < 6e-5, (err.max(), np.sort(err.ravel())[-8:])

@@ -1525,7 +1525,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                                                                 (size_t)P.tiles * TQ3_TILE + g * 16);
 #pragma unroll
             for (int j = 0; j < NB / 4; ++j) {
-                const uint4 m01 = __ldg(meta + j * 16), m23 = __ldg(meta + j * 16 + 8);
+                const uint4 m01 = meta[j * 16], m23 = meta[j * 16 + 8];
                 const uint32_t scp[4] = {m01.x, m01.z, m23.x, m23.z}, zpp[4] = {m01.y, m01.w, m23.y, m23.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {

@@ -88,8 +88,8 @@ __device__ __forceinline__ float push_magnitude(float acc, float step, float y, 
 
 template <int D, int FMT, bool BIG>
 __global__ void __launch_bounds__(32 * kDemoteWarps, D == 256 ? 3 : 4)
-demote_warp_kernel(const uint8_t* __restrict__ fp8, uint8_t* __restrict__ tq3, int fp8_pages, int tq3_pages, int hkv, int tiles,
-                   SigmaBits sigma, const int32_t* __restrict__ src_ids, const int32_t* __restrict__ dst_ids,
+demote_warp_kernel(const uint8_t* fp8, uint8_t* __restrict__ tq3, int fp8_pages, int tq3_pages, int hkv, int tiles,
+                   SigmaBits sigma, const int32_t* src_ids, const int32_t* dst_ids,
                    int32_t* block_table, uint8_t* tier_tag, const int64_t* entry_index, int64_t n_entries,
                    uint32_t* __restrict__ status, uint32_t* page_tickets)
 {

@@ -46,9 +46,9 @@ __device__ __forceinline__ void append_pair(uint8_t* __restrict__ rec, int slot,
 template <int D>
 __global__ void __launch_bounds__(D / 2) append_kernel(uint8_t* __restrict__ fp8, int fp8_pages, int hkv, int tiles,
                                                         float inv_k_scale, float inv_v_scale,
-                                                        const __nv_bfloat162* __restrict__ k,
-                                                        const __nv_bfloat162* __restrict__ v,
-                                                        const int32_t* __restrict__ slots,
+                                                        const __nv_bfloat162* k,
+                                                        const __nv_bfloat162* v,
+                                                        const int32_t* slots,
                                                         uint32_t* __restrict__ status)
 {
     pdl_begin();
@@ -92,9 +92,9 @@ __device__ __forceinline__ uint2 bf16x8_to_e4m3x8(uint4 in, float inv_scale)
 template <int D>
 __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ fp8, int fp8_pages, int hkv, int tiles,
                                                           float inv_k_scale, float inv_v_scale,
-                                                          const __nv_bfloat162* __restrict__ k,
-                                                          const __nv_bfloat162* __restrict__ v,
-                                                          const int32_t* __restrict__ slots, int n,
+                                                          const __nv_bfloat162* k,
+                                                          const __nv_bfloat162* v,
+                                                          const int32_t* slots, int n,
                                                           uint32_t* __restrict__ status)
 {
     constexpr int VROW = D + 4;                      // padded token row of the transposition tile
@@ -134,13 +134,20 @@ __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ f
     if (full >= 0) {
         const int gt = slot_s[full] >> 4, page = gt / tiles;
         uint8_t* rec = fp8 + (((size_t)page * hkv + h) * tiles + (gt - page * tiles)) * fp8_record_bytes(D);
-        constexpr int CPT = D / 8;                   // 16-byte input chunks per token
+        constexpr int CPT = D / 8, N = kPage * CPT / 128;      // 16-byte input chunks per token, and per thread
+        uint4 kin[N], vin[N];                        // all loads before the first store
 #pragma unroll
-        for (int c = tid; c < kPage * CPT; c += 128) {
-            const int t = c / CPT, c8 = c % CPT;
-            const size_t at = ((size_t)(t0 + full + t) * hkv + h) * (D / 8) + c8;
-            const uint2 kq = bf16x8_to_e4m3x8(reinterpret_cast<const uint4*>(k)[at], inv_k_scale);
-            const uint2 vq = bf16x8_to_e4m3x8(reinterpret_cast<const uint4*>(v)[at], inv_v_scale);
+        for (int u = 0; u < N; ++u) {
+            const int c = tid + 128 * u;
+            const size_t at = ((size_t)(t0 + full + c / CPT) * hkv + h) * CPT + c % CPT;
+            kin[u] = reinterpret_cast<const uint4*>(k)[at];
+            vin[u] = reinterpret_cast<const uint4*>(v)[at];
+        }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const int c = tid + 128 * u, t = c / CPT, c8 = c % CPT;
+            const uint2 kq = bf16x8_to_e4m3x8(kin[u], inv_k_scale);
+            const uint2 vq = bf16x8_to_e4m3x8(vin[u], inv_v_scale);
             *reinterpret_cast<uint2*>(rec + t * D + 8 * c8) = kq;
             *reinterpret_cast<uint32_t*>(vt + t * VROW + 8 * c8) = vq.x;
             *reinterpret_cast<uint32_t*>(vt + t * VROW + 8 * c8 + 4) = vq.y;
@@ -203,7 +210,7 @@ struct AppendLayers {
 
 template <int D>
 __global__ void __launch_bounds__(D / 2) append_layers_kernel(const AppendLayers A, int hkv, int tiles,
-                                                               const int32_t* __restrict__ slots)
+                                                               const int32_t* slots)
 {
     pdl_begin();
     const int tok = blockIdx.x, h = blockIdx.y, layer = blockIdx.z;
@@ -547,7 +554,7 @@ __device__ __forceinline__ uint32_t literal_value_code(float val, float scf, flo
 // scale/zero] in shared memory; all D threads of the block call it.  OWN_META: the value scale and zero come
 // from these 16 tokens (16-token pages); otherwise thread c passes the page's scale/zero of channel c.
 template <int D, bool OWN_META, int FMT>
-__device__ __forceinline__ void demote_tile(const uint8_t* __restrict__ rec8, uint8_t* img, uint8_t* kcode, uint8_t* vcode,
+__device__ __forceinline__ void demote_tile(const uint8_t* rec8, uint8_t* img, uint8_t* kcode, uint8_t* vcode,
                                             const DemoteLane<D, FMT>& K, float k_scale, float v_scale, uint16_t sc_page,
                                             uint16_t zp_page)
 {
@@ -705,11 +712,11 @@ __device__ __forceinline__ void demote_tile(const uint8_t* __restrict__ rec8, ui
 }
 
 template <int D, bool BIG, int FMT>
-__global__ void __launch_bounds__(D) demote_kernel(const uint8_t* __restrict__ fp8, uint8_t* __restrict__ tq3,
+__global__ void __launch_bounds__(D) demote_kernel(const uint8_t* fp8, uint8_t* __restrict__ tq3,
                                                       int fp8_pages, int tq3_pages, int hkv, int tiles, float k_scale,
                                                       float v_scale, SigmaBits sigma,
-                                                      const int32_t* __restrict__ src_ids,
-                                                      const int32_t* __restrict__ dst_ids, int32_t* block_table,
+                                                      const int32_t* src_ids,
+                                                      const int32_t* dst_ids, int32_t* block_table,
                                                       uint8_t* tier_tag, const int64_t* entry_index, int64_t n_entries,
                                                       uint32_t* __restrict__ status, uint32_t* page_tickets)
 {
@@ -814,10 +821,10 @@ __device__ __forceinline__ float ld_cluster_f32(const float* local, uint32_t ran
 }
 
 template <int D>
-__global__ void __launch_bounds__(D) demote_minmax_kernel(const uint8_t* __restrict__ fp8, uint8_t* __restrict__ tq3,
+__global__ void __launch_bounds__(D) demote_minmax_kernel(const uint8_t* fp8, uint8_t* __restrict__ tq3,
                                                            int fp8_pages, int tq3_pages, int hkv, int tiles,
-                                                           float v_scale, const int32_t* __restrict__ src_ids,
-                                                           const int32_t* __restrict__ dst_ids)
+                                                           float v_scale, const int32_t* src_ids,
+                                                           const int32_t* dst_ids)
 {
     __shared__ float part[2][D];
     const int csize = (int)cluster_size(), crank = (int)cluster_rank();
@@ -889,9 +896,9 @@ __global__ void __launch_bounds__(D) demote_minmax_kernel(const uint8_t* __restr
 
 // Pages of several tiles, last pass of Demote / Promote: the kernels before it in the stream have written the
 // whole page, so its id and tag may appear (copy-before-publish by stream order).
-__global__ void publish_kernel(int n, const int32_t* __restrict__ src_ids, const int32_t* __restrict__ dst_ids,
+__global__ void publish_kernel(int n, const int32_t* src_ids, const int32_t* dst_ids,
                                int src_cap, int dst_cap, int32_t* block_table, uint8_t* tier_tag,
-                               const int64_t* __restrict__ entry_index, int64_t n_entries, int tag, uint32_t* status)
+                               const int64_t* entry_index, int64_t n_entries, int tag, uint32_t* status)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_begin();

@@ -101,11 +101,14 @@ struct mkv_seq {
 };
 
 namespace mkv {
-// Programmatic dependent launch.  Every kernel of the library is launched so that it may start while the kernel
-// before it in the stream is still running, and begins with pdl_begin(): it lets the kernel behind it start in turn
-// and then waits until everything before it has completed and is visible.  What a kernel does not need to wait for
-// (its launch, shared-memory set-up) then overlaps its predecessor: an append + decode pair of a small call takes
-// 2 us less.  Order and visibility are those of ordinary stream order.
+// Programmatic dependent launch.  A kernel launched with `early` may start while the kernel before it in the stream is
+// still running, and begins with pdl_begin(): it lets the kernel behind it start in turn and then waits until everything
+// before it has completed and is visible.  What a kernel does not need to wait for (its launch, shared-memory set-up)
+// then overlaps its predecessor: an append + decode pair of a small call takes 2 us less.  Order and visibility are
+// those of ordinary stream order -- for coherent loads.  Such a kernel lives while its predecessor still writes, so the
+// memory it reads is not read-only for its lifetime: no const __restrict__ and no __ldg on anything that an earlier
+// kernel may have written (arenas, ids, entries, slots, page scales).  The CUDA-core and tensor-memory variants of the
+// scan are ordinary launches.
 __device__ __forceinline__ void pdl_begin()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -51,11 +51,11 @@ __device__ __forceinline__ void fetch_lane_words(const uint8_t* sec, int lane, u
     constexpr int LW = 3 * (D / 16) / 4;
 #pragma unroll
     for (int c = 0; c < LW / 4; ++c) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(sec + c * 512 + lane * 16));
+        const uint4 v = *reinterpret_cast<const uint4*>(sec + c * 512 + lane * 16);
         w[4 * c] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
     }
     if constexpr (LW % 4 != 0) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2*>(sec + (LW / 4) * 512 + lane * 8));
+        const uint2 v = *reinterpret_cast<const uint2*>(sec + (LW / 4) * 512 + lane * 8);
         w[LW - 2] = v.x; w[LW - 1] = v.y;
     }
 }
@@ -77,9 +77,9 @@ __device__ __forceinline__ uint32_t code_selector(uint32_t x, uint32_t y)
 
 template <int D, int FMT, bool BIG>
 __global__ void __launch_bounds__(32 * kDemoteWarps, D == 256 ? 3 : 4)
-promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, int tq3_pages, int fp8_pages, int hkv, int tiles,
-                    float inv_k_scale, float inv_v_scale, float rs, SigmaBits sigma, const int32_t* __restrict__ src_ids,
-                    const int32_t* __restrict__ dst_ids, int32_t* block_table, uint8_t* tier_tag, const int64_t* entry_index,
+promote_warp_kernel(const uint8_t* tq3, uint8_t* __restrict__ fp8, int tq3_pages, int fp8_pages, int hkv, int tiles,
+                    float inv_k_scale, float inv_v_scale, float rs, SigmaBits sigma, const int32_t* src_ids,
+                    const int32_t* dst_ids, int32_t* block_table, uint8_t* tier_tag, const int64_t* entry_index,
                     int64_t n_entries, uint32_t* __restrict__ status, uint32_t* page_tickets)
 {
     using G = PromoteWarp<D>;
@@ -125,12 +125,12 @@ promote_warp_kernel(const uint8_t* __restrict__ tq3, uint8_t* __restrict__ fp8, 
     uint16_t g0 = 0, g1 = 0;
     auto fetch_keys = [&](const uint8_t* rec3) {
         fetch_lane_words<D>(rec3, lane, kw);
-        g0 = __ldg(reinterpret_cast<const uint16_t*>(rec3 + 12 * D) + g);
-        g1 = __ldg(reinterpret_cast<const uint16_t*>(rec3 + 12 * D) + g + 8);
+        g0 = reinterpret_cast<const uint16_t*>(rec3 + 12 * D)[g];
+        g1 = reinterpret_cast<const uint16_t*>(rec3 + 12 * D)[g + 8];
     };
     auto fetch_meta = [&](const uint8_t* page3) {    // (16-token pages: right behind the one tile)
 #pragma unroll
-        for (int i = 0; i < D / 128; ++i) mt[i] = __ldg(reinterpret_cast<const uint4*>(page3 + (size_t)tiles * TILE) + lane + 32 * i);
+        for (int i = 0; i < D / 128; ++i) mt[i] = reinterpret_cast<const uint4*>(page3 + (size_t)tiles * TILE)[lane + 32 * i];
     };
     auto fetch_record = [&](int h, int m) {
         const uint8_t* page3 = page_of(h);

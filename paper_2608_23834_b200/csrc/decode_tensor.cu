@@ -405,6 +405,10 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, i
     const int rows = B * hkv;
     int blocks = useful_blocks(W, grid, min_pages);
     grid = blocks;
+    if (blocks == 0) {                                  // every request of the call is empty
+        if (lane == 0) pt->aligned = pt->blocks = 0;
+        return;
+    }
     // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
     // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
     // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).

@@ -236,3 +236,24 @@ def test_decode_one_long_row_and_the_page_limit():
         case.pool.decode_attention(case.q, wide_bt, wide_tg, case.lens, spec.scale)
     assert e.value.code == M.E_INVALID
     assert b"65535" in M.lib().mkv_last_cuda_error()
+
+
+@pytest.mark.parametrize("d,page", [(128, 16), (256, 16), (128, 48), (256, 832)])
+def test_a_batch_of_empty_requests_only(d, page):
+    """No pages at all: nothing to cut the grid over; outputs are zero and the log-sum-exps minus infinity."""
+    hkv, group, B = 2, 3, 5
+    pools = [M.Pool(d, hkv, hkv * group, 2, 2, np.ones(d, np.int8), max_batch=B, page_tokens=page) for _ in range(5)]
+    q = torch.randn((B, hkv * group, d), device="cuda:0", dtype=torch.bfloat16)
+    bt, tags = torch.full((B, 3), -1, dtype=torch.int32, device="cuda:0"), torch.zeros((B, 3), dtype=torch.uint8, device="cuda:0")
+    lens = torch.zeros(B, dtype=torch.int32, device="cuda:0")
+    new = lambda *shape: torch.full(shape, 7.0, device="cuda:0")
+    outs, lses = [new(B, hkv * group, d) for _ in range(8)], [new(B, hkv * group) for _ in range(8)]
+    pools[0].decode_attention(q, bt, tags, lens, 0.1, out=outs[0], lse=lses[0])
+    mass = pools[1].decode_attention_scored(q, bt, tags, lens, 0.1, out=outs[1], lse=lses[1])[2]
+    M.decode_attention_static(pools[2], q, bt, tags, lens, 0.1, out=outs[2], lse=lses[2])
+    for n in (2, 5):                          # every layer cut by itself, layers laid end to end
+        M.decode_attention_layers(pools[:n], [q] * n, [bt] * n, [tags] * n, lens, 0.1, outs[3:3 + n], lses[3:3 + n])
+        torch.cuda.synchronize()
+        for out, lse in zip(outs[:3 + n], lses[:3 + n]):
+            assert not out.any() and bool(torch.isneginf(lse).all())
+    assert not mass.any() and all(p.status() == M.OK for p in pools)

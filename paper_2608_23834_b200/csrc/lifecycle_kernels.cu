@@ -951,7 +951,7 @@ static cudaError_t launch_demote_warp(mkv_pool* p, const int32_t* src, const int
     const int smem = DemoteWarp<D>::OFF_WARPS + warps * DemoteWarp<D>::BYTES;
     static_assert(DemoteWarp<D>::OFF_WARPS + kDemoteWarps * DemoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
     return launch_pdl(demote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv) : 1), 32 * warps,
-                      (size_t)smem, c, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv,
+                      (size_t)smem, c, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv,
                       p->tiles, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }
 
@@ -966,7 +966,7 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
     }
     if (p->tiles == 1) {
         const int c = heads_cluster(p->hkv, n);
-        MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
+        MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, 1, p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, bt,
                                   tags, entry, n_entries, p->status_dev, (uint32_t*)nullptr));
         return MKV_OK;
@@ -978,7 +978,7 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
         // blocks per (page, head): up to a portable cluster of 8, fewer when the call fills the GPU anyway
         int cs = 8;
         while (cs > 1 && (cs > p->tiles || (long long)n * p->hkv * cs > 8LL * 148)) cs >>= 1;
-        MKV_CUDA(launch_pdl(demote_minmax_kernel<D>, dim3((unsigned)n * p->hkv * cs), D, 0, cs, n <= 148, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
+        MKV_CUDA(launch_pdl(demote_minmax_kernel<D>, dim3((unsigned)n * p->hkv * cs), D, 0, cs, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, p->tiles, p->cfg.v_scale, src, dst));
     }
     const int ch = heads_cluster(p->hkv, 0);
@@ -986,7 +986,7 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
         MKV_CUDA((launch_demote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
                                                    fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
     else
-    MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, n <= 148, s,
+    MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, false, s,
                                    (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv, p->tiles,
                                    p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr,
                                    fused ? tags : (uint8_t*)nullptr, fused ? entry : (const int64_t*)nullptr,
@@ -1022,7 +1022,7 @@ static cudaError_t launch_promote_warp(mkv_pool* p, const int32_t* src, const in
     static_assert(PromoteWarp<D>::OFF_WARPS + kDemoteWarps * PromoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
     const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale, rs = (float)(1.0 / sqrt((double)p->d));
     return launch_pdl(promote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv) : 1),
-                      32 * warps, (size_t)smem, c, n <= 148, s, (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages,
+                      32 * warps, (size_t)smem, c, false, s, (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages,
                       p->hkv, p->tiles, ik, iv, rs, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }
 

@@ -115,8 +115,10 @@ __device__ __forceinline__ void pdl_begin()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// early: start before the predecessor has ended.  Not for a grid of one or two waves of long blocks: blocks placed
-// while the predecessor still holds some SMs spread unevenly (Promote of 1,023 pages 33 -> 36 us).
+// early: start before the predecessor has ended.  Not for Demote and Promote: their blocks would be placed while the
+// predecessor still holds most SMs, up to four on one SM, and wait there, and behind a decode scan that has evicted
+// their code they start on it together: one page between decode calls, d = 256, 4 heads, Demote 40 -> 20 us, Promote
+// 15 -> 8 us without; 148 pages 37 -> 23 and 16 -> 10.5 us.
 // cluster: blocks per thread-block cluster along x (1: none)
 template <typename Kernel, typename... Args>
 static cudaError_t launch_pdl(Kernel kernel, dim3 grid, int threads, size_t smem, int cluster, bool early, cudaStream_t s,

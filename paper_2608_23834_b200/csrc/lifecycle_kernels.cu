@@ -960,7 +960,14 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
                                const int64_t* entry, int64_t n_entries, cudaStream_t s)
 {
     const bool unit_scales = p->cfg.k_scale == 1.0f && p->cfg.v_scale == 1.0f;      // what the warp kernel's exactness rests on
-    if (p->tiles == 1 && unit_scales) {
+    // Few records at d = 256 take the general kernel: eight warps share a record and its code is a loop, where the warp
+    // kernel runs 3,900 instructions in a row, which a call between two decode scans has to fetch anew.  Between decode
+    // calls one page of 4 heads takes 9 us in the general kernel, 20 (format 1) and 17 us in the warp kernel, a page of
+    // 1,792 tokens 22 against 29 and 23 against 25; the two meet at about 1,200 tile records in format 1 (24 us) and
+    // 800 in the shorter code of format 2 (18.5 us).  At d = 128 they differ by less than 1.5 us.
+    const bool few = D == 256 && (long long)n * p->hkv * p->tiles <= (FMT == 1 ? 8 : 5) * (long long)p->dev.sm_count;
+    const bool warp_per_record = unit_scales && !few;
+    if (p->tiles == 1 && warp_per_record) {
         MKV_CUDA((launch_demote_warp<D, FMT, false>(p, src, dst, n, bt, tags, entry, n_entries, nullptr, s)));
         return MKV_OK;
     }
@@ -982,11 +989,11 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
                                   p->cfg.tq3_pages, p->hkv, p->tiles, p->cfg.v_scale, src, dst));
     }
     const int ch = heads_cluster(p->hkv, 0);
-    if (unit_scales)
+    if (warp_per_record)
         MKV_CUDA((launch_demote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
                                                    fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
     else
-    MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, false, s,
+        MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, false, s,
                                    (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv, p->tiles,
                                    p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr,
                                    fused ? tags : (uint8_t*)nullptr, fused ? entry : (const int64_t*)nullptr,

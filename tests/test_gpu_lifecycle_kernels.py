@@ -372,3 +372,33 @@ def test_bulk_calls_write_the_same_bytes_as_small_calls(d, hkv):
         got = pool.page_read_raw(M.FMT_TQ3, p).reshape(hkv, -1)
         for h in range(hkv):
             assert np.array_equal(got[h], oracle.demote_record(src[h], d, sigma, 1.0, 1.0)), (p, h)
+
+
+@pytest.mark.parametrize("d,hkv,n,page,fmt", [(256, 4, 296, 16, 1), (256, 4, 297, 16, 1), (256, 4, 185, 16, 2), (256, 4, 186, 16, 2),
+                                              (256, 1, 37, 512, 1), (256, 1, 38, 512, 1), (128, 4, 300, 16, 2), (128, 1, 3, 512, 1)])
+def test_demote_is_the_same_on_both_sides_of_its_kernel_choice(d, hkv, n, page, fmt):
+    """One call of n pages and calls of at most four pages, which at d = 256 take different kernels (1,184 tile records
+    in format 1, 740 in format 2 on 148 SMs): the same bytes for every byte pattern, NaNs and saturated keys included."""
+    rng = np.random.default_rng(n + d)
+    sigma = (rng.integers(0, 2, d) * 2 - 1).astype(np.int8)
+    pool = M.Pool(d, hkv, hkv, n, 2 * n, sigma, page_tokens=page, tq3_format=fmt)
+    size = n * hkv * pool.fp8_rec
+    recs = rng.integers(0, 256, size).astype(np.uint8)                  # about one NaN in 128 bytes
+    recs = recs.reshape(n, hkv, page // 16, 2, 16 * d)
+    recs[1::2] = np.where((recs[1::2] & 0x7F) == 0x7F, 0, recs[1::2])   # every other page without
+    recs[2::4, :, :, 0] = recs[2::4, :, :, 0] & 0xBF                    # keys below 2
+    pool.fp8_arena[:size].copy_(torch.from_numpy(recs.reshape(-1)))
+    ids = torch.arange(n, dtype=torch.int32, device="cuda:0")
+    pool.demote(ids, ids)
+    for at in range(0, n, 4):
+        pool.demote(ids[at:at + 4].contiguous(), ids[at:at + 4] + n)
+    torch.cuda.synchronize()
+    assert pool.status() == M.OK
+    out = pool.tq3_arena[:2 * n * hkv * pool.tq3_rec].view(2, n, hkv, pool.tq3_rec)
+    assert torch.equal(out[0], out[1])
+    if page == 16:
+        with oracle.record_format(fmt):
+            for p in (1, 2, 3, n - 1):
+                if p % 2 or p % 4 == 2 and not (recs[p] & 0x7F == 0x7F).any():
+                    for h in range(hkv):
+                        assert np.array_equal(out[0, p, h].cpu().numpy(), oracle.demote_record(recs[p, h].reshape(-1), d, sigma)), (p, h)

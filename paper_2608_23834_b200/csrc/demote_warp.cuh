@@ -3,9 +3,12 @@
 //
 // The encoder is defined as a sequence of fp32 operations, and the records are those bit for bit; what changes is
 // how the same numbers are reached (per page and head at d = 256, 8,760 -> 3,870 warp instructions):
-//   * The Hadamard transform of an e4m3 vector is exact in fp32 as long as its coordinates are small: they are
-//     multiples of 2^-9, so with |x|^2 < 4096 (checked on the norm that the encoder needs anyway) no sum of
-//     signed coordinates needs more than 20 bits, and every order of summation gives the same value.  H_d is then
+//   * The Hadamard transform of an e4m3 vector is exact in fp32 as long as its coordinates are not huge: they are
+//     multiples of 2^-9, and with |x|^2 < kExactNorm2 = 2^22 (checked on the norm that the encoder needs anyway) a signed
+//     sum of n <= 256 of them is at most sqrt(n) |x| <= 2^15, that is 2^24 units of 2^-9: every partial sum is an integer
+//     that fp32 holds, and every order of summation gives the same value (the sums of 16 inside an MMA are at most
+//     2^22 units of products below 2^18).  Outlier channels of real keys stay far below; beyond are only records
+//     whose coordinates average more than 128 of e4m3's 448.  H_d is then
 //     taken as H_16 on the dims of a 16-dim block, by tensor-core products with a +-512 matrix (32 MMAs), times
 //     butterflies over the blocks, which a lane has all to itself (packed additions, no shuffles; the 16 shuffle
 //     stages per token were a quarter of the instructions).  The factor 512 makes every coordinate an integer, so a
@@ -16,7 +19,7 @@
 //     every quotient either exactly on a half-integer or at least 2^-16 away from one, so an approximate quotient
 //     rounded to 2^-18 decides like the correctly rounded one (checked over all ranges and values, tests): three packed
 //     operations per two tokens instead of two divisions.
-// Records with larger keys or NaNs take the literal sequence (per record for keys, per channel for values).
+// Records with such keys or with NaNs take the literal sequence (per record for keys, per channel for values).
 
 template <int D>
 struct DemoteWarp {
@@ -27,6 +30,7 @@ struct DemoteWarp {
     static_assert(kPage * KST >= kPage * D && OFF_V % 16 == 0 && OFF_META % 16 == 0, "value codes take the place of the keys");
 };
 constexpr int kDemoteWarps = 4;                      // warps per block, one head each
+constexpr float kExactNorm2 = 4194304.0f;
 
 __device__ __forceinline__ uint32_t e4m3x2_to_f16x2_bits(uint32_t two_bytes)
 {
@@ -183,7 +187,7 @@ demote_warp_kernel(const uint8_t* fp8, uint8_t* __restrict__ tq3, int fp8_pages,
                     e0[b] = __fadd_rn(e0[b], e0[b + o]);
                     e1[b] = __fadd_rn(e1[b], e1[b + o]);
                 }
-            if (__all_sync(FULL, e0[0] < 4096.0f && e1[0] < 4096.0f)) {
+            if (__all_sync(FULL, e0[0] < kExactNorm2 && e1[0] < kExactNorm2)) {
                 const float nx[2] = {__fsqrt_rn(e0[0]), __fsqrt_rn(e1[0])};
                 float nt[2][3];             // minus the thresholds, in units of 2^-9, rounded down
 #pragma unroll

@@ -46,7 +46,58 @@ def test_value_code_from_an_approximate_quotient():
             assert np.array_equal(r.view(np.uint32) - np.uint32(0x4B400000), want.astype(np.uint32)), (mn, ulps)
 
 
-def test_transform_sums_of_small_keys_are_exact_in_fp32():
-    """|x|^2 < 4096 with d <= 256 bounds every signed partial sum by sqrt(256 * 4096) = 1024; in units of 2^-9 that is
-    2^19, and the products with +-512 are integers of that size: far inside 24 bits."""
-    assert np.sqrt(256 * 4096.0) * 2 ** 9 <= 2 ** 19
+def _transform_f32(x):
+    """The kernel's order: H_16 on every block of 16 dims, then butterflies over the blocks, all in fp32."""
+    x, d = x.astype(F).copy(), x.shape[-1]
+    for strides in ([1, 2, 4, 8], [16 << i for i in range(d.bit_length() - 5)]):
+        for h in strides:
+            v = x.reshape(*x.shape[:-1], -1, 2, h)
+            x = np.stack([v[..., 0, :] + v[..., 1, :], v[..., 0, :] - v[..., 1, :]], -2).reshape(x.shape)
+            assert x.dtype == F
+    return x
+
+
+def _transform_units(x):
+    """The same in units of 2^-9, exactly."""
+    x, d = np.rint(x * 512.0).astype(np.int64), x.shape[-1]
+    for h in [1 << i for i in range(d.bit_length() - 1)]:
+        v = x.reshape(*x.shape[:-1], -1, 2, h)
+        x = np.stack([v[..., 0, :] + v[..., 1, :], v[..., 0, :] - v[..., 1, :]], -2).reshape(x.shape)
+    return x
+
+
+def _gate():
+    import os
+    import re
+
+    from conftest import ROOT
+    with open(os.path.join(ROOT, "paper_2608_23834_b200", "csrc", "demote_warp.cuh")) as f:
+        return float(re.search(r"kExactNorm2 = ([0-9.]+)f;", f.read()).group(1))
+
+
+def test_transform_is_exact_below_the_norm_gate_and_not_far_above():
+    """Vectors whose squared norm lies just below the kernel's gate, among them those that reach the largest sums: a
+    row of the transform's own signs scaled to the gate (one coordinate of 2^24 units), with the odd last bits that
+    small values bring.  Beyond the gate the fp32 sums do round, which is why there is one."""
+    gate, v, rng = _gate(), _e4m3_values(), np.random.default_rng(1)
+    assert gate == 2.0 ** 22
+    rows = []
+    for d in (128, 256):
+        signs = np.where(rng.random((64, d)) < 0.5, -1.0, 1.0)
+        for top in (96.0, 112.0, 120.0, 128.0, 144.0, 176.0, 448.0):
+            x = top * np.ones((64, d)) * np.where(np.arange(64)[:, None] % 2, signs, 1.0)
+            small = rng.random((64, d)) < rng.uniform(0, 0.5, (64, 1))
+            x = np.where(small, rng.choice(v[np.abs(v) < 0.1], (64, d)), x)
+            x[(x ** 2).sum(-1) >= gate] = 0.0
+            rows.append(x)
+        x = rng.choice(v, (4096, d))
+        rows.append(x[(x ** 2).sum(-1) < gate])
+    largest = 0
+    for x in rows:
+        want = _transform_units(x)
+        assert np.array_equal(_transform_f32(x).astype(np.float64) * 512.0, want.astype(np.float64))
+        largest = max(largest, int(np.abs(want).max()))
+    assert largest > 2 ** 23                                          # the cases do come near the 2^24 of the argument
+    x = np.full((1, 256), 448.0)
+    x[0, 3] = 2.0 ** -9                                               # an odd sum of 26 bits
+    assert not np.array_equal(_transform_f32(x).astype(np.float64) * 512.0, _transform_units(x).astype(np.float64))

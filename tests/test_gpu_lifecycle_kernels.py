@@ -402,3 +402,33 @@ def test_demote_is_the_same_on_both_sides_of_its_kernel_choice(d, hkv, n, page, 
                 if p % 2 or p % 4 == 2 and not (recs[p] & 0x7F == 0x7F).any():
                     for h in range(hkv):
                         assert np.array_equal(out[0, p, h].cpu().numpy(), oracle.demote_record(recs[p, h].reshape(-1), d, sigma)), (p, h)
+
+
+@pytest.mark.parametrize("d,hkv,n,fmt", [(256, 4, 300, 1), (256, 4, 200, 2), (128, 2, 24, 1), (128, 2, 24, 2)])
+def test_demote_of_keys_around_the_exact_transform_bound(d, hkv, n, fmt):
+    """Records whose largest token has a squared norm between 2^8 and beyond 2^22, where the tensor-core transform ends,
+    as single large channels, large tokens or large records: bit-exact with the oracle."""
+    rng = np.random.default_rng(d + n)
+    sigma = (rng.integers(0, 2, d) * 2 - 1).astype(np.int8)
+    pool = M.Pool(d, hkv, hkv, n, n, sigma, tq3_format=fmt)
+    checked = {}
+    for p in range(24):
+        recs = np.zeros((hkv, 32 * d), np.uint8)
+        for h in range(hkv):
+            k, v = rng.standard_normal((2, 16, d)).astype(np.float32)
+            if p % 3 == 0: k[:, 3] *= 2.0 ** (p / 2)
+            elif p % 3 == 1: k[5] = 2.0 ** 11 / np.sqrt(d) * (1 + (p - 12) / 64) * np.sign(k[5])      # |x|^2 around 2^22
+            else: k *= 2.0 ** (p / 2.6)
+            recs[h] = oracle.fp8_pack_record(k, v)
+        pool.page_write_raw(M.FMT_FP8, p, recs)
+        checked[p] = recs
+    pool.fp8_arena[24 * hkv * 32 * d:n * hkv * 32 * d].zero_()
+    ids = torch.arange(n, dtype=torch.int32, device="cuda:0")
+    pool.demote(ids, ids)
+    torch.cuda.synchronize()
+    assert pool.status() == M.OK
+    with oracle.record_format(fmt):
+        for p, recs in checked.items():
+            got = pool.page_read_raw(M.FMT_TQ3, p).reshape(hkv, -1)
+            for h in range(hkv):
+                assert np.array_equal(got[h], oracle.demote_record(recs[h], d, sigma)), (p, h)

@@ -39,9 +39,7 @@ namespace mkv {
 constexpr int kMaxBatch = 1024;      // requests per call
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-// the running maximum is only raised when exceeded by 2^8 (Stale records of 16-token pages, whose probabilities enter the
-// value product up to 2^8 larger: 2^7)
-constexpr float kRescaleSlack = 8.0f, kRescaleSlackStale = 7.0f;
+constexpr float kRescaleSlack = 8.0f;                        // the running maximum is only raised when exceeded by 2^8
 constexpr unsigned long long kDefaultWaitNs = 20000000ull;   // 20 ms: far beyond any copy that is going to arrive
 
 size_t decode_ws_tensor_bytes(int, int, int, int d)
@@ -256,8 +254,12 @@ __device__ __forceinline__ void key_lut4(uint32_t sel, uint32_t& r0, uint32_t& r
 }
 
 // Two 3-bit value codes sitting at bit POS of each 16-bit half of x -> half2 of the integer codes.
-// (x & mask) | 0x6400 is the fp16 number 1024 + code * 2^POS; one FMA recovers the code exactly.  (For operands that
-// have to be the codes themselves; the mma.sync scan uses value_bits.)
+// (x & mask) | 0x6400 is the fp16 number 1024 + code * 2^POS; one FMA recovers the code exactly.
+// (The masked bits alone are the exact operand code * 2^(POS - 24), a subnormal, and save the FMA: 2 x 59,008 tokens in
+// 16 layers 554 -> 592 us with it.  But the tensor core aligns the products of an MMA by the exponents of their factors,
+// and a subnormal has the exponent of the first binade: every bit that a code stands below bit 10 is a bit less of the
+// sum.  Rows of 30,000 equally weighted tokens came out 3 to 4 times as far from the fp64 result, 3e-6 to 5e-6 against
+// 1e-6, with codes at bits 5 to 8, and 100 times with codes left where they are.)
 template <int POS>
 __device__ __forceinline__ uint32_t value_code(uint32_t x)
 {
@@ -269,54 +271,15 @@ __device__ __forceinline__ uint32_t value_code(uint32_t x)
     return hfma2_u32(u, mul, add);
 }
 
-// The same two codes as they stand: bits below 2^11 read as an fp16 number are worth bits * 2^-24 (subnormals, and
-// the first binade above them, are one linear scale), so masking alone gives the exact operand code * 2^(POS - 24).
-// The powers of two are taken out again where they cost nothing or little (see value_operands).  Against value_code
-// this removes one half-rate FMA per two codes.  The tensor core aligns the products of an MMA by the exponents of their
-// factors, and a subnormal has the exponent of the first binade: every bit that a code stands below bit 10 is a bit less of
-// the sum.  Only positions 5 to 8 are used, which costs two or three bits of the 24 and more that a sum has (codes left
-// at positions 1 to 4 lost up to nine, 5e-5 of the result).
-template <int POS>
-__device__ __forceinline__ uint32_t value_bits(uint32_t x)
-{
-    static_assert(POS >= 5 && POS <= 8, "bits below 2^11 are linear; high ones keep the sum's precision");
-    return x & (0x00070007u << POS);
-}
-
-// A operands of the four channel blocks of a word triple, as code * 2^e.  In every row of every block the codes of
-// tokens 0-7 (registers 0, 1) stand two bits higher than those of tokens 8-15 (registers 2, 3), so the
-// probabilities of tokens 8-15 enter the product four times as large.  What is left is one power of two per row,
-// value_unit<row / 8>(), which goes into the row's scale.  Codes that stand low in their word are taken from the
-// word shifted by four (five shifts for sixteen registers).
+// A operands of the four channel blocks of a word triple
 template <int BLOCK>
 __device__ __forceinline__ void value_operands(uint32_t (&a)[4], uint32_t W0, uint32_t W1, uint32_t W2, uint32_t X)
 {
     if constexpr (BLOCK == 0) {          // X = bytes of W0, W1 between the two
-        a[0] = value_bits<8>(W0 << 8); a[1] = value_bits<7>(W0 << 4); a[2] = value_bits<6>(W0); a[3] = value_bits<5>(X << 4);
-    } else if constexpr (BLOCK == 1) {
-        a[0] = value_bits<8>(X << 4); a[1] = value_bits<7>(X); a[2] = value_bits<6>(W1 << 4); a[3] = value_bits<5>(W1);
-    } else if constexpr (BLOCK == 2) {   // X = bytes of W1, W2; its bytes 0 and 2 are bytes 1 and 3 of W1
-        a[0] = value_bits<8>(W1); a[1] = value_bits<7>(X << 4); a[2] = value_bits<6>(X); a[3] = value_bits<5>(W2 << 4);
-    } else {
-        a[0] = value_bits<8>(W2 << 4); a[1] = value_bits<7>(W2); a[2] = value_bits<6>(W2 >> 4); a[3] = value_bits<5>(W2 >> 8);
-    }
-}
-// What a unit of the sums is worth in codes: 2^(24 - POS) of the row's register 0 / 1, the probabilities entering
-// 2^6 (tokens 0-7) and 2^8 times as large: that keeps the units within fp16's powers of two, for half_times, and
-// the products within fp16's range (probabilities are at most 2^kRescaleSlackStale).
-template <int HI>
-__device__ __forceinline__ constexpr float value_unit() { return HI ? 2048.f : 1024.f; }
-
-// The operands of a long page, whose sums stay in the tensor core's accumulators over many tiles: the codes themselves
-// (the rounding of such a run depends on the operands' exponents; see the note at kOpens).
-template <int BLOCK>
-__device__ __forceinline__ void value_operands_plain(uint32_t (&a)[4], uint32_t W0, uint32_t W1, uint32_t W2, uint32_t X)
-{
-    if constexpr (BLOCK == 0) {
         a[0] = value_code<0>(W0); a[1] = value_code<3>(W0); a[2] = value_code<6>(W0); a[3] = value_code<1>(X);
     } else if constexpr (BLOCK == 1) {
         a[0] = value_code<4>(X); a[1] = value_code<7>(X); a[2] = value_code<2>(W1); a[3] = value_code<5>(W1);
-    } else if constexpr (BLOCK == 2) {
+    } else if constexpr (BLOCK == 2) {   // X = bytes of W1, W2
         a[0] = value_code<0>(X); a[1] = value_code<3>(X); a[2] = value_code<6>(X); a[3] = value_code<1>(W2);
     } else {
         const uint32_t X2 = W2 >> 8;
@@ -329,44 +292,15 @@ __device__ __forceinline__ float2 half2_to_float2(uint32_t x)
     return __half22float2(*reinterpret_cast<const __half2*>(&x));
 }
 
-// fp16 bits of a power of two from 1 to 2^15
-__device__ __forceinline__ constexpr uint32_t unit_bits(float x)
-{
-    uint32_t e = 15;
-    for (; x >= 2.f; x *= 0.5f) ++e;
-    return e << 10;
-}
-
-// h * 2^k in fp32, conversion and product in one mixed-precision FMA
-template <uint32_t UNIT>
-__device__ __forceinline__ float half_times(uint16_t h)
-{
-    float r;
-    asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(r) : "h"(h), "h"((uint16_t)UNIT), "f"(0.f));
-    return r;
-}
-
-// acc[channel rows g, g+8][heads] += scale_row * t + zero_row * psum_head, t in units of value_unit<row half>
-// MIXED: half_times instead of a conversion and a product.  (Not in the format-2 scan of more than four heads at
-// d = 256, where the compiler's schedule gets worse: 2 x 59,008 tokens in 16 layers 553 us with it, 540 us without.)
-template <bool MIXED>
+// acc[channel rows g, g+8][heads] += scale_row * t + zero_row * psum_head
 __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (&t)[4], uint32_t sc_pair, uint32_t zp_pair,
                                                   float ps0, float ps1)
 {
-    const float2 zp = half2_to_float2(zp_pair);
-    float s0, s1;                            // exact either way
-    if constexpr (MIXED) {
-        s0 = half_times<unit_bits(value_unit<0>())>((uint16_t)sc_pair);
-        s1 = half_times<unit_bits(value_unit<1>())>((uint16_t)(sc_pair >> 16));
-    } else {
-        const float2 sc = half2_to_float2(sc_pair);
-        s0 = sc.x * value_unit<0>();
-        s1 = sc.y * value_unit<1>();
-    }
-    acc[0] = fmaf(s0, t[0], fmaf(zp.x, ps0, acc[0]));
-    acc[1] = fmaf(s0, t[1], fmaf(zp.x, ps1, acc[1]));
-    acc[2] = fmaf(s1, t[2], fmaf(zp.y, ps0, acc[2]));
-    acc[3] = fmaf(s1, t[3], fmaf(zp.y, ps1, acc[3]));
+    const float2 sc = half2_to_float2(sc_pair), zp = half2_to_float2(zp_pair);
+    acc[0] = fmaf(sc.x, t[0], fmaf(zp.x, ps0, acc[0]));
+    acc[1] = fmaf(sc.x, t[1], fmaf(zp.x, ps1, acc[1]));
+    acc[2] = fmaf(sc.y, t[2], fmaf(zp.y, ps0, acc[2]));
+    acc[3] = fmaf(sc.y, t[3], fmaf(zp.y, ps1, acc[3]));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -597,20 +531,19 @@ struct PFrag {
 };
 
 // First half: raise the running maximum (and rescale the accumulators) if the page asks for it.
-template <int NB, bool TILED = false, bool STALE = false>
+template <int NB, bool TILED = false>
 __device__ __forceinline__ void softmax_rescale(WarpAcc<NB>& acc, const float (&s)[4])
 {
-    constexpr float SLACK = STALE && !TILED ? kRescaleSlackStale : kRescaleSlack;
     constexpr uint32_t FULL = 0xffffffffu;
     float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
     // the page maximum is only needed when some score exceeds the running maximum by more than the slack
-    if (__any_sync(FULL, mx0 > acc.m[0] + SLACK || mx1 > acc.m[1] + SLACK)) {
+    if (__any_sync(FULL, mx0 > acc.m[0] + kRescaleSlack || mx1 > acc.m[1] + kRescaleSlack)) {
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) {
             mx0 = fmaxf(mx0, __shfl_xor_sync(FULL, mx0, o));
             mx1 = fmaxf(mx1, __shfl_xor_sync(FULL, mx1, o));
         }
-        const bool up0 = mx0 > acc.m[0] + SLACK, up1 = mx1 > acc.m[1] + SLACK;
+        const bool up0 = mx0 > acc.m[0] + kRescaleSlack, up1 = mx1 > acc.m[1] + kRescaleSlack;
         const float f0 = up0 ? fast_exp2(acc.m[0] - mx0) : 1.f, f1 = up1 ? fast_exp2(acc.m[1] - mx1) : 1.f;
         if (up0) acc.m[0] = mx0;
         if (up1) acc.m[1] = mx1;
@@ -629,14 +562,11 @@ __device__ __forceinline__ void softmax_rescale(WarpAcc<NB>& acc, const float (&
 }
 
 // Second half, branch-free (so that it can be scheduled into the unpack work of the next page): P and its row sums.
-// STALE (Stale records of 16-token pages): the operands are 2^6 (second token half: 2^8) times the probabilities (value_operands, value_unit); the row
-// sums take the factors out again.
-template <int NB, bool STALE, bool SPLIT>
+template <int NB, bool SPLIT>
 __device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
-    const float up = STALE ? 6.f : 0.f, up2 = STALE ? 8.f : 0.f;
-    const float p0 = fast_exp2(s[0] - (acc.m[0] - up)), p1 = fast_exp2(s[1] - (acc.m[1] - up));
-    const float p2 = fast_exp2(s[2] - (acc.m[0] - up2)), p3 = fast_exp2(s[3] - (acc.m[1] - up2));
+    const float p0 = fast_exp2(s[0] - acc.m[0]), p1 = fast_exp2(s[1] - acc.m[1]);
+    const float p2 = fast_exp2(s[2] - acc.m[0]), p3 = fast_exp2(s[3] - acc.m[1]);
     const uint32_t ph01 = pack_f16x2(p0, p1), ph23 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(ph01), h23 = half2_to_float2(ph23);
     const uint32_t pl01 = pack_f16x2(p0 - h01.x, p1 - h01.y), pl23 = pack_f16x2(p2 - h23.x, p3 - h23.y);
@@ -650,7 +580,7 @@ __device__ __forceinline__ void softmax_probs(WarpAcc<NB>& acc, const float (&s)
         pf.c1 = movmatrix_trans(pl23);
     }
     // row sums through the tensor core: the same P that multiplies V
-    const uint32_t ones[4] = {STALE ? 0x24002400u : 0x3C003C00u, STALE ? 0x24002400u : 0x3C003C00u, STALE ? 0x1C001C00u : 0x3C003C00u, STALE ? 0x1C001C00u : 0x3C003C00u};
+    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
     if constexpr (!SPLIT) mma16816(ps, ones, pf.c0, pf.c1);
@@ -664,7 +594,7 @@ template <int NB, bool SPLIT>
 __device__ __forceinline__ void softmax_page(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
     softmax_rescale<NB>(acc, s);
-    softmax_probs<NB, false, SPLIT>(acc, s, pf, lane);
+    softmax_probs<NB, SPLIT>(acc, s, pf, lane);
 }
 
 // Scored variant (Section 3.1): log2 of the page's exponential sum, referred to an absolute origin
@@ -755,7 +685,7 @@ __device__ __forceinline__ void tq3_key_quad(float (&S0)[4], float (&S1)[4], uin
 // Output update of the four channel blocks 4j..4j+3 of a Stale page: integer codes through the tensor
 // core, then the fp16 scale and zero of every channel applied to the 16x8 result in fp32.
 // DEFER (long pages): sum p * code only, the accumulators are in code units until the page is left.
-template <bool DEFER, bool SPLIT, bool MIXED>
+template <bool DEFER, bool SPLIT>
 __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], float (&o2)[4], float (&o3)[4],
                                                uint32_t W0, uint32_t W1, uint32_t W2, uint32_t meta_quad, const PFrag& pf)
 {
@@ -770,26 +700,22 @@ __device__ __forceinline__ void tq3_value_quad(float (&o0)[4], float (&o1)[4], f
     {   // blocks 4j, 4j+1
         if constexpr (!DEFER) mt = lds128(meta_quad);
         const uint32_t X = prmt(W0, W1, 0x6341u);
-        if constexpr (DEFER) value_operands_plain<0>(a, W0, W1, W2, X);
-        else value_operands<0>(a, W0, W1, W2, X);
+        value_operands<0>(a, W0, W1, W2, X);
         product(DEFER ? o0 : t);
-        if constexpr (!DEFER) affine_accumulate<MIXED>(o0, t, mt.x, mt.y, pf.ps0, pf.ps1);
-        if constexpr (DEFER) value_operands_plain<1>(a, W0, W1, W2, X);
-        else value_operands<1>(a, W0, W1, W2, X);
+        if constexpr (!DEFER) affine_accumulate(o0, t, mt.x, mt.y, pf.ps0, pf.ps1);
+        value_operands<1>(a, W0, W1, W2, X);
         product(DEFER ? o1 : t);
-        if constexpr (!DEFER) affine_accumulate<MIXED>(o1, t, mt.z, mt.w, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) affine_accumulate(o1, t, mt.z, mt.w, pf.ps0, pf.ps1);
     }
     {   // blocks 4j+2, 4j+3
         if constexpr (!DEFER) mt = lds128(meta_quad + 128);
         const uint32_t X = prmt(W1, W2, 0x6341u);
-        if constexpr (DEFER) value_operands_plain<2>(a, W0, W1, W2, X);
-        else value_operands<2>(a, W0, W1, W2, X);
+        value_operands<2>(a, W0, W1, W2, X);
         product(DEFER ? o2 : t);
-        if constexpr (!DEFER) affine_accumulate<MIXED>(o2, t, mt.x, mt.y, pf.ps0, pf.ps1);
-        if constexpr (DEFER) value_operands_plain<3>(a, W0, W1, W2, X);
-        else value_operands<3>(a, W0, W1, W2, X);
+        if constexpr (!DEFER) affine_accumulate(o2, t, mt.x, mt.y, pf.ps0, pf.ps1);
+        value_operands<3>(a, W0, W1, W2, X);
         product(DEFER ? o3 : t);
-        if constexpr (!DEFER) affine_accumulate<MIXED>(o3, t, mt.z, mt.w, pf.ps0, pf.ps1);
+        if constexpr (!DEFER) affine_accumulate(o3, t, mt.z, mt.w, pf.ps0, pf.ps1);
     }
 }
 
@@ -881,10 +807,10 @@ __device__ __forceinline__ void softmax_rescale_v2(WarpAcc<NB>& acc, const float
 {
     constexpr uint32_t FULL = 0xffffffffu;
     float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
-    if (__any_sync(FULL, mx > acc.mr + kRescaleSlackStale)) {
+    if (__any_sync(FULL, mx > acc.mr + kRescaleSlack)) {
         mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, 2));
-        const bool up = mx > acc.mr + kRescaleSlackStale;
+        const bool up = mx > acc.mr + kRescaleSlack;
         const float f = up ? fast_exp2(acc.mr - mx) : 1.f;
         if (up) acc.mr = mx;
         const int tq = lane & 3;
@@ -905,13 +831,12 @@ __device__ __forceinline__ void softmax_rescale_v2(WarpAcc<NB>& acc, const float
     }
 }
 
-// P of head g for the lane's four tokens is the B fragment of the value product as it stands (tokens 8-15 four
-// times as large, see value_operands).
+// P of head g for the lane's four tokens is the B fragment of the value product as it stands.
 template <int NB>
 __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (&s)[4], PFrag& pf, int lane)
 {
-    const float p0 = fast_exp2(s[0] - (acc.mr - 6.f)), p1 = fast_exp2(s[1] - (acc.mr - 6.f));
-    const float p2 = fast_exp2(s[2] - (acc.mr - 8.f)), p3 = fast_exp2(s[3] - (acc.mr - 8.f));
+    const float p0 = fast_exp2(s[0] - acc.mr), p1 = fast_exp2(s[1] - acc.mr);
+    const float p2 = fast_exp2(s[2] - acc.mr), p3 = fast_exp2(s[3] - acc.mr);
     pf.b0 = pack_f16x2(p0, p1);
     pf.b1 = pack_f16x2(p2, p3);
     const float2 h01 = half2_to_float2(pf.b0), h23 = half2_to_float2(pf.b1);
@@ -919,7 +844,7 @@ __device__ __forceinline__ void softmax_probs_v2(WarpAcc<NB>& acc, const float (
     pf.c1 = pack_f16x2(p2 - h23.x, p3 - h23.y);
     pf.b0 = lane & 16 ? pf.c0 : pf.b0;       // rows 4-7 carry the low halves of heads 0-3
     pf.b1 = lane & 16 ? pf.c1 : pf.b1;
-    const uint32_t ones[4] = {0x24002400u, 0x24002400u, 0x1C001C00u, 0x1C001C00u};
+    const uint32_t ones[4] = {0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u};
     float ps[4];
     mma16816_zero(ps, ones, pf.b0, pf.b1);
     pf.ps0 = ps[0];
@@ -945,7 +870,7 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
     if constexpr (DO_V) load_lane_words<D>(rec_v + 6 * D, lane, vw);
     if constexpr (DO_V) {      // in one block with the key unpack of the next page
         if constexpr (FMT == 2 && SPLIT) softmax_probs_v2<NB>(acc, s_cur, pf, lane);
-        else softmax_probs<NB, !DEFER, SPLIT>(acc, s_cur, pf, lane);
+        else softmax_probs<NB, SPLIT>(acc, s_cur, pf, lane);
     }
     if constexpr (DO_V && DEFER) {
         acc.lp[0] += pf.ps0;
@@ -963,8 +888,8 @@ __device__ __forceinline__ void tq3_step(WarpAcc<D / 16>& acc, uint32_t rec_v, c
             else tq3_key_quad<SPLIT>(S0, S1, kw[3 * j], kw[3 * j + 1], kw[3 * j + 2], qt_lane + j * (SPLIT ? 1024 : 2048));
         }
         if constexpr (DO_V)
-            tq3_value_quad<DEFER, SPLIT, !(D == 256 && FMT == 2 && !SPLIT)>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
-                                  vw[3 * j + 2], meta + j * 256, pf);
+            tq3_value_quad<DEFER, SPLIT>(acc.o[4 * j], acc.o[4 * j + 1], acc.o[4 * j + 2], acc.o[4 * j + 3], vw[3 * j], vw[3 * j + 1],
+                                         vw[3 * j + 2], meta + j * 256, pf);
     }
     if constexpr (DO_K && FMT == 2 && SPLIT) {
         // head g % 4, tokens 2tq, 2tq+1 (I0) and 2tq+8, 2tq+9 (I1): the three query digits, then the token's norm
@@ -1688,7 +1613,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     const uint32_t cur = (uint32_t)i % NSTAGE, nxt = (uint32_t)(i + 1) % NSTAGE;
                     if ((i & 1) && !wait_slot(nxt / 2)) break;       // the next page opens a slot pair
                     if constexpr (FMT == 2 && SPLIT) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
-                    else softmax_rescale<NB, TILED, true>(acc, s_cur);
+                    else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
                         const int pg_i = list3[i];
                         if (pg_i != cur_page || (FLAT && i > 0 && (lpg3[i] & kOpens))) {
@@ -1707,7 +1632,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 if (!failed) {
                     if (n8 > 0) issue_fp8(0);
                     if constexpr (FMT == 2 && SPLIT) softmax_rescale_v2<NB, TILED>(acc, s_cur, lane);
-                    else softmax_rescale<NB, TILED, true>(acc, s_cur);
+                    else softmax_rescale<NB, TILED>(acc, s_cur);
                     if constexpr (TILED) {
                         const int pg_i = list3[n3 - 1];
                         if (pg_i != cur_page || (FLAT && n3 > 1 && (lpg3[n3 - 1] & kOpens))) {

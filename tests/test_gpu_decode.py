@@ -257,3 +257,19 @@ def test_a_batch_of_empty_requests_only(d, page):
         for out, lse in zip(outs[:3 + n], lses[:3 + n]):
             assert not out.any() and bool(torch.isneginf(lse).all())
     assert not mass.any() and all(p.status() == M.OK for p in pools)
+
+
+@pytest.mark.parametrize("fmt", [1, 2])
+@pytest.mark.parametrize("group", [4, 8])
+def test_long_flat_rows_keep_the_precision_of_the_sums(fmt, group):
+    """Rows of 30,000 tokens with about equal weights: the output is some hundredth of a value's size, so a bias of the
+    products of codes and probabilities shows enlarged.  fp32 sums of products that lose nothing below 2^-24 give
+    0.6e-6 to 1.6e-6 of the output here (four sources of 2^-24 = 6e-8 that grow with the square root of the enlargement,
+    about 100); operands that cost the products two or three bits gave 3e-6 to 5e-6."""
+    with oracle.record_format(fmt):
+        case = Case(W.config(1, seq_lens=(30000, 29899), head_dim=128, n_kv_heads=2, group=group, anchor_prefix=0,
+                             recent_tokens=64, anchor_spans=0))
+        out, _ = case.run(M.DECODE_TENSOR)
+        ref, _ = case.reference()
+    rel = np.linalg.norm(out - ref) / np.linalg.norm(ref)
+    assert rel < 2.2e-6, rel

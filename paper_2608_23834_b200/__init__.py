@@ -72,7 +72,7 @@ class LayerAppend(C.Structure):
 
 def lib():
     """Load libmkv.so; fails loudly if it has not been built (python paper_2608_23834_b200/build.py)."""
-    global _lib, _native
+    global _lib
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise ImportError(f"{_LIB_PATH} is missing: build it with `python -m paper_2608_23834_b200.build` "
@@ -127,10 +127,18 @@ def lib():
             fn.restype = C.c_int32
         L.mkv_last_cuda_error.restype = C.c_char_p
         L.mkv_last_cuda_error.argtypes = []
-        from . import _mkv_native
-        _native = _mkv_native
         _lib = L
     return _lib
+
+
+def native():
+    """The C++ binding of the calls on device pools (built with libmkv.so, tied to this PyTorch); fails loudly where it
+    is missing or does not load.  Host-only pools do without it."""
+    global _native
+    if _native is None:
+        from . import _mkv_native
+        _native = _mkv_native
+    return _native
 
 
 def _check(rc: int, where: str):
@@ -203,7 +211,7 @@ class Pool:
             _check(L.mkv_pool_create(C.byref(self.cfg), _ptr(self.fp8_arena), _ptr(self.tq3_arena), _stream(None),
                                      C.byref(h)), "mkv_pool_create")
             self.handle = h
-            self._ref = _native.pool_ref(h.value, n_kv_heads, n_q_heads, head_dim)     # what the native calls need of the pool
+            self._ref = native().pool_ref(h.value, n_kv_heads, n_q_heads, head_dim)     # what the native calls need of the pool
             _check(L.mkv_workspace_init(_ptr(self.workspace), self.ws_bytes, _stream(None)), "mkv_workspace_init")
 
     def close(self):
@@ -346,7 +354,7 @@ class Pool:
 def decode_attention_layers(pools, qs, block_tables, tier_tags, seq_lens, scale, outs, lses=None, stream=None):
     """mkv_decode_attention_layers: the decode attention of len(pools) layers in one launch; layer i reads
     pools[i], qs[i], block_tables[i], tier_tags[i] and writes outs[i] (and lses[i]); seq_lens is common."""
-    if _lib is not None and _native_rc(_native.decode_layers(pools, qs, block_tables, tier_tags, seq_lens, scale, outs, lses,
+    if _native is not None and _native_rc(_native.decode_layers(pools, qs, block_tables, tier_tags, seq_lens, scale, outs, lses,
                                                              stream), "mkv_decode_attention_layers"):
         return outs
     n = len(pools)
@@ -369,7 +377,7 @@ def decode_attention_layers(pools, qs, block_tables, tier_tags, seq_lens, scale,
 
 def append_layers(pools, ks, vs, slot_mapping, stream=None):
     """mkv_append_layers: Append of the same token positions into the pools of several layers in one launch."""
-    if _lib is not None and _native_rc(_native.append_layers(pools, ks, vs, slot_mapping, stream), "mkv_append_layers"):
+    if _native is not None and _native_rc(_native.append_layers(pools, ks, vs, slot_mapping, stream), "mkv_append_layers"):
         return
     n = len(pools)
     calls = (LayerAppend * n)()
@@ -385,8 +393,7 @@ def append_layers(pools, ks, vs, slot_mapping, stream=None):
 def page_score_update(page_mass, seq_lens, head_mask, beta, score, stream=None, page_tokens=16):
     """mkv_page_score_update[_paged] (Eq. attention-score): score <- beta * score + (1 - beta) * mean over the
     heads in head_mask of page_mass, in place, for the pages below each request's length."""
-    lib()
-    if _native_rc(_native.score_update(page_mass, seq_lens, int(head_mask), beta, score, stream, page_tokens),
+    if _native is not None and _native_rc(_native.score_update(page_mass, seq_lens, int(head_mask), beta, score, stream, page_tokens),
                   "mkv_page_score_update"):
         return score
     B, hq, max_pages = page_mass.shape

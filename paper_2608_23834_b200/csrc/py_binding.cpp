@@ -211,14 +211,13 @@ struct Items {
     PyObject* operator[](Py_ssize_t i) const { return PySequence_Fast_GET_ITEM(fast, i); }
 };
 
-// an attribute of a Pool; the Pool keeps the object alive
-PyObject* attr(PyObject* o, PyObject* name)
-{
-    PyObject* v = PyObject_GetAttr(o, name);
-    if (!v) PyErr_Clear();
-    Py_XDECREF(v);
-    return v;
-}
+// an attribute of a Pool, held while it is looked at (it may be a property that makes a new object)
+struct Attr {
+    PyObject* o;
+    Attr(PyObject* of, PyObject* name) : o(PyObject_GetAttr(of, name)) { if (!o) PyErr_Clear(); }
+    Attr(const Attr&) = delete;
+    ~Attr() { Py_XDECREF(o); }
+};
 
 // decode_layers(pools, qs, block_tables, tier_tags, seq_lens, scale, outs, lses, stream)
 PyObject* decode_layers(PyObject*, PyObject* const* a, Py_ssize_t n)
@@ -242,18 +241,18 @@ PyObject* decode_layers(PyObject*, PyObject* const* a, Py_ssize_t n)
     int64_t B = 0, width = 0;
     size_t ws_bytes = 0;
     for (Py_ssize_t i = 0; i < L; ++i) {
-        PyObject* ref = attr(pools[i], s_ref);
-        const PoolRef* r = ref ? ref_of(ref) : nullptr;
-        const at::Tensor *ws = tensor(attr(pools[i], s_workspace)), *q = tensor(qs[i]), *bt = tensor(bts[i]), *tg = tensor(tags[i]),
+        const Attr ref(pools[i], s_ref), workspace(pools[i], s_workspace);
+        const PoolRef* r = ref.o ? ref_of(ref.o) : nullptr;
+        const at::Tensor *ws = tensor(workspace.o), *q = tensor(qs[i]), *bt = tensor(bts[i]), *tg = tensor(tags[i]),
                          *out = tensor(outs[i]);
         if (!r || !ws || !is_dense(q, at::kBFloat16) || q->dim() != 3 || !is_dense(bt, at::kInt) || bt->dim() != 2)
             return result(kCheck);
         if (i == 0) {
             B = q->size(0);
             width = bt->size(1);
-            PyObject* nb = attr(pools[0], s_ws_bytes);
-            if (!nb) return result(kCheck);
-            ws_bytes = PyLong_AsSize_t(nb);
+            const Attr nb(pools[0], s_ws_bytes);
+            if (!nb.o) return result(kCheck);
+            ws_bytes = PyLong_AsSize_t(nb.o);
             if (PyErr_Occurred()) {
                 PyErr_Clear();
                 return result(kCheck);
@@ -287,8 +286,8 @@ PyObject* append_layers(PyObject*, PyObject* const* a, Py_ssize_t n)
     mkv_layer_append calls[MKV_MAX_LAYERS_PER_CALL];
     const int64_t tokens = slots->numel();
     for (Py_ssize_t i = 0; i < L; ++i) {
-        PyObject* ref = attr(pools[i], s_ref);
-        const PoolRef* r = ref ? ref_of(ref) : nullptr;
+        const Attr ref(pools[i], s_ref);
+        const PoolRef* r = ref.o ? ref_of(ref.o) : nullptr;
         const at::Tensor *k = tensor(ks[i]), *v = tensor(vs[i]);
         if (!r || !is_dense(k, at::kBFloat16) || !is_dense(v, at::kBFloat16) || !shape3(k, tokens, r->hkv, r->d) ||
             !v->sizes().equals(k->sizes()))

@@ -180,3 +180,15 @@ def test_sequence_bookkeeping_agrees_with_the_lifecycle_model_on_a_random_walk(p
         assert (st.fp8_pages_used, st.tq3_pages_used) == (used[0], used[1])
         model.check_invariants()
     hp.close()
+
+
+def test_host_only_pools_do_without_the_device_binding():
+    """The C++ binding of the device calls is tied to one PyTorch; the host bookkeeping needs libmkv.so alone."""
+    import subprocess
+    import sys
+    code = ("import sys; sys.modules['paper_2608_23834_b200._mkv_native'] = None\n"
+            "import paper_2608_23834_b200 as M\n"
+            "p = M.HostPool(128, 2, 8, 4, 4)\n"
+            "assert p.page_alloc(M.FMT_FP8, 2) is not None\n"
+            "p.close()\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)

@@ -466,7 +466,7 @@ struct Geo {
     static constexpr int FP8_HALF = 16 * D;
     static constexpr int SLOT = (TQ3_REC + 127) / 128 * 128;
     // pages of one warp whose table entries are compacted at a time (fewer where the ring leaves little room)
-    static constexpr int ROUND = (NW * NSTAGE * SLOT > 190000 || SHORT_ROUNDS) ? 64 : 128;
+    static constexpr int ROUND = SHORT_ROUNDS ? 64 : 128;
     // The ring is used in pairs of slots with one barrier each: a pair holds two Stale records, or the keys and values of one
     // FP8 page, asked for together and waited for once.
     static constexpr int NP = NSTAGE / 2, PAIR = 2 * SLOT;
@@ -1134,7 +1134,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     // 16-byte loads that a thread of the merge keeps in flight, within the registers of the launch shape
     constexpr int MERGE_LOADS = NW * MINB <= 8 ? 40 : NW * MINB <= 12 ? 24 : 16;
     using G = Geo<D, NW, NSTAGE, TILED>;     // pages of several tiles: short rounds leave room for the parked rows
-    constexpr int NB = G::NB, NBH = NB, NU = NW;
+    constexpr int NB = G::NB;
     constexpr uint32_t FULL = 0xffffffffu;
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
@@ -1147,7 +1147,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     float* red = reinterpret_cast<float*>(smem);            // [NW][D][8] over the ring, between segments
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
-    const int unit = warp, hf = 0;
     const int hkv = P0.hkv, GQ = P0.group, hq = hkv * GQ;
     const int n_layers = MAXL == 1 ? 1 : LS.n;
     // a length beyond the table row is cut to the row (and flagged), so that no entry past it is ever read
@@ -1670,7 +1669,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 start_round();
             }
         }
-        float (&oacc)[NBH][4] = acc.o;
+        float (&oacc)[NB][4] = acc.o;
         float (&lacc)[2] = acc.l;
         float (&m_run)[2] = acc.m;
 
@@ -1678,30 +1677,30 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         if (failed && drain()) last_s[1] = 1;      // a copy never arrived at all: the block must not touch the ring
         __syncthreads();
         if (last_s[1]) return;                     // (the call has failed; its workspace needs mkv_workspace_init again)
-        if (g == 0 && hf == 0) {           // both warps of a unit hold the same maximum and row sums
-            sm_m[unit * 8 + 2 * tq] = m_run[0];
-            sm_m[unit * 8 + 2 * tq + 1] = m_run[1];
+        if (g == 0) {
+            sm_m[warp * 8 + 2 * tq] = m_run[0];
+            sm_m[warp * 8 + 2 * tq + 1] = m_run[1];
         }
         __syncthreads();
         float M0 = -CUDART_INF_F, M1 = -CUDART_INF_F;
 #pragma unroll
-        for (int w = 0; w < NU; ++w) {
+        for (int w = 0; w < NW; ++w) {
             M0 = fmaxf(M0, sm_m[w * 8 + 2 * tq]);
             M1 = fmaxf(M1, sm_m[w * 8 + 2 * tq + 1]);
         }
         {
             const float f0 = m_run[0] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[0] - M0);
             const float f1 = m_run[1] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[1] - M1);
-            float* mine = red + (size_t)unit * D * 8 + (size_t)hf * NBH * 16 * 8;   // this warp's channel blocks
+            float* mine = red + (size_t)warp * D * 8;
 #pragma unroll
-            for (int i = 0; i < NBH; ++i) {
+            for (int i = 0; i < NB; ++i) {
                 // element (channel 16i + g + 8*(e>>1), head 2tq + (e&1)) at [channel][8 heads]
                 *reinterpret_cast<float2*>(mine + (16 * i + g) * 8 + 2 * tq) = make_float2(oacc[i][0] * f0, oacc[i][1] * f1);
                 *reinterpret_cast<float2*>(mine + (16 * i + g + 8) * 8 + 2 * tq) = make_float2(oacc[i][2] * f0, oacc[i][3] * f1);
             }
-            if (g == 0 && hf == 0) {
-                sm_l[unit * 8 + 2 * tq] = lacc[0] * f0;
-                sm_l[unit * 8 + 2 * tq + 1] = lacc[1] * f1;
+            if (g == 0) {
+                sm_l[warp * 8 + 2 * tq] = lacc[0] * f0;
+                sm_l[warp * 8 + 2 * tq + 1] = lacc[1] * f1;
             }
         }
         __syncthreads();
@@ -1713,7 +1712,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 if (head >= GQ) continue;
                 float acc = 0.f, l = 0.f;
 #pragma unroll
-                for (int w = 0; w < NU; ++w) {
+                for (int w = 0; w < NW; ++w) {
                     acc += red[(size_t)w * D * 8 + e];
                     l += sm_l[w * 8 + head];
                     if constexpr (SPLIT) {
@@ -1725,7 +1724,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             }
             if (P.lse && tid < GQ) {
                 float l = 0.f, M = -CUDART_INF_F;
-                for (int w = 0; w < NU; ++w) {
+                for (int w = 0; w < NW; ++w) {
                     l += sm_l[w * 8 + tid];
                     if constexpr (SPLIT) l += sm_l[w * 8 + tid + 4];
                     M = fmaxf(M, sm_m[w * 8 + tid]);
@@ -1739,7 +1738,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             for (int e = tid; e < 8 * D; e += NW * 32) {
                 float acc = 0.f;
 #pragma unroll
-                for (int w = 0; w < NU; ++w) {
+                for (int w = 0; w < NW; ++w) {
                     acc += red[(size_t)w * D * 8 + e];
                     if constexpr (SPLIT) acc += (e & 4) ? 0.f : red[(size_t)w * D * 8 + e + 4];
                 }
@@ -1747,7 +1746,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             }
             if (tid < 8) {
                 float l = 0.f, M = -CUDART_INF_F;
-                for (int w = 0; w < NU; ++w) {
+                for (int w = 0; w < NW; ++w) {
                     l += sm_l[w * 8 + tid];
                     if constexpr (SPLIT) l += tid < 4 ? sm_l[w * 8 + tid + 4] : 0.f;
                     M = fmaxf(M, sm_m[w * 8 + tid]);
@@ -1884,18 +1883,20 @@ static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_
     return MKV_OK;
 }
 
-// the pool's record format selects the instantiation
-template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false, int MAXL = 1, bool FLAT = false>
+// The pool's record format selects the instantiation, and for 16-token pages its group: groups of at most four query
+// heads use two column halves (see PFrag).  Not for long pages: their code sums stay in the tensor core's accumulators
+// over many tiles, and the split changes their rounding there.  GROUPS: which groups the caller sends here.
+enum Groups { kAnyGroup, kUpToFour, kMoreThanFour };
+template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false, int MAXL = 1, bool FLAT = false, Groups GROUPS = kAnyGroup>
 static int32_t run_tensor(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_t s)
 {
-    // groups of at most four query heads: two column halves (see PFrag).  Not for long pages: their code sums stay in
-    // the tensor core's accumulators over many tiles, and the split changes their rounding there.
-    if constexpr (!TILED)
-        if (p->group <= 4)
+    if constexpr (!TILED && GROUPS != kMoreThanFour)
+        if (GROUPS == kUpToFour || p->group <= 4)
             return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, true>(p, ls, s)
                                : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, true>(p, ls, s);
-    return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, false>(p, ls, s)
-                       : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, false>(p, ls, s);
+    if constexpr (GROUPS != kUpToFour)
+        return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, false>(p, ls, s)
+                           : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, false>(p, ls, s);
 }
 
 template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false>
@@ -2055,19 +2056,19 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
     // Two blocks of half the warps per SM: one's set-up, reduction and merge overlap the other's pages (16 layers x 2 x
     // 59,008 tokens, d 256: 540 -> 510 us; x 4 x 700..3,001: 86 -> 77 us).  Not at d = 128 with more than four query heads
-    // per KV head, whose scan spills in this shape (16 layers x 4 x 16,000 tokens, 1 head: 56 -> 60 us), and not at d = 256 with
-    // few rows, whose partials four warps take longer to merge (16 layers x 1 x 4,000 tokens: 48.6 -> 51 us).
+    // per KV head (16 layers x 4 x 16,000 tokens, 1 head: 56 -> 60 us; both shapes spill alike there), and not at d = 256 with
+    // few rows, whose partials four warps take longer to merge (64 rows, 16 layers x 1 x 4,000 tokens: 48.6 -> 51 us; the
+    // 128 rows above gain, and the line was set between the two).
     if (n_layers >= kMinFlatLayers)
-        return p0->d == 128 ? (p0->group > 4 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
-                                             : run_tensor<128, 8, 4, 2, false, false, kMaxLayers, true>(p0, ls, s))
+        return p0->d == 128 ? (p0->group > 4 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true, kMoreThanFour>(p0, ls, s)
+                                             : run_tensor<128, 8, 4, 2, false, false, kMaxLayers, true, kUpToFour>(p0, ls, s))
                             : (n_layers * B * p0->hkv < kRowsOfTwoBlocks
                                    ? run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
                                    : run_tensor<256, 4, 4, 2, false, false, kMaxLayers, true>(p0, ls, s));
-    if (two_blocks(p0, B, kMaxCtas))     // as a call of one layer (the results are the same bits)
-        return p0->d == 128 ? run_tensor<128, 8, 4, 2, false, false, kMaxLayers>(p0, ls, s)
-                            : run_tensor<256, 4, 4, 2, false, false, kMaxLayers>(p0, ls, s);
-    return p0->d == 128 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers>(p0, ls, s)
-                        : run_tensor<256, 8, 4, 1, false, false, kMaxLayers>(p0, ls, s);
+    // as a call of one layer (the results are the same bits); a workspace has room for two blocks per SM
+    if (p0->d == 128) return run_tensor<128, 8, 4, 2, false, false, kMaxLayers>(p0, ls, s);
+    return two_blocks(p0, B, kMaxCtas) ? run_tensor<256, 4, 4, 2, false, false, kMaxLayers>(p0, ls, s)
+                                       : run_tensor<256, 8, 4, 1, false, false, kMaxLayers>(p0, ls, s);
 }
 
 int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, const uint8_t* tags,
@@ -2095,10 +2096,9 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
             MKV_CUDA(launch_pdl(page_mass_clear_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, 1, true, s, mass, n));
             rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true, true>(p, prm, s);
         } else {
-            if (two_blocks(p, B, max_blocks))
-                rc = p->d == 128 ? run_tensor1<128, 8, 4, 2, true>(p, prm, s) : run_tensor1<256, 4, 4, 2, true>(p, prm, s);
-            else
-                rc = p->d == 128 ? run_tensor1<128, 16, 4, 1, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);
+            // (always with a caller's workspace, which has room for two blocks per SM)
+            if (p->d == 128) rc = run_tensor1<128, 8, 4, 2, true>(p, prm, s);
+            else rc = two_blocks(p, B, max_blocks) ? run_tensor1<256, 4, 4, 2, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true>(p, prm, s);
         }
         if (rc != MKV_OK) return rc;
         return launch_page_mass_finish(mass, lse, lens, B, p->hkv * p->group, max_pages, p->cfg.page_size, s);

@@ -86,8 +86,8 @@ __device__ __forceinline__ uint2 bf16x8_to_e4m3x8(uint4 in, float inv_scale)
 // such a run may reach up to 15 tokens into the next window.  A chunk of a request that starts anywhere inside a
 // page therefore still meets whole tiles, one per window.  A run that fills its tile leaves as whole rows: K with
 // 8-byte stores, V transposed through shared memory so that every channel's 16 tokens are one 16-byte store (HBM
-// bound: 6.3 of 6.55 TB/s).  Other runs (the ends of a request's chunk, scattered or skipped tokens) are stored
-// token by token.  (With windows cut at fixed tokens a chunk that starts inside a page had no whole tile at all
+// bound: 0.97 of the copy bandwidth on 196,608 tokens, 0.81 on 32,845 in five chunks).  Other runs (the ends of a
+// request's chunk, scattered or skipped tokens) are stored token by token.  (With windows cut at fixed tokens a chunk that starts inside a page had no whole tile at all
 // and every token took the second path: 147 us for 32,845 tokens in five chunks, d = 256.)
 template <int D>
 __global__ void __launch_bounds__(128) append_run_kernel(uint8_t* __restrict__ fp8, int fp8_pages, int hkv, int tiles,
@@ -299,9 +299,9 @@ __device__ __forceinline__ void cluster_barrier()
 // page go to the blocks of a cluster, the largest divisor of the head count that a portable cluster
 // allows.  A call that fills the GPU with one block per page anyway keeps the heads in one block, which
 // amortises the per-block set-up and overlaps one head's copy-out with the next head's encoding.
-static int heads_cluster(int hkv, int n_pages)
+static int heads_cluster(int hkv, int n_pages, int sms)
 {
-    if (n_pages > 2 * 148) return 1;
+    if (n_pages > 2 * sms) return 1;
     for (int c = 8; c > 1; --c)
         if (hkv % c == 0) return c;
     return 1;
@@ -921,24 +921,24 @@ constexpr int kPageTickets = 48;
 static uint32_t* page_tickets(mkv_pool* p) { return p->status_dev + 16; }
 
 // grid rows of the tile-parallel passes: at least 16, and enough to fill the GPU when few pages are converted
-static int tile_rows(int tiles, int n_pages, int hkv)
+static int tile_rows(int tiles, int n_pages, int hkv, int sms)
 {
-    int rows = (4 * 148 + n_pages * hkv - 1) / (n_pages * hkv);
+    int rows = (4 * sms + n_pages * hkv - 1) / (n_pages * hkv);
     if (rows < 16) rows = 16;
     return rows < tiles ? rows : tiles;
 }
 
 // blocks per page of the warp kernels: one, or a cluster that has a warp for every head when the call has few pages
-static int warp_cluster(int hkv, int n_pages)
+static int warp_cluster(int hkv, int n_pages, int sms)
 {
     const int c = (hkv + kDemoteWarps - 1) / kDemoteWarps;
-    return n_pages > 2 * 148 ? 1 : c < 8 ? c : 8;
+    return n_pages > 2 * sms ? 1 : c < 8 ? c : 8;
 }
 
 // grid rows of the tile-parallel warp kernels: enough for 12 warps on every SM
-static int warp_tile_rows(int tiles, int n_pages, int hkv)
+static int warp_tile_rows(int tiles, int n_pages, int hkv, int sms)
 {
-    int rows = (12 * 148 + n_pages * hkv - 1) / (n_pages * hkv);
+    int rows = (12 * sms + n_pages * hkv - 1) / (n_pages * hkv);
     if (rows < 16) rows = 16;
     return rows < tiles ? rows : tiles;
 }
@@ -947,10 +947,10 @@ template <int D, int FMT, bool BIG>
 static cudaError_t launch_demote_warp(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
                                       const int64_t* entry, int64_t n_entries, uint32_t* tickets, cudaStream_t s)
 {
-    const int warps = p->hkv < kDemoteWarps ? p->hkv : kDemoteWarps, c = warp_cluster(p->hkv, BIG ? 0 : n);
+    const int warps = p->hkv < kDemoteWarps ? p->hkv : kDemoteWarps, c = warp_cluster(p->hkv, BIG ? 0 : n, p->dev.sm_count);
     const int smem = DemoteWarp<D>::OFF_WARPS + warps * DemoteWarp<D>::BYTES;
     static_assert(DemoteWarp<D>::OFF_WARPS + kDemoteWarps * DemoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
-    return launch_pdl(demote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv) : 1), 32 * warps,
+    return launch_pdl(demote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv, p->dev.sm_count) : 1), 32 * warps,
                       (size_t)smem, c, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv,
                       p->tiles, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }
@@ -972,7 +972,7 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
         return MKV_OK;
     }
     if (p->tiles == 1) {
-        const int c = heads_cluster(p->hkv, n);
+        const int c = heads_cluster(p->hkv, n, p->dev.sm_count);
         MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, 1, p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, bt,
                                   tags, entry, n_entries, p->status_dev, (uint32_t*)nullptr));
@@ -984,16 +984,16 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
     {
         // blocks per (page, head): up to a portable cluster of 8, fewer when the call fills the GPU anyway
         int cs = 8;
-        while (cs > 1 && (cs > p->tiles || (long long)n * p->hkv * cs > 8LL * 148)) cs >>= 1;
+        while (cs > 1 && (cs > p->tiles || (long long)n * p->hkv * cs > 8LL * p->dev.sm_count)) cs >>= 1;
         MKV_CUDA(launch_pdl(demote_minmax_kernel<D>, dim3((unsigned)n * p->hkv * cs), D, 0, cs, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, p->tiles, p->cfg.v_scale, src, dst));
     }
-    const int ch = heads_cluster(p->hkv, 0);
+    const int ch = heads_cluster(p->hkv, 0, p->dev.sm_count);
     if (warp_per_record)
         MKV_CUDA((launch_demote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
                                                    fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
     else
-        MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv)), D, 0, ch, false, s,
+        MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv, p->dev.sm_count)), D, 0, ch, false, s,
                                    (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv, p->tiles,
                                    p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr,
                                    fused ? tags : (uint8_t*)nullptr, fused ? entry : (const int64_t*)nullptr,
@@ -1024,11 +1024,11 @@ template <int D, int FMT, bool BIG>
 static cudaError_t launch_promote_warp(mkv_pool* p, const int32_t* src, const int32_t* dst, int n, int32_t* bt, uint8_t* tags,
                                        const int64_t* entry, int64_t n_entries, uint32_t* tickets, cudaStream_t s)
 {
-    const int warps = p->hkv < kDemoteWarps ? p->hkv : kDemoteWarps, c = warp_cluster(p->hkv, BIG ? 0 : n);
+    const int warps = p->hkv < kDemoteWarps ? p->hkv : kDemoteWarps, c = warp_cluster(p->hkv, BIG ? 0 : n, p->dev.sm_count);
     const int smem = PromoteWarp<D>::OFF_WARPS + warps * PromoteWarp<D>::BYTES;
     static_assert(PromoteWarp<D>::OFF_WARPS + kDemoteWarps * PromoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
     const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale, rs = (float)(1.0 / sqrt((double)p->d));
-    return launch_pdl(promote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv) : 1),
+    return launch_pdl(promote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv, p->dev.sm_count) : 1),
                       32 * warps, (size_t)smem, c, false, s, (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages,
                       p->hkv, p->tiles, ik, iv, rs, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }

@@ -115,7 +115,7 @@ __device__ __forceinline__ void pdl_begin()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// early: start before the predecessor has ended.  Not for Demote and Promote: their blocks would be placed while the
+// early: start before the predecessor has ended.  Not for Demote and most calls of Promote: their blocks would be placed while the
 // predecessor still holds most SMs, up to four on one SM, and wait there, and behind a decode scan that has evicted
 // their code they start on it together: one page between decode calls, d = 256, 4 heads, Demote 40 -> 20 us, Promote
 // 15 -> 8 us without; 148 pages 37 -> 23 and 16 -> 10.5 us.

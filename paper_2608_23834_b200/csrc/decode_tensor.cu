@@ -211,6 +211,21 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// Arrival on a row's ticket: what this block has stored (before a block barrier) is released, what the others have is acquired
+__device__ __forceinline__ uint32_t ticket_add(uint32_t* p, uint32_t v)
+{
+    uint32_t old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
+
+__device__ __forceinline__ uint32_t ticket_or(uint32_t* p, uint32_t v)
+{
+    uint32_t old;
+    asm volatile("atom.or.acq_rel.gpu.global.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
+
 // bulk asynchronous copy global -> this block's shared memory, completion counted on an mbarrier
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
 {
@@ -315,115 +330,145 @@ __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (
 constexpr int kMaxAlignedRows = kMaxCtas / 4;
 
 //   flat (several layers): a linear cut of all layers' triples, the layers laid end to end.
+//
+// Every block works this out for itself before its first page can be asked for, so the arithmetic is kept short: one
+// 32-bit division per cut (quotient and remainder; block c starts at quo c + min(c, rem)), and warp 0 leaves the
+// block's own range and request in shared memory.  (With W c / blocks in 64 bits, a binary search for the row and a serial one for
+// the request, set-up took 11,600 cycles at 8 x 16,384 tokens and 18,900 in the flat cut of 64 rows, of 33 and 70 us in all.)
+struct Cut {
+    long long quo;
+    int rem, blocks;                    // blocks that get work (0: none)
+};
+
 struct Partition {
-    long long total;                    // flat: triples of all layers
-    int flat_blocks;                    // flat: blocks that get work
+    Cut flat;                           // flat: all layers' triples
+    Cut cut;                            // linear cut of one layer
     int aligned;                        // 1: row-aligned, 0: linear
-    int blocks;                         // blocks that get work
+    int start, end;                     // this block's range in the per-layer cut
+    int first_layer, end_layer;         // this block's layers in the flat cut
+    int first_b;                        // request of the block's first triple
     int base[kMaxAlignedRows + 1];      // row-aligned: first block of every row
 };
 
-// Called by warp 0 (all 32 lanes) after cum[] is complete; other warps wait at the next barrier.
 // Blocks that share W triples: all of the grid, but no more than give every block min_pages of them (a page per warp
 // of an SM: below that a row's partials cost more to merge than the spreading saves).
-__device__ __forceinline__ int useful_blocks(long long W, int grid, int min_pages)
+__device__ __forceinline__ Cut make_cut(long long W, int grid, int min_pages)
 {
-    const long long most = (W + min_pages - 1) / min_pages;
-    return (int)(most < (long long)grid ? most : (long long)grid);
+    Cut c;
+    if (W >> 31 == 0) {
+        const unsigned w = (unsigned)W, most = (w + min_pages - 1) / (unsigned)min_pages;
+        c.blocks = (int)min(most, (unsigned)grid);
+        const unsigned q = c.blocks ? w / (unsigned)c.blocks : 0u;
+        c.quo = q;
+        c.rem = (int)(w - q * (unsigned)c.blocks);
+    } else {
+        c.blocks = grid;
+        c.quo = W / grid;
+        c.rem = (int)(W - c.quo * grid);
+    }
+    return c;
 }
 
-__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, int B, int hkv, int grid, int min_pages, int straddle, int lane)
+__device__ __forceinline__ long long cut_start(const Cut& c, int block) { return c.quo * block + min(block, c.rem); }
+
+// the block that holds triple x
+__device__ __forceinline__ int cut_block_of(const Cut& c, long long x)
+{
+    const long long split = (c.quo + 1) * c.rem;          // the first `rem` blocks have one more; quo >= 1 where a triple exists
+    int b = x < split ? (int)__fdividef((float)x, (float)(c.quo + 1)) : c.rem + (int)__fdividef((float)(x - split), (float)c.quo);
+    b = min(b, c.blocks - 1);                             // near, then exact
+    while (b + 1 < c.blocks && cut_start(c, b + 1) <= x) ++b;
+    while (b > 0 && cut_start(c, b) > x) --b;
+    return b;
+}
+
+// Request that holds triple x of a layer: the number of requests that end at or before it.  All 32 lanes of a warp.
+__device__ __forceinline__ int request_of(const int* cum, int B, int x, int lane)
+{
+    int b = 0;
+    for (int b0 = 0; b0 < B; b0 += 32) {
+        const uint32_t m = __ballot_sync(0xffffffffu, b0 + lane < B && cum[b0 + lane + 1] <= x);
+        b += __popc(m);
+        if (m != 0xffffffffu) break;
+    }
+    return b;
+}
+
+// Called by warp 0 (all 32 lanes) after cum[] and lens[] are complete; other warps wait at the next barrier.
+__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, const int* lens, int B, int hkv, int grid,
+                                                int min_pages, int straddle, int me, int lane)
 {
     constexpr uint32_t FULL = 0xffffffffu;
-    const long long W = cum[B];
-    const int rows = B * hkv;
-    int blocks = useful_blocks(W, grid, min_pages);
-    grid = blocks;
-    if (blocks == 0) {                                  // every request of the call is empty
-        if (lane == 0) pt->aligned = pt->blocks = 0;
-        return;
-    }
+    const int W = cum[B], rows = B * hkv;
+    const Cut cut = make_cut(W, grid, min_pages);
+    grid = cut.blocks;
+    int start = 0, end = 0;                             // every request of the call is empty, or more blocks than work
     // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
     // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
     // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).
-    // The rounding to whole blocks costs about half a block's share in k of a block's pages; from `straddle` pages on that
-    // is dearer than the straddling (d 128, 8 heads, two blocks per SM: 8 x 4,096 tokens 28.9 us linear, 23.6 aligned;
-    // 8 x 32,768 of which half FP8 104.7 linear, 108 aligned).
-    const int aligned_loss = (int)(W * rows / (2ll * grid * grid));
-    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && W >= grid && aligned_loss < straddle) ? 1 : 0;
+    // The rounding to whole blocks costs about half a block's share in k of a block's pages, W rows / (2 grid^2); from
+    // `straddle` pages on that is dearer than the straddling (d 128, 8 heads, two blocks per SM: 8 x 4,096 tokens 28.9 us linear,
+    // 23.6 aligned; 8 x 32,768 of which half FP8 104.7 linear, 108 aligned).
+    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && W >= grid &&
+                   (long long)W * rows < 2ll * straddle * grid * grid) ? 1 : 0;
+    auto row_pages = [&](int b) { return (lens[b] + kPage - 1) / kPage; };
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_page(r) / W);
         // every row must end up with at least one block, otherwise the linear cut is used
         int bad = 0;
         const float scale = (float)grid / (float)W;
         for (int r = lane; r <= rows; r += 32) {
-            int first = (int)W;                                 // r == rows: one past the last row
+            int first = W;                                      // r == rows: one past the last row
             if (r < rows) {
-                const int b = r / hkv, h = r - b * hkv;
-                first = cum[b] + h * ((cum[b + 1] - cum[b]) / hkv);
+                const int b = r / hkv;
+                first = cum[b] + (r - b * hkv) * row_pages(b);
             }
             pt->base[r] = r == rows ? grid : (int)((float)first * scale + 0.5f);
         }
         __syncwarp();
+        int mine = -1;
         for (int r = lane; r < rows; r += 32) {
-            const int b = r / hkv;
-            if (cum[b + 1] > cum[b] && pt->base[r + 1] <= pt->base[r]) bad = 1;
+            const int b = r / hkv, c0 = pt->base[r], c1 = pt->base[r + 1];
+            if (cum[b + 1] > cum[b] && c1 <= c0) bad = 1;
+            if (c0 <= me && me < c1) mine = r;
         }
         if (__any_sync(FULL, bad)) aligned = 0;
-        else blocks = grid;
+        else if (mine >= 0) {                                   // the one lane that holds this block's row
+            const int b = mine / hkv, n = row_pages(b), row_start = cum[b] + (mine - b * hkv) * n;
+            const unsigned k = pt->base[mine + 1] - pt->base[mine], j = me - pt->base[mine];
+            pt->start = row_start + (int)(((unsigned)n * j) / k);
+            pt->end = row_start + (int)(((unsigned)n * (j + 1)) / k);
+            pt->first_b = b;
+        }
+        if (aligned && me >= grid && lane == 0) pt->start = pt->end = 0;
+    }
+    if (!aligned) {
+        if (me < grid) {
+            start = (int)cut_start(cut, me);
+            end = (int)cut_start(cut, me + 1);
+        }
+        const int b = request_of(cum, B, start, lane);
+        if (lane == 0) {
+            pt->start = start;
+            pt->end = end;
+            pt->first_b = b;
+        }
     }
     if (lane == 0) {
         pt->aligned = aligned;
-        pt->blocks = blocks;
+        pt->cut = cut;
     }
 }
 
-// linear range [start, end) of block c
-__device__ __forceinline__ void partition_range(const Partition* pt, const int* cum, int hkv, int B, int c, int& start,
-                                                int& end)
+// first triple of block c in the per-layer cut; row_start, n: the row of which block c is the first block
+__device__ __forceinline__ int layer_start_of_first_block(const Partition* pt, int c, int row_start)
 {
-    const long long W = cum[B];
-    if (!pt->aligned) {
-        start = (int)((W * c) / pt->blocks);
-        end = (int)((W * (c + 1)) / pt->blocks);
-        return;
-    }
-    const int rows = B * hkv;
-    int lo = 0;                                     // row of block c: base[r] <= c < base[r + 1]
-    for (int hi = rows - 1; lo < hi;) {
-        const int mid = (lo + hi) >> 1;
-        if (pt->base[mid + 1] <= c) lo = mid + 1; else hi = mid;
-    }
-    const int r = lo, b = r / hkv, h = r - b * hkv, n = (cum[b + 1] - cum[b]) / hkv;
-    const unsigned k = pt->base[r + 1] - pt->base[r], j = c - pt->base[r];
-    const int row_start = cum[b] + h * n;
-    start = row_start + (int)(((unsigned)n * j) / k);
-    end = row_start + (int)(((unsigned)n * (j + 1)) / k);
-}
-
-__device__ __forceinline__ int partition_start(const Partition* pt, const int* cum, int hkv, int B, int c)
-{
-    int s, e;
-    partition_range(pt, cum, hkv, B, c, s, e);
-    return s;
-}
-
-// flat cut: first triple of block c, counted over all layers
-__device__ __forceinline__ long long flat_start(const Partition* pt, int c) { return pt->total * c / pt->flat_blocks; }
-
-// block of a linear cut of W triples over C blocks that holds triple x: the last c with floor(W c / C) <= x
-__device__ __forceinline__ int linear_block_of(long long W, int C, long long x)
-{
-    int c = (int)((x * C) / W);
-    while (c + 1 < C && (W * (c + 1)) / C <= x) ++c;
-    while (c > 0 && (W * c) / C > x) --c;
-    return c;
+    return pt->aligned ? row_start : (int)cut_start(pt->cut, c);
 }
 
 // Whether position x of the row [row_start, row_end) (row index r) opens the run of some warp in the per-layer cut
 // with n_warps warps per block.
-__device__ __forceinline__ bool opens_warp_run(const Partition* pt, const int* cum, int B, int r, int row_start, int row_end,
-                                               int x, unsigned n_warps)
+__device__ __forceinline__ bool opens_warp_run(const Partition* pt, int r, int row_start, int row_end, int x, unsigned n_warps)
 {
     int first, n;                                   // the block's share of the row
     if (pt->aligned) {
@@ -432,26 +477,37 @@ __device__ __forceinline__ bool opens_warp_run(const Partition* pt, const int* c
         first = row_start + (int)(rows * j / k);
         n = row_start + (int)(rows * (j + 1) / k) - first;
     } else {
-        const long long W = cum[B];
-        const int c = linear_block_of(W, pt->blocks, x);
-        first = max((int)(W * c / pt->blocks), row_start);
-        n = min((int)(W * (c + 1) / pt->blocks), row_end) - first;
+        const int c = cut_block_of(pt->cut, x);
+        first = max((int)cut_start(pt->cut, c), row_start);
+        n = min((int)cut_start(pt->cut, c + 1), row_end) - first;
     }
     const unsigned w = ((unsigned)(x - first + 1) * n_warps - 1) / (unsigned)n;
     return (int)((unsigned)n * w / n_warps) == x - first;
 }
 
 // blocks c0..c1 that hold a part of the row [row_start, row_end) (row index r)
-__device__ __forceinline__ void partition_blocks_of_row(const Partition* pt, const int* cum, int B, int r, int row_start,
-                                                        int row_end, int& c0, int& c1)
+__device__ __forceinline__ void partition_blocks_of_row(const Partition* pt, int r, int row_start, int row_end, int& c0, int& c1)
 {
     if (pt->aligned) {
         c0 = pt->base[r];
         c1 = pt->base[r + 1] - 1;
         return;
     }
-    c0 = linear_block_of(cum[B], pt->blocks, row_start);
-    c1 = linear_block_of(cum[B], pt->blocks, row_end - 1);
+    c0 = cut_block_of(pt->cut, row_start);
+    c1 = cut_block_of(pt->cut, row_end - 1);
+}
+
+// Pages of a row are visited in an order that gives every contiguous range of positions the row's FP8 and TQ3 pages in
+// their overall proportion (spans of either format are contiguous), so that equal ranges cost equal time.  The row is cut into 32
+// strips of equal length (the first n % 32 are one page longer); position x is page x / 32 of strip x % 32, the strips
+// in bit-reversed order, and the pages that the longer strips have more come last.  A bijection without a division.  (Before: x
+// times a stride near 0.618 n and coprime to n, modulo n; finding it, seventeen remainders per try, kept all
+// warps waiting for 1,500 cycles.)
+__device__ __forceinline__ int page_at(int x, int n)
+{
+    const int len = n >> 5, longer = n & 31, at = x >> 5;
+    const int strip = at < len ? (int)(__brev((unsigned)x) >> 27) : x & 31;
+    return strip * len + min(strip, longer) + at;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -478,8 +534,8 @@ struct Geo {
     static constexpr int OFF_BAR = OFF_QF + QPLAIN;
     static constexpr int OFF_LIST = (OFF_BAR + NW * NP * 8 + 15) / 16 * 16;   // [warp][2 formats][ROUND] page ids, then [warp][2][ROUND] logical pages
     static constexpr int OFF_CUM = OFF_LIST + NW * 4 * ROUND * 4;
-    static constexpr int OFF_STRIDE = OFF_CUM + (kMaxBatch + 1) * 4;
-    static constexpr int OFF_M = OFF_STRIDE + kMaxBatch * 4;
+    static constexpr int OFF_LENS = OFF_CUM + (kMaxBatch + 1) * 4;
+    static constexpr int OFF_M = OFF_LENS + kMaxBatch * 4;
     static constexpr int OFF_L = OFF_M + NW * 8 * 4;
     static constexpr int OFF_PART = (OFF_L + NW * 8 * 4 + 15) / 16 * 16;    // holds 64-bit fields
     static constexpr int OFF_LAST = OFF_PART + ((int)sizeof(Partition) + 15) / 16 * 16;
@@ -1132,14 +1188,14 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 {
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
     // 16-byte loads that a thread of the merge keeps in flight, within the registers of the launch shape
-    constexpr int MERGE_LOADS = NW * MINB <= 8 ? 40 : NW * MINB <= 12 ? 24 : 16;
+    constexpr int MERGE_LOADS = NW * MINB <= 8 ? 20 : 16;
     using G = Geo<D, NW, NSTAGE, TILED>;     // pages of several tiles: short rounds leave room for the parked rows
     constexpr int NB = G::NB;
     constexpr uint32_t FULL = 0xffffffffu;
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     int* cum = reinterpret_cast<int*>(smem + G::OFF_CUM);
-    int* strides = reinterpret_cast<int*>(smem + G::OFF_STRIDE);
+    int* lens_s = reinterpret_cast<int*>(smem + G::OFF_LENS);
     float* sm_m = reinterpret_cast<float*>(smem + G::OFF_M);
     float* sm_l = reinterpret_cast<float*>(smem + G::OFF_L);
     Partition* pt = reinterpret_cast<Partition*>(smem + G::OFF_PART);
@@ -1160,7 +1216,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         return len < 0 ? 0 : len;
     };
 
-    // ---- prologue: barriers, prefix of pages, page strides ---------------------------------------
+    // ---- prologue: barriers, lengths, prefix of pages, this block's share ---------------------------------------
     if (tid == 0) {
         for (int i = 0; i < NW * G::NP; ++i) mbar_init(sbase + G::OFF_BAR + 8 * i, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1174,7 +1230,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             int n = 0;
             if (b < P0.B) {
                 const int len = length_of(b);
-                n = len > 0 ? ((len + kPage - 1) / kPage) * hkv : 0;
+                lens_s[b] = len;
+                n = ((len + kPage - 1) / kPage) * hkv;
             }
             int inc = n;
 #pragma unroll
@@ -1187,42 +1244,34 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         }
         if (lane == 0) cum[P0.B] = run;
         __syncwarp();
+        if constexpr (!FLAT || TILED)
+            build_partition(pt, cum, lens_s, P0.B, hkv, gridDim.x, NW * MINB, 4 * NW, blockIdx.x, lane);
         if constexpr (FLAT) {
+            const Cut cut = make_cut((long long)run * n_layers, gridDim.x, NW * MINB);
+            int first = 0, end = 0, b = 0;
+            if ((int)blockIdx.x < cut.blocks) {
+                const long long s = cut_start(cut, blockIdx.x), e = cut_start(cut, blockIdx.x + 1);
+                while (first + 1 < n_layers && (long long)(first + 1) * run <= s) ++first;
+                for (end = first + 1; end < n_layers && (long long)end * run < e;) ++end;
+                b = request_of(cum, P0.B, (int)(s - (long long)first * run), lane);
+            }
             if (lane == 0) {
-                pt->total = (long long)run * n_layers;
-                pt->flat_blocks = useful_blocks(pt->total, gridDim.x, NW * MINB);
+                pt->flat = cut;
+                pt->first_layer = first;
+                pt->end_layer = end;
+                pt->first_b = b;
             }
-        }
-        if constexpr (!FLAT || TILED) build_partition(pt, cum, P0.B, hkv, gridDim.x, NW * MINB, 4 * NW, lane);
-    } else {
-        // Pages of a row are visited in a strided order, page(i) = i * stride mod n_pages, the stride
-        // coprime to n_pages and near 0.618 n_pages: every contiguous range of positions then holds the
-        // row's FP8 and TQ3 pages in their overall proportion, so equal ranges cost equal time.
-        for (int b = tid - 32; b < P0.B; b += NW * 32 - 32) {
-            const int len = length_of(b), n = (len + kPage - 1) / kPage;
-            int st = (int)((float)n * 0.6180339f);
-            if (st < 1) st = 1;
-            if constexpr (TILED) st = 1;          // consecutive tiles: a warp's run stays inside one or two pages
-            for (; n > 1 && !TILED; ++st) {
-                int a = st, c = n;
-                while (c) { const int t = a % c; a = c; c = t; }
-                if (a == 1) break;
-            }
-            strides[b] = st;
         }
     }
     __syncthreads();
     int my_start = 0, my_end = 0;                          // more blocks than work: an empty range
     int layer_first = 0, layer_end = n_layers;
     if constexpr (FLAT) {
-        if ((int)blockIdx.x < pt->flat_blocks) {
-            layer_first = (int)(flat_start(pt, blockIdx.x) / cum[P0.B]);
-            layer_end = (int)((flat_start(pt, blockIdx.x + 1) - 1) / cum[P0.B]) + 1;
-        } else {
-            layer_end = 0;
-        }
-    } else if ((int)blockIdx.x < pt->blocks) {
-        partition_range(pt, cum, hkv, P0.B, blockIdx.x, my_start, my_end);
+        layer_first = pt->first_layer;
+        layer_end = pt->end_layer;
+    } else {
+        my_start = pt->start;
+        my_end = pt->end;
     }
 
     // per-warp ring of NP slot pairs; one bit per pair holds the mbarrier phase the next wait must see
@@ -1276,7 +1325,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     // rows of empty requests
     for (int i0 = blockIdx.x; i0 < P0.B * n_layers; i0 += gridDim.x) {
         const int b = i0 % P0.B;
-        if (P0.lens[b] > 0) continue;
+        if (lens_s[b] > 0) continue;
         const DecodeParams& P = LS.layer[MAXL == 1 ? 0 : i0 / P0.B];
         for (int i = tid; i < hq * D; i += NW * 32) P.out[(size_t)b * hq * D + i] = 0.f;
         if (P.lse)
@@ -1287,8 +1336,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     const DecodeParams& P = LS.layer[MAXL == 1 ? 0 : layer];
     if constexpr (FLAT) {                                  // this block's range inside the layer
         const long long w0 = (long long)layer * cum[P0.B];
-        my_start = (int)max(flat_start(pt, blockIdx.x) - w0, 0ll);
-        my_end = (int)min(flat_start(pt, blockIdx.x + 1) - w0, (long long)cum[P0.B]);
+        my_start = (int)max(cut_start(pt->flat, blockIdx.x) - w0, 0ll);
+        my_end = (int)min(cut_start(pt->flat, blockIdx.x + 1) - w0, (long long)cum[P0.B]);
     }
     auto wait_slot = [&](uint32_t s) -> bool {
         if (wait_bounded(s, P.wait_ns)) return true;
@@ -1297,21 +1346,20 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         return false;
     };
     int pos = my_start;
-    int b = 0;
+    int b = FLAT && layer > layer_first ? 0 : pt->first_b;
     while (pos < my_end) {
         // ---- locate the segment: request b, KV head h, positions [pg0, pg0 + n_seg) of the row ------
         while (cum[b + 1] <= pos) ++b;
-        const int len = min(max(P.lens[b], 0), len_cap), n_pages = (len + kPage - 1) / kPage;
-        const int h = (pos - cum[b]) / n_pages, pg0 = (pos - cum[b]) % n_pages;
+        const int len = lens_s[b], n_pages = (len + kPage - 1) / kPage;
+        const int h = (pos - cum[b]) / n_pages, pg0 = pos - cum[b] - h * n_pages;
         const int row_start = cum[b] + h * n_pages, row_end = row_start + n_pages;
         const int n_seg = min(my_end, row_end) - pos;
         const int32_t* bt_row = P.bt + (size_t)b * P.max_pages;
         const uint8_t* tag_row = P.tags + (size_t)b * P.max_pages;
-        // this warp's pages: a contiguous run of positions (a run of the strided order holds FP8 and TQ3
-        // pages in the row's proportion, so the warps of a block finish together)
+        // this warp's pages: a contiguous run of positions (which holds FP8 and TQ3 pages in the row's proportion,
+        // see page_at, so the warps of a block finish together)
         const int warp_first = (int)(((unsigned)n_seg * (unsigned)warp) / NW);
         const int n_my = (int)(((unsigned)n_seg * (unsigned)(warp + 1)) / NW) - warp_first;
-        const int stride = strides[b];
         constexpr int EPL = D / 32;
         constexpr int HPW = (8 + NW - 1) / NW;      // query heads a warp prepares (head warp, warp + NW, ...)
         float qx[HPW][EPL];       // loaded before anything else waits
@@ -1331,7 +1379,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         const size_t tq3_page = (size_t)P.tiles * TQ3_TILE + TQ3_META;
 
         // Table entries of up to G::ROUND of the warp's pages are compacted into two id lists, one per
-        // format (entry i of a 32-page chunk is read by lane i; ballots give the positions).
+        // format (entry i of a 32-page chunk is read by lane i, all chunks before the first is looked at; ballots give the positions).
         // Returns how many of the warp's pages (from `first` on) the lists cover.  Long pages in the flat cut: a Stale
         // tile that opens a warp's run of the per-layer cut is marked (kOpens); the scan leaves the page there, and
         // a round ends at the last such tile, so that code sums are gathered over the same runs of tiles as there
@@ -1341,24 +1389,38 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         auto build_lists = [&](int first) -> int {
             n3 = n8 = 0;
             int covered = min(G::ROUND, n_my - first), cut3 = 0, cut8 = 0, cut = 0;
-#pragma unroll 1
-            for (int c = 0; c < G::ROUND / 32; ++c) {
+            constexpr int CH = G::ROUND / 32;
+            int ids[CH], tg[CH], pgs[CH];
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
                 const int i = first + c * 32 + lane;
-                int kind = 0, id = 0, valid = kPage, pg = 0;
+                ids[c] = -1;
+                tg[c] = pgs[c] = 0;
                 if (i < n_my) {
-                    pg = (int)(((unsigned)(pg0 + warp_first + i) * (unsigned)stride) % (unsigned)n_pages);   // < 2^32: max_pages <= 65535
-                    // `pg` counts 16-token tiles of the row; the table has one entry per page of P.tiles tiles
+                    // `pg` counts 16-token tiles of the row (long pages: in their order, so that a warp's run stays inside one or
+                    // two pages); the table has one entry per page of P.tiles tiles
+                    const int pg = TILED ? pg0 + warp_first + i : page_at(pg0 + warp_first + i, n_pages);
                     const int entry = TILED ? pg / P.tiles : pg;
-                    id = bt_row[entry];
-                    const int tag = tag_row[entry];
+                    pgs[c] = pg;
+                    ids[c] = bt_row[entry];
+                    tg[c] = tag_row[entry];
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int i = first + c * 32 + lane;
+                if (first + c * 32 >= n_my) break;
+                int kind = 0, id = ids[c], valid = kPage, pg = pgs[c];
+                if (i < n_my) {
                     valid = min(kPage, len - pg * kPage);
-                    if (tag == MKV_TAG_STALE)
+                    if (tg[c] == MKV_TAG_STALE)
                         kind = (id >= 0 && id < P.tq3_pages && valid == kPage) ? 1 : 0;
                     else
-                        kind = (tag <= MKV_TAG_ANCHOR && id >= 0 && id < P.fp8_pages) ? 2 : 0;
+                        kind = (tg[c] <= MKV_TAG_ANCHOR && id >= 0 && id < P.fp8_pages) ? 2 : 0;
                     if (kind == 0) atomicOr(P.status, kStBounds);     // never dereferenced
                     if constexpr (TILED) {   // second list: tile inside its page | logical page << 16
-                        const bool opens = FLAT && opens_warp_run(pt, cum, P.B, b * hkv + h, row_start, row_end, row_start + pg, NW);
+                        const int entry = pg / P.tiles;
+                        const bool opens = FLAT && opens_warp_run(pt, b * hkv + h, row_start, row_end, row_start + pg, NW);
                         pg = (pg - entry * P.tiles) | (entry << 16) | (opens ? kOpens : 0);
                     }
                 }
@@ -1564,24 +1626,27 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     reinterpret_cast<uint32_t*>(qt8 + st * 768 + 512 + L * 8)[k >> 4] = word[2];
                 }
             }
+            if constexpr (FMT == 1) {       // rotated query, natural slot order: block i/16, slot s = i%16; per lane {hi b0, hi b1, lo b0, lo b1}
 #pragma unroll
-            for (int r = 0; r < EPL; ++r) {
-                const int i = lane * EPL + r;
-                if constexpr (FMT == 1) {   // rotated query, natural slot order: block i/16, slot s = i%16; per lane {hi b0, hi b1, lo b0, lo b1}
-                    const int kb = i >> 4, s = i & 15;
-                    const int at = (kb * 32 + 4 * hd + ((s & 7) >> 1)) * (SPLIT ? 4 : 8) + (s >> 3) * 2 + (s & 1);
+                for (int r = 0; r < EPL; r += 2) {
+                    const int i = lane * EPL + r, kb = i >> 4, s = i & 15;
+                    const int at = (kb * 32 + 4 * hd + ((s & 7) >> 1)) * (SPLIT ? 4 : 8) + (s >> 3) * 2;
                     // fp16 pair hi + lo carries the rotated query to ~2^-22
-                    const float v = a[r] * rs;
-                    const __half vh = __float2half_rn(v);
-                    qt[at] = vh;
-                    qt[at + (SPLIT ? 64 : 4)] = __float2half_rn(v - __half2float(vh));     // SPLIT: column hd + 4
+                    const float v0 = a[r] * rs, v1 = a[r + 1] * rs;
+                    const __half2 vh = __floats2half2_rn(v0, v1);
+                    *reinterpret_cast<__half2*>(qt + at) = vh;
+                    *reinterpret_cast<__half2*>(qt + at + (SPLIT ? 64 : 4)) =           // SPLIT: column hd + 4
+                        __floats2half2_rn(v0 - __low2float(vh), v1 - __high2float(vh));
                 }
-                {   // plain query in the slot order of the FP8 key loads: 16 consecutive dims per lane
-                    const int j = i >> 6, t4 = (i & 63) >> 4, wv = (i & 15) >> 2, e = i & 3;
-                    const int at = ((4 * j + wv) * 32 + 4 * hd + t4) * 4 + (e >> 1) * 2 + (e & 1);
-                    qf[at] = __float2half_rn(qx[k][r]);
-                    if constexpr (SPLIT) qf[at + 64] = qf[at];         // column hd + 4: the same scores
-                }
+            }
+            // plain query in the slot order of the FP8 key loads: 16 consecutive dims per lane
+#pragma unroll
+            for (int r = 0; r < EPL; r += 4) {
+                const int i = lane * EPL + r, j = i >> 6, t4 = (i & 63) >> 4, wv = (i & 15) >> 2;
+                __half* at = qf + ((4 * j + wv) * 32 + 4 * hd + t4) * 4;
+                const uint2 four = make_uint2(pack_f16x2(qx[k][r], qx[k][r + 1]), pack_f16x2(qx[k][r + 2], qx[k][r + 3]));
+                *reinterpret_cast<uint2*>(at) = four;
+                if constexpr (SPLIT) *reinterpret_cast<uint2*>(at + 64) = four;         // column hd + 4: the same scores
             }
         }
         __syncthreads();
@@ -1706,21 +1771,42 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         __syncthreads();
 
         const bool whole_row = (pos == row_start) && (pos + n_seg == row_end);
-        if (whole_row) {
-            for (int e = tid; e < 8 * D; e += NW * 32) {
-                const int head = e & 7, ch = e >> 3;
-                if (head >= GQ) continue;
-                float acc = 0.f, l = 0.f;
+        // sum of the warps for one channel (item e4 / 2) and four heads (first: 4 (e4 % 2)); SPLIT: columns 4 - 7 are the low
+        // halves of heads 0 - 3
+        auto sum_of_warps = [&](int e4) -> float4 {
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    acc += red[(size_t)w * D * 8 + e];
-                    l += sm_l[w * 8 + head];
-                    if constexpr (SPLIT) {
-                        acc += red[(size_t)w * D * 8 + e + 4];
-                        l += sm_l[w * 8 + head + 4];
-                    }
+            for (int w = 0; w < NW; ++w) {
+                const float4* row = reinterpret_cast<const float4*>(red + (size_t)w * D * 8);
+                const float4 hi = row[e4];
+                s.x += hi.x; s.y += hi.y; s.z += hi.z; s.w += hi.w;
+                if constexpr (SPLIT) {
+                    const float4 lo = row[e4 + 1];
+                    s.x += lo.x; s.y += lo.y; s.z += lo.z; s.w += lo.w;
                 }
-                P.out[((size_t)b * hq + h * GQ + head) * D + ch] = l > 0.f ? acc / l : 0.f;
+            }
+            return s;
+        };
+        constexpr int ITEMS = SPLIT ? D : 2 * D, PER_THREAD = (ITEMS + NW * 32 - 1) / (NW * 32);
+        if (whole_row) {
+#pragma unroll
+            for (int k = 0; k < PER_THREAD; ++k) {
+                const int i = tid + k * NW * 32, e4 = SPLIT ? 2 * i : i, ch = e4 >> 1;
+                if (i >= ITEMS) break;
+                const float4 s = sum_of_warps(e4);
+                const float v[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int head = 4 * (e4 & 1) + e;
+                    if (head >= GQ) continue;
+                    float l = 0.f;
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) {
+                        l += sm_l[w * 8 + head];
+                        if constexpr (SPLIT) l += sm_l[w * 8 + head + 4];
+                    }
+                    P.out[((size_t)b * hq + h * GQ + head) * D + ch] = l > 0.f ? v[e] / l : 0.f;
+                }
             }
             if (P.lse && tid < GQ) {
                 float l = 0.f, M = -CUDART_INF_F;
@@ -1735,14 +1821,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             // partial (m, l, O) of this block for the row; slot 2c if the segment opens the block's range (flat cut:
             // its range in this layer), 2c + 1 otherwise
             float* slot = P.partials + (size_t)(2 * blockIdx.x + (pos != my_start ? 1 : 0)) * (8 * D + 16);
-            for (int e = tid; e < 8 * D; e += NW * 32) {
-                float acc = 0.f;
 #pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    acc += red[(size_t)w * D * 8 + e];
-                    if constexpr (SPLIT) acc += (e & 4) ? 0.f : red[(size_t)w * D * 8 + e + 4];
-                }
-                slot[e] = acc;                 // (SPLIT: columns 4-7 are not read as heads)
+            for (int k = 0; k < PER_THREAD; ++k) {
+                const int i = tid + k * NW * 32, e4 = SPLIT ? 2 * i : i;
+                if (i >= ITEMS) break;
+                reinterpret_cast<float4*>(slot)[e4] = sum_of_warps(e4);
+                if constexpr (SPLIT) reinterpret_cast<float4*>(slot)[e4 + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
             if (tid < 8) {
                 float l = 0.f, M = -CUDART_INF_F;
@@ -1754,8 +1838,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 slot[8 * D + tid] = M;
                 slot[8 * D + 8 + tid] = l;
             }
-            // Ticket of the row (store -> fence -> ticket on the writers' side, ticket -> fence -> load on the
-            // merger's).  Who merges?  In the last layer of the launch the block that draws the row's last
+            // Ticket of the row (all threads' stores, block barrier, releasing ticket on the writers' side; acquiring ticket, block
+            // barrier, loads on the merger's).  Who merges?  In the last layer of the launch the block that draws the row's last
             // ticket.  In an earlier layer the row is left to the block that is FIRST to finish the same row in
             // the next layer -- the one that is ahead of the others, so that the merges do not keep falling on
             // the block that is already late.  That block finds the row complete and merges it, or it leaves a
@@ -1764,21 +1848,20 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             int c0, c1;
             if constexpr (FLAT) {                          // here the row's last arrival merges: no block is ahead of the others
                 const long long w0 = (long long)layer * cum[P0.B];
-                c0 = linear_block_of(pt->total, pt->flat_blocks, w0 + row_start);
-                c1 = linear_block_of(pt->total, pt->flat_blocks, w0 + row_end - 1);
+                c0 = cut_block_of(pt->flat, w0 + row_start);
+                c1 = cut_block_of(pt->flat, w0 + row_end - 1);
             } else {
-                partition_blocks_of_row(pt, cum, P.B, b * hkv + h, row_start, row_end, c0, c1);
+                partition_blocks_of_row(pt, b * hkv + h, row_start, row_end, c0, c1);
             }
             const int n_parts = c1 - c0 + 1;
             constexpr uint32_t kRequest = 0x80000000u;
             __syncthreads();
             if (tid == 0) {
-                __threadfence();
-                const uint32_t prev = atomicAdd(P.tickets + c0, 1u);
+                const uint32_t prev = ticket_add(P.tickets + c0, 1u);
                 int todo = 0;                          // 1: merge this layer's row, 2: merge the row of the layer before
                 if ((prev & ~kRequest) == (uint32_t)(n_parts - 1) && (FLAT || layer == n_layers - 1 || (prev & kRequest))) todo |= 1;
                 if (MAXL > 1 && !FLAT && layer > 0 && (prev & ~kRequest) == 0u) {
-                    const uint32_t old = atomicOr(LS.layer[layer - 1].tickets + c0, kRequest);
+                    const uint32_t old = ticket_or(LS.layer[layer - 1].tickets + c0, kRequest);
                     if (old == (uint32_t)n_parts) todo |= 2;
                 }
                 *last_s = todo;
@@ -1786,10 +1869,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             __syncthreads();
             const int todo = *last_s;
             if (todo) {
-                __threadfence();
                 // the row opens block c0's range of the layer where it starts at or before that range
-                const int c0_start = FLAT ? (int)max(flat_start(pt, c0) - (long long)layer * cum[P0.B], 0ll)
-                                          : partition_start(pt, cum, hkv, P.B, c0);
+                const int c0_start = FLAT ? (int)max(cut_start(pt->flat, c0) - (long long)layer * cum[P0.B], 0ll)
+                                          : layer_start_of_first_block(pt, c0, row_start);
                 const int first_slot = 2 * c0 + (row_start > c0_start ? 1 : 0);
                 if constexpr (MAXL > 1 && !FLAT) {
                     if (todo & 2) {

@@ -68,8 +68,8 @@ struct TG {
     static constexpr int OFF_LIST = OFF_BAR + ((kBarCount * 8 + 127) / 128) * 128;   // Stale ids, FP8 ids | valid << 27
     static constexpr int OFF_CNT = OFF_LIST + 2 * kRoundT * 4;         // n3, n8, 4 flags, 4 x 8 maxima
     static constexpr int OFF_CUM = OFF_CNT + 256;
-    static constexpr int OFF_STRIDE = OFF_CUM + (kMaxBatch + 1) * 4;
-    static constexpr int OFF_M = OFF_STRIDE + kMaxBatch * 4;
+    static constexpr int OFF_LENS = OFF_CUM + (kMaxBatch + 1) * 4;
+    static constexpr int OFF_M = OFF_LENS + kMaxBatch * 4;
     static constexpr int OFF_L = OFF_M + 8 * 4;
     static constexpr int OFF_PART = (OFF_L + 8 * 4 + 15) / 16 * 16;    // holds 64-bit fields
     static constexpr int OFF_LAST = OFF_PART + ((int)sizeof(Partition) + 15) / 16 * 16;
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     int* cum = reinterpret_cast<int*>(smem + G::OFF_CUM);
-    int* strides = reinterpret_cast<int*>(smem + G::OFF_STRIDE);
+    int* lens_s = reinterpret_cast<int*>(smem + G::OFF_LENS);
     float* sm_m = reinterpret_cast<float*>(smem + G::OFF_M);
     float* sm_l = reinterpret_cast<float*>(smem + G::OFF_L);
     Partition* pt = reinterpret_cast<Partition*>(smem + G::OFF_PART);
@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
             if (b < P.B) {
                 int len = P.lens[b];
                 if (len > P.max_pages * kPage) { atomicOr(P.status, kStBounds); len = P.max_pages * kPage; }   // a length beyond the table row is cut and flagged
+                lens_s[b] = max(len, 0);
                 n = len > 0 ? ((len + kPage - 1) / kPage) * hkv : 0;
             }
             int inc = n;
@@ -225,31 +226,17 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
         }
         if (lane == 0) cum[P.B] = run;
         __syncwarp();
-        build_partition(pt, cum, P.B, hkv, gridDim.x, 1, 1 << 30, lane);
-    } else {
-        for (int b = tid - 32; b < P.B; b += NT - 32) {
-            const int len = min(max(P.lens[b], 0), P.max_pages * kPage), n = (len + kPage - 1) / kPage;
-            int st = (int)((float)n * 0.6180339f);
-            if (st < 1) st = 1;
-            for (; n > 1; ++st) {
-                int a = st, c = n;
-                while (c) { const int t = a % c; a = c; c = t; }
-                if (a == 1) break;
-            }
-            strides[b] = st;
-        }
+        build_partition(pt, cum, lens_s, P.B, hkv, gridDim.x, 1, 1 << 30, blockIdx.x, lane);
     }
     __syncthreads();
-    if ((int)blockIdx.x >= pt->blocks) return;             // more blocks than work (nothing allocated yet)
+    const int my_start = pt->start, my_end = pt->end;
+    if (my_start >= my_end) return;                        // more blocks than work (nothing allocated yet)
     if (warp == kISS) tmem_alloc(smem_u32(tmem_s), 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tb = *tmem_s;
     const uint32_t my_lanes = (uint32_t)(32 * wq) << 16;    // lanes of this warp's subpartition
-
-    int my_start, my_end;
-    partition_range(pt, cum, hkv, P.B, blockIdx.x, my_start, my_end);
 
     bool failed = false;
     const float sc2 = P.scale * kLog2e;
@@ -287,16 +274,15 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
     };
 
     int pos = my_start;
-    int b = 0;
+    int b = pt->first_b;
     while (pos < my_end) {
         while (cum[b + 1] <= pos) ++b;
-        const int len = min(max(P.lens[b], 0), P.max_pages * kPage), n_pages = (len + kPage - 1) / kPage;
-        const int h = (pos - cum[b]) / n_pages, pg0 = (pos - cum[b]) % n_pages;
+        const int len = lens_s[b], n_pages = (len + kPage - 1) / kPage;
+        const int h = (pos - cum[b]) / n_pages, pg0 = pos - cum[b] - h * n_pages;
         const int row_start = cum[b] + h * n_pages, row_end = row_start + n_pages;
         const int n_seg = min(my_end, row_end) - pos;
         const int32_t* bt_row = P.bt + (size_t)b * P.max_pages;
         const uint8_t* tag_row = P.tags + (size_t)b * P.max_pages;
-        const int stride = strides[b];
         const int n_rounds = (n_seg + kRoundT - 1) / kRoundT;
         constexpr int EPL = D / 32;
         float qx[EPL];
@@ -363,7 +349,7 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
             if (tid == 0) { cnt[0] = 0; cnt[1] = 0; }
             __syncthreads();
             for (int i = round * kRoundT + tid; i < min(n_seg, (round + 1) * kRoundT); i += NT) {
-                const int pg = (int)(((unsigned)(pg0 + i) * (unsigned)stride) % (unsigned)n_pages);
+                const int pg = page_at(pg0 + i, n_pages);
                 const int id = bt_row[pg], tag = tag_row[pg], valid = min(kPage, len - pg * kPage);
                 int kind = 0;
                 if (tag == MKV_TAG_STALE) kind = (id >= 0 && id < P.tq3_pages && valid == kPage) ? 1 : 0;
@@ -784,20 +770,18 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
                 slot[8 * D + 8 + tid] = sm_l[tid];
             }
             int c0, c1;
-            partition_blocks_of_row(pt, cum, P.B, b * hkv + h, row_start, row_end, c0, c1);
+            partition_blocks_of_row(pt, b * hkv + h, row_start, row_end, c0, c1);
             const int n_parts = c1 - c0 + 1;
             __syncthreads();
             if (tid == 0) {
-                __threadfence();
-                const uint32_t prev = atomicAdd(P.tickets + c0, 1u);
+                const uint32_t prev = ticket_add(P.tickets + c0, 1u);
                 const int last = prev == (uint32_t)(n_parts - 1);
                 if (last) P.tickets[c0] = 0;
                 *last_s = last;
             }
             __syncthreads();
             if (*last_s) {
-                __threadfence();
-                const int first_slot = 2 * c0 + (row_start > partition_start(pt, cum, hkv, P.B, c0) ? 1 : 0);
+                const int first_slot = 2 * c0 + (row_start > layer_start_of_first_block(pt, c0, row_start) ? 1 : 0);
                 merge_row<D, NT, 16>(P, first_slot, 2 * c0, n_parts, red, b, h);
             }
         }

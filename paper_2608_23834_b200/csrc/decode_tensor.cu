@@ -333,8 +333,10 @@ constexpr int kMaxAlignedRows = kMaxCtas / 4;
 //
 // Every block works this out for itself before its first page can be asked for, so the arithmetic is kept short: one
 // 32-bit division per cut (quotient and remainder; block c starts at quo c + min(c, rem)), and warp 0 leaves the
-// block's own range and request in shared memory.  (With W c / blocks in 64 bits, a binary search for the row and a serial one for
-// the request, set-up took 11,600 cycles at 8 x 16,384 tokens and 18,900 in the flat cut of 64 rows, of 33 and 70 us in all.)
+// block's own range and request in shared memory.  (With W c / blocks in 64 bits, a binary search for the row, a serial one for the
+// request and the strides that page_at replaces, the time up to a block's first page was 11,600 cycles at 8 x 16,384 tokens, d 128,
+// and 18,900 in the flat cut of 16 layers x 16 rows, d 256; it is 8,400 and 10,100: 36.5 -> 34.3 and 75.6 -> 66.3 us a step, and
+// 650 -> 552 for 16 layers of long pages, where every tile asks which warp's run it opens.)
 struct Cut {
     long long quo;
     int rem, blocks;                    // blocks that get work (0: none)
@@ -1079,7 +1081,7 @@ __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, u
 // (one trip to L2: both are loaded together and kept in shared memory); a thread owns float4 groups (one channel,
 // four heads) of the [channel][8 heads] tile.  With twice as many threads as groups (16 warps at d = 128) every
 // other part goes to the second half of the threads.  KP loads per thread are in flight, issued before the weights
-// are worked out: 32 to 40 parts per block, bounded by the registers of the launch shape.
+// are worked out: as many as the launch shape has registers for, and no more than rows of few parts can use.
 template <int D, int NT, int KPMAX>
 __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot, int even_base, int n_parts,
                                           float* buf, int b, int h)
@@ -2006,18 +2008,29 @@ int decode_tensor_partial_floats(int d) { return 8 * d + 16; }
 // Second step of the scored variant: mass[b][hq][p] holds log2 of page p's exponential sum on an
 // absolute origin; with the row's log-sum-exp it becomes q_p = 2^(that - lse2), and q~_p = q_p / sum q_p
 // (Eq. score-global-weight and the normalisation over page-addressable mass that follows it).
-// One block per (query head, request); entries beyond the request's pages are set to zero.
-__global__ void __launch_bounds__(256) page_mass_finish_kernel(float* mass, const float* lse, const int32_t* lens,
+// One block per (query head, request); entries beyond the request's pages are set to zero.  The first 4,096 pages of a row
+// are loaded at once and stay in registers between the two steps; what is beyond is read twice.  (Bound by the trips to memory: four rows of
+// 2,501 pages x 24 heads with one load at a time and a second reading, and the score update behind it, took 4 us longer, 69.6 -> 65 us for
+// the whole scored step.)
+__global__ void __launch_bounds__(512) page_mass_finish_kernel(float* mass, const float* lse, const int32_t* lens,
                                                               int hq, int max_pages, int page_tokens)
 {
-    __shared__ float red[8];
+    constexpr int NT = 512, KEEP = 8;
+    __shared__ float red[NT / 32];
     pdl_begin();
     const int b = blockIdx.y, h = blockIdx.x, tid = threadIdx.x;
     const int len = lens[b], n_pages = len > 0 ? min((len + page_tokens - 1) / page_tokens, max_pages) : 0;
     float* row = mass + ((size_t)b * hq + h) * max_pages;
     const float lse2 = n_pages > 0 ? lse[(size_t)b * hq + h] * kLog2e : 0.f;
-    float sum = 0.f;
-    for (int p = tid; p < n_pages; p += 256) {
+    float kept[KEEP], sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) kept[k] = tid + k * NT < n_pages ? row[tid + k * NT] : -CUDART_INF_F;
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) {
+        kept[k] = tid + k * NT < n_pages ? fast_exp2(kept[k] - lse2) : 0.f;
+        sum += kept[k];
+    }
+    for (int p = tid + KEEP * NT; p < n_pages; p += NT) {
         const float qv = fast_exp2(row[p] - lse2);
         row[p] = qv;
         sum += qv;
@@ -2028,9 +2041,12 @@ __global__ void __launch_bounds__(256) page_mass_finish_kernel(float* mass, cons
     __syncthreads();
     float total = 0.f;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) total += red[w];
+    for (int w = 0; w < NT / 32; ++w) total += red[w];
     const float inv = total > 0.f ? 1.f / total : 0.f;
-    for (int p = tid; p < max_pages; p += 256) row[p] = p < n_pages ? row[p] * inv : 0.f;
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k)
+        if (tid + k * NT < max_pages) row[tid + k * NT] = kept[k] * inv;
+    for (int p = tid + KEEP * NT; p < max_pages; p += NT) row[p] = p < n_pages ? row[p] * inv : 0.f;
 }
 
 // Eq. (attention-score): r_p = mean over the sampled heads of q~_{h,p}; a_p <- beta a_p + (1 - beta) r_p.
@@ -2043,8 +2059,9 @@ __global__ void __launch_bounds__(256) page_score_kernel(const float* mass, cons
     const int len = lens[b], n_pages = len > 0 ? min((len + page_tokens - 1) / page_tokens, max_pages) : 0;
     if (p >= n_pages) return;
     float r = 0.f;
-    for (int h = 0; h < hq; ++h)
-        if ((head_mask >> h) & 1ull) r += mass[((size_t)b * hq + h) * max_pages + p];
+#pragma unroll 16
+    for (int h = 0; h < hq; ++h)            // many loads in flight
+        r += (head_mask >> h) & 1ull ? mass[((size_t)b * hq + h) * max_pages + p] : 0.f;
     float* a = score + (size_t)b * max_pages + p;
     *a = beta * *a + (1.f - beta) * (r * inv_heads);
 }
@@ -2060,7 +2077,7 @@ __global__ void page_mass_clear_kernel(float* mass, size_t n)
 int32_t launch_page_mass_finish(float* mass, const float* lse, const int32_t* lens, int B, int hq, int max_pages,
                                 int page_tokens, cudaStream_t s)
 {
-    MKV_CUDA(launch_pdl(page_mass_finish_kernel, dim3(hq, B), 256, 0, 1, true, s, mass, lse, lens, hq, max_pages, page_tokens));
+    MKV_CUDA(launch_pdl(page_mass_finish_kernel, dim3(hq, B), 512, 0, 1, true, s, mass, lse, lens, hq, max_pages, page_tokens));
     return MKV_OK;
 }
 

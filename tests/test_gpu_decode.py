@@ -238,6 +238,16 @@ def test_decode_one_long_row_and_the_page_limit():
     assert b"65535" in M.lib().mkv_last_cuda_error()
 
 
+@pytest.mark.parametrize("d,hkv,group", [(128, 2, 2), (256, 1, 6)])
+def test_rows_at_the_edges_of_the_page_order(d, hkv, group):
+    """Rows of one page more or less than a multiple of the 32 strips, behind more empty requests than a warp has lanes."""
+    lens = [0] * 35 + [16 * n + r for n in (1, 31, 32, 33, 63, 64, 65, 97) for r in (0, 7)]
+    case = Case(W.config(0, seq_lens=lens, head_dim=d, n_kv_heads=hkv, group=group, anchor_prefix=32, recent_tokens=120), extra_fp8=2,
+                extra_tq3=2)
+    out, lse = case.run()
+    check_case(case, out, lse, *case.reference())
+
+
 @pytest.mark.parametrize("d,page", [(128, 16), (256, 16), (128, 48), (256, 832)])
 def test_a_batch_of_empty_requests_only(d, page):
     """No pages at all: nothing to cut the grid over; outputs are zero and the log-sum-exps minus infinity."""

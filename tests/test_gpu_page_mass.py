@@ -21,6 +21,8 @@ CASES = {
     "cfg2": lambda: W.config(2, seq_lens=(5008, 4432), recent_tokens=512, n_layers=1),
     "cfg3": lambda: W.config(3, seq_lens=[int(1024 * 8 ** u) for u in np.random.default_rng(3).random(12)], recent_tokens=200),
     "cfg4_f95": lambda: W.config(4, batch=3, ctx=1024, stale_fraction=0.95),
+    # rows on both sides of the 4,096 pages that the finishing kernel keeps in registers
+    "4096_pages": lambda: W.config(0, seq_lens=(16 * 4096, 16 * 4095 + 1, 16 * 4610 + 3), head_dim=128, n_kv_heads=1, group=2, recent_tokens=200),
     "ragged": lambda: W.config(1, seq_lens=(1, 17, 0, 1000, 16, 333), recent_tokens=40, anchor_spans=0),
     # pages of several 16-token tiles: a page's mass is gathered from the warps and blocks that scan its tiles
     "pages_of_48": lambda: W.config(0, seq_lens=(21 * 48 + 37, 4 * 48, 0, 17), head_dim=128, n_kv_heads=2, group=4,

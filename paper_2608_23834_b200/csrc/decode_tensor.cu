@@ -352,6 +352,9 @@ struct Partition {
     int base[kMaxAlignedRows + 1];      // row-aligned: first block of every row
 };
 
+// a / b for 0 <= a < 2^20: (a + 1/2) / b is at least 1 / (2 b) away from the next integer, the approximate quotient less far off
+__device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
+
 // Blocks that share W triples: all of the grid, but no more than give every block min_pages of them (a page per warp
 // of an SM: below that a row's partials cost more to merge than the spreading saves).
 __device__ __forceinline__ Cut make_cut(long long W, int grid, int min_pages)
@@ -384,6 +387,17 @@ __device__ __forceinline__ int cut_block_of(const Cut& c, long long x)
     return b;
 }
 
+// a row of n pages (at most 65,535) over k whole blocks
+__device__ __forceinline__ Cut cut_row(int n, int k)
+{
+    Cut c;
+    c.blocks = k;
+    const int q = small_div(n, k);
+    c.quo = q;
+    c.rem = n - q * k;
+    return c;
+}
+
 // Request that holds triple x of a layer: the number of requests that end at or before it.  All 32 lanes of a warp.
 __device__ __forceinline__ int request_of(const int* cum, int B, int x, int lane)
 {
@@ -413,7 +427,7 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, c
     // 23.6 aligned; 8 x 32,768 of which half FP8 104.7 linear, 108 aligned).
     int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && W >= grid &&
                    (long long)W * rows < 2ll * straddle * grid * grid) ? 1 : 0;
-    auto row_pages = [&](int b) { return (lens[b] + kPage - 1) / kPage; };
+    auto row_pages = [&](int b) { return (int)((unsigned)(lens[b] + kPage - 1) / kPage); };
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_page(r) / W);
         // every row must end up with at least one block, otherwise the linear cut is used
@@ -422,7 +436,7 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, c
         for (int r = lane; r <= rows; r += 32) {
             int first = W;                                      // r == rows: one past the last row
             if (r < rows) {
-                const int b = r / hkv;
+                const int b = small_div(r, hkv);
                 first = cum[b] + (r - b * hkv) * row_pages(b);
             }
             pt->base[r] = r == rows ? grid : (int)((float)first * scale + 0.5f);
@@ -430,16 +444,17 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, c
         __syncwarp();
         int mine = -1;
         for (int r = lane; r < rows; r += 32) {
-            const int b = r / hkv, c0 = pt->base[r], c1 = pt->base[r + 1];
+            const int b = small_div(r, hkv), c0 = pt->base[r], c1 = pt->base[r + 1];
             if (cum[b + 1] > cum[b] && c1 <= c0) bad = 1;
             if (c0 <= me && me < c1) mine = r;
         }
         if (__any_sync(FULL, bad)) aligned = 0;
         else if (mine >= 0) {                                   // the one lane that holds this block's row
-            const int b = mine / hkv, n = row_pages(b), row_start = cum[b] + (mine - b * hkv) * n;
-            const unsigned k = pt->base[mine + 1] - pt->base[mine], j = me - pt->base[mine];
-            pt->start = row_start + (int)(((unsigned)n * j) / k);
-            pt->end = row_start + (int)(((unsigned)n * (j + 1)) / k);
+            const int b = small_div(mine, hkv), n = row_pages(b), row_start = cum[b] + (mine - b * hkv) * n;
+            const Cut row = cut_row(n, pt->base[mine + 1] - pt->base[mine]);
+            const int j = me - pt->base[mine];
+            pt->start = row_start + (int)cut_start(row, j);
+            pt->end = row_start + (int)cut_start(row, j + 1);
             pt->first_b = b;
         }
         if (aligned && me >= grid && lane == 0) pt->start = pt->end = 0;
@@ -474,10 +489,10 @@ __device__ __forceinline__ bool opens_warp_run(const Partition* pt, int r, int r
 {
     int first, n;                                   // the block's share of the row
     if (pt->aligned) {
-        const unsigned rows = row_end - row_start, k = pt->base[r + 1] - pt->base[r],
-                       j = ((unsigned)(x - row_start + 1) * k - 1) / rows;          // last j with floor(rows j / k) <= x - row_start
-        first = row_start + (int)(rows * j / k);
-        n = row_start + (int)(rows * (j + 1) / k) - first;
+        const Cut row = cut_row(row_end - row_start, pt->base[r + 1] - pt->base[r]);
+        const int j = cut_block_of(row, x - row_start);
+        first = row_start + (int)cut_start(row, j);
+        n = row_start + (int)cut_start(row, j + 1) - first;
     } else {
         const int c = cut_block_of(pt->cut, x);
         first = max((int)cut_start(pt->cut, c), row_start);
@@ -1253,8 +1268,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             int first = 0, end = 0, b = 0;
             if ((int)blockIdx.x < cut.blocks) {
                 const long long s = cut_start(cut, blockIdx.x), e = cut_start(cut, blockIdx.x + 1);
-                while (first + 1 < n_layers && (long long)(first + 1) * run <= s) ++first;
-                for (end = first + 1; end < n_layers && (long long)end * run < e;) ++end;
+                first = min((int)__fdividef((float)s, (float)run), n_layers - 1);
+                if ((long long)first * run > s) --first;
+                if ((long long)(first + 1) * run <= s) ++first;
+                for (end = first + 1; (long long)end * run < e;) ++end;
                 b = request_of(cum, P0.B, (int)(s - (long long)first * run), lane);
             }
             if (lane == 0) {
@@ -1353,8 +1370,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         // ---- locate the segment: request b, KV head h, positions [pg0, pg0 + n_seg) of the row ------
         while (cum[b + 1] <= pos) ++b;
         const int len = lens_s[b], n_pages = (len + kPage - 1) / kPage;
-        const int h = (pos - cum[b]) / n_pages, pg0 = pos - cum[b] - h * n_pages;
-        const int row_start = cum[b] + h * n_pages, row_end = row_start + n_pages;
+        int h = (int)__fdividef((float)(pos - cum[b]), (float)n_pages), pg0 = pos - cum[b] - h * n_pages;   // at most one off
+        if (pg0 < 0) --h, pg0 += n_pages;
+        if (pg0 >= n_pages) ++h, pg0 -= n_pages;
+        const int row_start = pos - pg0, row_end = row_start + n_pages;
         const int n_seg = min(my_end, row_end) - pos;
         const int32_t* bt_row = P.bt + (size_t)b * P.max_pages;
         const uint8_t* tag_row = P.tags + (size_t)b * P.max_pages;
@@ -1366,12 +1385,20 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         constexpr int HPW = (8 + NW - 1) / NW;      // query heads a warp prepares (head warp, warp + NW, ...)
         float qx[HPW][EPL];       // loaded before anything else waits
 #pragma unroll
-        for (int k = 0; k < HPW; ++k)
+        for (int k = 0; k < HPW; ++k) {
+            const int hd = warp + k * NW;
+            uint2 raw[EPL / 4];                     // (the entry points take queries on 16-byte boundaries)
 #pragma unroll
-            for (int r = 0; r < EPL; ++r) {
-                const int hd = warp + k * NW;
-                qx[k][r] = (hd < GQ) ? __bfloat162float(P.q[((size_t)b * hq + h * GQ + hd) * D + lane * EPL + r]) : 0.f;
+            for (int r = 0; r < EPL / 4; ++r)
+                raw[r] = hd < GQ ? reinterpret_cast<const uint2*>(P.q + ((size_t)b * hq + h * GQ + hd) * D + lane * EPL)[r]
+                                 : make_uint2(0u, 0u);
+#pragma unroll
+            for (int r = 0; r < EPL; r += 2) {
+                const uint32_t w = r & 2 ? raw[r / 4].y : raw[r / 4].x;
+                qx[k][r] = __uint_as_float(w << 16);
+                qx[k][r + 1] = __uint_as_float(w & 0xFFFF0000u);
             }
+        }
         float* mass_row = SCORED ? P.mass + ((size_t)b * hq + (size_t)h * GQ) * P.max_pages : nullptr;
         const uint8_t* tq3_base = P.tq3 + (size_t)h * G::TQ3_REC;
         const uint8_t* fp8_base = P.fp8 + (size_t)h * (2 * G::FP8_HALF);

@@ -321,8 +321,12 @@ __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (
 // ------------------------------------------------------------------------------------------------
 // Work partition (the scan and the merge of split rows use the same cut)
 // ------------------------------------------------------------------------------------------------
-// Work = (request, KV head, page) triples in row-major order; cum[b] = index of the first triple of
-// request b.  Two ways to cut it into one contiguous range per block:
+// Work = (request, KV head, page) triples in row-major order; cum[b] = position of the first triple of
+// request b.  A row of n pages takes row_cost + n positions: opening, reducing and storing a row (or a block's part of it)
+// costs a block as much time as row_cost pages, so that a block with many short rows gets fewer pages.  (64 requests of 1,024 to
+// 131,072 tokens, 8 heads: the blocks with the shortest requests took 520 us against 406 on average; 524 -> 480 us a step with
+// 32, the same with 48, 503 with 16.  16 layers x 4 x 700..3,001 tokens, d 256: 64.0 -> 60 with 16, 62 with 32, 66 with 48.
+// 16 layers x 8 x 512..16,384, one block of 16 warps per SM: 151 -> 139 with 32, 134 with 48, 136 with 64.)  Two ways to cut it into one contiguous range per block:
 //   row-aligned (few rows: B * hkv <= grid / 4): every row gets a whole number of blocks in proportion
 //     to its pages (cumulative rounding), so that no block straddles two rows and pays the per-row set-up
 //     and reduction twice;
@@ -355,13 +359,13 @@ struct Partition {
 // a / b for 0 <= a < 2^20: (a + 1/2) / b is at least 1 / (2 b) away from the next integer, the approximate quotient less far off
 __device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
 
-// Blocks that share W triples: all of the grid, but no more than give every block min_pages of them (a page per warp
-// of an SM: below that a row's partials cost more to merge than the spreading saves).
-__device__ __forceinline__ Cut make_cut(long long W, int grid, int min_pages)
+// Blocks that share W positions, `pages` of them pages: all of the grid, but no more than give every block min_pages pages (a page
+// per warp of an SM: below that a row's partials cost more to merge than the spreading saves).
+__device__ __forceinline__ Cut make_cut(long long W, long long pages, int grid, int min_pages)
 {
     Cut c;
     if (W >> 31 == 0) {
-        const unsigned w = (unsigned)W, most = (w + min_pages - 1) / (unsigned)min_pages;
+        const unsigned w = (unsigned)W, most = ((unsigned)pages + min_pages - 1) / (unsigned)min_pages;
         c.blocks = (int)min(most, (unsigned)grid);
         const unsigned q = c.blocks ? w / (unsigned)c.blocks : 0u;
         c.quo = q;
@@ -412,21 +416,21 @@ __device__ __forceinline__ int request_of(const int* cum, int B, int x, int lane
 
 // Called by warp 0 (all 32 lanes) after cum[] and lens[] are complete; other warps wait at the next barrier.
 __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, const int* lens, int B, int hkv, int grid,
-                                                int min_pages, int straddle, int me, int lane)
+                                                int pages, int row_cost, int min_pages, int straddle, int me, int lane)
 {
     constexpr uint32_t FULL = 0xffffffffu;
     const int W = cum[B], rows = B * hkv;
-    const Cut cut = make_cut(W, grid, min_pages);
+    const Cut cut = make_cut(W, pages, grid, min_pages);
     grid = cut.blocks;
     int start = 0, end = 0;                             // every request of the call is empty, or more blocks than work
     // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
     // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
     // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).
-    // The rounding to whole blocks costs about half a block's share in k of a block's pages, W rows / (2 grid^2); from
+    // The rounding to whole blocks costs about half a block's share in k of a block's pages, pages rows / (2 grid^2); from
     // `straddle` pages on that is dearer than the straddling (d 128, 8 heads, two blocks per SM: 8 x 4,096 tokens 28.9 us linear,
     // 23.6 aligned; 8 x 32,768 of which half FP8 104.7 linear, 108 aligned).
-    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && W >= grid &&
-                   (long long)W * rows < 2ll * straddle * grid * grid) ? 1 : 0;
+    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && pages >= grid &&
+                   (long long)pages * rows < 2ll * straddle * grid * grid) ? 1 : 0;
     auto row_pages = [&](int b) { return (int)((unsigned)(lens[b] + kPage - 1) / kPage); };
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_page(r) / W);
@@ -437,7 +441,7 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, c
             int first = W;                                      // r == rows: one past the last row
             if (r < rows) {
                 const int b = small_div(r, hkv);
-                first = cum[b] + (r - b * hkv) * row_pages(b);
+                first = cum[b] + (r - b * hkv) * (row_pages(b) + row_cost);
             }
             pt->base[r] = r == rows ? grid : (int)((float)first * scale + 0.5f);
         }
@@ -450,11 +454,11 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, c
         }
         if (__any_sync(FULL, bad)) aligned = 0;
         else if (mine >= 0) {                                   // the one lane that holds this block's row
-            const int b = small_div(mine, hkv), n = row_pages(b), row_start = cum[b] + (mine - b * hkv) * n;
+            const int b = small_div(mine, hkv), n = row_pages(b), row_start = cum[b] + (mine - b * hkv) * (n + row_cost);
             const Cut row = cut_row(n, pt->base[mine + 1] - pt->base[mine]);
             const int j = me - pt->base[mine];
-            pt->start = row_start + (int)cut_start(row, j);
-            pt->end = row_start + (int)cut_start(row, j + 1);
+            pt->start = row_start + (j > 0 ? row_cost + (int)cut_start(row, j) : 0);
+            pt->end = row_start + row_cost + (int)cut_start(row, j + 1);
             pt->first_b = b;
         }
         if (aligned && me >= grid && lane == 0) pt->start = pt->end = 0;
@@ -502,7 +506,7 @@ __device__ __forceinline__ bool opens_warp_run(const Partition* pt, int r, int r
     return (int)((unsigned)n * w / n_warps) == x - first;
 }
 
-// blocks c0..c1 that hold a part of the row [row_start, row_end) (row index r)
+// blocks c0..c1 that hold pages of the row with index r, whose first page is at row_start and whose last before row_end
 __device__ __forceinline__ void partition_blocks_of_row(const Partition* pt, int r, int row_start, int row_end, int& c0, int& c1)
 {
     if (pt->aligned) {
@@ -1206,6 +1210,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
     // 16-byte loads that a thread of the merge keeps in flight, within the registers of the launch shape
     constexpr int MERGE_LOADS = NW * MINB <= 8 ? 20 : 16;
+    // what a row costs besides its pages, in pages: more warps scan more of them in that time.  Long pages come in few rows.
+    constexpr int ROW_COST = TILED ? 0 : 8 + 3 * NW;
     using G = Geo<D, NW, NSTAGE, TILED>;     // pages of several tiles: short rounds leave room for the parked rows
     constexpr int NB = G::NB;
     constexpr uint32_t FULL = 0xffffffffu;
@@ -1241,15 +1247,16 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     }
     pdl_begin();
     if (warp == 0) {
-        int run = 0;
+        int run = 0, used = 0;                             // requests with tokens
         for (int b0 = 0; b0 < P0.B; b0 += 32) {
             const int b = b0 + lane;
             int n = 0;
             if (b < P0.B) {
                 const int len = length_of(b);
                 lens_s[b] = len;
-                n = ((len + kPage - 1) / kPage) * hkv;
+                n = len > 0 ? ((len + kPage - 1) / kPage + ROW_COST) * hkv : 0;
             }
+            used += __popc(__ballot_sync(FULL, n > 0));
             int inc = n;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -1262,9 +1269,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         if (lane == 0) cum[P0.B] = run;
         __syncwarp();
         if constexpr (!FLAT || TILED)
-            build_partition(pt, cum, lens_s, P0.B, hkv, gridDim.x, NW * MINB, 4 * NW, blockIdx.x, lane);
+            build_partition(pt, cum, lens_s, P0.B, hkv, gridDim.x, run - used * hkv * ROW_COST, ROW_COST, NW * MINB, 4 * NW, blockIdx.x, lane);
         if constexpr (FLAT) {
-            const Cut cut = make_cut((long long)run * n_layers, gridDim.x, NW * MINB);
+            const Cut cut = make_cut((long long)run * n_layers, (long long)(run - used * hkv * ROW_COST) * n_layers, gridDim.x,
+                                     NW * MINB);
             int first = 0, end = 0, b = 0;
             if ((int)blockIdx.x < cut.blocks) {
                 const long long s = cut_start(cut, blockIdx.x), e = cut_start(cut, blockIdx.x + 1);
@@ -1370,11 +1378,16 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         // ---- locate the segment: request b, KV head h, positions [pg0, pg0 + n_seg) of the row ------
         while (cum[b + 1] <= pos) ++b;
         const int len = lens_s[b], n_pages = (len + kPage - 1) / kPage;
-        int h = (int)__fdividef((float)(pos - cum[b]), (float)n_pages), pg0 = pos - cum[b] - h * n_pages;   // at most one off
-        if (pg0 < 0) --h, pg0 += n_pages;
-        if (pg0 >= n_pages) ++h, pg0 -= n_pages;
-        const int row_start = pos - pg0, row_end = row_start + n_pages;
-        const int n_seg = min(my_end, row_end) - pos;
+        const int row_len = n_pages + ROW_COST;
+        int h = (int)__fdividef((float)(pos - cum[b]), (float)row_len), off = pos - cum[b] - h * row_len;   // at most one off
+        if (off < 0) --h, off += row_len;
+        if (off >= row_len) ++h, off -= row_len;
+        const int row_start = pos - off, row_end = row_start + row_len, seg_end = min(my_end, row_end);
+        const int pg0 = max(off - ROW_COST, 0), n_seg = seg_end - row_start - ROW_COST - pg0;
+        if (n_seg <= 0) {                          // the block's range ends before the row's first page
+            pos = seg_end;
+            continue;
+        }
         const int32_t* bt_row = P.bt + (size_t)b * P.max_pages;
         const uint8_t* tag_row = P.tags + (size_t)b * P.max_pages;
         // this warp's pages: a contiguous run of positions (which holds FP8 and TQ3 pages in the row's proportion,
@@ -1799,7 +1812,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         }
         __syncthreads();
 
-        const bool whole_row = (pos == row_start) && (pos + n_seg == row_end);
+        const bool whole_row = n_seg == n_pages;
         // sum of the warps for one channel (item e4 / 2) and four heads (first: 4 (e4 % 2)); SPLIT: columns 4 - 7 are the low
         // halves of heads 0 - 3
         auto sum_of_warps = [&](int e4) -> float4 {
@@ -1877,10 +1890,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             int c0, c1;
             if constexpr (FLAT) {                          // here the row's last arrival merges: no block is ahead of the others
                 const long long w0 = (long long)layer * cum[P0.B];
-                c0 = cut_block_of(pt->flat, w0 + row_start);
+                c0 = cut_block_of(pt->flat, w0 + row_start + ROW_COST);
                 c1 = cut_block_of(pt->flat, w0 + row_end - 1);
             } else {
-                partition_blocks_of_row(pt, b * hkv + h, row_start, row_end, c0, c1);
+                partition_blocks_of_row(pt, b * hkv + h, row_start + ROW_COST, row_end, c0, c1);
             }
             const int n_parts = c1 - c0 + 1;
             constexpr uint32_t kRequest = 0x80000000u;
@@ -1916,7 +1929,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             }
         }
         __syncthreads();
-        pos += n_seg;
+        pos = seg_end;
     }
     }   // layers
 }

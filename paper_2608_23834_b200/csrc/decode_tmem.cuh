@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
         }
         if (lane == 0) cum[P.B] = run;
         __syncwarp();
-        build_partition(pt, cum, lens_s, P.B, hkv, gridDim.x, 1, 1 << 30, blockIdx.x, lane);
+        build_partition(pt, cum, lens_s, P.B, hkv, gridDim.x, run, 0, 1, 1 << 30, blockIdx.x, lane);
     }
     __syncthreads();
     const int my_start = pt->start, my_end = pt->end;

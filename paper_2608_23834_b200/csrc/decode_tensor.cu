@@ -1245,7 +1245,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         last_s[1] = 0;
     }
-    pdl_begin();
+    pdl_wait();
     if (warp == 0) {
         int run = 0, used = 0;                             // requests with tokens
         for (int b0 = 0; b0 < P0.B; b0 += 32) {
@@ -1776,6 +1776,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 start_round();
             }
         }
+        const bool last_segment = seg_end == my_end && layer + 1 == layer_end;
         float (&oacc)[NB][4] = acc.o;
         float (&lacc)[2] = acc.l;
         float (&m_run)[2] = acc.m;
@@ -1910,6 +1911,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             }
             __syncthreads();
             const int todo = *last_s;
+            if (last_segment) pdl_let_next_start();    // what is left of the block is at most a merge
             if (todo) {
                 // the row opens block c0's range of the layer where it starts at or before that range
                 const int c0_start = FLAT ? (int)max(cut_start(pt->flat, c0) - (long long)layer * cum[P0.B], 0ll)
@@ -2003,7 +2005,7 @@ static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_
         set_last_error("decode attention: the scan launches more blocks on this GPU than the partial area has slots for");
         return MKV_E_INVALID;
     }
-    MKV_CUDA(launch_pdl(kern, dim3((unsigned)grid), NW * 32, SMEM, 1, true, s, ls));
+    MKV_CUDA(launch_pdl(kern, dim3((unsigned)grid), NW * 32, SMEM, 1, s, ls));
     return MKV_OK;
 }
 
@@ -2117,7 +2119,7 @@ __global__ void page_mass_clear_kernel(float* mass, size_t n)
 int32_t launch_page_mass_finish(float* mass, const float* lse, const int32_t* lens, int B, int hq, int max_pages,
                                 int page_tokens, cudaStream_t s)
 {
-    MKV_CUDA(launch_pdl(page_mass_finish_kernel, dim3(hq, B), 512, 0, 1, true, s, mass, lse, lens, hq, max_pages, page_tokens));
+    MKV_CUDA(launch_pdl(page_mass_finish_kernel, dim3(hq, B), 512, 0, 1, s, mass, lse, lens, hq, max_pages, page_tokens));
     return MKV_OK;
 }
 
@@ -2127,7 +2129,7 @@ int32_t launch_page_score(const float* mass, const int32_t* lens, int B, int hq,
     int n = 0;
     for (int h = 0; h < hq; ++h) n += (int)((head_mask >> h) & 1ull);
     if (n == 0) return MKV_E_INVALID;
-    MKV_CUDA(launch_pdl(page_score_kernel, dim3((max_pages + 255) / 256, B), 256, 0, 1, true, s, mass, lens, hq, max_pages,
+    MKV_CUDA(launch_pdl(page_score_kernel, dim3((max_pages + 255) / 256, B), 256, 0, 1, s, mass, lens, hq, max_pages,
                         (unsigned long long)head_mask, beta, 1.f / (float)n, score, page_tokens));
     return MKV_OK;
 }
@@ -2232,7 +2234,7 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
         int32_t rc;
         if (p->tiles > 1) {
             const size_t n = (size_t)B * p->hkv * p->group * max_pages;
-            MKV_CUDA(launch_pdl(page_mass_clear_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, 1, true, s, mass, n));
+            MKV_CUDA(launch_pdl(page_mass_clear_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, 1, s, mass, n));
             rc = p->d == 128 ? run_tensor1<128, 12, 4, 1, true, true>(p, prm, s) : run_tensor1<256, 8, 4, 1, true, true>(p, prm, s);
         } else {
             // (always with a caller's workspace, which has room for two blocks per SM)

@@ -242,8 +242,8 @@ int32_t launch_append_layers(mkv_pool* const* pools, const void* const* k, const
     }
     const mkv_pool* p = pools[0];
     dim3 grid(n, p->hkv, n_layers);
-    if (p->d == 128) MKV_CUDA(launch_pdl(append_layers_kernel<128>, grid, 64, 0, 1, true, s, A, p->hkv, p->tiles, slots));
-    else MKV_CUDA(launch_pdl(append_layers_kernel<256>, grid, 128, 0, 1, true, s, A, p->hkv, p->tiles, slots));
+    if (p->d == 128) MKV_CUDA(launch_pdl(append_layers_kernel<128>, grid, 64, 0, 1, s, A, p->hkv, p->tiles, slots));
+    else MKV_CUDA(launch_pdl(append_layers_kernel<256>, grid, 128, 0, 1, s, A, p->hkv, p->tiles, slots));
     MKV_CUDA(cudaGetLastError());
     return MKV_OK;
 }
@@ -260,17 +260,17 @@ int32_t launch_append(mkv_pool* p, const void* k, const void* v, const int32_t* 
     if (n >= kAppendRun) {
         dim3 grid((n + kPage - 1) / kPage, p->hkv);
         if (p->d == 128)
-            MKV_CUDA(launch_pdl(append_run_kernel<128>, grid, 128, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
+            MKV_CUDA(launch_pdl(append_run_kernel<128>, grid, 128, 0, 1, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
                                                         p->status_dev));
         else
-            MKV_CUDA(launch_pdl(append_run_kernel<256>, grid, 128, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
+            MKV_CUDA(launch_pdl(append_run_kernel<256>, grid, 128, 0, 1, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, n,
                                                         p->status_dev));
     } else {
         dim3 grid(n, p->hkv);
         if (p->d == 128)
-            MKV_CUDA(launch_pdl(append_kernel<128>, grid, 64, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev));
+            MKV_CUDA(launch_pdl(append_kernel<128>, grid, 64, 0, 1, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev));
         else
-            MKV_CUDA(launch_pdl(append_kernel<256>, grid, 128, 0, 1, true, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev));
+            MKV_CUDA(launch_pdl(append_kernel<256>, grid, 128, 0, 1, s, p->fp8, p->cfg.fp8_pages, p->hkv, p->tiles, ik, iv, kk, vv, slots, p->status_dev));
     }
     MKV_CUDA(cudaGetLastError());
     return MKV_OK;
@@ -951,7 +951,7 @@ static cudaError_t launch_demote_warp(mkv_pool* p, const int32_t* src, const int
     const int smem = DemoteWarp<D>::OFF_WARPS + warps * DemoteWarp<D>::BYTES;
     static_assert(DemoteWarp<D>::OFF_WARPS + kDemoteWarps * DemoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
     return launch_pdl(demote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv, p->dev.sm_count) : 1), 32 * warps,
-                      (size_t)smem, c, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv,
+                      (size_t)smem, c, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv,
                       p->tiles, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }
 
@@ -973,7 +973,7 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
     }
     if (p->tiles == 1) {
         const int c = heads_cluster(p->hkv, n, p->dev.sm_count);
-        MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
+        MKV_CUDA(launch_pdl(demote_kernel<D, false, FMT>, dim3((unsigned)n * c), D, 0, c, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, 1, p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, bt,
                                   tags, entry, n_entries, p->status_dev, (uint32_t*)nullptr));
         return MKV_OK;
@@ -985,7 +985,7 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
         // blocks per (page, head): up to a portable cluster of 8, fewer when the call fills the GPU anyway
         int cs = 8;
         while (cs > 1 && (cs > p->tiles || (long long)n * p->hkv * cs > 8LL * p->dev.sm_count)) cs >>= 1;
-        MKV_CUDA(launch_pdl(demote_minmax_kernel<D>, dim3((unsigned)n * p->hkv * cs), D, 0, cs, false, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
+        MKV_CUDA(launch_pdl(demote_minmax_kernel<D>, dim3((unsigned)n * p->hkv * cs), D, 0, cs, s, (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages,
                                   p->cfg.tq3_pages, p->hkv, p->tiles, p->cfg.v_scale, src, dst));
     }
     const int ch = heads_cluster(p->hkv, 0, p->dev.sm_count);
@@ -993,13 +993,13 @@ static int32_t launch_demote_d(mkv_pool* p, const int32_t* src, const int32_t* d
         MKV_CUDA((launch_demote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
                                                    fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
     else
-        MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv, p->dev.sm_count)), D, 0, ch, false, s,
+        MKV_CUDA(launch_pdl(demote_kernel<D, true, FMT>, dim3((unsigned)n * ch, tile_rows(p->tiles, n, p->hkv, p->dev.sm_count)), D, 0, ch, s,
                                    (const uint8_t*)p->fp8, p->tq3, p->cfg.fp8_pages, p->cfg.tq3_pages, p->hkv, p->tiles,
                                    p->cfg.k_scale, p->cfg.v_scale, p->sigma, src, dst, fused ? bt : (int32_t*)nullptr,
                                    fused ? tags : (uint8_t*)nullptr, fused ? entry : (const int64_t*)nullptr,
                                    fused ? n_entries : (int64_t)0, p->status_dev, fused ? page_tickets(p) : (uint32_t*)nullptr));
     if (entry && !fused) {
-        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, true, s, n, src, dst, p->cfg.fp8_pages, p->cfg.tq3_pages, bt, tags, entry,
+        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, s, n, src, dst, p->cfg.fp8_pages, p->cfg.tq3_pages, bt, tags, entry,
                                                        n_entries, MKV_TAG_STALE, p->status_dev));
         MKV_CUDA(cudaGetLastError());
     }
@@ -1028,11 +1028,8 @@ static cudaError_t launch_promote_warp(mkv_pool* p, const int32_t* src, const in
     const int smem = PromoteWarp<D>::OFF_WARPS + warps * PromoteWarp<D>::BYTES;
     static_assert(PromoteWarp<D>::OFF_WARPS + kDemoteWarps * PromoteWarp<D>::BYTES <= 48 * 1024, "no opt-in needed");
     const float ik = 1.0f / p->cfg.k_scale, iv = 1.0f / p->cfg.v_scale, rs = (float)(1.0 / sqrt((double)p->d));
-    // long pages that give every SM its 16 warps and more are placed early: there is no SM to crowd on, and the launch is
-    // hidden (9 pages of 1,792 tokens, d = 256, 4 heads, back to back: about 4 us of 22)
-    const bool early = BIG && (long long)n * p->hkv * p->tiles >= 16ll * p->dev.sm_count;
     return launch_pdl(promote_warp_kernel<D, FMT, BIG>, dim3((unsigned)n * c, BIG ? warp_tile_rows(p->tiles, n, p->hkv, p->dev.sm_count) : 1),
-                      32 * warps, (size_t)smem, c, early, s, (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages,
+                      32 * warps, (size_t)smem, c, s, (const uint8_t*)p->tq3, p->fp8, p->cfg.tq3_pages, p->cfg.fp8_pages,
                       p->hkv, p->tiles, ik, iv, rs, p->sigma, src, dst, bt, tags, entry, n_entries, p->status_dev, tickets);
 }
 
@@ -1048,7 +1045,7 @@ static int32_t launch_promote_d(mkv_pool* p, const int32_t* src, const int32_t* 
     MKV_CUDA((launch_promote_warp<D, FMT, true>(p, src, dst, n, fused ? bt : nullptr, fused ? tags : nullptr,
                                                 fused ? entry : nullptr, fused ? n_entries : 0, fused ? page_tickets(p) : nullptr, s)));
     if (entry && !fused) {
-        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, true, s, n, src, dst, p->cfg.tq3_pages,
+        MKV_CUDA(launch_pdl(publish_kernel, dim3((n + 127) / 128), 128, 0, 1, s, n, src, dst, p->cfg.tq3_pages,
                             p->cfg.fp8_pages, bt, tags, entry, n_entries, MKV_TAG_ANCHOR, p->status_dev));
     }
     return MKV_OK;
@@ -1076,7 +1073,7 @@ __global__ void set_anchor_kernel(uint8_t* tags, int64_t entry, int flag, uint32
 
 int32_t launch_set_anchor(mkv_pool* p, uint8_t* tags, int64_t entry, int flag, cudaStream_t s)
 {
-    MKV_CUDA(launch_pdl(set_anchor_kernel, dim3(1), 1, 0, 1, true, s, tags, entry, flag, p->status_dev));
+    MKV_CUDA(launch_pdl(set_anchor_kernel, dim3(1), 1, 0, 1, s, tags, entry, flag, p->status_dev));
     MKV_CUDA(cudaGetLastError());
     return MKV_OK;
 }

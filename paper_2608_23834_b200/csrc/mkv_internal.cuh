@@ -101,27 +101,30 @@ struct mkv_seq {
 };
 
 namespace mkv {
-// Programmatic dependent launch.  A kernel launched with `early` may start while the kernel before it in the stream is
-// still running, and begins with pdl_begin(): it lets the kernel behind it start in turn and then waits until everything
-// before it has completed and is visible.  What a kernel does not need to wait for (its launch, shared-memory set-up)
-// then overlaps its predecessor: an append + decode pair of a small call takes 2 us less.  Order and visibility are
+// Programmatic dependent launch.  A kernel launched with launch_pdl may start while the kernel before it in the stream is
+// still running: as soon as all of that kernel's blocks have said so (pdl_let_next_start) or ended.  It waits (pdl_wait)
+// until everything before it has completed and is visible; what it does not need to wait for (its launch, shared-memory
+// set-up) then overlaps its predecessor: an append + decode pair of a small call takes 2 us less.  Order and visibility are
 // those of ordinary stream order -- for coherent loads.  Such a kernel lives while its predecessor still writes, so the
 // memory it reads is not read-only for its lifetime: no const __restrict__ and no __ldg on anything that an earlier
 // kernel may have written (arenas, ids, entries, slots, page scales).  The CUDA-core and tensor-memory variants of the
 // scan are ordinary launches.
+// Most kernels let the next one start at once (pdl_begin).  The scan does so when its blocks have done all but the merges:
+// blocks of a Demote or Promote that come while it still holds most SMs crowd on the first SMs that it leaves, up to four on one
+// SM, and wait there (one page between decode scans, d 256: Demote 40 us, ordinary launch 20).  Behind the late
+// signal they find the SMs free and their launch is hidden: Promote of 1,023 pages back to back 16.6 -> 14.3 us, 20 pages 6.4 -> 4.6,
+// Demote of 20 pages 8.4 -> 6.1, a page of each between scans 1.5 to 2.5 us less, steps of a small batch 1.8 to 2.8.
+__device__ __forceinline__ void pdl_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin()
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_let_next_start();
+    pdl_wait();
 }
 
-// early: start before the predecessor has ended.  Not for Demote and most calls of Promote: their blocks would be placed while the
-// predecessor still holds most SMs, up to four on one SM, and wait there, and behind a decode scan that has evicted
-// their code they start on it together: one page between decode calls, d = 256, 4 heads, Demote 40 -> 20 us, Promote
-// 15 -> 8 us without; 148 pages 37 -> 23 and 16 -> 10.5 us.
 // cluster: blocks per thread-block cluster along x (1: none)
 template <typename Kernel, typename... Args>
-static cudaError_t launch_pdl(Kernel kernel, dim3 grid, int threads, size_t smem, int cluster, bool early, cudaStream_t s,
+static cudaError_t launch_pdl(Kernel kernel, dim3 grid, int threads, size_t smem, int cluster, cudaStream_t s,
                               const Args&... args)
 {
     cudaLaunchConfig_t cfg = {};
@@ -131,10 +134,8 @@ static cudaError_t launch_pdl(Kernel kernel, dim3 grid, int threads, size_t smem
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     unsigned n = 0;
-    if (early) {
-        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[n++].val.programmaticStreamSerializationAllowed = 1;
-    }
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
     if (cluster > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
         attr[n].val.clusterDim.x = (unsigned)cluster;

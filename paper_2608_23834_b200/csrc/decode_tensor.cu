@@ -2012,17 +2012,16 @@ static int32_t run_tensor_fmt(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_
 // The pool's record format selects the instantiation, and for 16-token pages its group: groups of at most four query
 // heads use two column halves (see PFrag).  Not for long pages: their code sums stay in the tensor core's accumulators
 // over many tiles, and the split changes their rounding there.  GROUPS: which groups the caller sends here.
-enum Groups { kAnyGroup, kUpToFour, kMoreThanFour };
+enum Groups { kAnyGroup, kMoreThanFour };
 template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false, int MAXL = 1, bool FLAT = false, Groups GROUPS = kAnyGroup>
 static int32_t run_tensor(mkv_pool* p, const LayerSet<MAXL>& ls, cudaStream_t s)
 {
     if constexpr (!TILED && GROUPS != kMoreThanFour)
-        if (GROUPS == kUpToFour || p->group <= 4)
+        if (p->group <= 4)
             return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, true>(p, ls, s)
                                : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, true>(p, ls, s);
-    if constexpr (GROUPS != kUpToFour)
-        return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, false>(p, ls, s)
-                           : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, false>(p, ls, s);
+    return p->fmt == 2 ? run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 2, FLAT, false>(p, ls, s)
+                       : run_tensor_fmt<D, NW, NSTAGE, MINB, SCORED, TILED, MAXL, 1, FLAT, false>(p, ls, s);
 }
 
 template <int D, int NW, int NSTAGE, int MINB, bool SCORED = false, bool TILED = false>
@@ -2167,7 +2166,7 @@ static bool two_blocks(const mkv_pool* p, int B, int max_blocks)
     return max_blocks >= 2 * p->dev.sm_count && (p->d == 128 || B * p->hkv >= 32);
 }
 
-constexpr int kRowsOfTwoBlocks = 96;     // several layers laid end to end, d = 256
+constexpr int kRowsOfTwoBlocks = 64;     // several layers laid end to end
 
 // Decode attention of several layers in one launch: layer i reads pool[i], q[i], bt[i], tags[i] and writes
 // out[i], lse[i] (or none), with its own workspace ws[i]; the requests (lens, B, max_pages, scale) are common.
@@ -2195,17 +2194,20 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
     if (p0->tiles > 1)
         return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, true, kMaxLayers>(p0, ls, s)
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
-    // Two blocks of half the warps per SM: one's set-up, reduction and merge overlap the other's pages (16 layers x 2 x
-    // 59,008 tokens, d 256: 540 -> 510 us; x 4 x 700..3,001: 86 -> 77 us).  Not at d = 128 with more than four query heads
-    // per KV head (16 layers x 4 x 16,000 tokens, 1 head: 56 -> 60 us; both shapes spill alike there), and not at d = 256 with
-    // few rows, whose partials four warps take longer to merge (64 rows, 16 layers x 1 x 4,000 tokens: 48.6 -> 51 us; the
-    // 128 rows above gain, and the line was set between the two).
-    if (n_layers >= kMinFlatLayers)
-        return p0->d == 128 ? (p0->group > 4 ? run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true, kMoreThanFour>(p0, ls, s)
-                                             : run_tensor<128, 8, 4, 2, false, false, kMaxLayers, true, kUpToFour>(p0, ls, s))
-                            : (n_layers * B * p0->hkv < kRowsOfTwoBlocks
-                                   ? run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s)
-                                   : run_tensor<256, 4, 4, 2, false, false, kMaxLayers, true>(p0, ls, s));
+    // Two blocks of half the warps per SM from 64 rows on: one's set-up, reduction and merge overlap the other's pages, but few
+    // rows have partials that four warps take longer to merge.  d 256, us with one block and with two: 16 layers x 2 x 59,008
+    // tokens 540 / 510, 4 x 4 x 20,000 (64 rows) 109.0 / 102.7, 16 x 1 x 30,000 (64) 155 / 143.5, 16 x 1 x 4,000 (64) both 33.6, 4 x 1 x
+    // 3,000 (16) 17.7 / 21.2; d 128, eight query heads: 16 x 8 x 512..16,384 (512) 132 / 127.6, 16 x 2 x 2,000 (128) 24.5 / 23.3, 4 x 2 x
+    // 8,000 (8) 15.1 / 17.1.  Up to four query heads at d = 128 two blocks are better at any size.  (Long pages: 16 x 1 x 4,000
+    // 45.8 / 43.0, but 16 x 2 x 59,008 552 / 592: two blocks leave room for rounds of 32 tiles only.)
+    if (n_layers >= kMinFlatLayers) {
+        const bool two = n_layers * B * p0->hkv >= kRowsOfTwoBlocks;
+        if (p0->d == 256)
+            return two ? run_tensor<256, 4, 4, 2, false, false, kMaxLayers, true>(p0, ls, s)
+                       : run_tensor<256, 8, 4, 1, false, false, kMaxLayers, true>(p0, ls, s);
+        if (two || p0->group <= 4) return run_tensor<128, 8, 4, 2, false, false, kMaxLayers, true>(p0, ls, s);
+        return run_tensor<128, 16, 4, 1, false, false, kMaxLayers, true, kMoreThanFour>(p0, ls, s);
+    }
     // as a call of one layer (the results are the same bits); a workspace has room for two blocks per SM
     if (p0->d == 128) return run_tensor<128, 8, 4, 2, false, false, kMaxLayers>(p0, ls, s);
     return two_blocks(p0, B, kMaxCtas) ? run_tensor<256, 4, 4, 2, false, false, kMaxLayers>(p0, ls, s)

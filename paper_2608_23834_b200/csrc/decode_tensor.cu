@@ -433,35 +433,30 @@ __device__ __forceinline__ void build_partition(Partition* pt, const int* cum, c
                    (long long)pages * rows < 2ll * straddle * grid * grid) ? 1 : 0;
     auto row_pages = [&](int b) { return (int)((unsigned)(lens[b] + kPage - 1) / kPage); };
     if (aligned) {
-        // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_page(r) / W);
+        // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_position(r) / W);
         // every row must end up with at least one block, otherwise the linear cut is used
         int bad = 0;
         const float scale = (float)grid / (float)W;
-        for (int r = lane; r <= rows; r += 32) {
-            int first = W;                                      // r == rows: one past the last row
-            if (r < rows) {
-                const int b = small_div(r, hkv);
-                first = cum[b] + (r - b * hkv) * (row_pages(b) + row_cost);
-            }
-            pt->base[r] = r == rows ? grid : (int)((float)first * scale + 0.5f);
-        }
-        __syncwarp();
-        int mine = -1;
         for (int r = lane; r < rows; r += 32) {
-            const int b = small_div(r, hkv), c0 = pt->base[r], c1 = pt->base[r + 1];
-            if (cum[b + 1] > cum[b] && c1 <= c0) bad = 1;
-            if (c0 <= me && me < c1) mine = r;
+            const int b = small_div(r, hkv), n = row_pages(b), len = n > 0 ? n + row_cost : 0;
+            const int first = cum[b] + (r - b * hkv) * len;
+            const int c0 = (int)((float)first * scale + 0.5f), c1 = r + 1 == rows ? grid : (int)((float)(first + len) * scale + 0.5f);
+            pt->base[r] = c0;
+            if (n > 0 && c1 <= c0) bad = 1;
+            if (c0 <= me && me < c1) {                          // the one lane that holds this block's row
+                const Cut row = cut_row(n, c1 - c0);
+                const int j = me - c0;
+                pt->start = first + (j > 0 ? row_cost + (int)cut_start(row, j) : 0);
+                pt->end = first + row_cost + (int)cut_start(row, j + 1);
+                pt->first_b = b;
+            }
+        }
+        if (lane == 0) {
+            pt->base[rows] = grid;
+            if (me >= grid) pt->start = pt->end = 0;
         }
         if (__any_sync(FULL, bad)) aligned = 0;
-        else if (mine >= 0) {                                   // the one lane that holds this block's row
-            const int b = small_div(mine, hkv), n = row_pages(b), row_start = cum[b] + (mine - b * hkv) * (n + row_cost);
-            const Cut row = cut_row(n, pt->base[mine + 1] - pt->base[mine]);
-            const int j = me - pt->base[mine];
-            pt->start = row_start + (j > 0 ? row_cost + (int)cut_start(row, j) : 0);
-            pt->end = row_start + row_cost + (int)cut_start(row, j + 1);
-            pt->first_b = b;
-        }
-        if (aligned && me >= grid && lane == 0) pt->start = pt->end = 0;
+        __syncwarp();
     }
     if (!aligned) {
         if (me < grid) {

@@ -134,7 +134,7 @@ demote_warp_kernel(const uint8_t* fp8, uint8_t* __restrict__ tq3, int fp8_pages,
         hb[t][0] = h16_pair(4 * tq, 4 * tq + 1, n);
         hb[t][1] = h16_pair(4 * tq + 2, 4 * tq + 3, n);
     }
-    pdl_begin();
+    pdl_wait();
     __syncthreads();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < fp8_pages && dst >= 0 && dst < tq3_pages;
@@ -478,6 +478,7 @@ demote_warp_kernel(const uint8_t* fp8, uint8_t* __restrict__ tq3, int fp8_pages,
         }
     }
 
+    pdl_let_next_start();                   // (not sooner: see launch_pdl)
     // copy-before-publish, as in demote_kernel
     cluster_barrier();
     if (valid && crank == 0 && tid == 0 && entry_index != nullptr && (__threadfence(), last_cluster_of_page(page_tickets, page))) {

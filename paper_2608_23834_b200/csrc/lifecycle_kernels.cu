@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(D) demote_kernel(const uint8_t* fp8, uint8_t* 
 
     const int csize = (int)cluster_size(), crank = (int)cluster_rank();
     const int page = blockIdx.x / csize, tid = threadIdx.x, lane = tid & 31;
-    pdl_begin();
+    pdl_wait();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < fp8_pages && dst >= 0 && dst < tq3_pages;
     if (!valid && tid == 0 && crank == 0 && blockIdx.y == 0) atomicOr(status, kStBounds);
@@ -768,6 +768,7 @@ __global__ void __launch_bounds__(D) demote_kernel(const uint8_t* fp8, uint8_t* 
     // barrier (release / acquire) orders the record stores of every thread of the cluster before what the
     // publishing thread does next, and that thread's fence is cumulative: it orders them, device-wide, before its
     // own later stores.  (A fence in every thread would say the same and make each of them wait for its stores.)
+    pdl_let_next_start();                   // (not sooner: see launch_pdl)
     cluster_barrier();
     if (valid && crank == 0 && tid == 0 && entry_index != nullptr && (__threadfence(), last_cluster_of_page(page_tickets, page))) {
         const int64_t e = entry_index[page];
@@ -829,7 +830,7 @@ __global__ void __launch_bounds__(D) demote_minmax_kernel(const uint8_t* fp8, ui
     __shared__ float part[2][D];
     const int csize = (int)cluster_size(), crank = (int)cluster_rank();
     const int unit = blockIdx.x / csize, page = unit / hkv, h = unit % hkv, c = threadIdx.x;
-    pdl_begin();
+    pdl_wait();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < fp8_pages && dst >= 0 && dst < tq3_pages;      // flagged by demote_kernel
     const uint8_t* page8 = fp8 + ((size_t)(valid ? src : 0) * hkv + h) * fp8_page_bytes(D, tiles);
@@ -864,6 +865,7 @@ __global__ void __launch_bounds__(D) demote_minmax_kernel(const uint8_t* fp8, ui
     }
     part[0][c] = mn;
     part[1][c] = mx;
+    pdl_let_next_start();                   // (not sooner: see launch_pdl)
     cluster_barrier();
     if (crank == 0 && valid) {
         for (int k = 1; k < csize; ++k) {

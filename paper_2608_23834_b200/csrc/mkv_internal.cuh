@@ -109,13 +109,13 @@ namespace mkv {
 // memory it reads is not read-only for its lifetime: no const __restrict__ and no __ldg on anything that an earlier
 // kernel may have written (arenas, ids, entries, slots, page scales).  The CUDA-core and tensor-memory variants of the
 // scan are ordinary launches.
-// Most kernels let the next one start at once (pdl_begin).  Demote does so when its records are written: blocks placed while a grid of
-// about one block per SM still runs lie unevenly (12 pages of 1,792 tokens, d 256, 2 heads, back to back 29.5 -> 33 us, 120 pages
-// of 16 tokens 8.4 -> 9.2).  The scan does so when its blocks have done all but the merges:
+// Most kernels let the next one start at once (pdl_begin).  Demote and Promote do so when their records are written: blocks placed while a
+// grid of about one block per SM still runs lie unevenly (Demote of 12 pages of 1,792 tokens, d 256, 2 heads, back to back 29.5 -> 33
+// us, 120 pages of 16 tokens 8.4 -> 9.2; Promote of 700 pages, d 128, 8 heads, 12.8 us so and 11.2 with the late signal).  The scan does so when its blocks have done all but the merges:
 // blocks of a Demote or Promote that come while it still holds most SMs crowd on the first SMs that it leaves, up to four on one
 // SM, and wait there (one page between decode scans, d 256: Demote 40 us, ordinary launch 20).  Behind the late
-// signal they find the SMs free and their launch is hidden: Promote of 1,023 pages back to back 16.6 -> 14.3 us, 20 pages 6.4 -> 4.6,
-// Demote of 20 pages 8.4 -> 6.1, a page of each between scans 1.5 to 2.5 us less, steps of a small batch 1.8 to 2.8.
+// signal they find the SMs free and their launch is hidden: Promote of 1,023 pages back to back 16.7 -> 14.1 us, 300 pages 9.2 -> 7.5,
+// Demote of 20 pages 8.4 -> 5.8, a page of each between scans 1.5 to 2.5 us less, steps of a small batch 1.8 to 2.8.
 __device__ __forceinline__ void pdl_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin()

@@ -107,7 +107,7 @@ promote_warp_kernel(const uint8_t* tq3, uint8_t* __restrict__ fp8, int tq3_pages
         hb[t][0] = FMT == 2 ? h16_unit_pair(4 * tq, 4 * tq + 1, n) : h16_unit_pair(2 * tq, 2 * tq + 1, n);
         hb[t][1] = FMT == 2 ? h16_unit_pair(4 * tq + 2, 4 * tq + 3, n) : h16_unit_pair(2 * tq + 8, 2 * tq + 9, n);
     }
-    pdl_begin();
+    pdl_wait();
     __syncthreads();
     const int src = src_ids[page], dst = dst_ids[page];
     const bool valid = src >= 0 && src < tq3_pages && dst >= 0 && dst < fp8_pages;
@@ -300,6 +300,7 @@ promote_warp_kernel(const uint8_t* tq3, uint8_t* __restrict__ fp8, int tq3_pages
         }
     }
 
+    pdl_let_next_start();                   // (not sooner: see launch_pdl)
     // copy-before-publish, as in demote_kernel
     cluster_barrier();
     if (valid && crank == 0 && tid == 0 && entry_index != nullptr && (__threadfence(), last_cluster_of_page(page_tickets, page))) {

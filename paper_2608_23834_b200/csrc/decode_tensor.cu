@@ -2155,7 +2155,7 @@ static DecodeParams make_params(mkv_pool* p, const void* q, const int32_t* bt, c
 // Two blocks of half the warps per SM instead of one: the set-up, reduction and merge of one overlap the pages of the
 // other, which pays the more rows a block meets (d 128, 8 x 4 heads: 64 ragged requests 632 -> 579 us, 8 x 4,096 tokens
 // 30.7 -> 23.6 us).  At d = 256 a merge by four warps costs more, and few rows have many partials: from 32 rows (8 x
-// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows: 71 -> 76 us).  Partial areas for one block per SM only take one.
+// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows of 8,000 and 30,000: 20.9 -> 24.4, 47.6 -> 49.4).  Partial areas for one block per SM only take one.
 static bool two_blocks(const mkv_pool* p, int B, int max_blocks)
 {
     return max_blocks >= 2 * p->dev.sm_count && (p->d == 128 || B * p->hkv >= 32);

@@ -32,6 +32,7 @@
 #include <cstdlib>
 #include <mutex>
 
+#include "decode_cut.cuh"
 #include "mkv_internal.cuh"
 
 namespace mkv {
@@ -316,214 +317,6 @@ __device__ __forceinline__ void affine_accumulate(float (&acc)[4], const float (
     acc[1] = fmaf(sc.x, t[1], fmaf(zp.x, ps1, acc[1]));
     acc[2] = fmaf(sc.y, t[2], fmaf(zp.y, ps0, acc[2]));
     acc[3] = fmaf(sc.y, t[3], fmaf(zp.y, ps1, acc[3]));
-}
-
-// ------------------------------------------------------------------------------------------------
-// Work partition (the scan and the merge of split rows use the same cut)
-// ------------------------------------------------------------------------------------------------
-// Work = (request, KV head, page) triples in row-major order; cum[b] = position of the first triple of
-// request b.  A row of n pages takes row_cost + n positions: opening, reducing and storing a row (or a block's part of it)
-// costs a block as much time as row_cost pages, so that a block with many short rows gets fewer pages.  (64 requests of 1,024 to
-// 131,072 tokens, 8 heads: the blocks with the shortest requests took 520 us against 406 on average; 524 -> 480 us a step with
-// 32, the same with 48, 503 with 16.  16 layers x 4 x 700..3,001 tokens, d 256: 64.0 -> 60 with 16, 62 with 32, 66 with 48.
-// 16 layers x 8 x 512..16,384, one block of 16 warps per SM: 151 -> 139 with 32, 134 with 48, 136 with 64.)  Two ways to cut it into one contiguous range per block:
-//   row-aligned (few rows: B * hkv <= grid / 4): every row gets a whole number of blocks in proportion
-//     to its pages (cumulative rounding), so that no block straddles two rows and pays the per-row set-up
-//     and reduction twice;
-//   linear (many rows): grid equal ranges that may cross row boundaries.
-constexpr int kMaxAlignedRows = kMaxCtas / 4;
-
-//   flat (several layers): a linear cut of all layers' triples, the layers laid end to end.
-//
-// Every block works this out for itself before its first page can be asked for, so the arithmetic is kept short: one
-// 32-bit division per cut (quotient and remainder; block c starts at quo c + min(c, rem)), and warp 0 leaves the
-// block's own range and request in shared memory.  (With W c / blocks in 64 bits, a binary search for the row, a serial one for the
-// request and the strides that page_at replaces, the time up to a block's first page was 11,600 cycles at 8 x 16,384 tokens, d 128,
-// and 18,900 in the flat cut of 16 layers x 16 rows, d 256; it is 8,400 and 10,100: 36.5 -> 34.3 and 75.6 -> 66.3 us a step, and
-// 650 -> 552 for 16 layers of long pages, where every tile asks which warp's run it opens.)
-struct Cut {
-    long long quo;
-    int rem, blocks;                    // blocks that get work (0: none)
-};
-
-struct Partition {
-    Cut flat;                           // flat: all layers' triples
-    Cut cut;                            // linear cut of one layer
-    int aligned;                        // 1: row-aligned, 0: linear
-    int start, end;                     // this block's range in the per-layer cut
-    int first_layer, end_layer;         // this block's layers in the flat cut
-    int first_b;                        // request of the block's first triple
-    int base[kMaxAlignedRows + 1];      // row-aligned: first block of every row
-};
-
-// a / b for 0 <= a < 2^20: (a + 1/2) / b is at least 1 / (2 b) away from the next integer, the approximate quotient less far off
-__device__ __forceinline__ int small_div(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
-
-// Blocks that share W positions, `pages` of them pages: all of the grid, but no more than give every block min_pages pages (a page
-// per warp of an SM: below that a row's partials cost more to merge than the spreading saves).
-__device__ __forceinline__ Cut make_cut(long long W, long long pages, int grid, int min_pages)
-{
-    Cut c;
-    if (W >> 31 == 0) {
-        const unsigned w = (unsigned)W, most = ((unsigned)pages + min_pages - 1) / (unsigned)min_pages;
-        c.blocks = (int)min(most, (unsigned)grid);
-        const unsigned q = c.blocks ? w / (unsigned)c.blocks : 0u;
-        c.quo = q;
-        c.rem = (int)(w - q * (unsigned)c.blocks);
-    } else {
-        c.blocks = grid;
-        c.quo = W / grid;
-        c.rem = (int)(W - c.quo * grid);
-    }
-    return c;
-}
-
-__device__ __forceinline__ long long cut_start(const Cut& c, int block) { return c.quo * block + min(block, c.rem); }
-
-// the block that holds triple x
-__device__ __forceinline__ int cut_block_of(const Cut& c, long long x)
-{
-    const long long split = (c.quo + 1) * c.rem;          // the first `rem` blocks have one more; quo >= 1 where a triple exists
-    int b = x < split ? (int)__fdividef((float)x, (float)(c.quo + 1)) : c.rem + (int)__fdividef((float)(x - split), (float)c.quo);
-    b = min(b, c.blocks - 1);                             // near, then exact
-    while (b + 1 < c.blocks && cut_start(c, b + 1) <= x) ++b;
-    while (b > 0 && cut_start(c, b) > x) --b;
-    return b;
-}
-
-// a row of n pages (at most 65,535) over k whole blocks
-__device__ __forceinline__ Cut cut_row(int n, int k)
-{
-    Cut c;
-    c.blocks = k;
-    const int q = small_div(n, k);
-    c.quo = q;
-    c.rem = n - q * k;
-    return c;
-}
-
-// Request that holds triple x of a layer: the number of requests that end at or before it.  All 32 lanes of a warp.
-__device__ __forceinline__ int request_of(const int* cum, int B, int x, int lane)
-{
-    int b = 0;
-    for (int b0 = 0; b0 < B; b0 += 32) {
-        const uint32_t m = __ballot_sync(0xffffffffu, b0 + lane < B && cum[b0 + lane + 1] <= x);
-        b += __popc(m);
-        if (m != 0xffffffffu) break;
-    }
-    return b;
-}
-
-// Called by warp 0 (all 32 lanes) after cum[] and lens[] are complete; other warps wait at the next barrier.
-__device__ __forceinline__ void build_partition(Partition* pt, const int* cum, const int* lens, int B, int hkv, int grid,
-                                                int pages, int row_cost, int min_pages, int straddle, int me, int lane)
-{
-    constexpr uint32_t FULL = 0xffffffffu;
-    const int W = cum[B], rows = B * hkv;
-    const Cut cut = make_cut(W, pages, grid, min_pages);
-    grid = cut.blocks;
-    int start = 0, end = 0;                             // every request of the call is empty, or more blocks than work
-    // With k blocks per row the rows that get one block fewer run 1/k longer, but a block that straddles two rows
-    // pays the per-row set-up, reduction and partial twice (about 8 us, a quarter of a block's pages at config-1
-    // sizes).  Measured: from four blocks per row on, whole blocks per row win (16 rows: 71 -> 66 us, 32 rows: 74 -> 71).
-    // The rounding to whole blocks costs about half a block's share in k of a block's pages, pages rows / (2 grid^2); from
-    // `straddle` pages on that is dearer than the straddling (d 128, 8 heads, two blocks per SM: 8 x 4,096 tokens 28.9 us linear,
-    // 23.6 aligned; 8 x 32,768 of which half FP8 104.7 linear, 108 aligned).
-    int aligned = (rows * 4 <= grid && rows <= kMaxAlignedRows && pages >= grid &&
-                   (long long)pages * rows < 2ll * straddle * grid * grid) ? 1 : 0;
-    auto row_pages = [&](int b) { return (int)((unsigned)(lens[b] + kPage - 1) / kPage); };
-    if (aligned) {
-        // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_position(r) / W);
-        // every row must end up with at least one block, otherwise the linear cut is used
-        int bad = 0;
-        const float scale = (float)grid / (float)W;
-        for (int r = lane; r < rows; r += 32) {
-            const int b = small_div(r, hkv), n = row_pages(b), len = n > 0 ? n + row_cost : 0;
-            const int first = cum[b] + (r - b * hkv) * len;
-            const int c0 = (int)((float)first * scale + 0.5f), c1 = r + 1 == rows ? grid : (int)((float)(first + len) * scale + 0.5f);
-            pt->base[r] = c0;
-            if (n > 0 && c1 <= c0) bad = 1;
-            if (c0 <= me && me < c1) {                          // the one lane that holds this block's row
-                const Cut row = cut_row(n, c1 - c0);
-                const int j = me - c0;
-                pt->start = first + (j > 0 ? row_cost + (int)cut_start(row, j) : 0);
-                pt->end = first + row_cost + (int)cut_start(row, j + 1);
-                pt->first_b = b;
-            }
-        }
-        if (lane == 0) {
-            pt->base[rows] = grid;
-            if (me >= grid) pt->start = pt->end = 0;
-        }
-        if (__any_sync(FULL, bad)) aligned = 0;
-        __syncwarp();
-    }
-    if (!aligned) {
-        if (me < grid) {
-            start = (int)cut_start(cut, me);
-            end = (int)cut_start(cut, me + 1);
-        }
-        const int b = request_of(cum, B, start, lane);
-        if (lane == 0) {
-            pt->start = start;
-            pt->end = end;
-            pt->first_b = b;
-        }
-    }
-    if (lane == 0) {
-        pt->aligned = aligned;
-        pt->cut = cut;
-    }
-}
-
-// first triple of block c in the per-layer cut; row_start, n: the row of which block c is the first block
-__device__ __forceinline__ int layer_start_of_first_block(const Partition* pt, int c, int row_start)
-{
-    return pt->aligned ? row_start : (int)cut_start(pt->cut, c);
-}
-
-// Whether position x of the row [row_start, row_end) (row index r) opens the run of some warp in the per-layer cut
-// with n_warps warps per block.
-__device__ __forceinline__ bool opens_warp_run(const Partition* pt, int r, int row_start, int row_end, int x, unsigned n_warps)
-{
-    int first, n;                                   // the block's share of the row
-    if (pt->aligned) {
-        const Cut row = cut_row(row_end - row_start, pt->base[r + 1] - pt->base[r]);
-        const int j = cut_block_of(row, x - row_start);
-        first = row_start + (int)cut_start(row, j);
-        n = row_start + (int)cut_start(row, j + 1) - first;
-    } else {
-        const int c = cut_block_of(pt->cut, x);
-        first = max((int)cut_start(pt->cut, c), row_start);
-        n = min((int)cut_start(pt->cut, c + 1), row_end) - first;
-    }
-    const unsigned w = ((unsigned)(x - first + 1) * n_warps - 1) / (unsigned)n;
-    return (int)((unsigned)n * w / n_warps) == x - first;
-}
-
-// blocks c0..c1 that hold pages of the row with index r, whose first page is at row_start and whose last before row_end
-__device__ __forceinline__ void partition_blocks_of_row(const Partition* pt, int r, int row_start, int row_end, int& c0, int& c1)
-{
-    if (pt->aligned) {
-        c0 = pt->base[r];
-        c1 = pt->base[r + 1] - 1;
-        return;
-    }
-    c0 = cut_block_of(pt->cut, row_start);
-    c1 = cut_block_of(pt->cut, row_end - 1);
-}
-
-// Pages of a row are visited in an order that gives every contiguous range of positions the row's FP8 and TQ3 pages in
-// their overall proportion (spans of either format are contiguous), so that equal ranges cost equal time.  The row is cut into 32
-// strips of equal length (the first n % 32 are one page longer); position x is page x / 32 of strip x % 32, the strips
-// in bit-reversed order, and the pages that the longer strips have more come last.  A bijection without a division.  (Before: x
-// times a stride near 0.618 n and coprime to n, modulo n; finding it, seventeen remainders per try, kept all
-// warps waiting for 1,500 cycles.)
-__device__ __forceinline__ int page_at(int x, int n)
-{
-    const int len = n >> 5, longer = n & 31, at = x >> 5;
-    const int strip = at < len ? (int)(__brev((unsigned)x) >> 27) : x & 31;
-    return strip * len + min(strip, longer) + at;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1205,8 +998,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
     // 16-byte loads that a thread of the merge keeps in flight, within the registers of the launch shape
     constexpr int MERGE_LOADS = NW * MINB <= 8 ? 20 : 16;
-    // what a row costs besides its pages, in pages: more warps scan more of them in that time.  Long pages come in few rows.
-    constexpr int ROW_COST = TILED ? 0 : 8 + 3 * NW;
+    constexpr int ROW_COST = cut_row_cost(NW, TILED), MIN_PAGES = cut_min_pages(NW, MINB);
     using G = Geo<D, NW, NSTAGE, TILED>;     // pages of several tiles: short rounds leave room for the parked rows
     constexpr int NB = G::NB;
     constexpr uint32_t FULL = 0xffffffffu;
@@ -1242,48 +1034,19 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     }
     pdl_wait();
     if (warp == 0) {
-        int run = 0, used = 0;                             // requests with tokens
+        RowSums sum = {0, 0};
         for (int b0 = 0; b0 < P0.B; b0 += 32) {
             const int b = b0 + lane;
-            int n = 0;
-            if (b < P0.B) {
-                const int len = length_of(b);
-                lens_s[b] = len;
-                n = len > 0 ? ((len + kPage - 1) / kPage + ROW_COST) * hkv : 0;
-            }
-            used += __popc(__ballot_sync(FULL, n > 0));
-            int inc = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, inc, o);
-                if (lane >= o) inc += v;
-            }
-            if (b < P0.B) cum[b] = run + inc - n;
-            run += __shfl_sync(FULL, inc, 31);
+            int len = 0;
+            if (b < P0.B) lens_s[b] = len = length_of(b);
+            add_requests(sum, cum, P0.B, hkv, ROW_COST, b0, len, lane);
         }
-        if (lane == 0) cum[P0.B] = run;
+        if (lane == 0) cum[P0.B] = sum.positions;
         __syncwarp();
+        const int pages = sum.positions - sum.requests * hkv * ROW_COST;
         if constexpr (!FLAT || TILED)
-            build_partition(pt, cum, lens_s, P0.B, hkv, gridDim.x, run - used * hkv * ROW_COST, ROW_COST, NW * MINB, 4 * NW, blockIdx.x, lane);
-        if constexpr (FLAT) {
-            const Cut cut = make_cut((long long)run * n_layers, (long long)(run - used * hkv * ROW_COST) * n_layers, gridDim.x,
-                                     NW * MINB);
-            int first = 0, end = 0, b = 0;
-            if ((int)blockIdx.x < cut.blocks) {
-                const long long s = cut_start(cut, blockIdx.x), e = cut_start(cut, blockIdx.x + 1);
-                first = min((int)__fdividef((float)s, (float)run), n_layers - 1);
-                if ((long long)first * run > s) --first;
-                if ((long long)(first + 1) * run <= s) ++first;
-                for (end = first + 1; (long long)end * run < e;) ++end;
-                b = request_of(cum, P0.B, (int)(s - (long long)first * run), lane);
-            }
-            if (lane == 0) {
-                pt->flat = cut;
-                pt->first_layer = first;
-                pt->end_layer = end;
-                pt->first_b = b;
-            }
-        }
+            build_partition(pt, cum, lens_s, P0.B, hkv, gridDim.x, pages, ROW_COST, MIN_PAGES, cut_straddle(NW), blockIdx.x, lane);
+        if constexpr (FLAT) build_flat_partition(pt, cum, P0.B, n_layers, gridDim.x, pages, MIN_PAGES, blockIdx.x, lane);
     }
     __syncthreads();
     int my_start = 0, my_end = 0;                          // more blocks than work: an empty range
@@ -1356,11 +1119,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
 
     for (int layer = layer_first; layer < layer_end; ++layer) {
     const DecodeParams& P = LS.layer[MAXL == 1 ? 0 : layer];
-    if constexpr (FLAT) {                                  // this block's range inside the layer
-        const long long w0 = (long long)layer * cum[P0.B];
-        my_start = (int)max(cut_start(pt->flat, blockIdx.x) - w0, 0ll);
-        my_end = (int)min(cut_start(pt->flat, blockIdx.x + 1) - w0, (long long)cum[P0.B]);
-    }
+    if constexpr (FLAT) range_in_layer(pt, cum[P0.B], layer, blockIdx.x, my_start, my_end);
     auto wait_slot = [&](uint32_t s) -> bool {
         if (wait_bounded(s, P.wait_ns)) return true;
         failed = true;
@@ -1371,16 +1130,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
     int b = FLAT && layer > layer_first ? 0 : pt->first_b;
     while (pos < my_end) {
         // ---- locate the segment: request b, KV head h, positions [pg0, pg0 + n_seg) of the row ------
-        while (cum[b + 1] <= pos) ++b;
-        const int len = lens_s[b], n_pages = (len + kPage - 1) / kPage;
-        const int row_len = n_pages + ROW_COST;
-        int h = (int)__fdividef((float)(pos - cum[b]), (float)row_len), off = pos - cum[b] - h * row_len;   // at most one off
-        if (off < 0) --h, off += row_len;
-        if (off >= row_len) ++h, off -= row_len;
-        const int row_start = pos - off, row_end = row_start + row_len, seg_end = min(my_end, row_end);
-        const int pg0 = max(off - ROW_COST, 0), n_seg = seg_end - row_start - ROW_COST - pg0;
+        const Segment sg = segment_at(cum, lens_s, ROW_COST, pos, my_end, b);
+        const int len = lens_s[b], h = sg.h, n_pages = sg.n_pages, pg0 = sg.pg0, n_seg = sg.n;
         if (n_seg <= 0) {                          // the block's range ends before the row's first page
-            pos = seg_end;
+            pos = sg.end;
             continue;
         }
         const int32_t* bt_row = P.bt + (size_t)b * P.max_pages;
@@ -1457,7 +1210,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                     if (kind == 0) atomicOr(P.status, kStBounds);     // never dereferenced
                     if constexpr (TILED) {   // second list: tile inside its page | logical page << 16
                         const int entry = pg / P.tiles;
-                        const bool opens = FLAT && opens_warp_run(pt, b * hkv + h, row_start, row_end, row_start + pg, NW);
+                        const bool opens = FLAT && opens_warp_run(pt, b * hkv + h, sg.row_start, sg.row_end, sg.row_start + pg, NW);
                         pg = (pg - entry * P.tiles) | (entry << 16) | (opens ? kOpens : 0);
                     }
                 }
@@ -1771,7 +1524,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 start_round();
             }
         }
-        const bool last_segment = seg_end == my_end && layer + 1 == layer_end;
+        const bool last_segment = sg.end == my_end && layer + 1 == layer_end;
         float (&oacc)[NB][4] = acc.o;
         float (&lacc)[2] = acc.l;
         float (&m_run)[2] = acc.m;
@@ -1856,9 +1609,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 P.lse[(size_t)b * hq + h * GQ + tid] = l > 0.f ? (M + log2f(l)) * kLn2 : -CUDART_INF_F;
             }
         } else {
-            // partial (m, l, O) of this block for the row; slot 2c if the segment opens the block's range (flat cut:
-            // its range in this layer), 2c + 1 otherwise
-            float* slot = P.partials + (size_t)(2 * blockIdx.x + (pos != my_start ? 1 : 0)) * (8 * D + 16);
+            float* slot = P.partials + (size_t)partial_slot(blockIdx.x, pos, my_start) * (8 * D + 16);    // (m, l, O) of this block for the row
 #pragma unroll
             for (int k = 0; k < PER_THREAD; ++k) {
                 const int i = tid + k * NW * 32, e4 = SPLIT ? 2 * i : i;
@@ -1883,14 +1634,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             // the block that is already late.  That block finds the row complete and merges it, or it leaves a
             // request (the counter's top bit) and the row's last arrival, seeing the request, merges after all.
             // Either way exactly one block merges, and it leaves the counter at zero for the next call.
-            int c0, c1;
-            if constexpr (FLAT) {                          // here the row's last arrival merges: no block is ahead of the others
-                const long long w0 = (long long)layer * cum[P0.B];
-                c0 = cut_block_of(pt->flat, w0 + row_start + ROW_COST);
-                c1 = cut_block_of(pt->flat, w0 + row_end - 1);
-            } else {
-                partition_blocks_of_row(pt, b * hkv + h, row_start + ROW_COST, row_end, c0, c1);
-            }
+            int c0, c1;                                // (flat cut: the row's last arrival merges, no block is ahead of the others)
+            blocks_of_row<FLAT>(pt, cum[P0.B], layer, b * hkv + h, sg.row_start + ROW_COST, sg.row_end, c0, c1);
             const int n_parts = c1 - c0 + 1;
             constexpr uint32_t kRequest = 0x80000000u;
             __syncthreads();
@@ -1908,10 +1653,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             const int todo = *last_s;
             if (last_segment) pdl_let_next_start();    // what is left of the block is at most a merge
             if (todo) {
-                // the row opens block c0's range of the layer where it starts at or before that range
-                const int c0_start = FLAT ? (int)max(cut_start(pt->flat, c0) - (long long)layer * cum[P0.B], 0ll)
-                                          : layer_start_of_first_block(pt, c0, row_start);
-                const int first_slot = 2 * c0 + (row_start > c0_start ? 1 : 0);
+                const int first_slot = first_partial_slot<FLAT>(pt, cum[P0.B], layer, c0, sg.row_start);
                 if constexpr (MAXL > 1 && !FLAT) {
                     if (todo & 2) {
                         const DecodeParams& Q = LS.layer[layer - 1];
@@ -1926,7 +1668,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
             }
         }
         __syncthreads();
-        pos = seg_end;
+        pos = sg.end;
     }
     }   // layers
 }

@@ -205,28 +205,20 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
     // rows 8-15 of the plain query tiles stay zero for the whole launch
     for (int i = tid; i < G::QTILES / 4; i += NT) reinterpret_cast<uint32_t*>(smem + G::OFF_QF)[i] = 0;
     if (warp == 0) {
-        int run = 0;
+        RowSums sum = {0, 0};
         for (int b0 = 0; b0 < P.B; b0 += 32) {
             const int b = b0 + lane;
-            int n = 0;
+            int len = 0;
             if (b < P.B) {
-                int len = P.lens[b];
+                len = P.lens[b];
                 if (len > P.max_pages * kPage) { atomicOr(P.status, kStBounds); len = P.max_pages * kPage; }   // a length beyond the table row is cut and flagged
-                lens_s[b] = max(len, 0);
-                n = len > 0 ? ((len + kPage - 1) / kPage) * hkv : 0;
+                lens_s[b] = len = max(len, 0);
             }
-            int inc = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, inc, o);
-                if (lane >= o) inc += v;
-            }
-            if (b < P.B) cum[b] = run + inc - n;
-            run += __shfl_sync(FULL, inc, 31);
+            add_requests(sum, cum, P.B, hkv, 0, b0, len, lane);
         }
-        if (lane == 0) cum[P.B] = run;
+        if (lane == 0) cum[P.B] = sum.positions;
         __syncwarp();
-        build_partition(pt, cum, lens_s, P.B, hkv, gridDim.x, run, 0, 1, 1 << 30, blockIdx.x, lane);
+        build_partition(pt, cum, lens_s, P.B, hkv, gridDim.x, sum.positions, 0, 1, 1 << 30, blockIdx.x, lane);
     }
     __syncthreads();
     const int my_start = pt->start, my_end = pt->end;
@@ -276,11 +268,8 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
     int pos = my_start;
     int b = pt->first_b;
     while (pos < my_end) {
-        while (cum[b + 1] <= pos) ++b;
-        const int len = lens_s[b], n_pages = (len + kPage - 1) / kPage;
-        const int h = (pos - cum[b]) / n_pages, pg0 = pos - cum[b] - h * n_pages;
-        const int row_start = cum[b] + h * n_pages, row_end = row_start + n_pages;
-        const int n_seg = min(my_end, row_end) - pos;
+        const Segment sg = segment_at(cum, lens_s, 0, pos, my_end, b);
+        const int len = lens_s[b], h = sg.h, n_pages = sg.n_pages, pg0 = sg.pg0, n_seg = sg.n;
         const int32_t* bt_row = P.bt + (size_t)b * P.max_pages;
         const uint8_t* tag_row = P.tags + (size_t)b * P.max_pages;
         const int n_rounds = (n_seg + kRoundT - 1) / kRoundT;
@@ -752,7 +741,7 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
         }
         __syncthreads();
 
-        const bool whole_row = (pos == row_start) && (pos + n_seg == row_end);
+        const bool whole_row = n_seg == n_pages;
         if (whole_row) {
             for (int e = tid; e < 8 * D; e += NT) {
                 const int head = e & 7, ch = e >> 3;
@@ -763,14 +752,14 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
             if (P.lse && tid < GQ)
                 P.lse[(size_t)b * hq + h * GQ + tid] = sm_l[tid] > 0.f ? (sm_m[tid] + log2f(sm_l[tid])) * kLn2 : -CUDART_INF_F;
         } else {
-            float* slot = P.partials + (size_t)(2 * blockIdx.x + (pos != my_start ? 1 : 0)) * (8 * D + 16);
+            float* slot = P.partials + (size_t)partial_slot(blockIdx.x, pos, my_start) * (8 * D + 16);
             for (int e = tid; e < 8 * D; e += NT) slot[e] = red[e];
             if (tid < 8) {
                 slot[8 * D + tid] = sm_m[tid];
                 slot[8 * D + 8 + tid] = sm_l[tid];
             }
             int c0, c1;
-            partition_blocks_of_row(pt, b * hkv + h, row_start, row_end, c0, c1);
+            blocks_of_row<false>(pt, cum[P.B], 0, b * hkv + h, sg.row_start, sg.row_end, c0, c1);
             const int n_parts = c1 - c0 + 1;
             __syncthreads();
             if (tid == 0) {
@@ -781,12 +770,11 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
             }
             __syncthreads();
             if (*last_s) {
-                const int first_slot = 2 * c0 + (row_start > layer_start_of_first_block(pt, c0, row_start) ? 1 : 0);
-                merge_row<D, NT, 16>(P, first_slot, 2 * c0, n_parts, red, b, h);
+                merge_row<D, NT, 16>(P, first_partial_slot<false>(pt, cum[P.B], 0, c0, sg.row_start), 2 * c0, n_parts, red, b, h);
             }
         }
         __syncthreads();
-        pos += n_seg;
+        pos = sg.end;
     }
     tc_fence_before();
     __syncthreads();

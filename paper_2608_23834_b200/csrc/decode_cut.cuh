@@ -167,7 +167,8 @@ MKV_CUT void build_partition(Partition* pt, const int* cum, const int* lens, int
                    (long long)pages * rows < 2ll * straddle * grid * grid) ? 1 : 0;
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_position(r) / W);
-        // every row must end up with at least one block, otherwise the linear cut is used
+        // every row must end up with at least one block and with no more blocks than pages (a row's share also counts
+        // row_cost; a block without a page would never arrive at the row's merge), otherwise the linear cut is used
         int bad = 0;
         const float scale = (float)grid / (float)W;
         for (int r = lane; r < rows; r += kCutLanes) {
@@ -175,7 +176,7 @@ MKV_CUT void build_partition(Partition* pt, const int* cum, const int* lens, int
             const int first = cum[b] + (r - b * hkv) * len;
             const int c0 = (int)((float)first * scale + 0.5f), c1 = r + 1 == rows ? grid : (int)((float)(first + len) * scale + 0.5f);
             pt->base[r] = c0;
-            if (n > 0 && c1 <= c0) bad = 1;
+            if (n > 0 && (c1 <= c0 || c1 - c0 > n)) bad = 1;
             if (c0 <= me && me < c1) {                          // the one lane that holds this block's row
                 const Cut row = cut_row(n, c1 - c0);
                 const int j = me - c0;

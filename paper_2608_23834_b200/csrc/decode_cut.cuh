@@ -73,15 +73,17 @@ MKV_CUT constexpr int cut_min_pages(int warps, int per_sm) { return warps * per_
 MKV_CUT constexpr int cut_straddle(int warps) { return 4 * warps; }
 
 // Pages (16-token tiles) of a request of len tokens
-MKV_CUT int pages_of(int len) { return (int)((unsigned)(len + kPage - 1) / kPage); }
+MKV_CUT int pages_of(int len) { return (len + kPage - 1) / kPage; }
 
-// Running sums over the requests, kCutLanes at a time: request b0 + lane has len tokens; all lanes get the same sums.
+// Positions of a request's rows
+MKV_CUT int positions_of(int len, int hkv, int row_cost) { return len > 0 ? (pages_of(len) + row_cost) * hkv : 0; }
+
+// Running sums over the requests, kCutLanes at a time: request b0 + lane has n positions; all lanes get the same sums.
 struct RowSums {
     int positions, requests;            // positions so far, requests with pages so far
 };
-MKV_CUT void add_requests(RowSums& sum, int* cum, int B, int hkv, int row_cost, int b0, int len, int lane)
+MKV_CUT void add_requests(RowSums& sum, int* cum, int B, int b0, int n, int lane)
 {
-    const int n = len > 0 ? (pages_of(len) + row_cost) * hkv : 0;
     sum.requests += count_lanes(n > 0);
     int inc = n;                                            // over the lanes up to this one
 #pragma unroll

@@ -1037,9 +1037,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         RowSums sum = {0, 0};
         for (int b0 = 0; b0 < P0.B; b0 += 32) {
             const int b = b0 + lane;
-            int len = 0;
-            if (b < P0.B) lens_s[b] = len = length_of(b);
-            add_requests(sum, cum, P0.B, hkv, ROW_COST, b0, len, lane);
+            int n = 0;
+            if (b < P0.B) {
+                const int len = length_of(b);
+                lens_s[b] = len;
+                n = positions_of(len, hkv, ROW_COST);
+            }
+            add_requests(sum, cum, P0.B, b0, n, lane);
         }
         if (lane == 0) cum[P0.B] = sum.positions;
         __syncwarp();

@@ -208,13 +208,14 @@ __global__ void __launch_bounds__(tm::kThreads, 1) decode_tmem_kernel(const Deco
         RowSums sum = {0, 0};
         for (int b0 = 0; b0 < P.B; b0 += 32) {
             const int b = b0 + lane;
-            int len = 0;
+            int n = 0;
             if (b < P.B) {
-                len = P.lens[b];
+                int len = P.lens[b];
                 if (len > P.max_pages * kPage) { atomicOr(P.status, kStBounds); len = P.max_pages * kPage; }   // a length beyond the table row is cut and flagged
-                lens_s[b] = len = max(len, 0);
+                lens_s[b] = max(len, 0);
+                n = positions_of(len, hkv, 0);
             }
-            add_requests(sum, cum, P.B, hkv, 0, b0, len, lane);
+            add_requests(sum, cum, P.B, b0, n, lane);
         }
         if (lane == 0) cum[P.B] = sum.positions;
         __syncwarp();

@@ -24,7 +24,7 @@ int walk(const int* lens, int B, int hkv, int grid, int n_layers, int warps, int
     const int straddle = tensor_memory ? 1 << 30 : cut_straddle(warps);
     std::vector<int> cum(B + 1);
     RowSums sum = {0, 0};
-    for (int b = 0; b < B; ++b) add_requests(sum, cum.data(), B, hkv, cost, b, lens[b], 0);
+    for (int b = 0; b < B; ++b) add_requests(sum, cum.data(), B, b, positions_of(lens[b], hkv, cost), 0);
     const int W = cum[B] = sum.positions, pages = W - sum.requests * hkv * cost;
     std::vector<std::vector<RowParts>> part(n_layers, std::vector<RowParts>(B * hkv));
     std::vector<std::vector<std::vector<char>>> seen(n_layers, std::vector<std::vector<char>>(B * hkv));

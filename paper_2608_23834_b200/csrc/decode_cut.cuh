@@ -17,6 +17,7 @@ namespace mkv {
 //     and reduction twice;
 //   linear (many rows): grid equal ranges that may cross row boundaries.
 constexpr int kMaxAlignedRows = kMaxCtas / 4;
+constexpr int kMaxBatch = 1024;         // requests per call
 
 //   flat (several layers): a linear cut of all layers' triples, the layers laid end to end.
 //
@@ -71,6 +72,15 @@ MKV_CUT int small_div(int a, int b) { return (int)near_quotient((float)a + 0.5f,
 MKV_CUT constexpr int cut_row_cost(int warps, bool long_pages) { return long_pages ? 0 : 8 + 3 * warps; }
 MKV_CUT constexpr int cut_min_pages(int warps, int per_sm) { return warps * per_sm; }
 MKV_CUT constexpr int cut_straddle(int warps) { return 4 * warps; }
+
+// Positions are counted in 32 bits: requests that one launch may take where a table row has room for `tiles` 16-token tiles, so that
+// its positions stay below 2^31.  (A single request reaches 2^31 only with more than 32,700 KV heads.)
+inline int requests_per_launch(int hkv, int tiles)
+{
+    constexpr long long kLargestCost = cut_row_cost(16, false);
+    const long long most = 0x7FFFFFFFll / (hkv * (tiles + kLargestCost));
+    return most > 1 ? (int)(most < kMaxBatch ? most : kMaxBatch) : 1;
+}
 
 // Pages (16-token tiles) of a request of len tokens
 MKV_CUT int pages_of(int len) { return (len + kPage - 1) / kPage; }

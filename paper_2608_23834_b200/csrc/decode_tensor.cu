@@ -37,7 +37,6 @@
 
 namespace mkv {
 
-constexpr int kMaxBatch = 1024;      // requests per call
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleSlack = 8.0f;                        // the running maximum is only raised when exceeded by 2^8
@@ -1921,6 +1920,26 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
         set_last_error("mkv_decode_attention_layers: more than 65535 16-token tiles per table row (1,048,560 tokens per request)");
         return MKV_E_INVALID;
     }
+    if (const int most = requests_per_launch(p0->hkv, max_pages * p0->tiles); B > most) {      // one launch after the other, on the same workspaces
+        for (int b0 = 0; b0 < B; b0 += most) {
+            const size_t row = (size_t)b0 * max_pages, head = (size_t)b0 * p0->hkv * p0->group, vec = head * p0->d;
+            const void* qs[kMaxLayers];
+            const int32_t* bts[kMaxLayers];
+            const uint8_t* tagss[kMaxLayers];
+            float *outs[kMaxLayers], *lses[kMaxLayers];
+            for (int i = 0; i < n_layers; ++i) {
+                qs[i] = static_cast<const __nv_bfloat16*>(q[i]) + vec;
+                bts[i] = bt[i] + row;
+                tagss[i] = tags[i] + row;
+                outs[i] = out[i] + vec;
+                lses[i] = lse && lse[i] ? lse[i] + head : nullptr;
+            }
+            const int32_t rc = launch_decode_tensor_layers(pools, qs, bts, tagss, lens + b0, B - b0 < most ? B - b0 : most, max_pages,
+                                                           scale, outs, lse ? lses : nullptr, ws, n_layers, s);
+            if (rc != MKV_OK) return rc;
+        }
+        return MKV_OK;
+    }
     LayerSet<kMaxLayers> ls;
     ls.n = n_layers;
     for (int i = 0; i < n_layers; ++i) {
@@ -1971,6 +1990,16 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
     if (p->fmt == 2 && p->variant == MKV_DECODE_TMEM) {
         set_last_error("mkv_decode_attention: record format 2 is served by the tensor-core and the CUDA-core kernels");
         return MKV_E_INVALID;
+    }
+    if (const int most = requests_per_launch(p->hkv, max_pages * p->tiles); B > most) {        // one launch after the other, on the same workspace
+        for (int b0 = 0; b0 < B; b0 += most) {
+            const size_t row = (size_t)b0 * max_pages, head = (size_t)b0 * p->hkv * p->group, vec = head * p->d;
+            const int32_t rc = launch_decode_tensor_at(p, static_cast<const __nv_bfloat16*>(q) + vec, bt + row, tags + row, lens + b0,
+                                                       B - b0 < most ? B - b0 : most, max_pages, scale, out + vec, lse ? lse + head : nullptr,
+                                                       partials, tickets, max_blocks, mass ? mass + head * max_pages : nullptr, s);
+            if (rc != MKV_OK) return rc;
+        }
+        return MKV_OK;
     }
     DecodeParams prm = make_params(p, q, bt, tags, lens, B, max_pages, scale, out, lse, partials, tickets, max_blocks, mass);
     if (mass) {                          // scored variant: the default launch shapes only

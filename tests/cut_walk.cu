@@ -109,3 +109,23 @@ extern "C" int cut_walk(const int* lens, int B, int hkv, int grid, int n_layers,
     return (flat ? walk<true> : walk<false>)(lens, B, hkv, grid, n_layers, warps, per_sm, tiled, tensor_memory, idle_blocks,
                                              most_pages, blocks, why, why_size);
 }
+
+// The largest number of positions of a launch when B requests of `tiles` 16-token tiles each are decoded (negative: they do not fit)
+extern "C" long long cut_most_positions(int B, int hkv, int tiles)
+{
+    const int most = requests_per_launch(hkv, tiles);
+    long long largest = 0;
+    for (int b0 = 0; b0 < B; b0 += most) {
+        const int n = std::min(most, B - b0);
+        std::vector<int> cum(n);
+        RowSums sum = {0, 0};
+        long long exact = 0;
+        for (int b = 0; b < n; ++b) {
+            add_requests(sum, cum.data(), n, b, positions_of(tiles * kPage, hkv, cut_row_cost(16, false)), 0);
+            exact += ((long long)tiles + cut_row_cost(16, false)) * hkv;
+        }
+        if (exact != sum.positions) return -1;
+        largest = std::max(largest, exact);
+    }
+    return largest;
+}

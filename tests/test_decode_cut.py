@@ -18,13 +18,16 @@ SHAPES = {"d256": (8, 1, 0, 0, 0), "d256_two": (4, 2, 0, 0, 0), "d128_one": (16,
 
 
 @pytest.fixture(scope="module")
-def walk(tmp_path_factory):
+def lib(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("cut") / "cut_walk.so")
     subprocess.run([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-O1", "-std=c++17", "-shared", "-Xcompiler", "-fPIC",
                     "-gencode", "arch=compute_100a,code=sm_100a", "-I", os.path.join(ROOT, "paper_2608_23834_b200", "csrc"),
                     "-I", os.path.join(ROOT, "include"), os.path.join(ROOT, "tests", "cut_walk.cu"), "-o", so], check=True)
-    lib = C.CDLL(so)
+    return C.CDLL(so)
 
+
+@pytest.fixture(scope="module")
+def walk(lib):
     def run(shape, lens, hkv, n_layers=1):
         warps, per_sm, long_pages, flat, tensor_memory = SHAPES[shape]
         out = [C.c_int() for _ in range(3)]
@@ -71,3 +74,15 @@ def test_a_short_row_beside_long_ones(walk, shape):
     for _ in range(400):
         lens = [rng.randint(200, 3200) for _ in range(rng.randint(2, 7))] + [rng.randint(17, 64)]
         walk(shape, lens, rng.choice([1, 2, 4]))
+
+
+@pytest.mark.parametrize("B,hkv,tiles", [(1024, 32, 65535), (1024, 33, 65535), (300, 128, 65535), (1024, 8, 65535), (1024, 32, 256),
+                                         (1, 32700, 65535)])
+def test_positions_of_a_launch_fit_32_bits(lib, B, hkv, tiles):
+    """The largest tables that a call accepts: where the positions of all requests pass 2^31 they are decoded in several
+    launches, none of which does; smaller ones take one launch."""
+    lib.cut_most_positions.restype = C.c_longlong
+    most = lib.cut_most_positions(B, hkv, tiles)
+    assert 0 < most < 2 ** 31
+    one_launch = B * hkv * (tiles + 8 + 3 * 16)
+    assert (most == one_launch) == (one_launch < 2 ** 31)

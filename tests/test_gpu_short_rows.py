@@ -63,3 +63,42 @@ def test_a_short_row_beside_long_ones(d, hkv, group, fmt):
                     assert np.array_equal(got, first.setdefault((name, i, batch), got)), what
                     assert not _tickets(pools[i]).any(), what
     assert all(p.status() == M.OK for p in pools)
+
+
+def test_tables_of_more_positions_than_one_launch_counts():
+    """300 requests x 128 heads in tables of 65,535 pages a row may hold 2^31 pages and more: the call takes several launches
+    and gives what it gives for the same requests in a narrow table."""
+    d, hkv, B, wide = 128, 128, 300, 65535
+    rng = np.random.default_rng(5)
+    lens = torch.from_numpy(rng.integers(0, 65, B).astype(np.int32)).cuda()
+    sigma = (rng.integers(0, 2, d) * 2 - 1).astype(np.int8)
+    pools = [M.Pool(d, hkv, hkv, 8, 8, sigma, max_batch=B) for _ in range(2)]
+    gen = torch.Generator(device="cuda:0").manual_seed(5)
+    k, v = (torch.randn((8 * 16, hkv, d), generator=gen, device="cuda:0", dtype=torch.bfloat16) for _ in range(2))
+    for p in pools:
+        p.append(k, v, torch.arange(8 * 16, dtype=torch.int32, device="cuda:0"))
+        p.demote(torch.arange(8, dtype=torch.int32, device="cuda:0"), torch.arange(8, dtype=torch.int32, device="cuda:0"))
+    q = torch.randn((B, hkv, d), generator=gen, device="cuda:0", dtype=torch.bfloat16)
+    bt = torch.randint(0, 8, (B, 4), generator=gen, device="cuda:0", dtype=torch.int32)
+    tags = torch.full((B, 4), M.TAG_RECENT, dtype=torch.uint8, device="cuda:0")
+    tags[:, 0] = torch.where(lens >= 16, M.TAG_STALE, M.TAG_RECENT).to(torch.uint8)
+    results = []
+    for width in (4, wide):
+        bts, tgs = torch.full((B, width), -1, dtype=torch.int32, device="cuda:0"), torch.zeros((B, width), dtype=torch.uint8, device="cuda:0")
+        bts[:, :4], tgs[:, :4] = bt, tags
+        new = lambda: (torch.full((B, hkv, d), float("nan"), device="cuda:0"), torch.full((B, hkv), float("nan"), device="cuda:0"))
+        one, static, scored, layers = new(), new(), new(), (new(), new())
+        pools[0].decode_attention(q, bts, tgs, lens, 0.1, out=one[0], lse=one[1])
+        M.decode_attention_static(pools[0], q, bts, tgs, lens, 0.1, out=static[0], lse=static[1])
+        mass = pools[0].decode_attention_scored(q, bts, tgs, lens, 0.1, out=scored[0], lse=scored[1])[2]
+        M.decode_attention_layers(pools, [q] * 2, [bts] * 2, [tgs] * 2, lens, 0.1, [x[0] for x in layers], [x[1] for x in layers])
+        torch.cuda.synchronize()
+        assert all(p.status() == M.OK for p in pools) and not any(_tickets(p).any() for p in pools)
+        assert not mass[:, :, 4:].any()
+        results.append([*one, *static, *scored, *layers[0], *layers[1], mass[:, :, :4].clone()])
+        del mass, bts, tgs
+    for narrow, got in zip(*results):
+        same = torch.isneginf(narrow)
+        assert torch.equal(same, torch.isneginf(got))
+        # sums of at most 64 terms in fp32, cut over other blocks: a few 2^-24 of the largest term
+        assert (got[~same] - narrow[~same]).abs().max() < 1e-5

@@ -179,8 +179,9 @@ MKV_CUT void build_partition(Partition* pt, const int* cum, const int* lens, int
                    (long long)pages * rows < 2ll * straddle * grid * grid) ? 1 : 0;
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_position(r) / W);
-        // every row must end up with at least one block and with no more blocks than pages (a row's share also counts
-        // row_cost; a block without a page would never arrive at the row's merge), otherwise the linear cut is used
+        // every row must end up with at least one block, otherwise the linear cut is used.  (A row's share also counts row_cost, so
+        // that a row of a few pages may get more blocks than pages; those without a page do nothing, see blocks_of_row.  The linear cut for
+        // such batches: 2 x 32 and 2,000 to 8,000 tokens, d 256, 1 to 4 heads, 14.2 to 19.0 us a step, so 13.9 to 18.5.)
         int bad = 0;
         const float scale = (float)grid / (float)W;
         for (int r = lane; r < rows; r += kCutLanes) {
@@ -188,7 +189,7 @@ MKV_CUT void build_partition(Partition* pt, const int* cum, const int* lens, int
             const int first = cum[b] + (r - b * hkv) * len;
             const int c0 = (int)((float)first * scale + 0.5f), c1 = r + 1 == rows ? grid : (int)((float)(first + len) * scale + 0.5f);
             pt->base[r] = c0;
-            if (n > 0 && (c1 <= c0 || c1 - c0 > n)) bad = 1;
+            if (n > 0 && c1 <= c0) bad = 1;
             if (c0 <= me && me < c1) {                          // the one lane that holds this block's row
                 const Cut row = cut_row(n, c1 - c0);
                 const int j = me - c0;
@@ -289,7 +290,7 @@ MKV_CUT void blocks_of_row(const Partition* pt, int W, int layer, int r, int fir
         c1 = cut_block_of(pt->flat, w0 + row_end - 1);
     } else if (pt->aligned) {
         c0 = pt->base[r];
-        c1 = pt->base[r + 1] - 1;
+        c1 = c0 + smaller(pt->base[r + 1] - c0, row_end - first_page) - 1;      // no more blocks than pages
     } else {
         c0 = cut_block_of(pt->cut, first_page);
         c1 = cut_block_of(pt->cut, row_end - 1);

@@ -224,9 +224,8 @@ MKV_CUT void build_partition(Partition* pt, const int* cum, const int* lens, int
 }
 
 // Block `me` of the flat cut of n_layers layers: its layers, and the request of its first triple.  Warp 0, all lanes.
-MKV_CUT void build_flat_partition(Partition* pt, const int* cum, int B, int n_layers, int grid, int pages, int min_pages, int me, int lane)
+MKV_CUT void build_flat_partition(Partition* pt, const int* cum, int W, int B, int n_layers, int grid, int pages, int min_pages, int me, int lane)
 {
-    const int W = cum[B];
     const Cut cut = make_cut((long long)W * n_layers, (long long)pages * n_layers, grid, min_pages);
     int first = 0, end = 0, b = 0;
     if (me < cut.blocks) {
@@ -248,9 +247,9 @@ MKV_CUT void build_flat_partition(Partition* pt, const int* cum, int B, int n_la
 // Range [start, end) of block `me` of the flat cut in layer `layer`
 MKV_CUT void range_in_layer(const Partition* pt, int W, int layer, int me, int& start, int& end)
 {
-    const long long w0 = (long long)layer * W, s = cut_start(pt->flat, me) - w0, e = cut_start(pt->flat, me + 1) - w0;
-    start = (int)(s > 0 ? s : 0);
-    end = (int)(e < W ? e : W);
+    const long long w0 = (long long)layer * W;
+    start = (int)max(cut_start(pt->flat, me) - w0, 0ll);
+    end = (int)min(cut_start(pt->flat, me + 1) - w0, (long long)W);
 }
 
 // A block's part of a row

@@ -1049,7 +1049,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         const int pages = sum.positions - sum.requests * hkv * ROW_COST;
         if constexpr (!FLAT || TILED)
             build_partition(pt, cum, lens_s, P0.B, hkv, gridDim.x, pages, ROW_COST, MIN_PAGES, cut_straddle(NW), blockIdx.x, lane);
-        if constexpr (FLAT) build_flat_partition(pt, cum, P0.B, n_layers, gridDim.x, pages, MIN_PAGES, blockIdx.x, lane);
+        if constexpr (FLAT) build_flat_partition(pt, cum, sum.positions, P0.B, n_layers, gridDim.x, pages, MIN_PAGES, blockIdx.x, lane);
     }
     __syncthreads();
     int my_start = 0, my_end = 0;                          // more blocks than work: an empty range

@@ -36,7 +36,7 @@ int walk(const int* lens, int B, int hkv, int grid, int n_layers, int warps, int
         int layer_first = 0, layer_end = n_layers, scanned = 0;
         if (!FLAT || tiled) build_partition(&pt, cum.data(), lens, B, hkv, grid, pages, cost, least, straddle, me, 0);
         if (FLAT) {
-            build_flat_partition(&pt, cum.data(), B, n_layers, grid, pages, least, me, 0);
+            build_flat_partition(&pt, cum.data(), W, B, n_layers, grid, pages, least, me, 0);
             layer_first = pt.first_layer, layer_end = pt.end_layer;
         }
         *blocks = FLAT ? pt.flat.blocks : pt.cut.blocks;

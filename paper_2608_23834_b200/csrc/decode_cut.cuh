@@ -1,6 +1,6 @@
-// Cut of the decode scan's work into one contiguous range per block: which pages a block scans, which blocks hold a part of
-// a row, and where their partials lie.  Integer arithmetic only.  The scan kernels run it on the device; it also compiles for the host,
-// where a warp is one lane, so that every block of a grid can be walked without a GPU.
+// Cut of the decode scan's work into one contiguous range per block: which pages a block scans, which blocks hold a part
+// of a row, and where their partials lie.  The scan kernels run it on the device; it also compiles for the host, where a
+// warp is one lane, so that every block of a grid can be walked without a GPU.
 #pragma once
 #include "mkv_internal.cuh"
 
@@ -8,25 +8,28 @@ namespace mkv {
 
 // Work = (request, KV head, page) triples in row-major order; cum[b] = position of the first triple of
 // request b.  A row of n pages takes row_cost + n positions: opening, reducing and storing a row (or a block's part of it)
-// costs a block as much time as row_cost pages, so that a block with many short rows gets fewer pages.  (64 requests of 1,024 to
-// 131,072 tokens, 8 heads: the blocks with the shortest requests took 520 us against 406 on average; 524 -> 480 us a step with
-// 32, the same with 48, 503 with 16.  16 layers x 4 x 700..3,001 tokens, d 256: 64.0 -> 60 with 16, 62 with 32, 66 with 48.
-// 16 layers x 8 x 512..16,384, one block of 16 warps per SM: 151 -> 139 with 32, 134 with 48, 136 with 64.)  Two ways to cut it into one contiguous range per block:
+// costs a block as much time as row_cost pages, so that a block with many short rows gets fewer pages.  (us a step with
+// cost 0 and with row_cost: 64 requests of 1,024 to 131,072 tokens, 8 heads 524 / 480, as with 48, 503 with 16; 16 layers x
+// 4 x 700..3,001 tokens, d 256 64.0 / 60 with 16, 62 with 32, 66 with 48; 16 layers x 8 x 512..16,384, one block of 16
+// warps per SM 151 / 134 with 48, 139 with 32, 136 with 64.)  A block whose range lies inside a row's cost gets no page.
+// Where rows are few and short that is no loss: they are split over fewer blocks, whose partials take longer to merge than
+// the pages to scan.  (With the cost bounded so that every block gets pages: 4 layers x 1 x 700, d 256 13.5 -> 16.9 us;
+// 8 x 400, d 256 15.3 -> 17.6, d 128 13.8 -> 17.1; 16 layers x 1 x 500, d 128 9.9 -> 12.7; 16 x 64..8,000 25.0 -> 25.8.)
+//
+// Two ways to cut a layer into one contiguous range per block:
 //   row-aligned (few rows: B * hkv <= grid / 4): every row gets a whole number of blocks in proportion
-//     to its pages (cumulative rounding), so that no block straddles two rows and pays the per-row set-up
+//     to its positions (cumulative rounding), so that no block straddles two rows and pays the per-row set-up
 //     and reduction twice;
 //   linear (many rows): grid equal ranges that may cross row boundaries.
 constexpr int kMaxAlignedRows = kMaxCtas / 4;
 constexpr int kMaxBatch = 1024;         // requests per call
 
-//   flat (several layers): a linear cut of all layers' triples, the layers laid end to end.
+// and one for several layers: flat, a linear cut of all layers' triples, the layers laid end to end.
 //
 // Every block works this out for itself before its first page can be asked for, so the arithmetic is kept short: one
-// 32-bit division per cut (quotient and remainder; block c starts at quo c + min(c, rem)), and warp 0 leaves the
-// block's own range and request in shared memory.  (With W c / blocks in 64 bits, a binary search for the row, a serial one for the
-// request and the strides that page_at replaces, the time up to a block's first page was 11,600 cycles at 8 x 16,384 tokens, d 128,
-// and 18,900 in the flat cut of 16 layers x 16 rows, d 256; it is 8,400 and 10,100: 36.5 -> 34.3 and 75.6 -> 66.3 us a step, and
-// 650 -> 552 for 16 layers of long pages, where every tile asks which warp's run it opens.)
+// 32-bit division per cut (quotient and remainder; block c starts at quo c + min(c, rem)), and warp 0 leaves the block's
+// own range and request in shared memory.  (Time up to a block's first page with 64-bit divisions and serial searches, and
+// so: 8 x 16,384 tokens, d 128 11,600 / 8,400 cycles; flat cut of 16 layers x 16 rows, d 256 18,900 / 10,100.)
 struct Cut {
     long long quo;
     int rem, blocks;                    // blocks that get work (0: none)
@@ -73,8 +76,8 @@ MKV_CUT constexpr int cut_row_cost(int warps, bool long_pages) { return long_pag
 MKV_CUT constexpr int cut_min_pages(int warps, int per_sm) { return warps * per_sm; }
 MKV_CUT constexpr int cut_straddle(int warps) { return 4 * warps; }
 
-// Positions are counted in 32 bits: requests that one launch may take where a table row has room for `tiles` 16-token tiles, so that
-// its positions stay below 2^31.  (A single request reaches 2^31 only with more than 32,700 KV heads.)
+// Positions are counted in 32 bits: requests that one launch may take where a table row has room for `tiles` 16-token
+// tiles, so that its positions stay below 2^31.  (A single request reaches that only with more than 32,700 KV heads.)
 inline int requests_per_launch(int hkv, int tiles)
 {
     constexpr long long kLargestCost = cut_row_cost(16, false);
@@ -179,9 +182,10 @@ MKV_CUT void build_partition(Partition* pt, const int* cum, const int* lens, int
                    (long long)pages * rows < 2ll * straddle * grid * grid) ? 1 : 0;
     if (aligned) {
         // block boundaries at the rounded cumulative share of the rows: base[r] = round(grid * first_position(r) / W);
-        // every row must end up with at least one block, otherwise the linear cut is used.  (A row's share also counts row_cost, so
-        // that a row of a few pages may get more blocks than pages; those without a page do nothing, see blocks_of_row.  The linear cut for
-        // such batches: 2 x 32 and 2,000 to 8,000 tokens, d 256, 1 to 4 heads, 14.2 to 19.0 us a step, so 13.9 to 18.5.)
+        // every row must end up with at least one block, otherwise the linear cut is used.  (A row's share also counts
+        // row_cost, so that a row of a few pages may get more blocks than pages; those without a page do nothing, see
+        // blocks_of_row.  With the linear cut for such batches, and so: 2 requests of 32 and 2,000 to 8,000 tokens, d 256,
+        // 1 to 4 heads 14.2 .. 19.0 / 13.9 .. 18.5 us a step.)
         int bad = 0;
         const float scale = (float)grid / (float)W;
         for (int r = lane; r < rows; r += kCutLanes) {
@@ -332,9 +336,7 @@ MKV_CUT bool opens_warp_run(const Partition* pt, int r, int row_start, int row_e
 // Pages of a row are visited in an order that gives every contiguous range of positions the row's FP8 and TQ3 pages in
 // their overall proportion (spans of either format are contiguous), so that equal ranges cost equal time.  The row is cut into 32
 // strips of equal length (the first n % 32 are one page longer); position x is page x / 32 of strip x % 32, the strips
-// in bit-reversed order, and the pages that the longer strips have more come last.  A bijection without a division.  (Before: x
-// times a stride near 0.618 n and coprime to n, modulo n; finding it, seventeen remainders per try, kept all
-// warps waiting for 1,500 cycles.)
+// in bit-reversed order, and the pages that the longer strips have more come last.  A bijection without a division.
 MKV_CUT int page_at(int x, int n)
 {
     const int len = n >> 5, longer = n & 31, at = x >> 5;

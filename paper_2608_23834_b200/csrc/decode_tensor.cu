@@ -887,7 +887,7 @@ __device__ __forceinline__ void fp8_page(WarpAcc<D / 16>& acc, uint32_t kaddr, u
 // (one trip to L2: both are loaded together and kept in shared memory); a thread owns float4 groups (one channel,
 // four heads) of the [channel][8 heads] tile.  With twice as many threads as groups (16 warps at d = 128) every
 // other part goes to the second half of the threads.  KP loads per thread are in flight, issued before the weights
-// are worked out: as many as the launch shape has registers for, and no more than rows of few parts can use.
+// are worked out.
 template <int D, int NT, int KPMAX>
 __device__ __forceinline__ void merge_row(const DecodeParams& P, int first_slot, int even_base, int n_parts,
                                           float* buf, int b, int h)
@@ -995,7 +995,8 @@ template <int D, int NW, int NSTAGE, int MINB, bool SCORED, bool TILED, int MAXL
 __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const LayerSet<MAXL> LS)
 {
     const DecodeParams& P0 = LS.layer[0];    // requests and geometry are common to all layers
-    // 16-byte loads that a thread of the merge keeps in flight, within the registers of the launch shape
+    // 16-byte loads that a thread of the merge keeps in flight.  (d 256: 20 and 40 are alike also for rows of many parts, 37:
+    // 1 x 59,008 tokens 31.1 / 30.6 us a call, 1 x 131,072 53.4 / 53.1; 74: 33.2 / 33.1; 40 cost registers elsewhere.)
     constexpr int MERGE_LOADS = NW * MINB <= 8 ? 20 : 16;
     constexpr int ROW_COST = cut_row_cost(NW, TILED), MIN_PAGES = cut_min_pages(NW, MINB);
     using G = Geo<D, NW, NSTAGE, TILED>;     // pages of several tiles: short rounds leave room for the parked rows
@@ -1172,7 +1173,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
         const size_t tq3_page = (size_t)P.tiles * TQ3_TILE + TQ3_META;
 
         // Table entries of up to G::ROUND of the warp's pages are compacted into two id lists, one per
-        // format (entry i of a 32-page chunk is read by lane i, all chunks before the first is looked at; ballots give the positions).
+        // format (entry i of a 32-page chunk is read by lane i, all chunks before the first is looked at; ballots give the
+        // positions).
         // Returns how many of the warp's pages (from `first` on) the lists cover.  Long pages in the flat cut: a Stale
         // tile that opens a warp's run of the per-layer cut is marked (kOpens); the scan leaves the page there, and
         // a round ends at the last such tile, so that code sums are gathered over the same runs of tiles as there
@@ -1612,7 +1614,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) decode_tensor_kernel(const Laye
                 P.lse[(size_t)b * hq + h * GQ + tid] = l > 0.f ? (M + log2f(l)) * kLn2 : -CUDART_INF_F;
             }
         } else {
-            float* slot = P.partials + (size_t)partial_slot(blockIdx.x, pos, my_start) * (8 * D + 16);    // (m, l, O) of this block for the row
+            // partial (m, l, O) of this block for the row
+            float* slot = P.partials + (size_t)partial_slot(blockIdx.x, pos, my_start) * (8 * D + 16);
 #pragma unroll
             for (int k = 0; k < PER_THREAD; ++k) {
                 const int i = tid + k * NW * 32, e4 = SPLIT ? 2 * i : i;
@@ -1790,9 +1793,9 @@ int decode_tensor_partial_floats(int d) { return 8 * d + 16; }
 // absolute origin; with the row's log-sum-exp it becomes q_p = 2^(that - lse2), and q~_p = q_p / sum q_p
 // (Eq. score-global-weight and the normalisation over page-addressable mass that follows it).
 // One block per (query head, request); entries beyond the request's pages are set to zero.  The first 4,096 pages of a row
-// are loaded at once and stay in registers between the two steps; what is beyond is read twice.  (Bound by the trips to memory: four rows of
-// 2,501 pages x 24 heads with one load at a time and a second reading, and the score update behind it, took 4 us longer, 69.6 -> 65 us for
-// the whole scored step.)
+// are loaded at once and stay in registers between the two steps; what is beyond is read twice.  (Bound by the trips to
+// memory: with one load at a time and a second reading, the score update behind it likewise, a scored step over four rows
+// of 2,501 pages x 24 heads took 69.6 us, so 65.)
 __global__ void __launch_bounds__(512) page_mass_finish_kernel(float* mass, const float* lse, const int32_t* lens,
                                                               int hq, int max_pages, int page_tokens)
 {
@@ -1900,7 +1903,8 @@ static DecodeParams make_params(mkv_pool* p, const void* q, const int32_t* bt, c
 // Two blocks of half the warps per SM instead of one: the set-up, reduction and merge of one overlap the pages of the
 // other, which pays the more rows a block meets (d 128, 8 x 4 heads: 64 ragged requests 632 -> 579 us, 8 x 4,096 tokens
 // 30.7 -> 23.6 us).  At d = 256 a merge by four warps costs more, and few rows have many partials: from 32 rows (8 x
-// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows of 8,000 and 30,000: 20.9 -> 24.4, 47.6 -> 49.4).  Partial areas for one block per SM only take one.
+// 32,768 tokens, 4 heads: 78 -> 70 us; 16 rows of 8,000 and 30,000: 20.9 -> 24.4, 47.6 -> 49.4).  Partial areas for one
+// block per SM only take one.
 static bool two_blocks(const mkv_pool* p, int B, int max_blocks)
 {
     return max_blocks >= 2 * p->dev.sm_count && (p->d == 128 || B * p->hkv >= 32);
@@ -1920,7 +1924,8 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
         set_last_error("mkv_decode_attention_layers: more than 65535 16-token tiles per table row (1,048,560 tokens per request)");
         return MKV_E_INVALID;
     }
-    if (const int most = requests_per_launch(p0->hkv, max_pages * p0->tiles); B > most) {      // one launch after the other, on the same workspaces
+    // more positions than a launch counts: one launch after the other, on the same workspaces
+    if (const int most = requests_per_launch(p0->hkv, max_pages * p0->tiles); B > most) {
         for (int b0 = 0; b0 < B; b0 += most) {
             const size_t row = (size_t)b0 * max_pages, head = (size_t)b0 * p0->hkv * p0->group, vec = head * p0->d;
             const void* qs[kMaxLayers];
@@ -1954,12 +1959,13 @@ int32_t launch_decode_tensor_layers(mkv_pool* const* pools, const void* const* q
     if (p0->tiles > 1)
         return p0->d == 128 ? run_tensor<128, 12, 4, 1, false, true, kMaxLayers>(p0, ls, s)
                             : run_tensor<256, 8, 4, 1, false, true, kMaxLayers>(p0, ls, s);
-    // Two blocks of half the warps per SM from 64 rows on: one's set-up, reduction and merge overlap the other's pages, but few
-    // rows have partials that four warps take longer to merge.  d 256, us with one block and with two: 16 layers x 2 x 59,008
-    // tokens 540 / 510, 4 x 4 x 20,000 (64 rows) 109.0 / 102.7, 16 x 1 x 30,000 (64) 155 / 143.5, 16 x 1 x 4,000 (64) both 33.6, 4 x 1 x
-    // 3,000 (16) 17.7 / 21.2; d 128, eight query heads: 16 x 8 x 512..16,384 (512) 132 / 127.6, 16 x 2 x 2,000 (128) 24.5 / 23.3, 4 x 2 x
-    // 8,000 (8) 15.1 / 17.1.  Up to four query heads at d = 128 two blocks are better at any size.  (Long pages: 16 x 1 x 4,000
-    // 45.8 / 43.0, but 16 x 2 x 59,008 552 / 592: two blocks leave room for rounds of 32 tiles only.)
+    // Two blocks of half the warps per SM from 64 rows on: one's set-up, reduction and merge overlap the other's pages, but
+    // few rows have partials that four warps take longer to merge.  us with one block and with two (layers x requests x
+    // tokens): d 256, 16 x 2 x 59,008 540 / 510, 4 x 4 x 20,000 (64 rows) 109.0 / 102.7, 16 x 1 x 30,000 (64) 155 / 143.5,
+    // 16 x 1 x 4,000 (64) both 33.6, 4 x 1 x 3,000 (16) 17.7 / 21.2; d 128, eight query heads, 16 x 8 x 512..16,384 (512)
+    // 132 / 127.6, 16 x 2 x 2,000 (128) 24.5 / 23.3, 4 x 2 x 8,000 (8) 15.1 / 17.1.  Up to four query heads at d = 128 two
+    // blocks are better at any size.  (Long pages: 16 x 1 x 4,000 45.8 / 43.0, but 16 x 2 x 59,008 552 / 592: two blocks
+    // leave room for rounds of 32 tiles only.)
     if (n_layers >= kMinFlatLayers) {
         const bool two = n_layers * B * p0->hkv >= kRowsOfTwoBlocks;
         if (p0->d == 256)
@@ -1979,7 +1985,7 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
                                 float* partials, uint32_t* tickets, int max_blocks, float* mass, cudaStream_t s)
 {
     if (B > kMaxBatch) return MKV_E_INVALID;
-    if ((int64_t)max_pages * p->tiles > 65535) {   // the strided order multiplies two 16-token tile indices in 32 bits
+    if ((int64_t)max_pages * p->tiles > 65535) {   // tile counts: small_div takes up to 2^20, the lists of long pages 16 bits
         set_last_error("mkv_decode_attention: more than 65535 16-token tiles per table row (1,048,560 tokens per request)");
         return MKV_E_INVALID;
     }
@@ -1991,7 +1997,8 @@ int32_t launch_decode_tensor_at(mkv_pool* p, const void* q, const int32_t* bt, c
         set_last_error("mkv_decode_attention: record format 2 is served by the tensor-core and the CUDA-core kernels");
         return MKV_E_INVALID;
     }
-    if (const int most = requests_per_launch(p->hkv, max_pages * p->tiles); B > most) {        // one launch after the other, on the same workspace
+    // more positions than a launch counts: one launch after the other, on the same workspace
+    if (const int most = requests_per_launch(p->hkv, max_pages * p->tiles); B > most) {
         for (int b0 = 0; b0 < B; b0 += most) {
             const size_t row = (size_t)b0 * max_pages, head = (size_t)b0 * p->hkv * p->group, vec = head * p->d;
             const int32_t rc = launch_decode_tensor_at(p, static_cast<const __nv_bfloat16*>(q) + vec, bt + row, tags + row, lens + b0,

@@ -2,7 +2,7 @@
 // lifecycle_kernels.cu).
 //
 // The encoder is defined as a sequence of fp32 operations, and the records are those bit for bit; what changes is
-// how the same numbers are reached (per page and head at d = 256, 8,760 -> 3,870 warp instructions):
+// how the same numbers are reached (per page and head at d = 256, 8,760 -> 3,730 warp instructions):
 //   * The Hadamard transform of an e4m3 vector is exact in fp32 as long as its coordinates are not huge: they are
 //     multiples of 2^-9, and with |x|^2 < kExactNorm2 = 2^22 (checked on the norm that the encoder needs anyway) a signed
 //     sum of n <= 256 of them is at most sqrt(n) |x| <= 2^15, that is 2^24 units of 2^-9: every partial sum is an integer

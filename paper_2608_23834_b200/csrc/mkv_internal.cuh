@@ -109,13 +109,17 @@ namespace mkv {
 // memory it reads is not read-only for its lifetime: no const __restrict__ and no __ldg on anything that an earlier
 // kernel may have written (arenas, ids, entries, slots, page scales).  The CUDA-core and tensor-memory variants of the
 // scan are ordinary launches.
-// Most kernels let the next one start at once (pdl_begin).  Demote and Promote do so when their records are written: blocks placed while a
-// grid of about one block per SM still runs lie unevenly (Demote of 12 pages of 1,792 tokens, d 256, 2 heads, back to back 29.5 -> 33
-// us, 120 pages of 16 tokens 8.4 -> 9.2; Promote of 700 pages, d 128, 8 heads, 12.8 us so and 11.2 with the late signal).  The scan does so when its blocks have done all but the merges:
-// blocks of a Demote or Promote that come while it still holds most SMs crowd on the first SMs that it leaves, up to four on one
-// SM, and wait there (one page between decode scans, d 256: Demote 40 us, ordinary launch 20).  Behind the late
-// signal they find the SMs free and their launch is hidden: Promote of 1,023 pages back to back 16.7 -> 14.1 us, 300 pages 9.2 -> 7.5,
-// Demote of 20 pages 8.4 -> 5.8, a page of each between scans 1.5 to 2.5 us less, steps of a small batch 1.8 to 2.8.
+// Most kernels let the next one start at once (pdl_begin).  Demote and Promote do so when their records are written:
+// blocks placed while a grid of about one block per SM still runs lie unevenly (us with the signal at once, and so, back to
+// back: Demote of 12 pages of 1,792 tokens, d 256, 2 heads 33 / 29.5, of 120 pages of 16 tokens 9.2 / 8.4; Promote of 700
+// pages, d 128, 8 heads 12.8 / 11.2).  A block of the scan does so when the last partial of its range is stored, before it
+// may merge a row; a block whose range ends with a whole row, or inside what the next row costs in the cut, does so by
+// ending (the signal there, too: 8 x 400 tokens, d 256 15.3 -> 15.7 us, 4 layers x 1 x 700 13.3 -> 13.5).  Blocks of a
+// Demote or Promote that come while the scan still holds most SMs crowd on the first ones that it leaves, up to four on one
+// SM, and wait there (one page between decode scans, d 256: Demote 40 us, as an ordinary launch 20).  Behind the late
+// signal they find the SMs free and their launch is hidden (as ordinary launches, and so: Promote of 1,023 pages back to
+// back 18.6 / 16.7 us, 300 pages 9.2 / 7.5, Demote of 20 pages 8.4 / 5.8; a page of each between scans 1.5 to 2.5 us less,
+// steps of a small batch 1.8 to 2.8).
 __device__ __forceinline__ void pdl_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin()

@@ -11,7 +11,7 @@ from conftest import ROOT
 CSRC = os.path.join(ROOT, "paper_2608_23834_b200", "csrc")
 
 
-@pytest.mark.parametrize("name", ["lifecycle_kernels.cu", "demote_warp.cuh", "promote_warp.cuh", "decode_tensor.cu"])
+@pytest.mark.parametrize("name", ["lifecycle_kernels.cu", "demote_warp.cuh", "promote_warp.cuh", "decode_tensor.cu", "decode_cut.cuh"])
 def test_no_read_only_loads_in_kernels_that_start_early(name):
     with open(os.path.join(CSRC, name)) as f:
         code = re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
